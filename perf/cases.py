@@ -260,3 +260,67 @@ def tolerance(case):
     if case["keep"] >= 1.0 and case["kind"] != "pruned":
         return {"rel": 4e-5, "max": 4e-4}
     return {"rel": 1e-2, "max": 0.1, "differ": 0.01}
+
+
+# ---- the same in 64 bits, with plain torch -----------------------------------------------------------------------------
+def _stored(weights, wtype):
+    """The values that a stored matrix and its scales stand for."""
+    q, scale = weights
+    if wtype != "int4":
+        return q.double()
+    codes = torch.stack((q & 15, q >> 4), dim=2).view(q.shape[0], -1).double() - 8
+    return codes * scale.t().double().repeat_interleave(128, dim=1)
+
+
+def _kept(c, v, k):
+    """The 0/1 mask of the k largest keys of each row (cold caches: no column is resident yet), the lower column first among
+    equals, and whether another summation order of v could give another mask."""
+    key = v.float().abs()
+    if c["budget"] is not None:
+        key = key * torch.tensor(c["gamma"], dtype=torch.float32, device=key.device)
+    order = torch.argsort(key, dim=-1, descending=True, stable=True)
+    mask = torch.zeros_like(v).scatter_(-1, order[..., :k], 1.0)
+    if k == v.shape[-1]:
+        return mask, False
+    edge = key.gather(-1, order[..., k - 1:k + 1]).double()
+    size = torch.maximum(edge[..., 0], key.double().square().mean(-1).sqrt())
+    return mask, bool((edge[..., 0] - edge[..., 1] < (1e-4 if c["batch"] > 2 else 1e-5) * size).any())
+
+
+def exact(case, seed):
+    """What the first pass of a new state returns.  None for an output that hangs on the ranking of two columns whose keys are
+    equal to within the rounding of their sums, or for the case where that is every output."""
+    c = case
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    d_model, d_ff = c["d_model"], c["d_ff"]
+    stored = []
+    for _ in range(c["layers"]):
+        shapes = ((d_ff, d_model), (d_ff, d_model), (d_ff, d_model) if c["kind"] == "pruned" else (d_model, d_ff))
+        stored.append([_weights(gen, c["wtype"], *s) for s in shapes])
+    x = _tokens(c, gen)[0].double()
+    silu = torch.nn.functional.silu
+    near = False
+    for n, layer in enumerate(stored):
+        if n:
+            r = x + y
+            x = r / r.square().mean(-1, keepdim=True).sqrt()
+        gate, up, down = (_stored(m, c["wtype"]) for m in layer)
+        if c["kind"] == "pruned":
+            p = silu(x @ gate.t())
+            mask_h, tie_h = _kept(c, p, _keep(c, d_ff))
+            h = p * (x @ up.t()) * mask_h
+            y = h @ down
+        else:
+            mask_x, tie_x = _kept(c, x, _keep(c, d_model))
+            near = near or (n > 0 and tie_x)                  # (the first block's x is given: its mask is exact)
+            h = (x * mask_x) @ up.t() * silu((x * mask_x) @ gate.t())
+            mask_h, tie_h = _kept(c, h, _keep(c, d_ff))
+            y = (h * mask_h) @ down.t()
+        near = near or tie_h
+    if c["kind"] == "stack":
+        r = x + y
+        return None if near else {"y": r / r.square().mean(-1, keepdim=True).sqrt()}
+    if near:
+        return None if c["kind"] == "pruned" else {"y": None, "h": h}        # (there h itself is masked)
+    return {"y": y, "h": h}
