@@ -1,7 +1,7 @@
 // The select that builds a top-k bit mask (Sec. 3.1, Eq. 7-8; the cache-aware ranking of Eq. 10), as
 // device functions for CTAs of 1024 threads: the one-histogram select over the top 15 bits of the
 // rank keys with an exact ranking inside the threshold's bin, the general radix select for heavy
-// ties (also the cache update's victim search), and the residual scale of a chained layer.  Used by
+// ties, and the residual scale of a chained layer.  Used by
 // the stand-alone select kernels and by the product kernels that select for themselves.
 #pragma once
 
@@ -93,9 +93,8 @@ __device__ __forceinline__ void find_bin(TkShared &s, int krem)
 //
 // Radix select from the top bit down, up to 11 bits per pass: a shared-memory histogram of the
 // current digit over the keys that match the prefix found so far, then a suffix scan over the
-// bins (two per thread) to find the bin holding the k-th key.  The four smallest digits, which
-// are by far the most frequent ones when the keys are ages of cache lines, are counted in
-// registers instead of with contended atomics.
+// bins (two per thread) to find the bin holding the k-th key.  The four smallest digits are
+// counted in registers instead of with contended atomics (rows of zeros and denormals).
 __device__ void block_radix_select(const uint32_t *keys, int d, uint32_t keymask, int top_bit, int k,
                                    TkShared &s, uint32_t &T, int &quota, int &n_eq)
 {

@@ -100,120 +100,232 @@ select_fine_coarse_kernel(const float *__restrict__ x, const uint16_t *__restric
 
 // ---------------------------------------------------------------------------------------
 // cache_update_kernel: c' = cache_update(c, m) of Algorithm 1 with the LRU policy of Sec. 5.1
-// (or LFU when use counters are given), from the mask bits and the state alone.  One CTA; keys[] (dynamic shared memory, d words)
-// holds (resident flag << 31) | eviction key, the eviction key being the age of the column's
-// last use for columns that may be evicted (resident and outside the mask) and 0 otherwise.
+// (or LFU when use counters are given), from the mask bits and the state alone.  One CTA: it runs
+// beside a product that fills the other SMs, and a chain of exchanges between CTAs would cost
+// more than the few thousand columns an SM has to look at.
+// A warp owns NB consecutive blocks of 128 columns, a lane four consecutive columns of each (one
+// 16-byte load and one 16-byte store), and everything in between stays in registers.  The eviction
+// key of a column that may be evicted (resident and outside the mask) is the age of its last use
+// (LFU: t + 1 - uses), of any other column 0.
+// Bound by the SM's issue rate and its trips through shared memory.  Alone, LRU, after 38 updates:
+// 7.9 us at d = 17920 (load 1.5, histogram 2.1 + search 0.7, ties 1.2, stamps 2.1), 4.4 us at 5120;
+// one column per lane swept four times through shared memory with 4-byte stores took 14.4 and 6.6 us.
 // ---------------------------------------------------------------------------------------
+constexpr int CU_SPREAD = 8;                            // copies of the counters of the small digits,
+constexpr int CU_SMALL = 256;                           // which nearly all keys have: ages of a few updates
+
+template <int NB, bool LFU>
 __global__ void __launch_bounds__(TK_THREADS, 1)
 cache_update_kernel(const uint32_t *__restrict__ mask_bits, int d, int32_t *stamp, int32_t *count, int32_t *meta,
                     int capacity, unsigned long long *tr)
 {
-    DIP_TRACE_MIN(tr, 0);
-    DIP_TRACE_MIN(tr, 1);
-    extern __shared__ uint32_t keys[];
     __shared__ TkShared s;
+    __shared__ __align__(16) unsigned int small[CU_SMALL * CU_SPREAD];
+    static_assert(CU_SMALL * CU_SPREAD == 2 * TK_THREADS && RADIX_BINS == 2 * TK_THREADS, "two counters per thread");
+    DIP_TRACE_MIN(tr, 0);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const auto clear = [&]() {
+        s.hist[2 * tid] = s.hist[2 * tid + 1] = 0;
+        small[2 * tid] = small[2 * tid + 1] = 0;
+    };
+    clear();
+    dip_grid_dependency_wait();
+    DIP_TRACE_MIN(tr, 1);
+    dip_launch_dependents();
     const int n_res = meta[0];
     const int t_now = meta[1] + 1;
-    const int span = ((d + TK_THREADS - 1) / TK_THREADS) * 32;
-    const int base = warp * span;
-    const unsigned lt = lanemask_lt();
+    const int col0 = warp * (NB * 128) + lane * 4;      // this lane's first column; block i is 128 i further
 
-    int hits = 0, misses = 0;
-    constexpr int CU = 8;             // iterations whose loads are issued together
-    for (int it0 = 0; it0 < span && base + it0 < d; it0 += 32 * CU) {
-        unsigned mwv[CU];
-        int stv[CU], cnv[CU];
+    // ---- the state and the mask.  kv: LRU: t_now - stamp (the stamp can be had back), LFU: t_now - uses ----
+    uint32_t kv[NB][4];
+    uint32_t keep = 0u, res = 0u;                       // nibble i: block i's four columns in the mask / resident
+    {
+        int st[NB][4], cn[LFU ? NB : 1][4];
+        uint32_t word[NB];
 #pragma unroll
-        for (int u = 0; u < CU; ++u) {
-            const int it = it0 + 32 * u, e = base + it + lane;
-            const bool in_span = it < span && base + it < d;
-            mwv[u] = in_span ? mask_bits[(base + it) >> 5] : 0u;
-            stv[u] = in_span && e < d ? stamp[e] : -1;
-            cnv[u] = count && in_span && e < d ? count[e] : 0;
+        for (int i = 0; i < NB; ++i) {
+            const int c = col0 + 128 * i;
+            word[i] = 0u;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                st[i][e] = -1;
+                if (LFU) cn[i][e] = 0;
+            }
+            if (c < d) word[i] = mask_bits[c >> 5];
+            if (c + 4 <= d) {
+                const int4 q = *reinterpret_cast<const int4 *>(stamp + c);
+                st[i][0] = q.x; st[i][1] = q.y; st[i][2] = q.z; st[i][3] = q.w;
+                if (LFU) {
+                    const int4 n = *reinterpret_cast<const int4 *>(count + c);
+                    cn[i][0] = n.x; cn[i][1] = n.y; cn[i][2] = n.z; cn[i][3] = n.w;
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (c + e < d) {
+                        st[i][e] = stamp[c + e];
+                        if (LFU) cn[i][e] = count[c + e];
+                    }
+            }
         }
 #pragma unroll
-        for (int u = 0; u < CU; ++u) {
-            const int it = it0 + 32 * u, e = base + it + lane;
-            if (!(it < span && base + it < d)) break;          // uniform over the warp
-            const bool valid = e < d;
-            const unsigned mw = mwv[u];
-            const bool keep = valid && ((mw >> lane) & 1u);
-            const int st = stv[u];
-            const bool res = st >= 0;
-            // LRU: age of the last use.  LFU (count given): t + 1 - uses, so that the most rarely
-            // used column has the largest key (a column is used at most once per update: uses <= t)
-            uint32_t ek = 0u;
-            if (res && !keep) ek = count ? (uint32_t)(t_now - cnv[u]) : (uint32_t)(t_now - st);
-            if (valid) keys[e] = (res ? 0x80000000u : 0u) | ek;
-            const int hw = __popc(__ballot_sync(0xffffffffu, keep && res));
-            hits += hw;
-            misses += __popc(mw) - hw;
+        for (int i = 0; i < NB; ++i) {
+            const int c = col0 + 128 * i;
+            uint32_t nib = (word[i] >> ((4 * lane) & 31)) & 0xfu;
+            if (c + 4 > d) nib = c < d ? nib & ((1u << (d - c)) - 1u) : 0u;     // no column beyond d
+            keep |= nib << (4 * i);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (st[i][e] >= 0) res |= 1u << (4 * i + e);
+                // (a column is used at most once per update: uses <= t, so the most rarely used column has the
+                // largest key)
+                kv[i][e] = (uint32_t)(t_now - (LFU ? cn[i][e] : st[i][e]));
+            }
+            if (LFU && nib) {                           // used once more (resident or not)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) cn[i][e] += (int)((nib >> e) & 1u);
+                if (c + 4 <= d) {
+                    *reinterpret_cast<int4 *>(count + c) = make_int4(cn[i][0], cn[i][1], cn[i][2], cn[i][3]);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (c + e < d) count[c + e] = cn[i][e];
+                }
+            }
         }
     }
+    const uint32_t may_go = res & ~keep, misses = keep & ~res;
+    const auto evict_key = [&](int i, int e) { return (may_go >> (4 * i + e)) & 1u ? kv[i][e] & 0x7fffffffu : 0u; };
+
+    const int warp_hits = __reduce_add_sync(0xffffffffu, __popc(keep & res));
+    const int warp_misses = __reduce_add_sync(0xffffffffu, __popc(misses));
     if (lane == 0) {
-        s.wa[warp] = hits;
-        s.wc[warp] = misses;
+        s.wa[warp] = warp_hits;
+        s.wc[warp] = warp_misses;
     }
-    __syncthreads();
+    __syncthreads();                                    // the histogram is zero, the counts are there
     int total_hits, total_misses, tot;
     (void)warp_array_prefix(s.wa, warp, lane, total_hits);
-    int miss_before = warp_array_prefix(s.wc, warp, lane, total_misses);
+    const int miss_before = warp_array_prefix(s.wc, warp, lane, total_misses);
     const int free_slots = capacity - n_res;
     const int evictable = n_res - total_hits;
     const int n_evict = min(max(0, total_misses - free_slots), evictable);
     const int room = free_slots + n_evict;
-    __syncthreads();   // the warp arrays are reused by the select
 
-    // victims: the n_evict largest eviction keys (oldest stamps), lower index first among equals
+    // ---- victims: the n_evict largest eviction keys (oldest stamps), lower index first among equals:
+    //      radix select from the top bit down, up to 11 bits per pass ----
     uint32_t T2 = 0x7fffffffu;   // no key exceeds it: no victim
     int quota2 = 0, n_eq2 = 0;
     if (n_evict > 0) {
-        if (n_evict == evictable)
+        if (n_evict == evictable) {
             T2 = 0u;             // every evictable column (key > 0) goes
-        else
-            block_radix_select(keys, d, 0x7fffffffu, 32 - __clz(t_now), n_evict, s, T2, quota2, n_eq2);
-    }
-    // ordered rank of the eviction-key ties (needed only if some of them stay)
-    int veq_before = 0;
-    const bool ranked_ties = quota2 > 0 && quota2 < n_eq2;
-    if (ranked_ties) {
-        int veq = 0;
-        for (int it = 0; it < span; it += 32) {
-            const int e = base + it + lane;
-            veq += __popc(__ballot_sync(0xffffffffu, e < d && (keys[e] & 0x7fffffffu) == T2));
+        } else {
+            int hi = 32 - __clz(t_now), krem = n_evict;
+            uint32_t prefix = 0u, prefix_mask = 0u;
+            while (hi > 0) {
+                const int w = hi < RADIX_BITS ? hi : RADIX_BITS, shift = hi - w;
+                const uint32_t digit_mask = (1u << w) - 1u;
+#pragma unroll
+                for (int i = 0; i < NB; ++i)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const uint32_t ek = evict_key(i, e);
+                        if (ek != 0u && (ek & prefix_mask) == prefix) {
+                            const uint32_t dg = (ek >> shift) & digit_mask;
+                            atomicAdd(dg < CU_SMALL ? &small[dg * CU_SPREAD + (lane & (CU_SPREAD - 1))] : &s.hist[dg], 1u);
+                        }
+                    }
+                __syncthreads();
+                if (tid < CU_SMALL) {
+                    const uint4 p = *reinterpret_cast<const uint4 *>(small + tid * CU_SPREAD),
+                                q = *reinterpret_cast<const uint4 *>(small + tid * CU_SPREAD + 4);
+                    // (all other columns have key 0)
+                    s.hist[tid] = p.x + p.y + p.z + p.w + q.x + q.y + q.z + q.w + (tid == 0 && prefix == 0u ? (unsigned)d : 0u);
+                }
+                __syncthreads();
+                find_bin(s, krem);
+                prefix |= (uint32_t)s.bcast[0] << shift;
+                prefix_mask |= digit_mask << shift;
+                krem = s.bcast[1];
+                n_eq2 = s.bcast[2];        // after the last pass: the number of keys equal to T2
+                hi = shift;
+                if (hi > 0) {
+                    clear();
+                    __syncthreads();
+                }
+            }
+            T2 = prefix;
+            quota2 = krem;
         }
-        if (lane == 0) s.wb[warp] = veq;
+    }
+    // ---- if only the first quota2 ties go: the ties in front of each warp, and inside the one warp in
+    //      which the quota runs out, in front of each lane.  Likewise the misses, if some find no room ----
+    uint32_t ties = 0u;
+    if (quota2 > 0 && T2 != 0u) {
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (((may_go >> (4 * i + e)) & 1u) && (kv[i][e] & 0x7fffffffu) == T2) ties |= 1u << (4 * i + e);
+    }
+    // first `quota` of the flagged columns (ascending index) of which `before` lie in earlier warps
+    const auto first_of = [&](uint32_t flags, int before, int n_warp, int quota) {
+        if (before + n_warp <= quota) return flags;
+        if (before >= quota) return 0u;
+        uint32_t out = 0u;
+        int run = before;
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const uint32_t nib = (flags >> (4 * i)) & 0xfu;
+            int incl = __popc(nib);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int n = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += n;
+            }
+            int rank = run + incl - __popc(nib);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if ((nib >> e) & 1u) {
+                    if (rank < quota) out |= 1u << (4 * i + e);
+                    ++rank;
+                }
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        return out;
+    };
+    if (quota2 > 0 && quota2 < n_eq2) {                // (uniform over the block)
+        const int warp_ties = __reduce_add_sync(0xffffffffu, __popc(ties));
+        if (lane == 0) s.wb[warp] = warp_ties;
         __syncthreads();
-        veq_before = warp_array_prefix(s.wb, warp, lane, tot);
+        ties = first_of(ties, warp_array_prefix(s.wb, warp, lane, tot), warp_ties, quota2);
     }
-    const bool all_ties = quota2 > 0 && !ranked_ties;
+    // a hit, or a miss that still finds room (ascending index order), is stamped with this update
+    const uint32_t use = (keep & res) | (total_misses > room ? first_of(misses, miss_before, warp_misses, room) : misses);
 
-    for (int it = 0; it < span && base + it < d; it += 32) {
-        const int e = base + it + lane;
-        const bool valid = e < d;
-        const uint32_t kv = valid ? keys[e] : 0u;
-        const uint32_t vkey = kv & 0x7fffffffu;
-        const bool res = (kv >> 31) != 0u;
-        const bool keep = valid && ((mask_bits[(base + it) >> 5] >> lane) & 1u);
-        const bool vq = valid && vkey == T2 && vkey != 0u;
-        bool evict = valid && vkey > T2;
-        if (all_ties) evict = evict || vq;
-        if (ranked_ties) {
-            const unsigned bvq = __ballot_sync(0xffffffffu, vq);
-            evict = evict || (vq && (veq_before + __popc(bvq & lt)) < quota2);
-            veq_before += __popc(bvq);
+    // ---- the new stamps ----
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        const int c = col0 + 128 * i;
+        uint32_t gone = 0u;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (evict_key(i, e) > T2) gone |= 1u << e;
+        gone |= (ties >> (4 * i)) & 0xfu;
+        const uint32_t used = (use >> (4 * i)) & 0xfu;
+        if (!(gone | used)) continue;
+        if (LFU || c + 4 > d) {
+            // (LFU: the old stamps are not kept in registers)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (((gone | used) >> e) & 1u) stamp[c + e] = (gone >> e) & 1u ? -1 : t_now;
+        } else {
+            int v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                v[e] = (gone >> e) & 1u ? -1 : (used >> e) & 1u ? t_now : t_now - (int)kv[i][e];
+            *reinterpret_cast<int4 *>(stamp + c) = make_int4(v[0], v[1], v[2], v[3]);
         }
-        const bool miss = keep && !res;
-        const unsigned bm = __ballot_sync(0xffffffffu, miss);
-        if (evict) {
-            stamp[e] = -1;
-        } else if (keep) {
-            // a hit, or a miss that still finds room (ascending index order)
-            if (!miss || (miss_before + __popc(bm & lt)) < room) stamp[e] = t_now;
-        }
-        if (count && keep) count[e] += 1;       // used once more (resident or not)
-        miss_before += __popc(bm);
     }
     if (tid == 0) {
         const int inserted = min(total_misses, room);
@@ -324,9 +436,14 @@ dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, flo
 dip_status dip_launch_cache_update(dip_ctx *ctx, const uint32_t *mask_bits, int d, int32_t *stamp, int32_t *count,
                                    int32_t *meta, int capacity, cudaStream_t stream)
 {
-    cache_update_kernel<<<1, TK_THREADS, (size_t)d * sizeof(uint32_t), stream>>>(mask_bits, d, stamp, count, meta, capacity,
-                                                                                   dip_trace_slot(ctx, 3));
-    DIP_CUDA_TRY(ctx, cudaGetLastError());
+    unsigned long long *tr = dip_trace_slot(ctx, 3);
+    // blocks of 128 columns per warp: the smallest that covers d (a column's state is a register)
+    void (*kernel)(const uint32_t *, int, int32_t *, int32_t *, int32_t *, int, unsigned long long *);
+    if (d <= 2 * 128 * TK_WARPS) kernel = count ? cache_update_kernel<2, true> : cache_update_kernel<2, false>;
+    else if (d <= 5 * 128 * TK_WARPS) kernel = count ? cache_update_kernel<5, true> : cache_update_kernel<5, false>;
+    else kernel = count ? cache_update_kernel<8, true> : cache_update_kernel<8, false>;
+    static_assert(DIP_MAX_D <= 8 * 128 * TK_WARPS, "");
+    DIP_CUDA_TRY(ctx, dip_launch_pdl(kernel, dim3(1), dim3(TK_THREADS), 0, stream, mask_bits, d, stamp, count, meta, capacity, tr));
     return DIP_OK;
 }
 
@@ -334,7 +451,6 @@ dip_status dip_launch_cache_update(dip_ctx *ctx, const uint32_t *mask_bits, int 
 dip_status dip_init_mask_kernels(dip_ctx *ctx)
 {
     const int bytes = DIP_MAX_D * (int)sizeof(uint32_t);
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(cache_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     const int fine_bytes = bytes + (int)sizeof(TkFine);
     DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
     DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
