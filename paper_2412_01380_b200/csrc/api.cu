@@ -140,6 +140,8 @@ dip_status dip_create_ex(dip_ctx **out, int device, const dip_options *opt)
     ctx->n_tickets = N_TICKETS;
     const size_t vec = (size_t)ctx->max_batch * ctx->max_d;
     if ((st = dev_alloc(ctx, &ctx->partials, ctx->partials_floats)) != DIP_OK) return fail(st);
+    if ((st = dev_alloc(ctx, &ctx->mail, (size_t)ctx->sm_count * DIP_MAIL_FLOATS)) != DIP_OK) return fail(st);
+    if ((st = dev_alloc(ctx, &ctx->readers, (size_t)1)) != DIP_OK) return fail(st);
     if ((st = dev_alloc(ctx, &ctx->tickets, (size_t)N_TICKETS)) != DIP_OK) return fail(st);
     if ((st = dev_alloc(ctx, &ctx->h, vec)) != DIP_OK) return fail(st);
     if ((st = dev_alloc(ctx, &ctx->y, vec)) != DIP_OK) return fail(st);
@@ -172,6 +174,8 @@ dip_status dip_create_ex(dip_ctx **out, int device, const dip_options *opt)
         if (cudaEventCreateWithFlags(&ctx->ev_fork[i], cudaEventDisableTiming) != cudaSuccess) return fail(DIP_ERR_CUDA);
         if (cudaEventCreateWithFlags(&ctx->ev_join[i], cudaEventDisableTiming) != cudaSuccess) return fail(DIP_ERR_CUDA);
     }
+    if (cudaMemset(ctx->mail, 0xff, (size_t)ctx->sm_count * DIP_MAIL_FLOATS * sizeof(float)) != cudaSuccess) return fail(DIP_ERR_CUDA);
+    if (cudaMemset(ctx->readers, 0, sizeof(unsigned int)) != cudaSuccess) return fail(DIP_ERR_CUDA);
     if (cudaMemset(ctx->tickets, 0, N_TICKETS * sizeof(unsigned int)) != cudaSuccess) return fail(DIP_ERR_CUDA);
     if (cudaMemset(ctx->counts, 0, 8 * sizeof(int32_t)) != cudaSuccess) return fail(DIP_ERR_CUDA);
     if ((st = dip_init_mask_kernels(ctx)) != DIP_OK) return fail(st);
@@ -184,6 +188,8 @@ dip_status dip_destroy(dip_ctx *ctx)
 {
     if (!ctx) return DIP_ERR_INVALID_ARG;
     cudaFree(ctx->partials);
+    cudaFree(ctx->mail);
+    cudaFree(ctx->readers);
     cudaFree(ctx->tickets);
     cudaFree(ctx->h);
     cudaFree(ctx->y);
@@ -255,6 +261,9 @@ dip_status dip_reset_device_status(dip_ctx *ctx, void *stream)
 {
     if (!ctx_ok(ctx)) return DIP_ERR_INVALID_ARG;
     DIP_CUDA_TRY(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(int), (cudaStream_t)stream));
+    // (a launch that gave up a wait leaves behind what comes too late: counts, and sums nobody takes)
+    DIP_CUDA_TRY(ctx, cudaMemsetAsync(ctx->readers, 0, sizeof(unsigned int), (cudaStream_t)stream));
+    DIP_CUDA_TRY(ctx, cudaMemsetAsync(ctx->mail, 0xff, (size_t)ctx->sm_count * DIP_MAIL_FLOATS * sizeof(float), (cudaStream_t)stream));
     return DIP_OK;
 }
 
@@ -264,16 +273,24 @@ dip_status dip_selftest_bounded_wait(dip_ctx *ctx, int limit_us, unsigned long l
     return dip_launch_bounded_wait_selftest(ctx, 1000ull * (unsigned long long)limit_us, waited_ns, (cudaStream_t)stream);
 }
 
-// Run the cache update of one masked input beside the main stream (side stream `which`).
+// Run cache updates beside the main stream (side stream `which`).
+static dip_status fork_cache_updates(dip_ctx *ctx, int which, const dip_cache_updates &u, cudaStream_t main)
+{
+    if (u.n < 1) return DIP_OK;
+    DIP_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork[which], main));
+    DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->side[which], ctx->ev_fork[which], 0));
+    dip_status st = dip_launch_cache_updates(ctx, u, ctx->side[which]);
+    ctx->side_busy[which] = true;
+    return st;
+}
+
 static dip_status fork_cache_update(dip_ctx *ctx, int which, const uint32_t *mask_bits, const dip_cache_state *c,
                                     cudaStream_t main)
 {
-    DIP_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork[which], main));
-    DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->side[which], ctx->ev_fork[which], 0));
-    dip_status st = dip_launch_cache_update(ctx, mask_bits, c->d, c->stamp, c->policy == DIP_CACHE_LFU ? c->count : nullptr, c->meta,
-                                            c->capacity, ctx->side[which]);
-    ctx->side_busy[which] = true;
-    return st;
+    dip_cache_updates u;
+    u.n = 1;
+    u.at[0] = dip_update_of(c, mask_bits);
+    return fork_cache_updates(ctx, which, u, main);
 }
 
 // Make the main stream wait for the side streams' updates.
@@ -313,8 +330,10 @@ dip_status dip_ca_mask(dip_ctx *ctx, const float *x, int d, int k, float gamma,
     cudaStream_t s = (cudaStream_t)stream;
     uint32_t *m = mask_bits ? mask_bits : ctx->mask;
     dip_status rc = dip_launch_select(ctx, x, nullptr, nullptr, 1, d, k, gamma, st->stamp, m, s);
-    if (rc == DIP_OK) rc = dip_launch_cache_update(ctx, m, d, st->stamp, st->policy == DIP_CACHE_LFU ? st->count : nullptr, st->meta,
-                                                   st->capacity, s);
+    dip_cache_updates u;
+    u.n = 1;
+    u.at[0] = dip_update_of(st, m);
+    if (rc == DIP_OK) rc = dip_launch_cache_updates(ctx, u, s);
     if (rc == DIP_OK && kept_idx) rc = dip_launch_mask_to_idx(ctx, m, 1, 1, d, kept_idx, k, nullptr, s);
     return rc;
 }
@@ -366,7 +385,7 @@ dip_status dip_select_gemv_gate_up(dip_ctx *ctx, const dip_mlp_weights *w, const
     if (!fits(ctx, w->d_model, w->d_ff, 1)) return DIP_ERR_WORKSPACE;
     if (!dip_gemv_fused_supported(ctx, w, 0, false) || !dip_gemv_fused_supported(ctx, w, 1, false)) return DIP_ERR_UNSUPPORTED;
     dip_gemv_keys hk = {ctx->coarse, cache_d ? cache_d->stamp : nullptr, gamma, 0};
-    const dip_fused_select sx = {x, nullptr, nullptr, nullptr, k_x, gamma, cache_gu ? cache_gu->stamp : nullptr, mask_x};
+    const dip_fused_select sx = {x, nullptr, nullptr, nullptr, k_x, gamma, cache_gu ? cache_gu->stamp : nullptr, mask_x, nullptr, nullptr};
     return dip_launch_gemv_fused(ctx, w, 0, &sx, h, (cudaStream_t)stream, &hk);
 }
 
@@ -379,20 +398,22 @@ dip_status dip_select_gemv_down(dip_ctx *ctx, const dip_mlp_weights *w, const fl
     if (cache_d && !cache_ok(cache_d, w->d_ff)) return DIP_ERR_INVALID_ARG;
     if (!fits(ctx, w->d_model, w->d_ff, 1)) return DIP_ERR_WORKSPACE;
     if (!dip_gemv_fused_supported(ctx, w, 1, false)) return DIP_ERR_UNSUPPORTED;
-    const dip_fused_select sh = {h, nullptr, nullptr, ctx->coarse, k_h, gamma, cache_d ? cache_d->stamp : nullptr, mask_h};
+    const dip_fused_select sh = {h, nullptr, nullptr, ctx->coarse, k_h, gamma, cache_d ? cache_d->stamp : nullptr, mask_h, nullptr, nullptr};
     return dip_launch_gemv_fused(ctx, w, 1, &sh, y, (cudaStream_t)stream, nullptr);
 }
 
 // One sparse MLP step.  xb != nullptr: the step's input is formed first as
 // x = (xa + xb) / rms(xa + xb), written to x_norm, in the same launch as its mask.
 // slot_x / slot_h: where the masks go when the caller did not ask for them.  defer_join: leave
-// the cache updates running on the side streams (the caller joins them later).
+// the cache updates running on the side streams (the caller joins them later).  due: cache updates that
+// earlier blocks have left to later launches; this block leaves its own there too, unless it is the last
+// (of the call, or before the mask slots are used again).
 static dip_status step_impl(dip_ctx *ctx, const dip_mlp_weights *w,
                             const float *xa, const float *xb, float *x_norm,
                             int batch, int k_x, int k_h, float gamma,
                             const dip_cache_state *cache_gu, const dip_cache_state *cache_d,
                             float *y, const dip_step_outputs *out,
-                            uint32_t *slot_x, uint32_t *slot_h, bool defer_join, bool join_follows, void *stream)
+                            uint32_t *slot_x, uint32_t *slot_h, bool defer_join, dip_cache_updates *due, bool last, void *stream)
 {
     const float *x = xb ? x_norm : xa;
     if (!ctx || !weights_ok(w) || !xa || !x || !y || !dip_aligned16(xa) || !dip_aligned16(x) || !dip_aligned16(y))
@@ -415,27 +436,29 @@ static dip_status step_impl(dip_ctx *ctx, const dip_mlp_weights *w,
     dip_status st;
 
     if (batch == 1 && dip_gemv_fused_supported(ctx, w, 0, xb != nullptr) && dip_gemv_fused_supported(ctx, w, 1, false)) {
-        // The same four operations in two launches: each product builds the mask of its own input
-        // (Eq. 7 / Eq. 8, or the ranking of Algorithm 1) while it already streams the rows that are
-        // certain to be kept; the cache updates follow the launch that wrote their mask.
+        // The same operations in two launches: each product builds the mask of its own input (Eq. 7 / Eq. 8,
+        // or the ranking of Algorithm 1).
         dip_gemv_keys hk = {ctx->coarse, cache_d ? cache_d->stamp : nullptr, gamma, 0};
-        const dip_fused_select sx = {xa, xb, x_norm, nullptr, k_x, gamma, cache_gu ? cache_gu->stamp : nullptr, mask_x};
+        const dip_fused_select sx = {xa, xb, x_norm, nullptr, k_x, gamma, cache_gu ? cache_gu->stamp : nullptr, mask_x,
+                                     nullptr, nullptr};
         if ((st = dip_launch_gemv_fused(ctx, w, 0, &sx, h, s, &hk)) != DIP_OK) return st;
-        if (cache_gu && (st = fork_cache_update(ctx, 0, mask_x, cache_gu, s)) != DIP_OK) return st;
-        if (cache_d && join_follows) {
-            // The caller waits for this step's cache updates right after it: the update of the down input
-            // (the long one) then has to run BESIDE the down product, which it can only with the mask
-            // from a select kernel of its own.
-            st = dip_launch_select(ctx, h, nullptr, nullptr, 1, w->d_ff, k_h, gamma, cache_d->stamp, mask_h, s, ctx->coarse);
-            if (st != DIP_OK) return st;
-            if ((st = fork_cache_update(ctx, 1, mask_h, cache_d, s)) != DIP_OK) return st;
-            if ((st = dip_launch_gemv(ctx, w, 1, h, 1, mask_h, nmax_h, y, s)) != DIP_OK) return st;
-        } else {
-            const dip_fused_select sh = {h, nullptr, nullptr, ctx->coarse, k_h, gamma, cache_d ? cache_d->stamp : nullptr, mask_h};
-            if ((st = dip_launch_gemv_fused(ctx, w, 1, &sh, y, s, nullptr)) != DIP_OK) return st;
-            if (cache_d && (st = fork_cache_update(ctx, 1, mask_h, cache_d, s)) != DIP_OK) return st;
+        if (cache_gu) due->at[due->n++] = dip_update_of(cache_gu, mask_x);
+        // the updates that are due ride with the last block's down product, if that has a cache and SMs to spare; else a
+        // launch beside the products takes them
+        const bool ride = last && cache_d && dip_gemv_fused_update_room(ctx, w) > due->n;
+        if (!ride && (last || due->n + 2 > DIP_CACHE_UPDATES)) {
+            if ((st = fork_cache_updates(ctx, 0, *due, s)) != DIP_OK) return st;
+            due->n = 0;
         }
+        const dip_fused_select sh = {h, nullptr, nullptr, ctx->coarse, k_h, gamma, cache_d ? cache_d->stamp : nullptr, mask_h,
+                                     ride ? cache_d : nullptr, due};
+        if ((st = dip_launch_gemv_fused(ctx, w, 1, &sh, y, s, nullptr)) != DIP_OK) return st;
+        if (ride) due->n = 0;
+        else if (last && cache_d && (st = fork_cache_update(ctx, 1, mask_h, cache_d, s)) != DIP_OK) return st;
+        else if (!last && cache_d) due->at[due->n++] = dip_update_of(cache_d, mask_h);
     } else {
+        if ((st = fork_cache_updates(ctx, 0, *due, s)) != DIP_OK) return st;
+        due->n = 0;
         // m_x = topK(score(x))            (Eq. 7; the ranking of Algorithm 1 when a cache is given)
         st = dip_launch_select(ctx, xa, xb, x_norm, batch, w->d_model, k_x, gamma,
                                cache_gu ? cache_gu->stamp : nullptr, mask_x, s);
@@ -475,8 +498,10 @@ dip_status dip_mlp_step(dip_ctx *ctx, const dip_mlp_weights *w,
                         float *y, const dip_step_outputs *out, void *stream)
 {
     if (!ctx_ok(ctx)) return DIP_ERR_INVALID_ARG;
+    dip_cache_updates due;
+    due.n = 0;
     return step_impl(ctx, w, x, nullptr, nullptr, batch, k_x, k_h, gamma, cache_gu, cache_d, y, out,
-                     ctx->mask, ctx->mask_h, false, true, stream);
+                     ctx->mask, ctx->mask_h, false, &due, true, stream);
 }
 
 // One masked input of the two-tier step.  On the step's path: the hit / miss split, the list of
@@ -499,9 +524,10 @@ static dip_status tiered_half(dip_ctx *ctx, const dip_mlp_weights *w, int which,
     DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(sb, ctx->ev_tier_fork[which], 0));
     if ((st = dip_launch_tier_fetch(ctx, t, sf)) != DIP_OK) return st;
     DIP_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_tier_fetched[which], sf));
-    st = dip_launch_cache_update(ctx, mask_bits, c->d, c->stamp, c->policy == DIP_CACHE_LFU ? c->count : nullptr,
-                                 c->meta, c->capacity, sb);
-    if (st != DIP_OK) return st;
+    dip_cache_updates u;
+    u.n = 1;
+    u.at[0] = dip_update_of(c, mask_bits);
+    if ((st = dip_launch_cache_updates(ctx, u, sb)) != DIP_OK) return st;
     if ((st = dip_launch_tier_assign(ctx, t, mask_bits, c->stamp, sb)) != DIP_OK) return st;
     DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(sb, ctx->ev_tier_fetched[which], 0));
     if ((st = dip_launch_tier_install(ctx, t, sb)) != DIP_OK) return st;
@@ -634,6 +660,8 @@ static dip_status stack_impl(dip_ctx *ctx, int n_layers, const dip_mlp_weights *
     const float *x_prev = x_in;
     const float *y_prev = nullptr;
     const bool ca = cache_gu || cache_d;
+    dip_cache_updates due;
+    due.n = 0;
     if (probe) DIP_CUDA_TRY(ctx, cudaMemcpyAsync(probe->x, x_in, sizeof(float) * (size_t)batch * d, cudaMemcpyDeviceToDevice, s));
     for (int l = 0; l < n_layers; ++l) {
         float *y = (l == n_layers - 1 && y_last) ? y_last : ((l & 1) ? ctx->y2 : ctx->y);
@@ -653,7 +681,7 @@ static dip_status stack_impl(dip_ctx *ctx, int n_layers, const dip_mlp_weights *
         }
         dip_status st = step_impl(ctx, &layers[l], x_prev, y_prev, y_prev ? x_l : nullptr, batch, k_x, k_h, gamma,
                                   cache_gu ? &cache_gu[l] : nullptr, cache_d ? &cache_d[l] : nullptr,
-                                  y, probe ? &po : nullptr, slot_x, slot_h, true,
+                                  y, probe ? &po : nullptr, slot_x, slot_h, true, &due,
                                   l == n_layers - 1 || (ca && slot == DIP_RING_LAYERS - 1), stream);
         if (st != DIP_OK) return st;
         if (ca && slot == DIP_RING_LAYERS - 1 && (st = join_cache_updates(ctx, s)) != DIP_OK) return st;

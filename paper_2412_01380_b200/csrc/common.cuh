@@ -11,6 +11,8 @@
 
 constexpr int DIP_RING_LAYERS = 128;
 constexpr int DIP_TRACE_SLOTS = 1024;
+constexpr uint32_t DIP_MAIL_EMPTY = 0xffffffffu;
+constexpr int DIP_MAIL_FLOATS = 256;   // boxes per SM: one CTA's segment of sums
 constexpr int DIP_TRACE_WORDS = 4;   // first start, dependency ready, last end, auxiliary
 
 // Scratch workspace of a context.  All device memory the library itself owns.
@@ -25,6 +27,8 @@ struct dip_ctx {
     // split-row partial sums of the two GEMVs (binary32)
     float *partials;
     size_t partials_floats;
+    float *mail;         // [sm_count][DIP_MAIL_FLOATS] row parts of the fused products on their way to the CTA that adds them up
+    unsigned int *readers; // [1] CTAs of a fused product that have read the stamps; zero between launches
     // one arrival counter per output slab; zero between launches
     unsigned int *tickets;
     int n_tickets;
@@ -151,10 +155,22 @@ dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, flo
                              float gamma, const int32_t *stamp, uint32_t *mask_bits, cudaStream_t stream,
                              const uint16_t *coarse = nullptr);
 
-// topk.cu: LRU cache update from (mask, state).
-// count != nullptr: LFU (use counters), else LRU.
-dip_status dip_launch_cache_update(dip_ctx *ctx, const uint32_t *mask_bits, int d, int32_t *stamp, int32_t *count,
-                                   int32_t *meta, int capacity, cudaStream_t stream);
+// topk.cu: cache updates from (mask, state), a block per cache.  count != nullptr: LFU (use counters), else LRU.
+struct dip_cache_update {
+    const uint32_t *mask;
+    int32_t *stamp, *count, *meta;
+    int d, capacity;
+};
+constexpr int DIP_CACHE_UPDATES = 7;   // the caches of three blocks and a half; beside 140 products' CTAs on 148 SMs
+struct dip_cache_updates {
+    int n;
+    dip_cache_update at[DIP_CACHE_UPDATES];
+};
+static inline dip_cache_update dip_update_of(const dip_cache_state *c, const uint32_t *mask)
+{
+    return {mask, c->stamp, c->policy == DIP_CACHE_LFU ? c->count : nullptr, c->meta, c->d, c->capacity};
+}
+dip_status dip_launch_cache_updates(dip_ctx *ctx, const dip_cache_updates &u, cudaStream_t stream);
 
 // topk.cu: per-device set-up of the mask kernels (dynamic shared memory limit).
 dip_status dip_init_mask_kernels(dip_ctx *ctx);
@@ -206,7 +222,13 @@ struct dip_fused_select {
     float gamma;
     const int32_t *stamp;    // cache state of the input (cache-aware ranking) or nullptr
     uint32_t *mask_out;      // receives the mask
+    // down with a cache only: the launch also updates that cache, and those of `beside`, on which nothing in the
+    // launch depends (n = 0: none)
+    const dip_cache_state *update;
+    const dip_cache_updates *beside;
 };
+// gemv_fused.cu: how many cache updates (its own among them) find an SM beside a down launch's products.
+int dip_gemv_fused_update_room(const dip_ctx *ctx, const dip_mlp_weights *w);
 bool dip_gemv_fused_supported(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool norm);
 dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int which, const dip_fused_select *sel,
                                  float *out, cudaStream_t stream, dip_gemv_keys *keys);

@@ -70,6 +70,69 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity, unsign
     }
 }
 
+// Sums that one CTA of a launch hands to another through global memory: the value itself is the message.
+// A box holds DIP_MAIL_EMPTY (a NaN pattern that no arithmetic produces) until its sum arrives; who
+// takes a sum empties its box again.
+__device__ __forceinline__ void mail_put(float *box, float v)
+{
+    asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(box), "f"(v) : "memory");
+}
+// The sums of the first min(n, N) of the boxes box[0], box[stride], ... (the others: zero).  Waits at most
+// limit_ns for them, after which it records status 1 and takes what is there.
+template <int N>
+__device__ __forceinline__ void mail_take(float *box, size_t stride, int n, float (&a)[N], int *status, unsigned long long limit_ns)
+{
+    unsigned long long t0 = 0;
+    for (unsigned i = 0;; ++i) {
+        bool all = true;
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            a[q] = 0.f;
+            if (q < n) asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(a[q]) : "l"(box + (size_t)q * stride) : "memory");
+        }
+#pragma unroll
+        for (int q = 0; q < N; ++q) all = all && __float_as_uint(a[q]) != DIP_MAIL_EMPTY;
+        if (all) break;
+        if ((i & 63u) == 63u) {
+            const unsigned long long now = dip_gtime();
+            if (t0 == 0) {
+                t0 = now;
+            } else if (now - t0 > limit_ns) {
+                atomicExch(status, 1);
+                break;
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+        if (q < n) mail_put(box + (size_t)q * stride, __uint_as_float(DIP_MAIL_EMPTY));
+}
+
+// One more at a counter in global memory, after what this thread (and those it has synchronised with) has read.
+__device__ __forceinline__ void count_one(unsigned int *counter)
+{
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
+}
+// Waits until the counter has reached n; false (and status 1) if limit_ns ran out.
+__device__ __forceinline__ bool wait_count(const unsigned int *counter, unsigned int n, int *status, unsigned long long limit_ns)
+{
+    unsigned long long t0 = 0;
+    for (unsigned i = 0;; ++i) {
+        unsigned int v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
+        if (v >= n) return true;
+        if ((i & 63u) == 63u) {
+            const unsigned long long now = dip_gtime();
+            if (t0 == 0) {
+                t0 = now;
+            } else if (now - t0 > limit_ns) {
+                atomicExch(status, 1);
+                return false;
+            }
+        }
+    }
+}
+
 __device__ __forceinline__ float silu_f32(float g) { return g / (1.0f + expf(-g)); }
 
 __device__ __forceinline__ float half_bits_to_float(uint16_t h)

@@ -4,20 +4,34 @@
 // ranking of Algorithm 1), and a select kernel in front of it costs a kernel boundary, the mask's
 // trip through global memory, and a device that idles while one CTA selects.  The select by one
 // 15-bit histogram (select_core.cuh) is short enough for every CTA of the product to run it for
-// itself - same code, same inputs, hence the same mask everywhere, with nothing to wait for -
-// and to go straight on to its rows.  CTA 0 also writes the mask (and, for the gate/up input of a
-// chained layer, the normalised x) to global memory for the cache update and the caller.  The
-// mask is bit for bit the stand-alone select's, and the product is gemv_direct_kernel's: a CTA owns
-// a 512-byte segment of the packed rows and a share of the kept rows, 32 warps x 4 loads in flight.
+// itself - same code, same inputs, hence the same rows everywhere, with nothing to wait for -
+// and to go straight on to its rows.  The kept set is the stand-alone select's, bit for bit.
+//
+// Memory is idle until the first row is asked for, so what lies between the threshold's bin and that
+// moment is kept short: the columns above the bin ("sure") go from the flags in registers into the
+// CTA's row list with one block-wide prefix sum, and the bin's few dozen columns ("ties") are ranked
+// by one warp while the others already stream.  What bounds these phases is the number of instructions, as
+// all 32 warps issue them (1200 per warp, 9600 of a scheduler's cycles, when each key was tested by itself and
+// each warp searched the histogram).  List order: sure columns, then the kept ties by rank; a CTA owns a
+// 512-byte segment of the packed rows and a share of that list (32 warps x 4 loads in flight).  Its sums
+// meet in a fixed order: warps in shared memory, row parts in the CTA of the last part, which the others
+// send theirs to.
+//
+// The updates of column caches ride along with the last down product of a call, as blocks without rows
+// (UPD).  The down input's own cache is among them: its block makes the mask together with the others and
+// writes the cache's state once all of them have read it.  Other launches do without that code, which would
+// cost each of them 1.3 us (block_f32 shapes, 14.3 against 16.9 us per step of two launches).
+#include <type_traits>
+
+#include "cache_update.cuh"
 #include "gemv_common.cuh"
-#include "select_core.cuh"
 
 namespace {
 
 constexpr int GF_SEG = 512;
 constexpr int GF_NW = TK_THREADS / 32;     // 32 warps
 constexpr int GF_U = 4;                    // loads in flight per lane
-constexpr size_t GF_SMEM_LIMIT = (size_t)220 * 1024;   // dynamic shared memory a launch may ask for
+constexpr size_t GF_SMEM_LIMIT = (size_t)224 * 1024;   // dynamic shared memory a launch may ask for
 
 struct FusedParams {
     // product
@@ -25,9 +39,11 @@ struct FusedParams {
     size_t row_bytes;
     int d_in, d_out;
     int n_slabs, nparts;
+    int x_near;                  // gate/up: room in shared memory for the values of x
     float *out;
-    float *partials;             // [nparts][n_slabs][segment elements]
-    unsigned int *tickets;
+    float *mail;                 // [nparts][n_slabs][segment elements]; DIP_MAIL_EMPTY outside a launch
+    int *status;
+    unsigned long long wait_limit_ns;
     unsigned long long *tr;
     uint16_t *key_coarse;        // gate/up: top 16 bits of the rank keys of h (nullptr: not wanted)
     const int32_t *key_stamp;
@@ -43,26 +59,32 @@ struct FusedParams {
     uint32_t *mask_out;
 };
 
-struct __align__(16) FusedSmem {
-    TkFine fine;                           // the select's histogram; afterwards the warps' sums ([warp][lane * E + e])
-    TkShared ts;
-    unsigned int maskw[DIP_MAX_D / 32];    // the mask
-    int wsum[GF_NW];
-    int last;
-    float sum[32 * 8];
+struct FusedUpdates {            // UPD
+    unsigned int *readers;       // CTAs that have read the stamps; zero between launches
+    dip_cache_update own;        // this input's cache (its mask is made here)
+    dip_cache_updates beside;    // caches that nothing in the launch depends on
 };
-static_assert(sizeof(float) * GF_NW * 32 * 8 <= sizeof(unsigned int) * TK_FINE_WORDS, "the warps' sums fit the histogram");
 
-// This part's share of the rows in `words` (a bit set in shared memory, complete and visible), by
-// rank, as a list in idx[]; returns the share's size.  One word per thread (DIP_MAX_D / 32 words at
-// most); all threads call it; ends with a barrier.
-__device__ __forceinline__ int list_rows(FusedSmem &s, const unsigned int *words, int mask_words, int d_in, int part,
-                                         int nparts, uint16_t *idx)
+struct __align__(16) FusedSmem {
+    TkFine fine;                           // the select's histogram; afterwards the warps' sums [32][segment elements]
+                                           // and, in its second half, their partial sums [1024]
+    TkShared ts;
+    unsigned int maskw[DIP_MAX_D / 32];    // the mask (in the CTA that writes it, and under heavy ties)
+    int wsum[GF_NW];
+    uint16_t tie[TK_TIE_LIMIT];            // the kept columns of the threshold's bin, by rank
+    int go;                                // UPD: all have read the stamps
+};
+static_assert(GF_NW * 32 * 8 <= TK_FINE_WORDS / 2 && TK_THREADS <= TK_FINE_WORDS / 2, "the sums fit the histogram");
+
+// Ranks [lo, hi) of the rows in `words` (a bit set in shared memory, complete and visible) as a list
+// in idx[].  One word per thread (DIP_MAX_D / 32 words at most); all threads call it; ends with a
+// barrier.  (Heavy ties only: otherwise the list is built from the flags in registers.)
+__device__ __forceinline__ void list_rows(FusedSmem &s, const unsigned int *words, int mask_words, int lo, int hi,
+                                          uint16_t *idx)
 {
     static_assert(DIP_MAX_D / 32 <= TK_THREADS, "one mask word per thread");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t u = tid < mask_words ? words[tid] : 0u;
-    if (tid == mask_words - 1 && (d_in & 31)) u &= (1u << (d_in & 31)) - 1u;
     const int c = __popc(u);
     int incl = c;
 #pragma unroll
@@ -73,28 +95,80 @@ __device__ __forceinline__ int list_rows(FusedSmem &s, const unsigned int *words
     if (lane == 31) s.wsum[warp] = incl;
     __syncthreads();
     int total;
-    const int before = warp_array_prefix(s.wsum, warp, lane, total);
-    int lo = 0, hi = total;
-    if (nparts > 1) {
-        // (part * total fits 32 bits: at most one part per SM, at most DIP_MAX_D rows)
-        lo = (int)((unsigned)part * (unsigned)total / (unsigned)nparts);
-        hi = (int)((unsigned)(part + 1) * (unsigned)total / (unsigned)nparts);
+    int rank = warp_array_prefix(s.wsum, warp, lane, total) + incl - c;
+    for (; u; u &= u - 1, ++rank)
+        if (rank >= lo && rank < hi) idx[rank - lo] = (uint16_t)(tid * 32 + __ffs(u) - 1);
+    __syncthreads();
+}
+
+// The sure columns (c of them flagged by this thread) whose rank among them lies in [lo, hi) to idx[], in the
+// order of the warps, their lanes, and the flags of put(emit)'s calls emit(base, flags, bit, column).
+// Deterministic, which is all that is asked of the order.  All threads call it; the barrier inside also
+// publishes what was written before the call; does not end with one.
+template <typename Put>
+__device__ __forceinline__ void list_sure(FusedSmem &s, int c, int lo, int hi, uint16_t *idx, const Put &put)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += n;
     }
-    int rank = before + incl - c;
-    if (rank < hi && rank + c > lo) {
-        uint16_t *out = idx + (rank - lo);
-        int col = tid * 32;
-        while (u) {
-            const int sh = __ffs(u);             // 1-based position of the next row's bit
-            col += sh;
-            u = sh < 32 ? u >> sh : 0u;
-            if (rank >= lo && rank < hi) *out = (uint16_t)(col - 1);
-            ++out;
-            ++rank;
+    if (lane == 31) s.wsum[warp] = incl;
+    __syncthreads();
+    const int at = (int)__reduce_add_sync(0xffffffffu, lane < warp ? (unsigned)s.wsum[lane] : 0u) + incl - c - lo;   // list place of the first
+    const unsigned n = (unsigned)(hi - lo);
+    // (every flag finds its place by itself: a walk from one set bit to the next is a chain of latencies)
+    if (at < hi - lo && at + c > 0)
+        put(at, [&](int base, uint32_t flags, int bit, int col) {
+            const unsigned place = (unsigned)(base + __popc(flags & ((1u << bit) - 1u)));
+            if (((flags >> bit) & 1u) && place < n) idx[place] = (uint16_t)col;
+        });
+}
+
+// One warp: the n_c columns of the threshold's bin (f.cand) are ranked by (full key descending,
+// column ascending), which inside one bin is the order of (low 16 key bits, column) in one word;
+// the first krem go to tie[] by rank, and into maskw when that is given.
+template <typename KeyOf>
+__device__ __forceinline__ void rank_ties(TkFine &f, int n_c, int krem, uint16_t *tie, unsigned int *maskw, const KeyOf &key_of)
+{
+    constexpr int PER = TK_TIE_LIMIT / 32;
+    const int lane = threadIdx.x & 31;
+    int col[PER];
+    uint32_t rk[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int c = lane + 32 * i;
+        rk[i] = 0u;
+        if (c < n_c) {
+            col[i] = f.cand[c];
+            rk[i] = key_of(col[i], c);
         }
     }
-    __syncthreads();
-    return hi - lo;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int c = lane + 32 * i;
+        if (c < n_c) rk[i] = ((rk[i] & 0xffffu) << 15) | (uint32_t)(0x7fff - col[i]);
+        if (32 * i < n_c) f.ckey[c] = rk[i];               // (zeros up to the end of the last 32: nobody's rank)
+    }
+    __syncwarp();
+    int rank[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) rank[i] = 0;
+    for (int j = 0; j < n_c; j += 4) {
+        const uint4 q = *reinterpret_cast<const uint4 *>(f.ckey + j);
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (32 * i < n_c) rank[i] += (int)(q.x > rk[i]) + (int)(q.y > rk[i]) + (int)(q.z > rk[i]) + (int)(q.w > rk[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+        if (lane + 32 * i < n_c && rank[i] < krem) {
+            tie[rank[i]] = (uint16_t)col[i];
+            if (maskw) atomicOr(&maskw[col[i] >> 5], 1u << (col[i] & 31));
+        }
+    __syncwarp();
 }
 
 // acc += sum over rows idx[first], idx[first + stride], ... below n_rows of row segment x value,
@@ -129,163 +203,418 @@ __device__ __forceinline__ void stream_rows(const uint16_t *idx, int first, int 
     }
 }
 
-// Block part * n_slabs + slab owns segment `slab`, row part `part`.  Dynamic shared memory:
-// FusedSmem, then keys[] (d_in words rounded up to four: rank keys, later this CTA's row list),
-// then for a chained gate/up input the d_in values of x.
-template <int WT, int WHICH, bool CA, bool NORM>
+// Block part * n_slabs + slab owns segment `slab`, row part `part`.  UPD: then come the blocks without rows, one
+// for each cache of u.beside, and last the one that completes the mask and updates this input's cache.  NQ =
+// chunks of columns per thread (gate/up: 4 columns each, down: 8).  Dynamic shared memory: FusedSmem, then d_in
+// words (rounded up to four: the CTA's row list; the updating block's copy of the stamps; under heavy ties the rank
+// keys before that), then for gate/up (x_near) the d_in values of x.  Shared memory is kept small: what it does not
+// take is L1, which the rows in flight pass through (with the 72 KB of h beside the rest, 224 KB in all, the down
+// product of 17920 dense rows took 11 us longer).
+template <int WT, int WHICH, bool CA, bool NORM, int NQ, bool UPD>
 __global__ void __launch_bounds__(TK_THREADS, 1)
-gemv_fused_kernel(const FusedParams p)
+gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdates, Int<0>> u)
 {
     constexpr int E = WTraits<WT>::E;
     constexpr int SLAB = 32 * E;
     constexpr int OUT_PER_SLAB = WHICH == 0 ? SLAB / 2 : SLAB;
-    constexpr int C = WTraits<WT>::C;
+    constexpr int W = WHICH == 0 ? 4 : 8;
+    static_assert(WTraits<WT>::C == E, "a lane's elements are all gate or all up, the next lane's their partners");
+    static_assert(!UPD || (CA && WHICH == 1), "updates ride with a down product that has a cache");
     extern __shared__ __align__(16) unsigned char dyn[];
     FusedSmem &s = *reinterpret_cast<FusedSmem *>(dyn);
     const int dpad = (p.d_in + 3) & ~3;
     uint32_t *keys = reinterpret_cast<uint32_t *>(dyn + sizeof(FusedSmem));
+    uint16_t *idx = reinterpret_cast<uint16_t *>(keys);
     float *xs = reinterpret_cast<float *>(keys + dpad);
 
     DIP_TRACE_MIN(p.tr, 0);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int slab = (int)blockIdx.x % p.n_slabs, part = (int)blockIdx.x / p.n_slabs, nparts = p.nparts;
-    const bool first = blockIdx.x == 0;
+    const int n_prod = p.n_slabs * nparts;
+    const bool updater = UPD && blockIdx.x == gridDim.x - 1;
+    const bool writer = UPD ? updater : (int)blockIdx.x == n_prod - 1;   // writes the mask (the last part ranks the ties anyway)
     const int mask_words = (p.d_in + 31) >> 5;
     const size_t byte_off = (size_t)slab * GF_SEG + lane * 16;
     const bool lane_ok = byte_off < p.row_bytes;
+    // this part's share of the k rows (part * k fits 32 bits: at most one part per SM, at most DIP_MAX_D rows)
+    const int lo = updater ? p.k : (int)((unsigned)part * (unsigned)p.k / (unsigned)nparts);
+    const int hi = updater ? p.k : (int)((unsigned)(part + 1) * (unsigned)p.k / (unsigned)nparts);
+    const bool every = p.k == p.d_in;                         // nothing to select
+    // position tid of a segment's sums (see below) is element `el`; gate/up: of output `o` if it is a gate element
+    const int el = E == 8 ? ((tid & 127) >> 2) * 8 + (tid >> 7) * 4 + (tid & 3) : tid;
+    const int o = WHICH == 0 ? (el / (2 * E)) * E + el % E : el;
+    const int j_out = slab * OUT_PER_SLAB + o;
+    const bool out_ok = tid < SLAB && (WHICH == 1 || ((tid >> 2) & 1) == 0) && j_out < p.d_out;
 
-    fine_zero(s.fine);
-    dip_grid_dependency_wait();
-    DIP_TRACE_MIN(p.tr, 1);
-    dip_launch_dependents();
+    bool staged = false;                                       // updater: keys[] is a copy of the stamps
+    if constexpr (UPD) {
+        if ((int)blockIdx.x >= n_prod) {
+            // (small[], like the select's histogram that lies there otherwise, and the counters)
+            if (!updater) cache_update_clear(s.ts, s.fine.hist);
+            else if (!every) fine_zero(s.fine);
+            dip_grid_dependency_wait();
+            dip_launch_dependents();
+            if (!updater) {
+                const dip_cache_update &c = u.beside.at[(int)blockIdx.x - n_prod];
+                block_cache_update_any(c.mask, c.d, c.stamp, c.stamp, c.count, c.meta, c.capacity, s.ts, s.fine.hist, []() {},
+                                       []() { return true; });
+                return;
+            }
+            // the stamps on their way to shared memory while the mask is made: once the other CTAs stream, a trip to
+            // global memory takes several microseconds
+            for (int q = tid; q < p.d_in / 4; q += TK_THREADS)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(keys + 4 * q)), "l"(p.stamp + 4 * q) : "memory");
+            staged = true;
+        }
+    }
+    if (!updater) {
+        if (!every) fine_zero(s.fine);
+        dip_grid_dependency_wait();
+        DIP_TRACE_MIN(p.tr, 1);
+        dip_launch_dependents();
+    }
 
     // the stamp that the epilogue's rank key needs travels while the rows stream
     int key_stamp = 0;
-    if (WHICH == 0 && p.key_coarse && p.key_stamp && tid < OUT_PER_SLAB && slab * OUT_PER_SLAB + tid < p.d_out)
-        key_stamp = __ldcg(p.key_stamp + slab * OUT_PER_SLAB + tid);
+    if (WHICH == 0 && p.key_coarse && p.key_stamp && out_ok) key_stamp = __ldcg(p.key_stamp + j_out);
 
-    // ---- the mask of the input, in every CTA ----
-    if (WHICH == 0) {
-        float *x_out = NORM && first ? p.x_out : nullptr;
-        if (NORM && (p.d_in & 3) == 0 && p.d_in <= 8 * TK_THREADS) {
-            __syncthreads();                                  // histogram zeroed
-            select_fine_chained<CA>(p.xa, p.xb, x_out, xs, p.d_in, p.k, p.gamma, p.stamp, keys, s.ts, s.fine, s.maskw);
+    // ---- the rank keys of the input and their histogram, in every CTA ----
+    const int n_q = p.d_in / W;
+    uint32_t kk[NQ][4];                    // gate/up: full keys of four columns; down: 16-bit keys of eight
+    if constexpr (WHICH == 0) {
+        // one trip to memory for x (or the two vectors that make it) and the stamps
+        float4 r[NQ];
+        int4 st[NQ];
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) {
+            const int q = tid + j * TK_THREADS;
+            r[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            st[j] = make_int4(0, 0, 0, 0);
+            if (q < n_q) {
+                r[j] = reinterpret_cast<const float4 *>(p.xa)[q];
+                if (CA) st[j] = reinterpret_cast<const int4 *>(p.stamp)[q];
+                if (NORM) {
+                    const float4 vb = reinterpret_cast<const float4 *>(p.xb)[q];
+                    r[j] = make_float4(r[j].x + vb.x, r[j].y + vb.y, r[j].z + vb.z, r[j].w + vb.w);
+                }
+            }
+        }
+        float scale = 1.0f;
+        if (NORM) {
+            // 1 / rms, summed in block_residual_scale's order
+            float ss = 0.f;
+#pragma unroll
+            for (int j = 0; j < NQ; ++j)
+                if (tid + j * TK_THREADS < n_q) {
+                    ss = fmaf(r[j].x, r[j].x, ss);
+                    ss = fmaf(r[j].y, r[j].y, ss);
+                    ss = fmaf(r[j].z, r[j].z, ss);
+                    ss = fmaf(r[j].w, r[j].w, ss);
+                }
+            scale = block_rms_scale(ss, p.d_in, s.ts.wf, &s.ts.scale);
         } else {
-            float scale = 1.0f;
-            if (NORM)
-                scale = block_residual_scale(p.xa, p.xb, p.d_in, keys, s.ts.wf, &s.ts.scale);   // ends with a barrier
-            else
-                __syncthreads();
-            select_fine<CA, NORM>(p.xa, x_out, NORM ? xs : nullptr, p.d_in, p.k, p.gamma, p.stamp, scale, keys, s.ts,
-                                  s.fine, s.maskw);
+            __syncthreads();               // histogram zeroed
+        }
+        float *x_out = NORM && blockIdx.x == 0 ? p.x_out : nullptr;
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) {
+            const int q = tid + j * TK_THREADS;
+            if (q < n_q) {
+                if (NORM) r[j] = make_float4(r[j].x * scale, r[j].y * scale, r[j].z * scale, r[j].w * scale);
+                if (x_out) reinterpret_cast<float4 *>(x_out)[q] = r[j];
+                if (NORM || p.x_near) reinterpret_cast<float4 *>(xs)[q] = r[j];
+                kk[j][0] = rank_key<CA>(r[j].x, st[j].x, p.gamma);
+                kk[j][1] = rank_key<CA>(r[j].y, st[j].y, p.gamma);
+                kk[j][2] = rank_key<CA>(r[j].z, st[j].z, p.gamma);
+                kk[j][3] = rank_key<CA>(r[j].w, st[j].w, p.gamma);
+                if (!every) {
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) fine_count_hi(s.fine, kk[j][t]);
+                }
+            }
         }
     } else {
-        __syncthreads();
-        select_fine_coarse<CA>(p.coarse, p.xa, p.stamp, p.gamma, p.d_in, p.k, keys, s.ts, s.fine, s.maskw);
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) {
+            const int q = tid + j * TK_THREADS;
+            if (q < n_q && !every) {
+                const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(p.coarse) + q);
+                kk[j][0] = v.x; kk[j][1] = v.y; kk[j][2] = v.z; kk[j][3] = v.w;
+            }
+        }
+        __syncthreads();                   // histogram zeroed
+#pragma unroll
+        for (int j = 0; j < NQ; ++j)
+            if (tid + j * TK_THREADS < n_q && !every) {
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    fine_count_lo(s.fine, kk[j][t]);
+                    fine_count_hi(s.fine, kk[j][t]);
+                }
+            }
     }
-    if (first)
-        for (int w = tid; w < mask_words; w += TK_THREADS) p.mask_out[w] = s.maskw[w];
 
-    // ---- this part's rows (the list lives where the rank keys were: d_in 16-bit entries always fit) ----
-    const float *xsrc = (WHICH == 0 && NORM) ? xs : p.xa;
-    uint16_t *idx = reinterpret_cast<uint16_t *>(keys);
-    float acc[E];
+    // ---- this part's rows: n_list of them in idx[], and ranks tie_lo .. tie_hi - 1 of the ties in s.tie ----
+    int n_list = hi - lo, tie_lo = 0, tie_hi = 0;
+    int krem = 0, n_c = 0;
+    if (every) {
+        for (int r = tid; r < n_list; r += TK_THREADS) idx[r] = (uint16_t)(lo + r);
+        if (writer)
+            for (int w = tid; w < mask_words; w += TK_THREADS) s.maskw[w] = 0xffffffffu;
+        __syncthreads();
+    } else {
+        __syncthreads();
+        fine_find(s.fine, s.ts, p.k);
+        const uint32_t b = (uint32_t)s.ts.bcast[0];
+        krem = s.ts.bcast[1];
+        n_c = s.ts.bcast[2];
+        if (n_c > TK_TIE_LIMIT) {
+            // masses of equal keys: the general select on full keys
+            if (staged) {
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                staged = false;
+            }
+            __syncthreads();
+            if constexpr (WHICH == 0) {
 #pragma unroll
-    for (int e = 0; e < E; ++e) acc[e] = 0.f;
-    const int n_rows = list_rows(s, s.maskw, mask_words, p.d_in, part, nparts, idx);
-    stream_rows<WT>(idx, warp, GF_NW, n_rows, p.W + byte_off, p.row_bytes, lane_ok, xsrc, acc);
-    DIP_TRACE_MAX(p.tr, 3);            // streaming done
-
-    // ---- the warps' sums, in warp order ----
-    float (*red)[32 * 8] = reinterpret_cast<float (*)[32 * 8]>(s.fine.hist);
+                for (int j = 0; j < NQ; ++j)
+                    if (tid + j * TK_THREADS < n_q)
+                        *reinterpret_cast<uint4 *>(keys + 4 * (tid + j * TK_THREADS)) = make_uint4(kk[j][0], kk[j][1], kk[j][2], kk[j][3]);
+            } else {
+                for (int e = tid; e < p.d_in; e += TK_THREADS) keys[e] = rank_key<CA>(p.xa[e], CA ? p.stamp[e] : 0, p.gamma);
+            }
+            __syncthreads();
+            general_select(keys, p.d_in, p.k, s.ts, s.maskw);
+            __syncthreads();
+            list_rows(s, s.maskw, mask_words, lo, hi, idx);
+            n_c = 0;
+        } else {
+            // Columns above the bin: flags gt; the bin's columns: candidates (in any order).  Flag bit of column
+            // t of a group: gate/up: t; down, whose keys are compared two at a time (the top bit of each half
+            // survives the subtraction where the key is no smaller): 12 + t / 2, in the upper half for odd t
+            uint32_t gt[NQ], eqs[NQ];
+            int c_gt = 0, c_eq = 0;
+            const uint32_t above = (b << 16) | 0xffffu;       // a full key above the bin is larger than this
+            const uint32_t ge1 = (b + 1) * 0x10001u, ge0 = b * 0x10001u;
+            constexpr uint32_t TOP = 0x80008000u;
 #pragma unroll
-    for (int e = 0; e < E; ++e) red[warp][lane * E + e] = acc[e];
-    __syncthreads();
-    if (tid < SLAB) {
-        float t = 0.f;
+            for (int j = 0; j < NQ; ++j) {
+                gt[j] = eqs[j] = 0u;
+                const int q = tid + j * TK_THREADS;
+                if (q < n_q) {
+                    uint32_t eq = 0u;
+                    if constexpr (WHICH == 0) {
 #pragma unroll
-        for (int w = 0; w < GF_NW; ++w) t += red[w][tid];
-        if (nparts > 1) p.partials[((size_t)part * p.n_slabs + slab) * SLAB + tid] = t;
-        else s.sum[tid] = t;
+                        for (int t = 0; t < 4; ++t) {
+                            if (kk[j][t] > above) gt[j] |= 1u << t;
+                            if (kk[j][t] >= (b << 16)) eq |= 1u << t;
+                        }
+                    } else {
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) {
+                            const uint32_t w = kk[j][t] | TOP;
+                            gt[j] |= ((w - ge1) & TOP) >> (3 - t);
+                            eq |= ((w - ge0) & TOP) >> (3 - t);
+                        }
+                    }
+                    eqs[j] = eq & ~gt[j];
+                    c_gt += __popc(gt[j]);
+                    c_eq += __popc(eqs[j]);
+                }
+                if (writer && (tid & ~31) + j * TK_THREADS < n_q) {      // (the whole warp or none of it)
+                    constexpr int LANES = 32 / W;                        // lanes per mask word
+                    uint32_t w = gt[j];
+                    if (WHICH == 1) {
+                        w = 0u;
+#pragma unroll
+                        for (int t = 0; t < 8; ++t) w |= ((gt[j] >> (12 + t / 2 + 16 * (t & 1))) & 1u) << t;
+                    }
+                    w <<= W * (lane % LANES);
+#pragma unroll
+                    for (int m = 1; m < LANES; m <<= 1) w |= __shfl_xor_sync(0xffffffffu, w, m);
+                    if (lane % LANES == 0 && q < n_q) s.maskw[q / LANES] = w;
+                }
+            }
+            if (c_eq) {
+                int slot = atomicAdd(&s.fine.n_cand, c_eq);
+#pragma unroll
+                for (int j = 0; j < NQ; ++j)
+                    for (uint32_t eq = eqs[j]; eq; eq &= eq - 1, ++slot) {
+                        const int f = __ffs(eq) - 1, t = WHICH == 0 ? f : 2 * (f & 3) + (f >> 4);
+                        s.fine.cand[slot] = (uint16_t)(W * (tid + j * TK_THREADS) + t);
+                        if (WHICH == 0) s.fine.ckey[slot] = t == 0 ? kk[j][0] : t == 1 ? kk[j][1] : t == 2 ? kk[j][2] : kk[j][3];
+                    }
+            }
+            const int n_sure = p.k - krem;
+            n_list = max(0, min(hi, n_sure) - lo);
+            tie_lo = max(lo, n_sure) - n_sure;
+            tie_hi = max(hi, n_sure) - n_sure;
+            list_sure(s, c_gt, lo, hi, idx, [&](int base, const auto &emit) {
+#pragma unroll
+                for (int j = 0; j < NQ; ++j) {
+                    if (j * TK_THREADS >= n_q) break;
+#pragma unroll
+                    for (int t = 0; t < W; ++t)
+                        emit(base, gt[j], WHICH == 0 ? t : 12 + t / 2 + 16 * (t & 1), W * (tid + j * TK_THREADS) + t);
+                    base += __popc(gt[j]);
+                }
+            });
+            __syncthreads();
+        }
     }
-    // ---- the parts, in part order, by the last CTA of the segment ----
-    if (nparts > 1) {
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) s.last = atomicAdd(&p.tickets[slab], 1u) == (unsigned)(nparts - 1);
-        __syncthreads();
-        if (!s.last) {
+
+    const bool ranks = n_c > 0 && (tie_lo < tie_hi || writer);
+    const auto tie_key = [&](int col, int c) {
+        return WHICH == 0 ? s.fine.ckey[c] : rank_key<CA>(__ldcg(p.xa + col), CA ? __ldcg(p.stamp + col) : 0, p.gamma);
+    };
+    if constexpr (UPD) {
+        if (updater) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            if (ranks && warp == 0) rank_ties(s.fine, n_c, krem, s.tie, s.maskw, tie_key);
+            __syncthreads();
+            for (int w = tid; w < mask_words; w += TK_THREADS) p.mask_out[w] = s.maskw[w];
+            cache_update_clear(s.ts, s.fine.hist);
+            // The stamps may change once every block with rows has read them.  Blocks start in index order and this is
+            // the last one, so all the others are running or done
+            block_cache_update_any(
+                s.maskw, p.d_in, staged ? reinterpret_cast<const int32_t *>(keys) : p.stamp, u.own.stamp, u.own.count, u.own.meta,
+                u.own.capacity, s.ts, s.fine.hist,
+                [&]() {
+                    if (lane == 0) {
+                        s.go = wait_count(u.readers, (unsigned)n_prod, p.status, p.wait_limit_ns);
+                        *u.readers = 0u;                       // ready for the next launch
+                    }
+                },
+                [&]() {
+                    __syncthreads();
+                    return s.go != 0;
+                });
             DIP_TRACE_MAX(p.tr, 2);
             return;
         }
-        __threadfence();
-        if (tid < SLAB) {
-            const size_t stride = (size_t)p.n_slabs * SLAB;
-            const float *pp = p.partials + (size_t)slab * SLAB + tid;
-            float t = 0.f;
-            for (int q0 = 0; q0 < nparts; q0 += 8) {
-                float a[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) a[q] = q0 + q < nparts ? __ldcg(pp + (size_t)(q0 + q) * stride) : 0.f;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) t += a[q];
-            }
-            s.sum[tid] = t;
-        }
-        if (tid == 0) p.tickets[slab] = 0;                    // ready for the next launch
     }
+
+    // ---- stream.  Where this CTA ranks ties, warp 0 does that first, takes their rows, and gets so many fewer of
+    //      the listed ones ----
+    const float *xsrc = WHICH == 0 && (NORM || p.x_near) ? xs : p.xa;
+    const char *base = p.W + byte_off;
+    float acc[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) acc[e] = 0.f;
+    int n_even = n_list;                                       // rows shared out over all warps
+    if (ranks) {
+        n_even = min(n_list, max(0, (n_list + tie_hi - tie_lo) / GF_NW - (tie_hi - tie_lo) - GF_U) * GF_NW);
+        if (warp == 0) {
+            rank_ties(s.fine, n_c, krem, s.tie, writer ? s.maskw : nullptr, tie_key);
+            if constexpr (UPD) {
+                if (lane == 0) count_one(u.readers);
+            }
+            stream_rows<WT>(s.tie, tie_lo, 1, tie_hi, base, p.row_bytes, lane_ok, xsrc, acc);
+        }
+    } else if constexpr (UPD) {
+        if (tid == 0) count_one(u.readers);                    // (the stamps were read before the last barrier)
+    }
+    stream_rows<WT>(idx, warp, GF_NW, n_even, base, p.row_bytes, lane_ok, xsrc, acc);
+    if (warp > 0 && n_even < n_list)
+        stream_rows<WT>(idx, n_even + warp - 1, GF_NW - 1, n_list, base, p.row_bytes, lane_ok, xsrc, acc);
+    DIP_TRACE_MAX(p.tr, 3);            // streaming done
+
+    // ---- the warps' sums, in warp order.  Element e of lane l lies at position (e / 4) * 128 + 4 l + e % 4 ----
+    float *red = reinterpret_cast<float *>(s.fine.hist), *psum = red + TK_FINE_WORDS / 2;
+#pragma unroll
+    for (int h = 0; h < E / 4; ++h)
+        *reinterpret_cast<float4 *>(red + warp * SLAB + h * 128 + lane * 4) =
+            make_float4(acc[4 * h], acc[4 * h + 1], acc[4 * h + 2], acc[4 * h + 3]);
     __syncthreads();
+    constexpr int G = TK_THREADS / SLAB;                       // threads per position
+    {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < GF_NW / G; ++w) t += red[((tid / SLAB) * (GF_NW / G) + w) * SLAB + tid % SLAB];
+        psum[tid] = t;
+    }
+    if (writer)
+        for (int w = tid; w < mask_words; w += TK_THREADS) p.mask_out[w] = s.maskw[w];
+    __syncthreads();
+    if (tid >= SLAB) return;
+    float t = 0.f;
+#pragma unroll
+    for (int g = 0; g < G; ++g) t += psum[g * SLAB + tid];
+    // ---- the parts, in part order, in the last part's CTA.  A sum is its own message: the CTA that adds them up
+    //      waits until none of its inputs is "empty" any more, and empties them for the next launch.  Blocks start
+    //      in index order and only the last ones wait, so what they wait for is running or done ----
+    if (nparts > 1) {
+        const size_t stride = (size_t)p.n_slabs * SLAB;
+        float *box = p.mail + (size_t)slab * SLAB + tid;
+        if (part != nparts - 1) {
+            mail_put(box + (size_t)part * stride, t);
+            DIP_TRACE_MAX(p.tr, 2);
+            return;
+        }
+        float sum = 0.f;
+        for (int q0 = 0; q0 < nparts - 1; q0 += 8) {
+            float a[8];
+            mail_take<8>(box + (size_t)q0 * stride, stride, nparts - 1 - q0, a, p.status, p.wait_limit_ns);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) sum += a[q];
+        }
+        t = sum + t;
+    }
     // ---- epilogue ----
-    if (tid < OUT_PER_SLAB) {
-        const int o = tid, j = slab * OUT_PER_SLAB + o;
-        if (j < p.d_out) {
-            float r;
-            if (WHICH == 0) {
-                const int e0 = (o / C) * 2 * C + (o % C);     // gate element; its up element is C further
-                r = silu_f32(s.sum[e0]) * s.sum[e0 + C];
-            } else {
-                r = s.sum[o];
-            }
-            p.out[j] = r;
-            if (WHICH == 0 && p.key_coarse) {
-                // what the select would form from h_j and the stamp, cut to its top 16 bits
-                float a = fabsf(r);
-                if (p.key_stamp) a = __fmul_rn(a, key_stamp >= 0 ? 1.0f : p.key_gamma);
-                p.key_coarse[j] = (uint16_t)((__float_as_uint(a) & 0x7fffffffu) >> 16);
-            }
+    const float up = __shfl_down_sync(0xffffffffu, t, 4);      // gate/up: a gate element's up element is four positions on
+    if (out_ok) {
+        const float r = WHICH == 0 ? silu_f32(t) * up : t;
+        p.out[j_out] = r;
+        if (WHICH == 0 && p.key_coarse) {
+            // what the select would form from h_j and the stamp, cut to its top 16 bits
+            float a = fabsf(r);
+            if (p.key_stamp) a = __fmul_rn(a, key_stamp >= 0 ? 1.0f : p.key_gamma);
+            p.key_coarse[j_out] = (uint16_t)((__float_as_uint(a) & 0x7fffffffu) >> 16);
         }
     }
     DIP_TRACE_MAX(p.tr, 2);
 }
 
-template <int WT, int WHICH, bool CA, bool NORM>
-dip_status launch_fused(dip_ctx *ctx, const FusedParams &p, size_t smem, cudaStream_t stream)
+template <int WT, int WHICH, bool CA, bool NORM, int NQ, bool UPD>
+dip_status launch_fused(dip_ctx *ctx, const FusedParams &p, const std::conditional_t<UPD, FusedUpdates, Int<0>> &u, int extra,
+                        size_t smem, cudaStream_t stream)
 {
     static dip_per_device_once once;
-    DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once, ctx->device, gemv_fused_kernel<WT, WHICH, CA, NORM>, GF_SMEM_LIMIT));
-    DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_fused_kernel<WT, WHICH, CA, NORM>, dim3(p.n_slabs * p.nparts),
-                                     dim3(TK_THREADS), smem, stream, p));
+    DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once, ctx->device, gemv_fused_kernel<WT, WHICH, CA, NORM, NQ, UPD>, GF_SMEM_LIMIT));
+    DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_fused_kernel<WT, WHICH, CA, NORM, NQ, UPD>, dim3(p.n_slabs * p.nparts + extra),
+                                     dim3(TK_THREADS), smem, stream, p, u));
     return DIP_OK;
 }
 
-template <int WT>
-dip_status launch_fused_wt(dip_ctx *ctx, const FusedParams &p, int which, bool ca, bool norm, size_t smem,
-                           cudaStream_t stream)
+// Columns per thread: a row's keys stay in registers, so the variant for wide inputs (which spills) only takes
+// what the narrow one cannot.
+template <int WT, bool CA, bool NORM>
+dip_status launch_fused_gate_up(dip_ctx *ctx, const FusedParams &p, size_t smem, cudaStream_t stream)
 {
-    if (which == 0) {
-        if (ca) return norm ? launch_fused<WT, 0, true, true>(ctx, p, smem, stream)
-                            : launch_fused<WT, 0, true, false>(ctx, p, smem, stream);
-        return norm ? launch_fused<WT, 0, false, true>(ctx, p, smem, stream)
-                    : launch_fused<WT, 0, false, false>(ctx, p, smem, stream);
-    }
-    return ca ? launch_fused<WT, 1, true, false>(ctx, p, smem, stream)
-              : launch_fused<WT, 1, false, false>(ctx, p, smem, stream);
+    if (p.d_in <= 2 * 4 * TK_THREADS) return launch_fused<WT, 0, CA, NORM, 2, false>(ctx, p, Int<0>(), 0, smem, stream);
+    return launch_fused<WT, 0, CA, NORM, TK_VEC_ITERS, false>(ctx, p, Int<0>(), 0, smem, stream);
 }
 
-size_t fused_smem_bytes(int which, int d_in, bool norm)
+template <int WT>
+dip_status launch_fused_wt(dip_ctx *ctx, const FusedParams &p, int which, bool ca, bool norm, const FusedUpdates *u,
+                           size_t smem, cudaStream_t stream)
+{
+    if (which == 0) {
+        if (ca) return norm ? launch_fused_gate_up<WT, true, true>(ctx, p, smem, stream)
+                            : launch_fused_gate_up<WT, true, false>(ctx, p, smem, stream);
+        return norm ? launch_fused_gate_up<WT, false, true>(ctx, p, smem, stream)
+                    : launch_fused_gate_up<WT, false, false>(ctx, p, smem, stream);
+    }
+    constexpr int NQ = TK_COARSE_ITERS;
+    if (u) return launch_fused<WT, 1, true, false, NQ, true>(ctx, p, *u, u->beside.n + 1, smem, stream);
+    return ca ? launch_fused<WT, 1, true, false, NQ, false>(ctx, p, Int<0>(), 0, smem, stream)
+              : launch_fused<WT, 1, false, false, NQ, false>(ctx, p, Int<0>(), 0, smem, stream);
+}
+
+size_t fused_smem_bytes(int d_in, bool x_near)
 {
     const size_t dpad = ((size_t)d_in + 3) & ~(size_t)3;
-    return sizeof(FusedSmem) + dpad * 4 + (which == 0 && norm ? dpad * 4 : 0);
+    return sizeof(FusedSmem) + dpad * 4 + (x_near ? dpad * 4 : 0);
 }
 
 // Segments and row parts of a launch; false when the shape does not fit this path.
@@ -296,20 +625,26 @@ bool fused_plan(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool no
     p.d_in = which == 0 ? w->d_model : w->d_ff;
     p.d_out = which == 0 ? w->d_ff : w->d_model;
     if (which == 1 && ((p.d_in & 31) != 0 || p.d_in > 8 * TK_COARSE_ITERS * TK_THREADS)) return false;
-    if (fused_smem_bytes(which, p.d_in, norm) > GF_SMEM_LIMIT) return false;
+    p.x_near = which == 0 && fused_smem_bytes(p.d_in, true) <= GF_SMEM_LIMIT;
+    if ((norm && !p.x_near) || fused_smem_bytes(p.d_in, false) > GF_SMEM_LIMIT) return false;
     const size_t row_elems = which == 0 ? (size_t)2 * w->d_ff : (size_t)w->d_model;
     p.row_bytes = w->wtype == DIP_W_F32 ? row_elems * 4 : row_elems * 2;
     p.n_slabs = (int)((p.row_bytes + GF_SEG - 1) / GF_SEG);
-    if (p.n_slabs > ctx->n_tickets) return false;
-    const int slab_elems = w->wtype == DIP_W_F32 ? 128 : 256;
-    int nparts = ctx->sm_count / p.n_slabs;
-    if (nparts < 1) nparts = 1;
-    while (nparts > 1 && (size_t)nparts * p.n_slabs * slab_elems > ctx->partials_floats) --nparts;
-    p.nparts = nparts;
+    // one CTA per SM, and where that is cheap two SMs to spare for the blocks that update caches
+    p.nparts = ctx->sm_count / p.n_slabs;              // (DIP_MAIL_FLOATS per SM suffice)
+    if (p.nparts > 4 && p.nparts * p.n_slabs > ctx->sm_count - 2) --p.nparts;
+    if (p.nparts < 1) p.nparts = 1;
     return true;
 }
 
 }  // namespace
+
+int dip_gemv_fused_update_room(const dip_ctx *ctx, const dip_mlp_weights *w)
+{
+    FusedParams p;
+    // (a wave of products that fills the SMs to the last one leaves none)
+    return fused_plan(ctx, w, 1, false, p) ? (ctx->sm_count - p.n_slabs * p.nparts % ctx->sm_count) % ctx->sm_count : 0;
+}
 
 bool dip_gemv_fused_supported(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool norm)
 {
@@ -326,8 +661,9 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
     if (p.nparts > sel->k) p.nparts = sel->k;
     p.W = (const char *)(which == 0 ? w->gate_up : w->down);
     p.out = out;
-    p.partials = ctx->partials;
-    p.tickets = ctx->tickets;
+    p.mail = ctx->mail;
+    p.status = ctx->status;
+    p.wait_limit_ns = ctx->wait_limit_ns;
     p.tr = dip_trace_slot(ctx, which == 0 ? 4 : 5);
     p.key_coarse = nullptr;
     p.key_stamp = nullptr;
@@ -347,7 +683,15 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
     p.gamma = sel->gamma;
     p.stamp = sel->stamp;
     p.mask_out = sel->mask_out;
-    const size_t smem = fused_smem_bytes(which, p.d_in, norm);
-    return w->wtype == DIP_W_F32 ? launch_fused_wt<DIP_W_F32>(ctx, p, which, sel->stamp != nullptr, norm, smem, stream)
-                                 : launch_fused_wt<DIP_W_BF16>(ctx, p, which, sel->stamp != nullptr, norm, smem, stream);
+    const size_t smem = fused_smem_bytes(p.d_in, p.x_near);
+    FusedUpdates u;
+    if (sel->update) {
+        u.readers = ctx->readers;
+        u.own = dip_update_of(sel->update, nullptr);
+        u.beside.n = 0;
+        if (sel->beside) u.beside = *sel->beside;
+    }
+    const FusedUpdates *up = sel->update ? &u : nullptr;
+    return w->wtype == DIP_W_F32 ? launch_fused_wt<DIP_W_F32>(ctx, p, which, sel->stamp != nullptr, norm, up, smem, stream)
+                                 : launch_fused_wt<DIP_W_BF16>(ctx, p, which, sel->stamp != nullptr, norm, up, smem, stream);
 }

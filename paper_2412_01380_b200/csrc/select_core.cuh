@@ -14,6 +14,8 @@ constexpr int TK_WARPS = TK_THREADS / 32;
 constexpr int RADIX_BITS = 11;
 constexpr int RADIX_BINS = 1 << RADIX_BITS;   // two bins per thread
 
+template <int N> struct Int { static constexpr int value = N; };
+
 struct TkShared {
     unsigned int hist[RADIX_BINS];
     int bcast[4];
@@ -147,6 +149,28 @@ __device__ void block_radix_select(const uint32_t *keys, int d, uint32_t keymask
 constexpr int TK_VEC_ITERS = DIP_MAX_D / 4 / TK_THREADS;   // float4 loads per thread at the largest d
 constexpr int TK_VEC_BATCH = 5;                            // of which this many are in flight together
 
+// 1 / rms of d elements whose squares the threads of the CTA have summed up in ss: a shuffle tree per
+// warp, then one over the warps; the same bits on every thread.  Ends with a barrier (two inside).
+__device__ __forceinline__ float block_rms_scale(float ss, int d, float *wf, float *scale_slot)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if (lane == 0) wf[warp] = ss;
+    __syncthreads();
+    if (warp == 0) {
+        float v = wf[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) {
+            const float rms = sqrtf(v / (float)d);
+            *scale_slot = rms > 0.f ? 1.0f / rms : 1.0f;
+        }
+    }
+    __syncthreads();
+    return *scale_slot;
+}
+
 // scale = 1 / rms(xa + xb) over d elements, the same bits on every thread of the CTA.  The sums
 // r = xa + xb are optionally parked in stash[] (as bit patterns).  Summation order: each thread
 // adds its elements in index order (16-byte groups tid, tid + 1024, ... when d % 4 == 0, single
@@ -155,7 +179,7 @@ constexpr int TK_VEC_BATCH = 5;                            // of which this many
 __device__ float block_residual_scale(const float *__restrict__ xa, const float *__restrict__ xb, int d,
                                       uint32_t *stash, float *wf, float *scale_slot)
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x;
     float ss = 0.f;
     if ((d & 3) == 0) {
         const float4 *a4 = reinterpret_cast<const float4 *>(xa), *b4 = reinterpret_cast<const float4 *>(xb);
@@ -192,21 +216,7 @@ __device__ float block_residual_scale(const float *__restrict__ xa, const float 
             ss = fmaf(r, r, ss);
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if (lane == 0) wf[warp] = ss;
-    __syncthreads();
-    if (warp == 0) {
-        float v = wf[lane];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) {
-            const float rms = sqrtf(v / (float)d);
-            *scale_slot = rms > 0.f ? 1.0f / rms : 1.0f;
-        }
-    }
-    __syncthreads();
-    return *scale_slot;
+    return block_rms_scale(ss, d, wf, scale_slot);
 }
 
 // General path (very many keys tied around the threshold): full radix select on all d keys in
@@ -289,61 +299,67 @@ __device__ __forceinline__ void fine_zero(TkFine &f)
     if (tid == 0) f.n_cand = 0;
 }
 
-// Counter of bin c15: logical word w = c15 / 2 (low half: even bin) is stored at (w % 16) * 1024 + w / 16, so
-// that the 16 words of thread t = w / 16 in fine_find are a conflict-free stride apart.
-__device__ __forceinline__ void fine_count(TkFine &f, uint32_t c15)
+// Counter of bin c15: half c15 % 2 of word c15 / 2.  fine_count_lo / _hi take the bin from the lower /
+// upper 16 bits of w (top bit zero): the byte offset of the word is a shift and a mask.
+__device__ __forceinline__ void fine_count_at(TkFine &f, uint32_t byte_off, bool odd)
 {
-    const uint32_t w = c15 >> 1;
-    atomicAdd(&f.hist[((w & 15u) << 10) | (w >> 4)], (c15 & 1u) ? 0x10000u : 1u);
+    atomicAdd(reinterpret_cast<unsigned int *>(reinterpret_cast<char *>(f.hist) + byte_off), odd ? 0x10000u : 1u);
 }
+__device__ __forceinline__ void fine_count_lo(TkFine &f, uint32_t w) { fine_count_at(f, (w << 1) & 0xfffcu, w & 1u); }
+__device__ __forceinline__ void fine_count_hi(TkFine &f, uint32_t w) { fine_count_at(f, (w >> 15) & 0xfffcu, w & 0x10000u); }
 
 // The bin of the k-th largest key: s.bcast[0] = bin, [1] = rank of the wanted key inside it (from
-// the top, 1-based), [2] = keys in the bin.  Thread t owns bins 32 t .. 32 t + 31.  All threads
-// call it; the histogram must be complete and visible; ends with a barrier.
+// the top, 1-based), [2] = keys in the bin.  Warp w owns bins 1024 w .. 1024 w + 1023 and only adds them
+// up (every instruction here costs 32 warps' issue slots); the one warp that holds the wanted key looks
+// closer.  All threads call it; the histogram must be complete and visible; ends with a barrier.
 __device__ __forceinline__ void fine_find(const TkFine &f, TkShared &s, int k)
 {
     static_assert(TK_FINE_WORDS == 16 * TK_THREADS, "sixteen words per thread");
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t wv[16];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // 16 bytes = 8 bins, ascending over (block i of 256 bins, lane)
+    const uint4 *own = reinterpret_cast<const uint4 *>(f.hist) + warp * 128 + lane;
+    uint32_t sum[4];                             // both halves of a word counted in one (each at most DIP_MAX_D)
 #pragma unroll
-    for (int i = 0; i < 16; ++i) wv[i] = f.hist[(i << 10) | tid];
-    int own = 0;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) own += (int)(wv[i] & 0xffffu) + (int)(wv[i] >> 16);
-    int suf = own;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int n = __shfl_down_sync(0xffffffffu, suf, o);
-        if (lane + o < 32) suf += n;
+    for (int i = 0; i < 4; ++i) {
+        const uint4 v = own[32 * i];
+        sum[i] = (v.x + v.y) + (v.z + v.w);
     }
-    if (lane == 0) s.wa[warp] = suf;
+    const uint32_t all = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+    const int total = (int)__reduce_add_sync(0xffffffffu, (all & 0xffffu) + (all >> 16));
+    if (lane == 0) s.wa[warp] = total;
     __syncthreads();
-    int wsum = s.wa[lane], wsuf = wsum;
+    int cum = (int)__reduce_add_sync(0xffffffffu, lane > warp ? (unsigned)s.wa[lane] : 0u);   // keys above this warp's bins
+    if (cum < k && k <= cum + total) {
+        int in_lane = 0, blk = 3;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int n = __shfl_down_sync(0xffffffffu, wsuf, o);
-        if (lane + o < 32) wsuf += n;
-    }
-    const int cum = __shfl_sync(0xffffffffu, wsuf - wsum, warp) + suf - own;     // keys in bins above this thread's
-    // the owner of the k-th key's bins hands them to its warp: a lane per bin
-    const unsigned owner = __ballot_sync(0xffffffffu, cum < k && k <= cum + own);
-    if (owner) {
-        const int ol = __ffs(owner) - 1;
-        const int ot = (tid & ~31) | ol;
-        const int ocum = __shfl_sync(0xffffffffu, cum, ol);
-        const uint32_t wl = f.hist[((lane >> 1) << 10) | ot];
-        const int cnt = (lane & 1) ? (int)(wl >> 16) : (int)(wl & 0xffffu);
-        int bsuf = cnt;                          // inclusive suffix over the 32 bins, top bin = lane 31
+        for (int i = 3; i >= 0; --i) {
+            const int mine = (int)((sum[i] & 0xffffu) + (sum[i] >> 16));
+            const int t = (int)__reduce_add_sync(0xffffffffu, (unsigned)mine);
+            in_lane = mine;
+            blk = i;
+            if (k <= cum + t) break;             // (uniform)
+            cum += t;
+        }
+        int suf = in_lane;                       // inclusive suffix over the lanes
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            int n = __shfl_down_sync(0xffffffffu, bsuf, o);
-            if (lane + o < 32) bsuf += n;
+            const int n = __shfl_down_sync(0xffffffffu, suf, o);
+            if (lane + o < 32) suf += n;
         }
-        const int above = ocum + bsuf - cnt;
-        if (above < k && k <= above + cnt) {
-            s.bcast[0] = 32 * ot + lane;
-            s.bcast[1] = k - above;
-            s.bcast[2] = cnt;
+        cum += suf - in_lane;                    // keys above this lane's eight bins
+        if (cum < k && k <= cum + in_lane) {
+            const uint4 v = own[32 * blk];
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 7; i >= 0; --i) {
+                const int c = (int)((i & 1) ? w[i >> 1] >> 16 : w[i >> 1] & 0xffffu);
+                if (cum < k && k <= cum + c) {
+                    s.bcast[0] = 8 * (warp * 128 + 32 * blk + lane) + i;
+                    s.bcast[1] = k - cum;
+                    s.bcast[2] = c;
+                }
+                cum += c;
+            }
         }
     }
     __syncthreads();
@@ -423,10 +439,10 @@ __device__ __forceinline__ void select_fine_tail(const uint32_t *keys, int d, in
 
 // The whole select of one row from full rank keys.  On entry f is zero (and that is visible); with
 // NORM, keys[] holds the bits of r = xa + xb and `scale` is 1 / rms(r), without NORM the row is
-// xa.  The row's values go to x_out and / or x_keep when given, the rank keys to keys[], the mask
-// (complete) to maskw[], all in shared memory except x_out.  Ends with a barrier.
+// xa.  The row's values go to x_out when given, the rank keys to keys[], the mask (complete) to maskw[],
+// all in shared memory except x_out.  Ends with a barrier.
 template <bool CA, bool NORM>
-__device__ __forceinline__ void select_fine(const float *__restrict__ xa, float *__restrict__ x_out, float *x_keep, int d,
+__device__ __forceinline__ void select_fine(const float *__restrict__ xa, float *__restrict__ x_out, int d,
                                             int k, float gamma, const int32_t *__restrict__ stamp, float scale,
                                             uint32_t *keys, TkShared &s, TkFine &f, unsigned int *maskw)
 {
@@ -455,14 +471,13 @@ __device__ __forceinline__ void select_fine(const float *__restrict__ xa, float 
             const int q = tid + (j0 + j) * TK_THREADS;
             if (q < n4) {
                 if (x_out) reinterpret_cast<float4 *>(x_out)[q] = v4[j];
-                if (x_keep) reinterpret_cast<float4 *>(x_keep)[q] = v4[j];
                 const float vv[4] = {v4[j].x, v4[j].y, v4[j].z, v4[j].w};
                 const int sv[4] = {CA ? st4[j].x : 0, CA ? st4[j].y : 0, CA ? st4[j].z : 0, CA ? st4[j].w : 0};
                 uint32_t kk[4];
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     kk[t] = rank_key<CA>(vv[t], sv[t], gamma);
-                    fine_count(f, kk[t] >> 16);
+                    fine_count_hi(f, kk[t]);
                 }
                 *reinterpret_cast<uint4 *>(keys + 4 * q) = make_uint4(kk[0], kk[1], kk[2], kk[3]);
             }
@@ -474,10 +489,9 @@ __device__ __forceinline__ void select_fine(const float *__restrict__ xa, float 
             if (NORM) v = __uint_as_float(keys[e]) * scale;
             else v = xa[e];
             if (x_out) x_out[e] = v;
-            if (x_keep) x_keep[e] = v;
             const uint32_t key = rank_key<CA>(v, CA ? stamp[e] : 0, gamma);
             keys[e] = key;
-            fine_count(f, key >> 16);
+            fine_count_hi(f, key);
         }
     }
     select_fine_tail(keys, d, k, s, f, maskw);
@@ -488,11 +502,11 @@ __device__ __forceinline__ void select_fine(const float *__restrict__ xa, float 
 // one trip to memory instead of two.  Same summation order as block_residual_scale, same bits.
 template <bool CA>
 __device__ __forceinline__ void select_fine_chained(const float *__restrict__ xa, const float *__restrict__ xb,
-                                                    float *__restrict__ x_out, float *x_keep, int d, int k, float gamma,
+                                                    float *__restrict__ x_out, int d, int k, float gamma,
                                                     const int32_t *__restrict__ stamp, uint32_t *keys, TkShared &s,
                                                     TkFine &f, unsigned int *maskw)
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x;
     const int n4 = d >> 2;
     float4 r[2];
     int4 st[2];
@@ -517,35 +531,20 @@ __device__ __forceinline__ void select_fine_chained(const float *__restrict__ xa
             ss = fmaf(r[j].w, r[j].w, ss);
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if (lane == 0) s.wf[warp] = ss;
-    __syncthreads();
-    if (warp == 0) {
-        float v = s.wf[lane];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) {
-            const float rms = sqrtf(v / (float)d);
-            s.scale = rms > 0.f ? 1.0f / rms : 1.0f;
-        }
-    }
-    __syncthreads();
-    const float scale = s.scale;
+    const float scale = block_rms_scale(ss, d, s.wf, &s.scale);
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         const int q = tid + j * TK_THREADS;
         if (q < n4) {
             const float4 v4 = make_float4(r[j].x * scale, r[j].y * scale, r[j].z * scale, r[j].w * scale);
             if (x_out) reinterpret_cast<float4 *>(x_out)[q] = v4;
-            if (x_keep) reinterpret_cast<float4 *>(x_keep)[q] = v4;
             const float vv[4] = {v4.x, v4.y, v4.z, v4.w};
             const int sv[4] = {st[j].x, st[j].y, st[j].z, st[j].w};
             uint32_t kk[4];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 kk[t] = rank_key<CA>(vv[t], sv[t], gamma);
-                fine_count(f, kk[t] >> 16);
+                fine_count_hi(f, kk[t]);
             }
             *reinterpret_cast<uint4 *>(keys + 4 * q) = make_uint4(kk[0], kk[1], kk[2], kk[3]);
         }
@@ -577,8 +576,8 @@ __device__ __forceinline__ void select_fine_coarse(const uint16_t *__restrict__ 
             const uint32_t wv[4] = {ck[j].x, ck[j].y, ck[j].z, ck[j].w};
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
-                fine_count(f, wv[t] & 0xffffu);
-                fine_count(f, wv[t] >> 16);
+                fine_count_lo(f, wv[t]);
+                fine_count_hi(f, wv[t]);
             }
         }
     }

@@ -1,0 +1,99 @@
+"""Single-token steps whose products select for themselves, at the sizes where the kernel's branches meet: one and several
+chunks of columns per thread (8192 / 8224 columns), the variants of the cache update that rides along (8192, 20480), rows
+of one segment up to one per SM (where the update gets a launch of its own), row parts of one row, keep counts 1 and d,
+and threshold bins of 256 and 257 columns (the last that is ranked in place, the first that is not)."""
+import numpy as np
+import pytest
+
+import dip_inputs as di
+import oracle
+from gpu_util import check_step, upload_layer
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+SHAPES = [
+    (di.W_BF16, 8192, 96, 0.3), (di.W_BF16, 8224, 64, 0.3), (di.W_F32, 12288, 64, 0.2), (di.W_BF16, 32, 20512, 0.2),
+    (di.W_BF16, 64, 8192, 0.25), (di.W_BF16, 64, 8224, 0.25), (di.W_BF16, 64, 9472, 0.25), (di.W_BF16, 32, 18944, 0.1),
+    (di.W_F32, 96, 160, 0.02), (di.W_F32, 160, 96, 1.0), (di.W_BF16, 2080, 5472, 0.999),
+]
+
+
+def _layer(d_model, d_ff, wtype, seed):
+    return di.layer_weights(di.WORKLOADS["phi3_mini"].scaled(seed=seed, d_model=d_model, d_ff=d_ff, wtype=wtype, n_layers=1), 0)
+
+
+@pytest.mark.parametrize("policy", [None, "lru", "lfu"])
+@pytest.mark.parametrize("wtype,d_model,d_ff,rho", SHAPES)
+def test_steps_at_the_kernels_edges(wtype, d_model, d_ff, rho, policy):
+    import paper_2412_01380_b200 as dip
+    ctx = dip.Context(0)
+    lw = _layer(d_model, d_ff, wtype, d_model + d_ff)
+    w = upload_layer(dip, ctx, lw)
+    k_x, k_h = max(1, int(rho * d_model)), max(1, int(rho * d_ff))
+    refs, mine = [None, None], [None, None]
+    if policy:
+        for i, d in enumerate((d_model, d_ff)):
+            refs[i] = oracle.Cache(d, int(0.4 * d), policy)
+            mine[i] = dip.CacheState(d, int(0.4 * d), "cuda", policy)
+    for t in range(4):
+        check_step(dip, ctx, lw, w, di.heavy_tail_vector(70 + t, d_model), k_x, k_h, 0.2, *refs, *mine)
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("n_tied", [1, 32, 33, 255, 256, 257])
+@pytest.mark.parametrize("kept", ["one", "half", "all"])
+def test_threshold_bins_of_every_size(n_tied, kept):
+    """n_tied columns share the threshold's magnitude; one, half or all of them are kept."""
+    import paper_2412_01380_b200 as dip
+    ctx = dip.Context(0)
+    d_model, d_ff, above = 1024, 320, 200
+    lw = _layer(d_model, d_ff, di.W_BF16, n_tied)
+    w = upload_layer(dip, ctx, lw)
+    rng = np.random.default_rng(n_tied)
+    x = np.concatenate([rng.uniform(4.0, 9.0, above), np.full(n_tied, 1.5), rng.uniform(0.01, 1.0, d_model - above - n_tied)])
+    x = (rng.permutation(x) * rng.choice([-1, 1], d_model)).astype(np.float32)
+    k = above + {"one": 1, "half": (n_tied + 1) // 2, "all": n_tied}[kept]
+    for policy in (None, "lru"):
+        refs = [None, None] if policy is None else [oracle.Cache(d, d // 3) for d in (d_model, d_ff)]
+        mine = [None, None] if policy is None else [dip.CacheState(d, d // 3, "cuda") for d in (d_model, d_ff)]
+        for _ in range(2):
+            check_step(dip, ctx, lw, w, x, k, 80, 0.25, *refs, *mine)
+    ctx.close()
+
+
+@pytest.mark.parametrize("caches", ["both", "x", "h"])
+@pytest.mark.parametrize("n_layers", [1, 3, 4, 9])
+def test_stacks_leave_their_cache_updates_to_later_launches(n_layers, caches):
+    """A stack's cache states equal those of its blocks stepped one by one (blocks whose updates ride with the last down
+    product, fill a launch beside the products, or have no product with a cache to ride with)."""
+    import paper_2412_01380_b200 as dip
+    ctx = dip.Context(0)
+    d_model, d_ff = 256, 704
+    k_x, k_h = 64, 200
+    ws = [upload_layer(dip, ctx, _layer(d_model, d_ff, di.W_BF16, 100 + l)) for l in range(n_layers)]
+
+    def states():
+        return [[dip.CacheState(d, d // 2, "cuda") for _ in ws] if caches in (c, "both") else None
+                for d, c in ((d_model, "x"), (d_ff, "h"))]
+    gu, d = states()
+    gu1, d1 = states()
+    stack = dip.Stack(ws, gu, d)
+    out = torch.empty(d_model, device="cuda")
+    y = torch.empty(d_model, device="cuda")
+    for t in range(5):
+        x = torch.from_numpy(di.heavy_tail_vector(300 + t, d_model)).cuda()
+        dip.dip_stack_step(ctx, stack, x, k_x, k_h, 0.2, out)
+        for l, w in enumerate(ws):
+            dip.dip_mlp_step(ctx, w, x, k_x, k_h, 0.2, gu1[l] if gu1 else None, d1[l] if d1 else None, y)
+            nxt = torch.empty_like(x)
+            dip.dip_residual_rmsnorm(ctx, x, y, nxt)
+            x = nxt
+        torch.cuda.synchronize()
+        assert torch.equal(out, x), t
+        for a, b in ((gu, gu1), (d, d1)):
+            for p, q in zip(a or [], b or []):
+                assert torch.equal(p.stamp, q.stamp) and torch.equal(p.meta, q.meta), t
+    assert ctx.device_status() == 0
+    ctx.close()
