@@ -383,6 +383,7 @@ dip_status dip_select_gemv_gate_up(dip_ctx *ctx, const dip_mlp_weights *w, const
     if (cache_gu && !cache_ok(cache_gu, w->d_model)) return DIP_ERR_INVALID_ARG;
     if (cache_d && !cache_ok(cache_d, w->d_ff)) return DIP_ERR_INVALID_ARG;
     if (!fits(ctx, w->d_model, w->d_ff, 1)) return DIP_ERR_WORKSPACE;
+    if (w->wtype == DIP_W_INT4_G128) return DIP_ERR_UNSUPPORTED;
     if (!dip_gemv_fused_supported(ctx, w, 0, false) || !dip_gemv_fused_supported(ctx, w, 1, false)) return DIP_ERR_UNSUPPORTED;
     dip_gemv_keys hk = {ctx->coarse, cache_d ? cache_d->stamp : nullptr, gamma, 0};
     const dip_fused_select sx = {x, nullptr, nullptr, nullptr, k_x, gamma, cache_gu ? cache_gu->stamp : nullptr, mask_x, nullptr, nullptr};
@@ -397,6 +398,7 @@ dip_status dip_select_gemv_down(dip_ctx *ctx, const dip_mlp_weights *w, const fl
     if (k_h < 1 || k_h > w->d_ff || !(gamma >= 0.0f) || !isfinite(gamma)) return DIP_ERR_INVALID_ARG;
     if (cache_d && !cache_ok(cache_d, w->d_ff)) return DIP_ERR_INVALID_ARG;
     if (!fits(ctx, w->d_model, w->d_ff, 1)) return DIP_ERR_WORKSPACE;
+    if (w->wtype == DIP_W_INT4_G128) return DIP_ERR_UNSUPPORTED;
     if (!dip_gemv_fused_supported(ctx, w, 1, false)) return DIP_ERR_UNSUPPORTED;
     const dip_fused_select sh = {h, nullptr, nullptr, ctx->coarse, k_h, gamma, cache_d ? cache_d->stamp : nullptr, mask_h, nullptr, nullptr};
     return dip_launch_gemv_fused(ctx, w, 1, &sh, y, (cudaStream_t)stream, nullptr);
@@ -445,17 +447,25 @@ static dip_status step_impl(dip_ctx *ctx, const dip_mlp_weights *w,
         if (cache_gu) due->at[due->n++] = dip_update_of(cache_gu, mask_x);
         // the updates that are due ride with the last block's down product, if that has a cache and SMs to spare; else a
         // launch beside the products takes them
-        const bool ride = last && cache_d && dip_gemv_fused_update_room(ctx, w) > due->n;
+        const bool ride = last && cache_d && w->wtype != DIP_W_INT4_G128 && dip_gemv_fused_update_room(ctx, w) > due->n;
         if (!ride && (last || due->n + 2 > DIP_CACHE_UPDATES)) {
             if ((st = fork_cache_updates(ctx, 0, *due, s)) != DIP_OK) return st;
             due->n = 0;
         }
+        if (last && cache_d && w->wtype == DIP_W_INT4_G128) {
+            // (no updates inside the 4-bit launches: with a mask from a select kernel this one runs beside the product)
+            st = dip_launch_select(ctx, h, nullptr, nullptr, 1, w->d_ff, k_h, gamma, cache_d->stamp, mask_h, s, ctx->coarse);
+            if (st != DIP_OK) return st;
+            if ((st = fork_cache_update(ctx, 1, mask_h, cache_d, s)) != DIP_OK) return st;
+            if ((st = dip_launch_gemv(ctx, w, 1, h, 1, mask_h, nmax_h, y, s)) != DIP_OK) return st;
+        } else {
         const dip_fused_select sh = {h, nullptr, nullptr, ctx->coarse, k_h, gamma, cache_d ? cache_d->stamp : nullptr, mask_h,
                                      ride ? cache_d : nullptr, due};
         if ((st = dip_launch_gemv_fused(ctx, w, 1, &sh, y, s, nullptr)) != DIP_OK) return st;
         if (ride) due->n = 0;
         else if (last && cache_d && (st = fork_cache_update(ctx, 1, mask_h, cache_d, s)) != DIP_OK) return st;
         else if (!last && cache_d) due->at[due->n++] = dip_update_of(cache_d, mask_h);
+        }
     } else {
         if ((st = fork_cache_updates(ctx, 0, *due, s)) != DIP_OK) return st;
         due->n = 0;

@@ -12,7 +12,7 @@
 constexpr int DIP_RING_LAYERS = 128;
 constexpr int DIP_TRACE_SLOTS = 1024;
 constexpr uint32_t DIP_MAIL_EMPTY = 0xffffffffu;
-constexpr int DIP_MAIL_FLOATS = 256;   // boxes per SM: one CTA's segment of sums
+constexpr int DIP_MAIL_FLOATS = 2048;  // boxes per SM: one CTA's segment of sums (INT4: up to 2048, F32 / BF16: 256)
 constexpr int DIP_TRACE_WORDS = 4;   // first start, dependency ready, last end, auxiliary
 
 // Scratch workspace of a context.  All device memory the library itself owns.
@@ -229,6 +229,7 @@ struct dip_fused_select {
 };
 // gemv_fused.cu: how many cache updates (its own among them) find an SM beside a down launch's products.
 int dip_gemv_fused_update_room(const dip_ctx *ctx, const dip_mlp_weights *w);
+// (INT4: gemv_int4.cu.  Its launches update no caches.)
 bool dip_gemv_fused_supported(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool norm);
 dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int which, const dip_fused_select *sel,
                                  float *out, cudaStream_t stream, dip_gemv_keys *keys);

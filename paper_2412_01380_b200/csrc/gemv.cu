@@ -851,6 +851,7 @@ dip_status dip_launch_gemv(dip_ctx *ctx, const dip_mlp_weights *w, int which,
     p.d_out = which == 0 ? w->d_ff : w->d_model;
     p.mask_words = (p.d_in + 31) / 32;
     p.partials = ctx->partials;
+    p.mail = ctx->mail;
     p.tickets = ctx->tickets;
     p.status = ctx->status;
     p.wait_limit_ns = ctx->wait_limit_ns;
@@ -886,7 +887,7 @@ dip_status dip_launch_gemv(dip_ctx *ctx, const dip_mlp_weights *w, int which,
                 p.key_stamp = keys->stamp;
                 p.key_gamma = keys->gamma;
             }
-            st = dip_launch_gemv_int4(ctx, p, which, n_kept_max, mode, stream);
+            st = dip_launch_gemv_int4(ctx, p, which, n_kept_max, mode, nullptr, stream);
             if (st == DIP_OK && p.key_coarse && !mode) keys->written = 1;
         }
         else if (ctx->gemv_direct && p.batch == 2 && !rows) {

@@ -21,6 +21,7 @@ struct GemvParams {
     int d_out;
     int batch;                 // tokens in this launch (<= BT)
     float *partials;
+    float *mail;               // row parts on their way between CTAs of a launch; DIP_MAIL_EMPTY outside one
     unsigned int *tickets;
     int *status;               // device status word (0 = fine)
     unsigned long long wait_limit_ns;   // a wait on a copy's arrival gives up after this long
@@ -108,6 +109,45 @@ __device__ __forceinline__ void mail_take(float *box, size_t stride, int n, floa
         if (q < n) mail_put(box + (size_t)q * stride, __uint_as_float(DIP_MAIL_EMPTY));
 }
 
+// The same for groups of four.
+__device__ __forceinline__ void mail_put4(float *box, const float4 &v)
+{
+    asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(box), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void mail_take4(float *box, size_t stride, int n, float4 (&a)[N], int *status, unsigned long long limit_ns)
+{
+    unsigned long long t0 = 0;
+    for (unsigned i = 0;; ++i) {
+        bool all = true;
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            a[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (q < n)
+                asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a[q].x), "=f"(a[q].y), "=f"(a[q].z), "=f"(a[q].w)
+                             : "l"(box + (size_t)q * stride) : "memory");
+        }
+#pragma unroll
+        for (int q = 0; q < N; ++q)
+            all = all && __float_as_uint(a[q].x) != DIP_MAIL_EMPTY && __float_as_uint(a[q].y) != DIP_MAIL_EMPTY &&
+                  __float_as_uint(a[q].z) != DIP_MAIL_EMPTY && __float_as_uint(a[q].w) != DIP_MAIL_EMPTY;
+        if (all) break;
+        if ((i & 63u) == 63u) {
+            const unsigned long long now = dip_gtime();
+            if (t0 == 0) {
+                t0 = now;
+            } else if (now - t0 > limit_ns) {
+                atomicExch(status, 1);
+                break;
+            }
+        }
+    }
+    const float e = __uint_as_float(DIP_MAIL_EMPTY);
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+        if (q < n) mail_put4(box + (size_t)q * stride, make_float4(e, e, e, e));
+}
+
 // One more at a counter in global memory, after what this thread (and those it has synchronised with) has read.
 __device__ __forceinline__ void count_one(unsigned int *counter)
 {
@@ -179,4 +219,7 @@ dip_status dip_launch_gemv_direct_bt(dip_ctx *ctx, GemvParams &p, int wtype, int
 dip_status dip_launch_gemv_tc(dip_ctx *ctx, GemvParams &p, int which, int n_kept_max, cudaStream_t stream);
 
 // gemv_int4.cu: the single-token product for INT4-g128 weights.  mode as dip_gemv_rows.mode.
-dip_status dip_launch_gemv_int4(dip_ctx *ctx, GemvParams &p, int which, int n_kept_max, int mode, cudaStream_t stream);
+// sel != nullptr (mode 0): the product builds its own mask, as gemv_fused.cu's do (p.mask_bits is not read).
+dip_status dip_launch_gemv_int4(dip_ctx *ctx, GemvParams &p, int which, int n_kept_max, int mode, const dip_fused_select *sel,
+                                cudaStream_t stream);
+bool dip_gemv_int4_selects(const dip_ctx *ctx, const dip_mlp_weights *w, int which);

@@ -127,50 +127,6 @@ __device__ __forceinline__ void list_sure(FusedSmem &s, int c, int lo, int hi, u
         });
 }
 
-// One warp: the n_c columns of the threshold's bin (f.cand) are ranked by (full key descending,
-// column ascending), which inside one bin is the order of (low 16 key bits, column) in one word;
-// the first krem go to tie[] by rank, and into maskw when that is given.
-template <typename KeyOf>
-__device__ __forceinline__ void rank_ties(TkFine &f, int n_c, int krem, uint16_t *tie, unsigned int *maskw, const KeyOf &key_of)
-{
-    constexpr int PER = TK_TIE_LIMIT / 32;
-    const int lane = threadIdx.x & 31;
-    int col[PER];
-    uint32_t rk[PER];
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const int c = lane + 32 * i;
-        rk[i] = 0u;
-        if (c < n_c) {
-            col[i] = f.cand[c];
-            rk[i] = key_of(col[i], c);
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const int c = lane + 32 * i;
-        if (c < n_c) rk[i] = ((rk[i] & 0xffffu) << 15) | (uint32_t)(0x7fff - col[i]);
-        if (32 * i < n_c) f.ckey[c] = rk[i];               // (zeros up to the end of the last 32: nobody's rank)
-    }
-    __syncwarp();
-    int rank[PER];
-#pragma unroll
-    for (int i = 0; i < PER; ++i) rank[i] = 0;
-    for (int j = 0; j < n_c; j += 4) {
-        const uint4 q = *reinterpret_cast<const uint4 *>(f.ckey + j);
-#pragma unroll
-        for (int i = 0; i < PER; ++i)
-            if (32 * i < n_c) rank[i] += (int)(q.x > rk[i]) + (int)(q.y > rk[i]) + (int)(q.z > rk[i]) + (int)(q.w > rk[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < PER; ++i)
-        if (lane + 32 * i < n_c && rank[i] < krem) {
-            tie[rank[i]] = (uint16_t)col[i];
-            if (maskw) atomicOr(&maskw[col[i] >> 5], 1u << (col[i] & 31));
-        }
-    __syncwarp();
-}
-
 // acc += sum over rows idx[first], idx[first + stride], ... below n_rows of row segment x value,
 // U rows in flight per lane.
 template <int WT>
@@ -648,6 +604,7 @@ int dip_gemv_fused_update_room(const dip_ctx *ctx, const dip_mlp_weights *w)
 
 bool dip_gemv_fused_supported(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool norm)
 {
+    if (w->wtype == DIP_W_INT4_G128) return dip_gemv_int4_selects(ctx, w, which);
     FusedParams p;
     return fused_plan(ctx, w, which, norm, p);
 }
@@ -656,6 +613,33 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
                                  float *out, cudaStream_t stream, dip_gemv_keys *keys)
 {
     const bool norm = which == 0 && sel->xb != nullptr;
+    if (w->wtype == DIP_W_INT4_G128) {
+        const size_t row_elems = which == 0 ? (size_t)2 * w->d_ff : (size_t)w->d_model;
+        GemvParams g = {};
+        g.W = (const char *)(which == 0 ? w->gate_up : w->down);
+        g.row_bytes = row_elems / 2;
+        g.scales = (const uint16_t *)(which == 0 ? w->gate_up_scales : w->down_scales);
+        g.scale_row_elems = row_elems;
+        g.v = sel->xa;                                  // (down; gate/up keeps x in shared memory)
+        g.d_in = which == 0 ? w->d_model : w->d_ff;
+        g.d_out = which == 0 ? w->d_ff : w->d_model;
+        g.mask_words = (g.d_in + 31) / 32;
+        g.out = out;
+        g.batch = 1;
+        g.mail = ctx->mail;
+        g.status = ctx->status;
+        g.wait_limit_ns = ctx->wait_limit_ns;
+        g.tr = dip_trace_slot(ctx, which == 0 ? 4 : 5);
+        g.key_gamma = 1.0f;
+        if (keys) keys->written = 0;
+        if (which == 0 && keys && keys->coarse) {
+            g.key_coarse = keys->coarse;
+            g.key_stamp = keys->stamp;
+            g.key_gamma = keys->gamma;
+            keys->written = 1;
+        }
+        return dip_launch_gemv_int4(ctx, g, which, sel->k, 0, sel, stream);
+    }
     FusedParams p;
     if (!fused_plan(ctx, w, which, norm, p)) return DIP_ERR_UNSUPPORTED;
     if (p.nparts > sel->k) p.nparts = sel->k;

@@ -48,15 +48,22 @@ __device__ __forceinline__ int warp_array_prefix(const int *arr, int warp, int l
     return __shfl_sync(0xffffffffu, excl, warp);
 }
 
-// Find the histogram bin holding the krem-th largest key: suffix scan over the RADIX_BINS bins,
-// two per thread.  Leaves bcast[0] = bin, bcast[1] = rank of the wanted key inside the bin
-// (1-based, from the top), bcast[2] = keys in the bin.  All threads call it; ends with a barrier.
+// Find the histogram bin holding the krem-th largest key: suffix scan over the RADIX_BINS bins, a few
+// per thread.  Leaves bcast[0] = bin, bcast[1] = rank of the wanted key inside the bin
+// (1-based, from the top), bcast[2] = keys in the bin.  All T threads of the CTA call it (with fewer than
+// 1024, the per-warp arrays beyond the CTA's warps are zero); ends with a barrier.
+template <int T = TK_THREADS>
 __device__ __forceinline__ void find_bin(TkShared &s, int krem)
 {
+    constexpr int B = RADIX_BINS / T;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // suffix scan: thread t owns bins 2t and 2t+1
-    const unsigned h0 = s.hist[2 * tid], h1 = s.hist[2 * tid + 1];
-    const int own = (int)(h0 + h1);
+    // suffix scan: thread t owns bins B t .. B t + B - 1
+    int h[B], own = 0;
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+        h[i] = (int)s.hist[B * tid + i];
+        own += h[i];
+    }
     int suf = own;   // inclusive suffix within the warp
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -73,17 +80,15 @@ __device__ __forceinline__ void find_bin(TkShared &s, int krem)
         if (lane + o < 32) wsuf += n;
     }
     const int above_warp = __shfl_sync(0xffffffffu, wsuf - wv, warp);
-    int cum = above_warp + suf - own;         // keys in bins above 2t+1
-    if (cum < krem && krem <= cum + (int)h1) {
-        s.bcast[0] = 2 * tid + 1;
-        s.bcast[1] = krem - cum;
-        s.bcast[2] = (int)h1;
-    }
-    cum += (int)h1;
-    if (cum < krem && krem <= cum + (int)h0) {
-        s.bcast[0] = 2 * tid;
-        s.bcast[1] = krem - cum;
-        s.bcast[2] = (int)h0;
+    int cum = above_warp + suf - own;         // keys in bins above this thread's
+#pragma unroll
+    for (int i = B - 1; i >= 0; --i) {
+        if (cum < krem && krem <= cum + h[i]) {
+            s.bcast[0] = B * tid + i;
+            s.bcast[1] = krem - cum;
+            s.bcast[2] = h[i];
+        }
+        cum += h[i];
     }
     __syncthreads();
 }
@@ -97,6 +102,7 @@ __device__ __forceinline__ void find_bin(TkShared &s, int krem)
 // current digit over the keys that match the prefix found so far, then a suffix scan over the
 // bins (two per thread) to find the bin holding the k-th key.  The four smallest digits are
 // counted in registers instead of with contended atomics (rows of zeros and denormals).
+template <int T_ = TK_THREADS>
 __device__ void block_radix_select(const uint32_t *keys, int d, uint32_t keymask, int top_bit, int k,
                                    TkShared &s, uint32_t &T, int &quota, int &n_eq)
 {
@@ -108,11 +114,10 @@ __device__ void block_radix_select(const uint32_t *keys, int d, uint32_t keymask
         const int w = hi < RADIX_BITS ? hi : RADIX_BITS;
         const int shift = hi - w;
         const uint32_t dmask = (1u << w) - 1u;
-        s.hist[2 * tid] = 0;
-        s.hist[2 * tid + 1] = 0;
+        for (int i = tid; i < RADIX_BINS; i += T_) s.hist[i] = 0;
         __syncthreads();
         int c0 = 0, c1 = 0, c2 = 0, c3 = 0;
-        for (int e = tid; e < d; e += TK_THREADS) {
+        for (int e = tid; e < d; e += T_) {
             const uint32_t key = keys[e] & keymask;
             if ((key & prefmask) == prefix) {
                 const uint32_t dg = (key >> shift) & dmask;
@@ -134,7 +139,7 @@ __device__ void block_radix_select(const uint32_t *keys, int d, uint32_t keymask
             if (c3) atomicAdd(&s.hist[3], (unsigned)c3);
         }
         __syncthreads();
-        find_bin(s, krem);
+        find_bin<T_>(s, krem);
         prefix |= (uint32_t)s.bcast[0] << shift;
         prefmask |= dmask << shift;
         krem = s.bcast[1];
@@ -221,15 +226,16 @@ __device__ float block_residual_scale(const float *__restrict__ xa, const float 
 
 // General path (very many keys tied around the threshold): full radix select on all d keys in
 // keys[], then an ordered sweep that ranks the ties by column.
+template <int T_ = TK_THREADS>
 __device__ void general_select(const uint32_t *keys, int d, int k, TkShared &s, uint32_t *__restrict__ mask_bits)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // warp w owns columns [w*span, (w+1)*span), span a multiple of 32: one ballot = one mask word
-    const int span = ((d + TK_THREADS - 1) / TK_THREADS) * 32;
+    const int span = ((d + T_ - 1) / T_) * 32;
     const int base = warp * span;
     uint32_t T;
     int quota, n_eq;
-    block_radix_select(keys, d, 0x7fffffffu, 31, k, s, T, quota, n_eq);
+    block_radix_select<T_>(keys, d, 0x7fffffffu, 31, k, s, T, quota, n_eq);
     if (quota == n_eq) {
         // every column tied with the threshold is kept: the mask is key >= T
         for (int it = 0; it < span && base + it < d; it += 32) {
@@ -290,12 +296,13 @@ struct __align__(16) TkFine {
     int n_cand;
 };
 
+template <int T = TK_THREADS>
 __device__ __forceinline__ void fine_zero(TkFine &f)
 {
     const int tid = threadIdx.x;
     uint4 *h4 = reinterpret_cast<uint4 *>(f.hist);
 #pragma unroll
-    for (int i = 0; i < TK_FINE_WORDS / 4 / TK_THREADS; ++i) h4[tid + i * TK_THREADS] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 0; i < TK_FINE_WORDS / 4 / T; ++i) h4[tid + i * T] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) f.n_cand = 0;
 }
 
@@ -309,30 +316,32 @@ __device__ __forceinline__ void fine_count_lo(TkFine &f, uint32_t w) { fine_coun
 __device__ __forceinline__ void fine_count_hi(TkFine &f, uint32_t w) { fine_count_at(f, (w >> 15) & 0xfffcu, w & 0x10000u); }
 
 // The bin of the k-th largest key: s.bcast[0] = bin, [1] = rank of the wanted key inside it (from
-// the top, 1-based), [2] = keys in the bin.  Warp w owns bins 1024 w .. 1024 w + 1023 and only adds them
-// up (every instruction here costs 32 warps' issue slots); the one warp that holds the wanted key looks
-// closer.  All threads call it; the histogram must be complete and visible; ends with a barrier.
+// the top, 1-based), [2] = keys in the bin.  Each of the T / 32 warps owns a run of bins and only adds them
+// up (every instruction here costs all warps' issue slots); the one warp that holds the wanted key looks
+// closer.  All threads call it (T < 1024: s.wa is zero beyond the CTA's warps); the histogram must be complete
+// and visible; ends with a barrier.
+template <int T = TK_THREADS>
 __device__ __forceinline__ void fine_find(const TkFine &f, TkShared &s, int k)
 {
-    static_assert(TK_FINE_WORDS == 16 * TK_THREADS, "sixteen words per thread");
+    constexpr int NB = TK_FINE_WORDS / 4 / T;    // blocks of 256 bins per warp
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // 16 bytes = 8 bins, ascending over (block i of 256 bins, lane)
-    const uint4 *own = reinterpret_cast<const uint4 *>(f.hist) + warp * 128 + lane;
-    uint32_t sum[4];                             // both halves of a word counted in one (each at most DIP_MAX_D)
+    const uint4 *own = reinterpret_cast<const uint4 *>(f.hist) + warp * (32 * NB) + lane;
+    uint32_t sum[NB], all = 0u;                  // both halves of a word counted in one (each at most DIP_MAX_D)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < NB; ++i) {
         const uint4 v = own[32 * i];
         sum[i] = (v.x + v.y) + (v.z + v.w);
+        all += sum[i];
     }
-    const uint32_t all = (sum[0] + sum[1]) + (sum[2] + sum[3]);
     const int total = (int)__reduce_add_sync(0xffffffffu, (all & 0xffffu) + (all >> 16));
     if (lane == 0) s.wa[warp] = total;
     __syncthreads();
     int cum = (int)__reduce_add_sync(0xffffffffu, lane > warp ? (unsigned)s.wa[lane] : 0u);   // keys above this warp's bins
     if (cum < k && k <= cum + total) {
-        int in_lane = 0, blk = 3;
+        int in_lane = 0, blk = NB - 1;
 #pragma unroll
-        for (int i = 3; i >= 0; --i) {
+        for (int i = NB - 1; i >= 0; --i) {
             const int mine = (int)((sum[i] & 0xffffu) + (sum[i] >> 16));
             const int t = (int)__reduce_add_sync(0xffffffffu, (unsigned)mine);
             in_lane = mine;
@@ -354,7 +363,7 @@ __device__ __forceinline__ void fine_find(const TkFine &f, TkShared &s, int k)
             for (int i = 7; i >= 0; --i) {
                 const int c = (int)((i & 1) ? w[i >> 1] >> 16 : w[i >> 1] & 0xffffu);
                 if (cum < k && k <= cum + c) {
-                    s.bcast[0] = 8 * (warp * 128 + 32 * blk + lane) + i;
+                    s.bcast[0] = 8 * (warp * (32 * NB) + 32 * blk + lane) + i;
                     s.bcast[1] = k - cum;
                     s.bcast[2] = c;
                 }
@@ -390,6 +399,50 @@ __device__ __forceinline__ void fine_complete(TkFine &f, int n_c, int krem, unsi
         if (rank < krem) atomicOr(&maskw[mc >> 5], 1u << (mc & 31));
     }
     __syncthreads();
+}
+
+// One warp: the n_c columns of the threshold's bin (f.cand) are ranked by (full key descending,
+// column ascending), which inside one bin is the order of (low 16 key bits, column) in one word;
+// the first krem go to tie[] by rank, and into maskw when that is given.
+template <typename KeyOf>
+__device__ __forceinline__ void rank_ties(TkFine &f, int n_c, int krem, uint16_t *tie, unsigned int *maskw, const KeyOf &key_of)
+{
+    constexpr int PER = TK_TIE_LIMIT / 32;
+    const int lane = threadIdx.x & 31;
+    int col[PER];
+    uint32_t rk[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int c = lane + 32 * i;
+        rk[i] = 0u;
+        if (c < n_c) {
+            col[i] = f.cand[c];
+            rk[i] = key_of(col[i], c);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int c = lane + 32 * i;
+        if (c < n_c) rk[i] = ((rk[i] & 0xffffu) << 15) | (uint32_t)(0x7fff - col[i]);
+        if (32 * i < n_c) f.ckey[c] = rk[i];               // (zeros up to the end of the last 32: nobody's rank)
+    }
+    __syncwarp();
+    int rank[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) rank[i] = 0;
+    for (int j = 0; j < n_c; j += 4) {
+        const uint4 q = *reinterpret_cast<const uint4 *>(f.ckey + j);
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (32 * i < n_c) rank[i] += (int)(q.x > rk[i]) + (int)(q.y > rk[i]) + (int)(q.z > rk[i]) + (int)(q.w > rk[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+        if (lane + 32 * i < n_c && rank[i] < krem) {
+            tie[rank[i]] = (uint16_t)col[i];
+            if (maskw) atomicOr(&maskw[col[i] >> 5], 1u << (col[i] & 31));
+        }
+    __syncwarp();
 }
 
 // Second part of select_fine: keys[] and the histogram are complete (not yet synchronised).

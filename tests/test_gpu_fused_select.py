@@ -16,6 +16,11 @@ SHAPES = [
     (di.W_BF16, 8192, 96, 0.3), (di.W_BF16, 8224, 64, 0.3), (di.W_F32, 12288, 64, 0.2), (di.W_BF16, 32, 20512, 0.2),
     (di.W_BF16, 64, 8192, 0.25), (di.W_BF16, 64, 8224, 0.25), (di.W_BF16, 64, 9472, 0.25), (di.W_BF16, 32, 18944, 0.1),
     (di.W_F32, 96, 160, 0.02), (di.W_F32, 160, 96, 1.0), (di.W_BF16, 2080, 5472, 0.999),
+    # 4-bit: 8, 32 and 64 columns per thread of the list, more rows than one round, quads beyond 32, and a width whose
+    # keys do not fit beside the tables (select kernels in front)
+    (di.W_INT4_G128, 128, 256, 0.01), (di.W_INT4_G128, 4096, 4224, 0.25), (di.W_INT4_G128, 384, 16512, 0.3),
+    (di.W_INT4_G128, 4224, 384, 0.9), (di.W_INT4_G128, 16512, 128, 0.2), (di.W_INT4_G128, 256, 18048, 1.0),
+    (di.W_INT4_G128, 128, 32768, 0.1),
 ]
 
 
@@ -42,14 +47,15 @@ def test_steps_at_the_kernels_edges(wtype, d_model, d_ff, rho, policy):
     ctx.close()
 
 
+@pytest.mark.parametrize("wtype", [di.W_BF16, di.W_INT4_G128])
 @pytest.mark.parametrize("n_tied", [1, 32, 33, 255, 256, 257])
 @pytest.mark.parametrize("kept", ["one", "half", "all"])
-def test_threshold_bins_of_every_size(n_tied, kept):
+def test_threshold_bins_of_every_size(n_tied, kept, wtype):
     """n_tied columns share the threshold's magnitude; one, half or all of them are kept."""
     import paper_2412_01380_b200 as dip
     ctx = dip.Context(0)
-    d_model, d_ff, above = 1024, 320, 200
-    lw = _layer(d_model, d_ff, di.W_BF16, n_tied)
+    d_model, d_ff, above = 1024, 384, 200
+    lw = _layer(d_model, d_ff, wtype, n_tied)
     w = upload_layer(dip, ctx, lw)
     rng = np.random.default_rng(n_tied)
     x = np.concatenate([rng.uniform(4.0, 9.0, above), np.full(n_tied, 1.5), rng.uniform(0.01, 1.0, d_model - above - n_tied)])
@@ -65,14 +71,15 @@ def test_threshold_bins_of_every_size(n_tied, kept):
 
 @pytest.mark.parametrize("caches", ["both", "x", "h"])
 @pytest.mark.parametrize("n_layers", [1, 3, 4, 9])
-def test_stacks_leave_their_cache_updates_to_later_launches(n_layers, caches):
+@pytest.mark.parametrize("wtype", [di.W_BF16, di.W_INT4_G128])
+def test_stacks_leave_their_cache_updates_to_later_launches(n_layers, caches, wtype):
     """A stack's cache states equal those of its blocks stepped one by one (blocks whose updates ride with the last down
     product, fill a launch beside the products, or have no product with a cache to ride with)."""
     import paper_2412_01380_b200 as dip
     ctx = dip.Context(0)
-    d_model, d_ff = 256, 704
+    d_model, d_ff = 256, 640
     k_x, k_h = 64, 200
-    ws = [upload_layer(dip, ctx, _layer(d_model, d_ff, di.W_BF16, 100 + l)) for l in range(n_layers)]
+    ws = [upload_layer(dip, ctx, _layer(d_model, d_ff, wtype, 100 + l)) for l in range(n_layers)]
 
     def states():
         return [[dip.CacheState(d, d // 2, "cuda") for _ in ws] if caches in (c, "both") else None
