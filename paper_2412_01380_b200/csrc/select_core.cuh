@@ -389,25 +389,33 @@ __device__ __forceinline__ void fine_complete(TkFine &f, int n_c, int krem, unsi
         f.ckey[tid] = my;
     }
     __syncthreads();
-    if (tid < n_c) {
+    // eight lanes count for one column (a chain of n_c steps by one thread each took 1 us)
+    const int part = tid & 7;
+    for (int c0 = 0; c0 < n_c; c0 += TK_THREADS / 8) {
+        const int c = c0 + (tid >> 3);
         int rank = 0;
-        for (int j = 0; j < n_c; ++j) {
-            const uint32_t kj = f.ckey[j];
-            const int cj = f.cand[j];
-            rank += (kj > my) || (kj == my && cj < mc);
+        if (c < n_c) {
+            my = f.ckey[c];
+            mc = f.cand[c];
+            for (int j = part; j < n_c; j += 8) {
+                const uint32_t kj = f.ckey[j];
+                const int cj = f.cand[j];
+                rank += (kj > my) || (kj == my && cj < mc);
+            }
         }
-        if (rank < krem) atomicOr(&maskw[mc >> 5], 1u << (mc & 31));
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+        if (part == 0 && c < n_c && rank < krem) atomicOr(&maskw[mc >> 5], 1u << (mc & 31));
     }
     __syncthreads();
 }
 
 // One warp: the n_c columns of the threshold's bin (f.cand) are ranked by (full key descending,
 // column ascending), which inside one bin is the order of (low 16 key bits, column) in one word;
-// the first krem go to tie[] by rank, and into maskw when that is given.
-template <typename KeyOf>
-__device__ __forceinline__ void rank_ties(TkFine &f, int n_c, int krem, uint16_t *tie, unsigned int *maskw, const KeyOf &key_of)
+// the first krem go to tie[] by rank, and into maskw when that is given.  PER columns per lane.
+template <int PER, typename KeyOf>
+__device__ __forceinline__ void rank_ties_per(TkFine &f, int n_c, int krem, uint16_t *tie, unsigned int *maskw, const KeyOf &key_of)
 {
-    constexpr int PER = TK_TIE_LIMIT / 32;
     const int lane = threadIdx.x & 31;
     int col[PER];
     uint32_t rk[PER];
@@ -443,6 +451,13 @@ __device__ __forceinline__ void rank_ties(TkFine &f, int n_c, int krem, uint16_t
             if (maskw) atomicOr(&maskw[col[i] >> 5], 1u << (col[i] & 31));
         }
     __syncwarp();
+}
+// (two variants: the usual few dozen columns should not pay for the code of 256)
+template <typename KeyOf>
+__device__ __forceinline__ void rank_ties(TkFine &f, int n_c, int krem, uint16_t *tie, unsigned int *maskw, const KeyOf &key_of)
+{
+    if (n_c <= 64) rank_ties_per<2>(f, n_c, krem, tie, maskw, key_of);
+    else rank_ties_per<TK_TIE_LIMIT / 32>(f, n_c, krem, tie, maskw, key_of);
 }
 
 // Second part of select_fine: keys[] and the histogram are complete (not yet synchronised).
