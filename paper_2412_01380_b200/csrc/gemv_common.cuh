@@ -71,6 +71,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity, unsign
     }
 }
 
+// Asks for `bytes` at p to be brought into L2 (a hint: nothing to wait for).  p on a 16-byte boundary, bytes a
+// multiple of 16, the range inside one allocation.
+__device__ __forceinline__ void l2_prefetch(const void *p, unsigned bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 // Sums that one CTA of a launch hands to another through global memory: the value itself is the message.
 // A box holds DIP_MAIL_EMPTY (a NaN pattern that no arithmetic produces) until its sum arrives; who
 // takes a sum empties its box again.

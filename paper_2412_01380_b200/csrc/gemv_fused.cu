@@ -31,6 +31,7 @@ namespace {
 constexpr int GF_SEG = 512;
 constexpr int GF_NW = TK_THREADS / 32;     // 32 warps
 constexpr int GF_U = 4;                    // loads in flight per lane
+constexpr double GF_AHEAD_BYTES = 15e6;   // rows asked for ahead of the stream, see own_ahead
 constexpr size_t GF_SMEM_LIMIT = (size_t)224 * 1024;   // dynamic shared memory a launch may ask for
 
 struct FusedParams {
@@ -39,6 +40,7 @@ struct FusedParams {
     size_t row_bytes;
     int d_in, d_out;
     int n_slabs, nparts;
+    int own_ahead;               // gate/up: quads of columns whose rows are asked for as soon as the threshold's bin is known
     int x_near;                  // gate/up: room in shared memory for the values of x
     float *out;
     float *mail;                 // [nparts][n_slabs][segment elements]; DIP_MAIL_EMPTY outside a launch
@@ -324,6 +326,20 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
         const uint32_t b = (uint32_t)s.ts.bcast[0];
         krem = s.ts.bcast[1];
         n_c = s.ts.bcast[2];
+        if constexpr (WHICH == 0) {
+            // The first rows on their way to L2 while the list is made: whole rows, shared out over the CTAs.  As many as
+            // come in that time: with 15 MB three Phi-3-Medium blocks took 112.7 us, with none 115.4, with 30 MB 116.1,
+            // with 60 MB 120.9 (what is still under way delays the first rows that are waited for)
+#pragma unroll
+            for (int j = 0; j < NQ; ++j) {
+                const int q = tid + j * TK_THREADS;
+                if (q < p.own_ahead && q % n_prod == (int)blockIdx.x) {
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+                        if (kk[j][t] > ((b << 16) | 0xffffu)) l2_prefetch(p.W + (size_t)(4 * q + t) * p.row_bytes, (unsigned)p.row_bytes);
+                }
+            }
+        }
         if (n_c > TK_TIE_LIMIT) {
             // masses of equal keys: the general select on full keys
             if (staged) {
@@ -659,6 +675,9 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
         p.key_gamma = keys->gamma;
         keys->written = 1;
     }
+    const double quads = GF_AHEAD_BYTES / (double)p.row_bytes / sel->k * p.d_in / 4;
+    // (a product of fewer bytes than that gains nothing, and 0.4 us go into asking: two blocks of 1088 / 2816)
+    p.own_ahead = which == 0 && quads < p.d_in / 4 ? (int)quads : 0;
     p.xa = sel->xa;
     p.xb = sel->xb;
     p.x_out = sel->x_out;
