@@ -766,6 +766,26 @@ def main_two_tier(args, dip, ctx, torch, w, keep_ratio, budget, rank, world, loc
     print(json.dumps(line))
 
 
+def launches_per_token(n_layers, batch, caches, int4):
+    """Kernels of one dip_stack_step.  One token: two products per layer that build their own masks; the cache updates
+    ride with the last down product, seven at a time in a launch of their own before that (4-bit weights: the last layer's
+    down half is select, update and product, and a launch for the updates that are due).  Several tokens: two selects
+    and two products (their value gathers and part sums not counted).  One residual + rmsnorm closes the stack."""
+    if batch > 1:
+        return 4 * n_layers + 1
+    n, due = 2 * n_layers + 1, 0
+    for layer in range(n_layers if caches else 0):
+        last = layer == n_layers - 1 or layer % 128 == 127        # (the mask slots are used again)
+        due += 1
+        if (last and int4) or (not last and due + 2 > 7):
+            n, due = n + 1, 0
+        if last:
+            n, due = n + (2 if int4 else 0), 0
+        else:
+            due += 1
+    return n
+
+
 def print_timeline(dip, ctx, torch, w, layers, xs_host, keep_ratio, budget):
     """One decode token through the stack as a CUDA graph, with the library's device-side
     timeline on: per kernel, when it started, when its inputs were ready, when it ended."""
@@ -978,10 +998,7 @@ def main():
         gu_us = None
         achieved = head.get("union_gbs", head["step_gbs"])
     fused = bool(head.get("select_in_product"))
-    # per layer: two selects and two products (or two launches that do both), two cache updates when a
-    # cache is on; one residual + rmsnorm closes the stack
-    # (with a cache the last layer's down half keeps its select kernel: one launch more per token)
-    launches_per_step = L * ((2 if fused else 4) + (2 if budget is not None else 0)) + 1 + (1 if fused and budget is not None else 0)
+    launches_per_step = launches_per_token(L, args.batch, budget is not None, w.wtype == di.W_INT4_G128)
     kernel_name = GATE_UP_KERNEL(w, args.batch, fused) + (" (select of x + gate/up bundle)" if fused else " (gate/up bundle)")
     line = {
         "metric": METRIC, "value": whole_job_rate(L * args.steps, world, head["ms_total"]), "unit": UNIT, "n_gpus": world,
