@@ -617,15 +617,15 @@ dip_status dip_mlp_step_neuron_pruned(dip_ctx *ctx, const dip_neuron_weights *w,
     dip_status st;
     // the dense, ranking activation: p = silu(W^g x) (Gate pruning) or W^u x (Up pruning)
     st = dip_launch_rowdot(ctx, w->wtype, by_gate ? w->gate : w->up, w->d_model, w->d_ff, x, nullptr, w->d_ff,
-                           by_gate ? 1 : 0, nullptr, p, s);
+                           by_gate ? 1 : 0, nullptr, p, h, s);
     if (st != DIP_OK) return st;
     // m = topK(|p|) over the neurons (Eq. 5), as a bit set and as an ascending list
     if ((st = dip_launch_select(ctx, p, nullptr, nullptr, 1, w->d_ff, k, 1.0f, nullptr, mask, s)) != DIP_OK) return st;
     if ((st = dip_launch_mask_to_idx(ctx, mask, 1, 1, w->d_ff, idx, k, nullptr, s)) != DIP_OK) return st;
-    // the kept rows of the other matrix: h_j = p_j * (W^u x)_j, or p_j * silu((W^g x)_j); 0 elsewhere
-    DIP_CUDA_TRY(ctx, cudaMemsetAsync(h, 0, sizeof(float) * (size_t)w->d_ff, s));
+    // the kept rows of the other matrix: h_j = p_j * (W^u x)_j, or p_j * silu((W^g x)_j); 0 elsewhere (from the
+    // dense product's launch)
     st = dip_launch_rowdot(ctx, w->wtype, by_gate ? w->up : w->gate, w->d_model, w->d_ff, x, idx, k,
-                           by_gate ? 0 : 1, p, h, s);
+                           by_gate ? 0 : 1, p, h, nullptr, s);
     if (st != DIP_OK) return st;
     // y = sum over the kept neurons of W^d[:, j] h_j
     dip_mlp_weights wd = {};

@@ -255,9 +255,9 @@ dip_status dip_launch_tier_fetch(dip_ctx *ctx, const dip_tier *t, cudaStream_t s
 dip_status dip_launch_tier_install(dip_ctx *ctx, const dip_tier *t, cudaStream_t stream);
 
 // rowdot.cu: out_j = [silu](W[j, :] . x) [* mul_j] for the listed rows (rows == nullptr: rows
-// 0 .. n_rows-1) of a row-major [d_ff][d_model] matrix; F32 or BF16.
+// 0 .. n_rows-1) of a row-major [d_ff][d_model] matrix; F32 or BF16.  zero != nullptr: also zero_j = 0 for these rows.
 dip_status dip_launch_rowdot(dip_ctx *ctx, int wtype, const void *W, int d_model, int d_ff, const float *x,
-                             const int32_t *rows, int n_rows, int silu, const float *mul, float *out,
+                             const int32_t *rows, int n_rows, int silu, const float *mul, float *out, float *zero,
                              cudaStream_t stream);
 
 // pack.cu

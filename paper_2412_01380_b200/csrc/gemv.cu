@@ -664,13 +664,28 @@ dip_status dip_launch_bounded_wait_selftest(dip_ctx *ctx, unsigned long long lim
 
 namespace {
 
-// Bit set from an ascending index list (the list-based entry points).
-__global__ void idx_to_mask_kernel(const int32_t *__restrict__ idx, int n, int d, uint32_t *__restrict__ mask)
+// Bit set from an ascending index list (the list-based entry points).  One CTA: the set is made in shared
+// memory and written once, so nothing has to clear it first (a memset and a grid of atomics were two launches).
+__global__ void __launch_bounds__(1024, 1)
+idx_to_mask_kernel(const int32_t *__restrict__ idx, int n, int d, uint32_t *__restrict__ mask)
 {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-        const int i = idx[r];
-        if (i >= 0 && i < d) atomicOr(&mask[i >> 5], 1u << (i & 31));   // out-of-range entries are ignored
+    __shared__ unsigned int words[DIP_MAX_D / 32];
+    const int tid = threadIdx.x, n_words = (d + 31) >> 5;
+    for (int w = tid; w < n_words; w += 1024) words[w] = 0u;
+    dip_grid_dependency_wait();
+    dip_launch_dependents();
+    __syncthreads();
+    constexpr int U = 8;                       // loads that go out together
+    for (int r0 = tid; r0 < n; r0 += U * 1024) {
+        int i[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) i[u] = r0 + u * 1024 < n ? idx[r0 + u * 1024] : -1;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i[u] >= 0 && i[u] < d) atomicOr(&words[i[u] >> 5], 1u << (i[u] & 31));   // out-of-range entries are ignored
     }
+    __syncthreads();
+    for (int w = tid; w < n_words; w += 1024) mask[w] = words[w];
 }
 
 // Sum of the row parts and the epilogue as a kernel of its own (large batches; the two launches
@@ -915,8 +930,6 @@ dip_status dip_launch_gemv(dip_ctx *ctx, const dip_mlp_weights *w, int which,
 
 dip_status dip_launch_idx_to_mask(dip_ctx *ctx, const int32_t *idx, int n, int d, uint32_t *mask, cudaStream_t stream)
 {
-    DIP_CUDA_TRY(ctx, cudaMemsetAsync(mask, 0, sizeof(uint32_t) * ((d + 31) / 32), stream));
-    idx_to_mask_kernel<<<(n + 255) / 256, 256, 0, stream>>>(idx, n, d, mask);
-    DIP_CUDA_TRY(ctx, cudaGetLastError());
+    DIP_CUDA_TRY(ctx, dip_launch_pdl(idx_to_mask_kernel, dim3(1), dim3(1024), 0, stream, idx, n, d, mask));
     return DIP_OK;
 }

@@ -21,6 +21,7 @@ struct RowdotParams {
     int silu;                  // apply silu to the product
     const float *mul;          // [d_ff] or nullptr: out_j *= mul_j
     float *out;                // [d_ff]
+    float *zero;               // [d_ff] or nullptr: zero_j = 0 for each row done
     unsigned long long *tr;
 };
 
@@ -96,6 +97,7 @@ rowdot_kernel(const RowdotParams p)
             float v = p.silu ? rd_silu(acc) : acc;
             if (p.mul) v *= p.mul[j];
             p.out[j] = v;
+            if (p.zero) p.zero[j] = 0.f;
         }
     }
     DIP_TRACE_MAX(p.tr, 2);
@@ -104,7 +106,7 @@ rowdot_kernel(const RowdotParams p)
 }  // namespace
 
 dip_status dip_launch_rowdot(dip_ctx *ctx, int wtype, const void *W, int d_model, int d_ff, const float *x,
-                             const int32_t *rows, int n_rows, int silu, const float *mul, float *out,
+                             const int32_t *rows, int n_rows, int silu, const float *mul, float *out, float *zero,
                              cudaStream_t stream)
 {
     if (wtype != DIP_W_F32 && wtype != DIP_W_BF16) return DIP_ERR_UNSUPPORTED;
@@ -118,6 +120,7 @@ dip_status dip_launch_rowdot(dip_ctx *ctx, int wtype, const void *W, int d_model
     p.silu = silu;
     p.mul = mul;
     p.out = out;
+    p.zero = zero;
     p.tr = dip_trace_slot(ctx, 9);
     const size_t smem = sizeof(float) * (size_t)d_model;
     const int warps_needed = n_rows;

@@ -128,6 +128,8 @@ mask_to_idx_kernel(const uint32_t *__restrict__ mask_bits, int nb, int d,
     __shared__ int wsum[TK_WARPS];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_words = (d + 31) >> 5;
+    dip_grid_dependency_wait();
+    dip_launch_dependents();
     mask_bits += (size_t)blockIdx.x * nb * n_words;
     uint32_t u = 0;
     if (tid < n_words)
@@ -235,8 +237,8 @@ dip_status dip_init_mask_kernels(dip_ctx *ctx)
 dip_status dip_launch_mask_to_idx(dip_ctx *ctx, const uint32_t *mask_bits, int rows, int nb, int d,
                                   int32_t *idx_out, int out_stride, int32_t *count_out, cudaStream_t stream)
 {
-    mask_to_idx_kernel<<<rows, TK_THREADS, 0, stream>>>(mask_bits, nb, d, idx_out, out_stride, count_out);
-    DIP_CUDA_TRY(ctx, cudaGetLastError());
+    DIP_CUDA_TRY(ctx, dip_launch_pdl(mask_to_idx_kernel, dim3(rows), dim3(TK_THREADS), 0, stream, mask_bits, nb, d, idx_out, out_stride,
+                                     count_out));
     return DIP_OK;
 }
 
