@@ -429,7 +429,6 @@ template <int NW> struct __align__(16) GemvDirectSmem {
     int pre[DIP_MAX_D / 32];
     int wsum[GV_SCAN_THREADS / 32];
     int n_total;
-    int last;
     float red[NW][32 * 8];           // [warp][lane * E + e], E <= 8
     float sum[32 * 8];
 };
@@ -554,39 +553,32 @@ gemv_direct_kernel(const GemvParams p)
 #pragma unroll
     for (int e = 0; e < E; ++e) s.red[warp][lane * E + e] = acc[e];
     __syncthreads();
+    float t = 0.f;
     if (tid < SLAB) {
-        float t = 0.f;
 #pragma unroll
         for (int w = 0; w < NW; ++w) t += s.red[w][tid];
-        if (nparts > 1) p.partials[((size_t)part * gridDim.x + slab) * SLAB + tid] = t;
-        else s.sum[tid] = t;
     }
-    // ---- 5. the parts, in part order, by the last CTA of the segment ----
+    // ---- 5. the parts, in part order, in the last part's CTA: a sum is its own message (see gemv_fused.cu) ----
     if (nparts > 1) {
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) s.last = atomicAdd(&p.tickets[slab], 1u) == (unsigned)(nparts - 1);
-        __syncthreads();
-        if (!s.last) {
+        const size_t stride = (size_t)gridDim.x * SLAB;
+        float *box = p.mail + (size_t)slab * SLAB + tid;
+        if (part != nparts - 1) {
+            if (tid < SLAB) mail_put(box + (size_t)part * stride, t);
             DIP_TRACE_MAX(p.tr, 2);
             return;
         }
-        __threadfence();
         if (tid < SLAB) {
-            const size_t stride = (size_t)gridDim.x * SLAB;
-            const float *pp = p.partials + (size_t)slab * SLAB + tid;
-            float t = 0.f;
-            for (int q0 = 0; q0 < nparts; q0 += 8) {
+            float sum = 0.f;
+            for (int q0 = 0; q0 < nparts - 1; q0 += 8) {
                 float a[8];
+                mail_take<8>(box + (size_t)q0 * stride, stride, nparts - 1 - q0, a, p.status, p.wait_limit_ns);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) a[q] = q0 + q < nparts ? __ldcg(pp + (size_t)(q0 + q) * stride) : 0.f;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) t += a[q];
+                for (int q = 0; q < 8; ++q) sum += a[q];
             }
-            s.sum[tid] = t;
+            t = sum + t;
         }
-        if (tid == 0) p.tickets[slab] = 0;                    // ready for the next launch
     }
+    if (tid < SLAB) s.sum[tid] = t;
     __syncthreads();
     // ---- 6. epilogue ----
     if (tid < OUT_PER_SLAB) {
@@ -615,12 +607,11 @@ template <int WT, int WHICH, int NW, int U>
 dip_status launch_direct_cfg(dip_ctx *ctx, GemvParams &p, int n_kept_max, cudaStream_t stream)
 {
     constexpr int SLAB = 32 * WTraits<WT>::E;
-    const int n_slabs = (int)((p.row_bytes + GD_SEG - 1) / GD_SEG);
+    const int n_slabs = (int)((p.row_bytes + GD_SEG - 1) / GD_SEG);   // (parts only with one CTA per SM: the mail boxes suffice)
     int nparts = ctx->sm_count / n_slabs;
     if (nparts > n_kept_max) nparts = n_kept_max;
     if (nparts < 1) nparts = 1;
-    if (n_slabs > ctx->n_tickets) return DIP_ERR_WORKSPACE;
-    if (nparts > 1 && (size_t)nparts * n_slabs * SLAB > ctx->partials_floats) return DIP_ERR_WORKSPACE;
+    static_assert(SLAB <= DIP_MAIL_FLOATS, "");
     p.defer = 0;
     p.part_base = 0;
     DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_direct_kernel<WT, WHICH, NW, U>, dim3(n_slabs, nparts), dim3(NW * 32), 0,
