@@ -21,7 +21,6 @@ struct __align__(16) GemvBtSmem {
     int pre[DIP_MAX_D / 32];
     int wsum[GV_SCAN_THREADS / 32];
     int n_total;
-    int last;
 };
 // after GemvBtSmem (dynamic): float red[NW][BT][SLAB], float sum[BT][SLAB]
 
@@ -165,39 +164,30 @@ gemv_direct_bt_kernel(const GemvParams p)
 #pragma unroll
         for (int e = 0; e < E; ++e) s_red[(warp * BT + b) * SLAB + lane * E + e] = acc[b][e];
     __syncthreads();
+    // ---- 5. the parts, in part order, in the last part's CTA: a sum is its own message (see gemv_fused.cu) ----
     for (int i = tid; i < BT * SLAB; i += THREADS) {
         const int b = i / SLAB, el = i % SLAB;
         float t = 0.f;
 #pragma unroll
         for (int w = 0; w < NW; ++w) t += s_red[(w * BT + b) * SLAB + el];
-        if (nparts > 1) p.partials[((size_t)part * gridDim.x + slab) * (BT * SLAB) + i] = t;
-        else s_sum[i] = t;
+        const size_t stride = (size_t)gridDim.x * (BT * SLAB);
+        float *box = p.mail + (size_t)slab * (BT * SLAB) + i;
+        if (part != nparts - 1) {
+            mail_put(box + (size_t)part * stride, t);
+            continue;
+        }
+        float sum = 0.f;
+        for (int q0 = 0; q0 < nparts - 1; q0 += 8) {
+            float a[8];
+            mail_take<8>(box + (size_t)q0 * stride, stride, nparts - 1 - q0, a, p.status, p.wait_limit_ns);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) sum += a[q];
+        }
+        s_sum[i] = nparts > 1 ? sum + t : t;
     }
-    // ---- 5. the parts, in part order, by the last CTA of the segment ----
-    if (nparts > 1) {
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) s.last = atomicAdd(&p.tickets[slab], 1u) == (unsigned)(nparts - 1);
-        __syncthreads();
-        if (!s.last) {
-            DIP_TRACE_MAX(p.tr, 2);
-            return;
-        }
-        __threadfence();
-        for (int i = tid; i < BT * SLAB; i += THREADS) {
-            const size_t stride = (size_t)gridDim.x * (BT * SLAB);
-            const float *pp = p.partials + (size_t)slab * (BT * SLAB) + i;
-            float t = 0.f;
-            for (int q0 = 0; q0 < nparts; q0 += 8) {
-                float a[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) a[q] = q0 + q < nparts ? __ldcg(pp + (size_t)(q0 + q) * stride) : 0.f;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) t += a[q];
-            }
-            s_sum[i] = t;
-        }
-        if (tid == 0) p.tickets[slab] = 0;                    // ready for the next launch
+    if (part != nparts - 1) {
+        DIP_TRACE_MAX(p.tr, 2);
+        return;
     }
     __syncthreads();
     // ---- 6. epilogue ----
@@ -228,8 +218,7 @@ dip_status launch_cfg(dip_ctx *ctx, GemvParams &p, int n_kept_max, cudaStream_t 
     int nparts = ctx->sm_count / n_slabs;
     if (nparts > n_kept_max) nparts = n_kept_max;
     if (nparts < 1) nparts = 1;
-    if (n_slabs > ctx->n_tickets) return DIP_ERR_WORKSPACE;
-    if (nparts > 1 && (size_t)nparts * n_slabs * BT * SLAB > ctx->partials_floats) return DIP_ERR_WORKSPACE;
+    static_assert(BT * SLAB <= DIP_MAIL_FLOATS, "");        // (parts only with one CTA per SM: the mail boxes suffice)
     p.defer = 0;
     p.part_base = 0;
     const size_t smem = sizeof(GemvBtSmem) + sizeof(float) * (NW + 1) * BT * SLAB;
