@@ -447,7 +447,7 @@ static dip_status step_impl(dip_ctx *ctx, const dip_mlp_weights *w,
         if (cache_gu) due->at[due->n++] = dip_update_of(cache_gu, mask_x);
         // the updates that are due ride with the last block's down product, if that has a cache and SMs to spare; else a
         // launch beside the products takes them
-        const bool ride = last && cache_d && w->wtype != DIP_W_INT4_G128 && dip_gemv_fused_update_room(ctx, w) > due->n;
+        const bool ride = last && cache_d && w->wtype != DIP_W_INT4_G128 && dip_gemv_fused_update_room(ctx, w, k_h) > due->n;
         if (!ride && (last || due->n + 2 > DIP_CACHE_UPDATES)) {
             if ((st = fork_cache_updates(ctx, 0, *due, s)) != DIP_OK) return st;
             due->n = 0;

@@ -227,8 +227,8 @@ struct dip_fused_select {
     const dip_cache_state *update;
     const dip_cache_updates *beside;
 };
-// gemv_fused.cu: how many cache updates (its own among them) find an SM beside a down launch's products.
-int dip_gemv_fused_update_room(const dip_ctx *ctx, const dip_mlp_weights *w);
+// gemv_fused.cu: how many cache updates (its own among them) find an SM beside the products of a down launch of k rows.
+int dip_gemv_fused_update_room(const dip_ctx *ctx, const dip_mlp_weights *w, int k);
 // (INT4: gemv_int4.cu.  Its launches update no caches.)
 bool dip_gemv_fused_supported(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool norm);
 dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int which, const dip_fused_select *sel,

@@ -561,22 +561,14 @@ gemv_direct_kernel(const GemvParams p)
     // ---- 5. the parts, in part order, in the last part's CTA: a sum is its own message (see gemv_fused.cu) ----
     if (nparts > 1) {
         const size_t stride = (size_t)gridDim.x * SLAB;
-        float *box = p.mail + (size_t)slab * SLAB + tid;
+        float *boxes = p.mail + (size_t)slab * SLAB;
         if (part != nparts - 1) {
-            if (tid < SLAB) mail_put(box + (size_t)part * stride, t);
+            if (tid < SLAB) mail_put(boxes + (size_t)part * stride + tid, t);
             DIP_TRACE_MAX(p.tr, 2);
             return;
         }
-        if (tid < SLAB) {
-            float sum = 0.f;
-            for (int q0 = 0; q0 < nparts - 1; q0 += 8) {
-                float a[8];
-                mail_take<8>(box + (size_t)q0 * stride, stride, nparts - 1 - q0, a, p.status, p.wait_limit_ns);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) sum += a[q];
-            }
-            t = sum + t;
-        }
+        if (nparts - 1 > MAIL_N) __syncthreads();               // everyone has read s.red
+        t = mail_sum<SLAB, THREADS>(boxes, stride, nparts - 1, t, &s.red[0][0], p.status, p.wait_limit_ns);
     }
     if (tid < SLAB) s.sum[tid] = t;
     __syncthreads();
@@ -608,9 +600,7 @@ dip_status launch_direct_cfg(dip_ctx *ctx, GemvParams &p, int n_kept_max, cudaSt
 {
     constexpr int SLAB = 32 * WTraits<WT>::E;
     const int n_slabs = (int)((p.row_bytes + GD_SEG - 1) / GD_SEG);   // (parts only with one CTA per SM: the mail boxes suffice)
-    int nparts = ctx->sm_count / n_slabs;
-    if (nparts > n_kept_max) nparts = n_kept_max;
-    if (nparts < 1) nparts = 1;
+    const int nparts = row_parts(ctx->sm_count / n_slabs, n_kept_max, NW);
     static_assert(SLAB <= DIP_MAIL_FLOATS, "");
     p.defer = 0;
     p.part_base = 0;

@@ -165,30 +165,25 @@ gemv_direct_bt_kernel(const GemvParams p)
         for (int e = 0; e < E; ++e) s_red[(warp * BT + b) * SLAB + lane * E + e] = acc[b][e];
     __syncthreads();
     // ---- 5. the parts, in part order, in the last part's CTA: a sum is its own message (see gemv_fused.cu) ----
-    for (int i = tid; i < BT * SLAB; i += THREADS) {
-        const int b = i / SLAB, el = i % SLAB;
-        float t = 0.f;
+    float t = 0.f;
+    static_assert(BT * SLAB <= THREADS, "one sum per thread");
+    if (tid < BT * SLAB) {
+        const int b = tid / SLAB, el = tid % SLAB;
 #pragma unroll
         for (int w = 0; w < NW; ++w) t += s_red[(w * BT + b) * SLAB + el];
+    }
+    if (nparts > 1) {
         const size_t stride = (size_t)gridDim.x * (BT * SLAB);
-        float *box = p.mail + (size_t)slab * (BT * SLAB) + i;
+        float *boxes = p.mail + (size_t)slab * (BT * SLAB);
         if (part != nparts - 1) {
-            mail_put(box + (size_t)part * stride, t);
-            continue;
+            if (tid < BT * SLAB) mail_put(boxes + (size_t)part * stride + tid, t);
+            DIP_TRACE_MAX(p.tr, 2);
+            return;
         }
-        float sum = 0.f;
-        for (int q0 = 0; q0 < nparts - 1; q0 += 8) {
-            float a[8];
-            mail_take<8>(box + (size_t)q0 * stride, stride, nparts - 1 - q0, a, p.status, p.wait_limit_ns);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) sum += a[q];
-        }
-        s_sum[i] = nparts > 1 ? sum + t : t;
+        if (nparts - 1 > MAIL_N) __syncthreads();               // everyone has read s_red
+        t = mail_sum<BT * SLAB, THREADS>(boxes, stride, nparts - 1, t, s_red, p.status, p.wait_limit_ns);
     }
-    if (part != nparts - 1) {
-        DIP_TRACE_MAX(p.tr, 2);
-        return;
-    }
+    if (tid < BT * SLAB) s_sum[tid] = t;
     __syncthreads();
     // ---- 6. epilogue ----
     for (int i = tid; i < BT * OUT_PER_SLAB; i += THREADS) {
@@ -215,9 +210,7 @@ dip_status launch_cfg(dip_ctx *ctx, GemvParams &p, int n_kept_max, cudaStream_t 
 {
     constexpr int SLAB = 32 * WTraits<WT>::E;
     const int n_slabs = (int)((p.row_bytes + GB_SEG - 1) / GB_SEG);
-    int nparts = ctx->sm_count / n_slabs;
-    if (nparts > n_kept_max) nparts = n_kept_max;
-    if (nparts < 1) nparts = 1;
+    const int nparts = row_parts(ctx->sm_count / n_slabs, n_kept_max, NW);
     static_assert(BT * SLAB <= DIP_MAIL_FLOATS, "");        // (parts only with one CTA per SM: the mail boxes suffice)
     p.defer = 0;
     p.part_base = 0;

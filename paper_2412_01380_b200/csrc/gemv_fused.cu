@@ -508,29 +508,25 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
     if (writer)
         for (int w = tid; w < mask_words; w += TK_THREADS) p.mask_out[w] = s.maskw[w];
     __syncthreads();
-    if (tid >= SLAB) return;
+    if (tid >= SLAB && (part != nparts - 1 || nparts - 1 <= MAIL_N)) return;
     float t = 0.f;
+    if (tid < SLAB) {
 #pragma unroll
-    for (int g = 0; g < G; ++g) t += psum[g * SLAB + tid];
+        for (int g = 0; g < G; ++g) t += psum[g * SLAB + tid];
+    }
     // ---- the parts, in part order, in the last part's CTA.  A sum is its own message: the CTA that adds them up
     //      waits until none of its inputs is "empty" any more, and empties them for the next launch.  Blocks start
     //      in index order and only the last ones wait, so what they wait for is running or done ----
     if (nparts > 1) {
         const size_t stride = (size_t)p.n_slabs * SLAB;
-        float *box = p.mail + (size_t)slab * SLAB + tid;
+        float *boxes = p.mail + (size_t)slab * SLAB;
         if (part != nparts - 1) {
-            mail_put(box + (size_t)part * stride, t);
+            mail_put(boxes + (size_t)part * stride + tid, t);
             DIP_TRACE_MAX(p.tr, 2);
             return;
         }
-        float sum = 0.f;
-        for (int q0 = 0; q0 < nparts - 1; q0 += 8) {
-            float a[8];
-            mail_take<8>(box + (size_t)q0 * stride, stride, nparts - 1 - q0, a, p.status, p.wait_limit_ns);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) sum += a[q];
-        }
-        t = sum + t;
+        t = mail_sum<SLAB, TK_THREADS>(boxes, stride, nparts - 1, t, red, p.status, p.wait_limit_ns);
+        if (tid >= SLAB) return;
     }
     // ---- epilogue ----
     const float up = __shfl_down_sync(0xffffffffu, t, 4);      // gate/up: a gate element's up element is four positions on
@@ -589,8 +585,8 @@ size_t fused_smem_bytes(int d_in, bool x_near)
     return sizeof(FusedSmem) + dpad * 4 + (x_near ? dpad * 4 : 0);
 }
 
-// Segments and row parts of a launch; false when the shape does not fit this path.
-bool fused_plan(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool norm, FusedParams &p)
+// Segments and row parts of a launch of k rows; false when the shape does not fit this path.
+bool fused_plan(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool norm, int k, FusedParams &p)
 {
     if (!ctx->gemv_direct || !ctx->fuse_select) return false;
     if (w->wtype != DIP_W_F32 && w->wtype != DIP_W_BF16) return false;
@@ -603,26 +599,26 @@ bool fused_plan(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool no
     p.row_bytes = w->wtype == DIP_W_F32 ? row_elems * 4 : row_elems * 2;
     p.n_slabs = (int)((p.row_bytes + GF_SEG - 1) / GF_SEG);
     // one CTA per SM, and where that is cheap two SMs to spare for the blocks that update caches
-    p.nparts = ctx->sm_count / p.n_slabs;              // (DIP_MAIL_FLOATS per SM suffice)
-    if (p.nparts > 4 && p.nparts * p.n_slabs > ctx->sm_count - 2) --p.nparts;
-    if (p.nparts < 1) p.nparts = 1;
+    int most = ctx->sm_count / p.n_slabs;              // (DIP_MAIL_FLOATS per SM suffice)
+    if (most > 4 && most * p.n_slabs > ctx->sm_count - 2) --most;
+    p.nparts = row_parts(most, k, GF_NW);
     return true;
 }
 
 }  // namespace
 
-int dip_gemv_fused_update_room(const dip_ctx *ctx, const dip_mlp_weights *w)
+int dip_gemv_fused_update_room(const dip_ctx *ctx, const dip_mlp_weights *w, int k)
 {
     FusedParams p;
     // (a wave of products that fills the SMs to the last one leaves none)
-    return fused_plan(ctx, w, 1, false, p) ? (ctx->sm_count - p.n_slabs * p.nparts % ctx->sm_count) % ctx->sm_count : 0;
+    return fused_plan(ctx, w, 1, false, k, p) ? (ctx->sm_count - p.n_slabs * p.nparts % ctx->sm_count) % ctx->sm_count : 0;
 }
 
 bool dip_gemv_fused_supported(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool norm)
 {
     if (w->wtype == DIP_W_INT4_G128) return dip_gemv_int4_selects(ctx, w, which);
     FusedParams p;
-    return fused_plan(ctx, w, which, norm, p);
+    return fused_plan(ctx, w, which, norm, 1, p);
 }
 
 dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int which, const dip_fused_select *sel,
@@ -657,8 +653,7 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
         return dip_launch_gemv_int4(ctx, g, which, sel->k, 0, sel, stream);
     }
     FusedParams p;
-    if (!fused_plan(ctx, w, which, norm, p)) return DIP_ERR_UNSUPPORTED;
-    if (p.nparts > sel->k) p.nparts = sel->k;
+    if (!fused_plan(ctx, w, which, norm, sel->k, p)) return DIP_ERR_UNSUPPORTED;
     p.W = (const char *)(which == 0 ? w->gate_up : w->down);
     p.out = out;
     p.mail = ctx->mail;
