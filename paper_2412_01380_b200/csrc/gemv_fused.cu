@@ -600,7 +600,7 @@ bool fused_plan(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool no
     p.n_slabs = (int)((p.row_bytes + GF_SEG - 1) / GF_SEG);
     // one CTA per SM, and where that is cheap two SMs to spare for the blocks that update caches
     int most = ctx->sm_count / p.n_slabs;              // (DIP_MAIL_FLOATS per SM suffice)
-    if (most > 4 && most * p.n_slabs > ctx->sm_count - 2) --most;
+    if (most > 4 && most * p.n_slabs > ctx->sm_count - 2) most = (ctx->sm_count - 2) / p.n_slabs;
     p.nparts = row_parts(most, k, GF_NW);
     return true;
 }

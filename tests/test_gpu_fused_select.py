@@ -104,3 +104,28 @@ def test_stacks_leave_their_cache_updates_to_later_launches(n_layers, caches, wt
                 assert torch.equal(p.stamp, q.stamp) and torch.equal(p.meta, q.meta), t
     assert ctx.device_status() == 0
     ctx.close()
+
+
+def launch_kinds(ctx, call):
+    """The kinds of the library's launches in a call, as its own timeline records them."""
+    ctx.trace_begin()
+    call()
+    torch.cuda.synchronize()
+    kinds = [r["kind"] for r in ctx.trace_read()]
+    ctx.trace_end()
+    return kinds
+
+
+def test_rows_of_one_segment_leave_room_for_both_updates():
+    """A part per SM would leave none: 5000 rows of 256 BF16 outputs."""
+    import paper_2412_01380_b200 as dip
+    ctx = dip.Context(0)
+    d_model, d_ff = 256, 8192
+    lw = _layer(d_model, d_ff, di.W_BF16, 5)
+    w = upload_layer(dip, ctx, lw)
+    refs = [oracle.Cache(d, d // 2) for d in (d_model, d_ff)]
+    mine = [dip.CacheState(d, d // 2, "cuda") for d in (d_model, d_ff)]
+    for t in range(2):
+        kinds = launch_kinds(ctx, lambda: check_step(dip, ctx, lw, w, di.heavy_tail_vector(t, d_model), 100, 5000, 0.3, *refs, *mine))
+        assert kinds == ["gemv_gate_up", "gemv_down"]           # (no launch for the updates)
+    ctx.close()
