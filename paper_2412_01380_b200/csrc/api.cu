@@ -663,6 +663,14 @@ static dip_status stack_impl(dip_ctx *ctx, int n_layers, const dip_mlp_weights *
                   !dip_aligned16(probe->mask_x) || !dip_aligned16(probe->h) || !dip_aligned16(probe->mask_h) ||
                   !dip_aligned16(probe->y) || (d & 127) || (d_ff & 127)))
         return DIP_ERR_INVALID_ARG;      // (per-layer slices of the arrays stay 16-byte aligned)
+    // What a block's step would refuse is refused here, before the blocks in front of it are launched: a call that fails
+    // half-way would leave their masks made and their caches as they were.
+    if (k_x < 1 || k_x > d || k_h < 1 || k_h > d_ff || !(gamma >= 0.0f) || !isfinite(gamma)) return DIP_ERR_INVALID_ARG;
+    for (int l = 0; l < n_layers; ++l) {
+        if (cache_gu && !cache_ok(&cache_gu[l], d)) return DIP_ERR_INVALID_ARG;
+        if (cache_d && !cache_ok(&cache_d[l], d_ff)) return DIP_ERR_INVALID_ARG;
+        if (batch > 1 && (cache_gu || cache_d || layers[l].wtype == DIP_W_INT4_G128)) return DIP_ERR_UNSUPPORTED;
+    }
     cudaStream_t s = (cudaStream_t)stream;
     const size_t ring_words = (size_t)ctx->max_d / 32;
     // x_0 = x_in; for l > 0 the chaining x_l = rmsnorm(x_{l-1} + y_{l-1}) runs inside layer l's

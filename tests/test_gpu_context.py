@@ -134,3 +134,37 @@ def test_misaligned_pointers_are_rejected_before_any_launch(dip):
     finally:
         torch.cuda.synchronize()
         c.close()
+
+
+@pytest.mark.parametrize("wtype", [di.W_BF16, di.W_INT4_G128])
+def test_a_stack_with_a_bad_block_launches_nothing(dip, wtype):
+    """A cache state that only the last block refuses: an error code, no launch, states untouched; the next good call is right."""
+    c = dip.Context(0)
+    try:
+        wl = di.WORKLOADS["phi3_mini"].scaled(seed=12, d_model=256, d_ff=640, wtype=wtype, n_layers=3)
+        ws = [upload_layer(dip, c, di.layer_weights(wl, l)) for l in range(3)]
+        caches = [[dip.CacheState(d, d // 2, "cuda") for _ in range(3)] for d in (256, 640)]
+        x, y = torch.from_numpy(di.heavy_tail_vector(1, 256)).cuda(), torch.empty(256, device="cuda")
+        for which in (0, 1):
+            stack = dip.Stack(ws, *caches)
+            arr = (stack.gu_arr, stack.d_arr)[which]
+            arr[2].capacity = arr[2].d + 1
+            c.trace_begin()
+            with pytest.raises(dip.DipError) as e:
+                dip.dip_stack_step(c, stack, x, 64, 160, 0.2, y)
+            assert e.value.status == dip.ERR_INVALID_ARG
+            assert c.trace_read() == []
+            c.trace_end()
+        with pytest.raises(dip.DipError) as e:
+            dip.dip_stack_step(c, dip.Stack(ws, *caches), x, 64, 641, 0.2, y)
+        assert e.value.status == dip.ERR_INVALID_ARG
+        with pytest.raises(dip.DipError) as e:
+            dip.dip_stack_step(c, dip.Stack(ws, *caches), x.expand(2, 256).contiguous(), 64, 160, 0.2, y.expand(2, 256).contiguous())
+        assert e.value.status == dip.ERR_UNSUPPORTED
+        assert all(int(s.meta.abs().sum()) == 0 and int(s.stamp.max()) == -1 for half in caches for s in half)
+        dip.dip_stack_step(c, dip.Stack(ws, *caches), x, 64, 160, 0.2, y)
+        torch.cuda.synchronize()
+        assert all(int(s.meta[1]) == 1 for half in caches for s in half) and c.device_status() == dip.DEVICE_OK
+    finally:
+        torch.cuda.synchronize()
+        c.close()
