@@ -118,16 +118,23 @@ const char *dip_status_string(dip_status s);
 const char *dip_last_error(const dip_ctx *ctx);
 /* Number of streaming multiprocessors of the context's device. */
 int dip_sm_count(const dip_ctx *ctx);
-/* Every wait inside a kernel (on the arrival of an asynchronous copy) is bounded.  If one runs
- * out, the kernel stops early, its outputs are invalid and a sticky status word on the device
- * becomes non-zero.  This call waits for `stream`, then copies the word to *status_out (host). */
+/* Every wait inside a kernel is bounded: on the arrival of an asynchronous copy, and on another thread
+ * block of the same launch (the blocks of a one- or two-token product hand their row parts to the
+ * block that adds them up; the block that updates a cache waits until the others have read its state).
+ * If a wait runs out, the kernel goes on without what it waited for and a sticky status word on the
+ * device becomes non-zero.  From then on the outputs of that call AND OF EVERY LATER CALL on the context
+ * are invalid (what came too late is still under way in its workspace) until dip_reset_device_status;
+ * a cache state that the failed call was to update may or may not be updated: restore or clear it.
+ * No call looks at the word by itself.
+ * This call waits for `stream`, then copies the word to *status_out (host). */
 typedef enum {
     DIP_DEVICE_OK = 0,
     DIP_DEVICE_WAIT_TIMEOUT = 1,        /* a kernel gave up a bounded wait                          */
     DIP_DEVICE_TIER_INCONSISTENT = 2    /* two-tier step: slot table and cache state disagree       */
 } dip_device_status_word;
 dip_status dip_device_status(dip_ctx *ctx, int *status_out, void *stream);
-/* Clears the sticky word (enqueued on `stream`). */
+/* Clears the sticky word and what a wait that ran out has left in the workspace (enqueued on `stream`;
+ * like any call, not while work of this context is in flight on another stream). */
 dip_status dip_reset_device_status(dip_ctx *ctx, void *stream);
 /* Self-test of the bounded wait (diagnostics): enqueues one tiny kernel that waits, with the
  * given limit, for a copy that is never issued.  The wait runs out, the kernel returns, and the
@@ -251,6 +258,12 @@ typedef struct {
     int32_t policy;     /* dip_cache_policy                                 */
     int32_t reserved;
 } dip_cache_state;
+
+/* Self-test of the waits between thread blocks (see dip_device_status): enqueues one kernel in which a row part and a reader of the
+ * cache state `st` come too late for the limit.  The status word becomes DIP_DEVICE_WAIT_TIMEOUT and the
+ * workspace is as after a real failure (call dip_reset_device_status); the state, whose update with the mask
+ * mask_bits [ceil(st->d/32)] is given up, stays as it is.  1 <= limit_us <= 1000000. */
+dip_status dip_selftest_block_waits(dip_ctx *ctx, int limit_us, const dip_cache_state *st, const uint32_t *mask_bits, void *stream);
 
 /* ------------------------------------------------------------------------
  * dip_mask_topk — per-token magnitude top-k (Sec. 3.1; the masks of Eq. 7-8).

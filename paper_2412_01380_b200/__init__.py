@@ -62,6 +62,8 @@ _lib.dip_reset_device_status.restype = _i32
 _lib.dip_reset_device_status.argtypes = [_vp, _vp]
 _lib.dip_selftest_bounded_wait.restype = _i32
 _lib.dip_selftest_bounded_wait.argtypes = [_vp, _i32, _vp, _vp]
+_lib.dip_selftest_block_waits.restype = _i32
+_lib.dip_selftest_block_waits.argtypes = [_vp, _i32, C.POINTER(CacheStateStruct), _vp, _vp]
 _lib.dip_destroy.restype = _i32
 _lib.dip_destroy.argtypes = [_vp]
 _lib.dip_status_string.restype = C.c_char_p
@@ -130,7 +132,7 @@ _lib.dip_sparse_gemv_down_noalloc.restype = _i32
 _lib.dip_sparse_gemv_down_noalloc.argtypes = [C.POINTER(MlpWeightsStruct), _vp, _vp, _i32, _vp, _vp]
 
 EXPORTED = ["dip_create", "dip_create_ex", "dip_destroy", "dip_status_string", "dip_last_error", "dip_sm_count",
-            "dip_device_status", "dip_reset_device_status", "dip_selftest_bounded_wait", "dip_stack_step_probed",
+            "dip_device_status", "dip_reset_device_status", "dip_selftest_bounded_wait", "dip_selftest_block_waits", "dip_stack_step_probed",
             "dip_trace_begin", "dip_trace_reset", "dip_trace_read", "dip_trace_end",
             "dip_packed_bytes", "dip_pack_weights", "dip_mask_topk", "dip_ca_mask",
             "dip_sparse_gemv_gate_up", "dip_sparse_gemv_down", "dip_select_gemv_gate_up", "dip_select_gemv_down",
@@ -206,6 +208,10 @@ class Context:
     def selftest_bounded_wait(self, limit_us: int, waited_ns: Optional[torch.Tensor] = None) -> None:
         """Enqueue the tiny kernel whose bounded wait runs out (device status becomes 1)."""
         self.check(_lib.dip_selftest_bounded_wait(self.handle, int(limit_us), _ptr(waited_ns), _stream()))
+
+    def selftest_block_waits(self, limit_us: int, st: "CacheState", mask_bits: torch.Tensor) -> None:
+        """Enqueue the kernel whose waits between thread blocks run out (device status becomes 1, st stays as it is)."""
+        self.check(_lib.dip_selftest_block_waits(self.handle, int(limit_us), C.byref(st.struct), _ptr(mask_bits), _stream()))
 
     def trace_begin(self) -> None:
         self.check(_lib.dip_trace_begin(self.handle))

@@ -273,6 +273,13 @@ dip_status dip_selftest_bounded_wait(dip_ctx *ctx, int limit_us, unsigned long l
     return dip_launch_bounded_wait_selftest(ctx, 1000ull * (unsigned long long)limit_us, waited_ns, (cudaStream_t)stream);
 }
 
+dip_status dip_selftest_block_waits(dip_ctx *ctx, int limit_us, const dip_cache_state *st, const uint32_t *mask_bits, void *stream)
+{
+    if (!ctx_ok(ctx) || limit_us < 1 || limit_us > 1000000 || !mask_bits || !dip_aligned16(mask_bits)) return DIP_ERR_INVALID_ARG;
+    if (!st || st->d < 1 || st->d > DIP_MAX_D || !cache_ok(st, st->d)) return DIP_ERR_INVALID_ARG;
+    return dip_launch_block_waits_selftest(ctx, 1000ull * (unsigned long long)limit_us, dip_update_of(st, mask_bits), (cudaStream_t)stream);
+}
+
 // Run cache updates beside the main stream (side stream `which`).
 static dip_status fork_cache_updates(dip_ctx *ctx, int which, const dip_cache_updates &u, cudaStream_t main)
 {

@@ -27,7 +27,7 @@ struct dip_ctx {
     // split-row partial sums of the two GEMVs (binary32)
     float *partials;
     size_t partials_floats;
-    float *mail;         // [sm_count][DIP_MAIL_FLOATS] row parts of the fused products on their way to the CTA that adds them up
+    float *mail;         // [sm_count][DIP_MAIL_FLOATS] row parts of one- and two-token products on their way to the CTA that adds them up
     unsigned int *readers; // [1] CTAs of a fused product that have read the stamps; zero between launches
     // one arrival counter per output slab; zero between launches
     unsigned int *tickets;
@@ -237,6 +237,9 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
 // gemv.cu: one tiny kernel whose bounded wait runs out (sets the status word to 1).
 dip_status dip_launch_bounded_wait_selftest(dip_ctx *ctx, unsigned long long limit_ns, unsigned long long *waited_ns,
                                             cudaStream_t stream);
+
+// gemv_fused.cu: one kernel whose waits between blocks run out (sets the status word to 1, leaves the cache state as it is).
+dip_status dip_launch_block_waits_selftest(dip_ctx *ctx, unsigned long long limit_ns, const dip_cache_update &c, cudaStream_t stream);
 
 // gemv.cu: bit set from an ascending index list.
 dip_status dip_launch_idx_to_mask(dip_ctx *ctx, const int32_t *idx, int n, int d, uint32_t *mask, cudaStream_t stream);

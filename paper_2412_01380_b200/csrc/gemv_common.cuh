@@ -81,6 +81,9 @@ __device__ __forceinline__ void l2_prefetch(const void *p, unsigned bytes)
 // Sums that one CTA of a launch hands to another through global memory: the value itself is the message.
 // A box holds DIP_MAIL_EMPTY (a NaN pattern that no arithmetic produces) until its sum arrives; who
 // takes a sum empties its box again.
+// The block that waits is the last part of its segment.  It cannot keep those that it waits for from running: a launch with
+// parts has at most one block per SM, and where something else holds SMs, blocks are started in index order, so the earlier
+// parts are running or done when it starts.  The order is what the hardware does, not a promise, hence the limit.
 __device__ __forceinline__ void mail_put(float *box, float v)
 {
     asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(box), "f"(v) : "memory");

@@ -605,7 +605,50 @@ bool fused_plan(const dip_ctx *ctx, const dip_mlp_weights *w, int which, bool no
     return true;
 }
 
+// Self-test of the waits between blocks.  Block 0 collects ten row parts of which one is missing, and sends that one too
+// late; block 1 updates a cache whose readers (two are expected) have not all counted, and the missing one counts too late.
+__global__ void __launch_bounds__(TK_THREADS, 1)
+block_waits_selftest_kernel(float *mail, unsigned int *readers, int *status, unsigned long long limit_ns, const dip_cache_update c)
+{
+    constexpr int SLAB = 256, N = MAIL_N + 2, MISSING = MAIL_N;
+    __shared__ TkShared ts;
+    __shared__ __align__(16) unsigned int small[CU_SMALL * CU_SPREAD];
+    __shared__ float sum[TK_THREADS];
+    __shared__ int go;
+    const int tid = threadIdx.x;
+    if (blockIdx.x == 0) {
+        if (tid < SLAB)
+            for (int q = 0; q < N; ++q)
+                if (q != MISSING) mail_put(mail + q * SLAB + tid, 1.f);
+        (void)mail_sum<SLAB, TK_THREADS>(mail, SLAB, N, 1.f, sum, status, limit_ns);
+        if (tid < SLAB) mail_put(mail + MISSING * SLAB + tid, 1e30f);
+        return;
+    }
+    cache_update_clear(ts, small);
+    block_cache_update_any(
+        c.mask, c.d, c.stamp, c.stamp, c.count, c.meta, c.capacity, ts, small,
+        [&]() {
+            if (tid % 32 == 0) {
+                count_one(readers);
+                go = wait_count(readers, 2u, status, limit_ns);
+                *readers = 0u;
+            }
+        },
+        [&]() {
+            __syncthreads();
+            return go != 0;
+        });
+    if (tid == TK_THREADS - 32) count_one(readers);
+}
+
 }  // namespace
+
+dip_status dip_launch_block_waits_selftest(dip_ctx *ctx, unsigned long long limit_ns, const dip_cache_update &c, cudaStream_t stream)
+{
+    block_waits_selftest_kernel<<<2, TK_THREADS, 0, stream>>>(ctx->mail, ctx->readers, ctx->status, limit_ns, c);
+    DIP_CUDA_TRY(ctx, cudaGetLastError());
+    return DIP_OK;
+}
 
 int dip_gemv_fused_update_room(const dip_ctx *ctx, const dip_mlp_weights *w, int k)
 {

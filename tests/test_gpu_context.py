@@ -6,7 +6,7 @@ import torch
 
 import dip_inputs as di
 import oracle
-from gpu_util import check_step, upload_layer
+from gpu_util import cache_equal, check_step, upload_layer
 
 pytestmark = pytest.mark.gpu
 
@@ -42,6 +42,40 @@ def test_bounded_wait_runs_out_and_the_context_stays_usable(dip):
             c.selftest_bounded_wait(0)
         with pytest.raises(dip.DipError):
             c.selftest_bounded_wait(2_000_000)
+    finally:
+        torch.cuda.synchronize()
+        c.close()
+
+
+@pytest.mark.parametrize("policy", ["lru"])
+@pytest.mark.parametrize("d", [1056, 17920])
+def test_block_waits_run_out_and_a_reset_mends_the_context(dip, d, policy):
+    """Row parts and readers of a cache state that come too late: status 1, the state as it was, and after a reset the same
+    boxes and the same counter serve correct steps (33 parts per segment, updates that ride along)."""
+    c = dip.Context(0)
+    try:
+        ref, st = oracle.Cache(d, d // 2, policy), dip.CacheState(d, d // 2, "cuda", policy)
+        bits = torch.zeros((d + 31) // 32, dtype=torch.int32, device="cuda")
+        for t in range(3):
+            v = di.heavy_tail_vector(20 + t, d)
+            dip.dip_ca_mask(c, torch.from_numpy(v).cuda(), d // 3, 0.2, st, bits, None)
+            oracle.dip_ca_mask(v, d // 3, 0.2, ref)
+        dip.dip_mask_topk(c, torch.from_numpy(di.heavy_tail_vector(30, d)).cuda(), d // 3, bits, None)
+        assert c.device_status() == dip.DEVICE_OK and cache_equal(st, ref)
+        c.selftest_block_waits(1000, st, bits)
+        assert c.device_status() == dip.DEVICE_WAIT_TIMEOUT
+        assert cache_equal(st, ref)
+        c.reset_device_status()
+        lw = di.layer_weights(di.WORKLOADS["phi3_mini"].scaled(seed=4, d_model=256, d_ff=1536, n_layers=1), 0)
+        w = upload_layer(dip, c, lw)
+        refs = [oracle.Cache(n, n // 2) for n in (256, 1536)]
+        mine = [dip.CacheState(n, n // 2, "cuda") for n in (256, 1536)]
+        for t in range(2):
+            check_step(dip, c, lw, w, di.heavy_tail_vector(40 + t, 256), 128, 1056, 0.2, *refs, *mine)
+        assert c.device_status() == dip.DEVICE_OK
+        for bad in (0, 2_000_000):
+            with pytest.raises(dip.DipError):
+                c.selftest_block_waits(bad, st, bits)
     finally:
         torch.cuda.synchronize()
         c.close()
