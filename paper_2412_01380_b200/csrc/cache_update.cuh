@@ -20,8 +20,9 @@ namespace {
 //
 // mask_bits and stamp_now (the stamps as they are) may lie in shared memory.  s.hist and small[] are zero on
 // entry (cache_update_clear), though not yet synchronised.  poll() is called by the last warp (which seldom has
-// columns) some time before may_write(), which all threads call before the first stamp is written; if it says
-// no, the call ends there.  (The counters, which only this function reads, are written before that.)
+// columns) some time before may_write(), which all threads call before the first stamp is written (and which is a
+// barrier unless it always says yes); if it says no, the state is left as it was.  (The counters, which only this
+// function reads, are written before that, and restored.)
 constexpr int CU_SPREAD = 8;                            // copies of the counters of the small digits,
 constexpr int CU_SMALL = 256;                           // which nearly all keys have: ages of a few updates
 
@@ -219,7 +220,12 @@ __device__ __forceinline__ void block_cache_update(const uint32_t *mask_bits, in
     const uint32_t use = (keep & res) | (total_misses > room ? first_of(misses, miss_before, warp_misses, room) : misses);
 
     // ---- the new stamps ----
-    if (!may_write()) return;
+    if (!may_write()) {
+        if (LFU)                                        // the uses are taken back (from the mask: nothing is kept for this)
+            for (int c = tid; c < d; c += TK_THREADS)
+                if ((mask_bits[c >> 5] >> (c & 31)) & 1u) --count[c];
+        return;
+    }
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
         const int c = col0 + 128 * i;

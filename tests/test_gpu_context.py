@@ -47,7 +47,7 @@ def test_bounded_wait_runs_out_and_the_context_stays_usable(dip):
         c.close()
 
 
-@pytest.mark.parametrize("policy", ["lru"])
+@pytest.mark.parametrize("policy", ["lru", "lfu"])
 @pytest.mark.parametrize("d", [1056, 17920])
 def test_block_waits_run_out_and_a_reset_mends_the_context(dip, d, policy):
     """Row parts and readers of a cache state that come too late: status 1, the state as it was, and after a reset the same
