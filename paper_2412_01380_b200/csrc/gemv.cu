@@ -567,8 +567,12 @@ gemv_direct_kernel(const GemvParams p)
             DIP_TRACE_MAX(p.tr, 2);
             return;
         }
-        if (nparts - 1 > MAIL_N) __syncthreads();               // everyone has read s.red
-        t = mail_sum<SLAB, THREADS>(boxes, stride, nparts - 1, t, &s.red[0][0], p.status, p.wait_limit_ns);
+        if (nparts - 1 > MAIL_N) {
+            __syncthreads();           // everyone has read s.red
+            t = mail_sum_wide<SLAB, THREADS>(boxes, stride, nparts - 1, &s.red[0][0], p.status, p.wait_limit_ns) + t;
+        } else if (tid < SLAB) {
+            t = mail_sum(boxes + tid, stride, nparts - 1, p.status, p.wait_limit_ns) + t;
+        }
     }
     if (tid < SLAB) s.sum[tid] = t;
     __syncthreads();

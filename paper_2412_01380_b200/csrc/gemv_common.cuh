@@ -119,33 +119,41 @@ __device__ __forceinline__ void mail_take(float *box, size_t stride, int n, floa
         if (q < n) mail_put(box + (size_t)q * stride, __uint_as_float(DIP_MAIL_EMPTY));
 }
 
-// The row parts of a segment of SLAB elements in the last part's CTA of T threads (all call it): the n sums in boxes[0],
-// boxes[stride], ... and this part's own (thread e < SLAB has element e's, and gets the result; the others' is void).
-// Up to MAIL_N parts are one trip of the first SLAB threads; more are shared out, MAIL_N at a time, over the CTA's
-// T / SLAB groups, whose sums meet in order of the groups.  (Narrow rows have up to one part per SM, and the first SLAB
-// threads alone paid a trip to L2 for every eight: the down product of 704 rows of 256 BF16 outputs took 12.3 us, with
-// both this and row_parts 5.8.)  scratch: T floats of shared memory that nobody reads or writes any more.
+// Up to MAIL_N row parts are one trip of a segment's threads, one per element.  More are shared out, MAIL_N at a time,
+// over the T / SLAB groups of the last part's CTA (all T threads call it): the sum of the n boxes boxes[0], boxes[stride], ...
+// of element tid % SLAB, the groups' sums in order of the groups.  (Narrow rows have up to one part per SM, and a trip to L2
+// for every eight added up: the down product of 704 rows of 256 BF16 outputs took 12.3 us, with both this and row_parts
+// 5.8.)  Out of line: in line it cost the launches that carry cache updates, which never come here at these widths, 0.4 us
+// (one step with caches, 3072 / 8192: 19.1 us, 18.8 like this).
+// scratch: T floats of shared memory that nobody reads or writes any more.
 constexpr int MAIL_N = 8;
 template <int SLAB, int T>
-__device__ __forceinline__ float mail_sum(float *boxes, size_t stride, int n, float own, float *scratch, int *status, unsigned long long limit_ns)
+__device__ __noinline__ float mail_sum_wide(float *boxes, size_t stride, int n, float *scratch, int *status, unsigned long long limit_ns)
 {
     static_assert(T % SLAB == 0, "");
-    const int tid = threadIdx.x, el = tid % SLAB, group = tid / SLAB;
+    const int tid = threadIdx.x, el = tid % SLAB;
     float sum = 0.f;
-    for (int q0 = group * MAIL_N; q0 < n; q0 += T / SLAB * MAIL_N) {
+    for (int q0 = tid / SLAB * MAIL_N; q0 < n; q0 += T / SLAB * MAIL_N) {
         float a[MAIL_N];
         mail_take<MAIL_N>(boxes + (size_t)q0 * stride + el, stride, n - q0, a, status, limit_ns);
 #pragma unroll
         for (int q = 0; q < MAIL_N; ++q) sum += a[q];
     }
-    if (n > MAIL_N) {
-        scratch[tid] = sum;
-        __syncthreads();
-        sum = 0.f;
+    scratch[tid] = sum;
+    __syncthreads();
+    sum = 0.f;
 #pragma unroll
-        for (int g = 0; g < T / SLAB; ++g) sum += scratch[g * SLAB + el];
-    }
-    return sum + own;
+    for (int g = 0; g < T / SLAB; ++g) sum += scratch[g * SLAB + el];
+    return sum;
+}
+// The same for n <= MAIL_N by one thread for its element.
+__device__ __forceinline__ float mail_sum(float *box, size_t stride, int n, int *status, unsigned long long limit_ns)
+{
+    float a[MAIL_N], sum = 0.f;
+    mail_take<MAIL_N>(box, stride, n, a, status, limit_ns);
+#pragma unroll
+    for (int q = 0; q < MAIL_N; ++q) sum += a[q];
+    return sum;
 }
 
 // Parts of n rows by CTAs of `warps` warps, at most `most`: with less than a row per warp a part takes no less time, and one

@@ -180,8 +180,12 @@ gemv_direct_bt_kernel(const GemvParams p)
             DIP_TRACE_MAX(p.tr, 2);
             return;
         }
-        if (nparts - 1 > MAIL_N) __syncthreads();               // everyone has read s_red
-        t = mail_sum<BT * SLAB, THREADS>(boxes, stride, nparts - 1, t, s_red, p.status, p.wait_limit_ns);
+        if (nparts - 1 > MAIL_N) {
+            __syncthreads();           // everyone has read s_red
+            t = mail_sum_wide<BT * SLAB, THREADS>(boxes, stride, nparts - 1, s_red, p.status, p.wait_limit_ns) + t;
+        } else if (tid < BT * SLAB) {
+            t = mail_sum(boxes + tid, stride, nparts - 1, p.status, p.wait_limit_ns) + t;
+        }
     }
     if (tid < BT * SLAB) s_sum[tid] = t;
     __syncthreads();

@@ -508,25 +508,26 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
     if (writer)
         for (int w = tid; w < mask_words; w += TK_THREADS) p.mask_out[w] = s.maskw[w];
     __syncthreads();
-    if (tid >= SLAB && (part != nparts - 1 || nparts - 1 <= MAIL_N)) return;
+    const size_t stride = (size_t)p.n_slabs * SLAB;
+    float *boxes = p.mail + (size_t)slab * SLAB;
+    float others = 0.f;
+    if (nparts - 1 > MAIL_N && part == nparts - 1)
+        others = mail_sum_wide<SLAB, TK_THREADS>(boxes, stride, nparts - 1, red, p.status, p.wait_limit_ns);
+    if (tid >= SLAB) return;
     float t = 0.f;
-    if (tid < SLAB) {
 #pragma unroll
-        for (int g = 0; g < G; ++g) t += psum[g * SLAB + tid];
-    }
+    for (int g = 0; g < G; ++g) t += psum[g * SLAB + tid];
     // ---- the parts, in part order, in the last part's CTA.  A sum is its own message: the CTA that adds them up
     //      waits until none of its inputs is "empty" any more, and empties them for the next launch.  Blocks start
     //      in index order and only the last ones wait, so what they wait for is running or done ----
     if (nparts > 1) {
-        const size_t stride = (size_t)p.n_slabs * SLAB;
-        float *boxes = p.mail + (size_t)slab * SLAB;
         if (part != nparts - 1) {
             mail_put(boxes + (size_t)part * stride + tid, t);
             DIP_TRACE_MAX(p.tr, 2);
             return;
         }
-        t = mail_sum<SLAB, TK_THREADS>(boxes, stride, nparts - 1, t, red, p.status, p.wait_limit_ns);
-        if (tid >= SLAB) return;
+        if (nparts - 1 <= MAIL_N) others = mail_sum(boxes + tid, stride, nparts - 1, p.status, p.wait_limit_ns);
+        t = others + t;
     }
     // ---- epilogue ----
     const float up = __shfl_down_sync(0xffffffffu, t, 4);      // gate/up: a gate element's up element is four positions on
@@ -620,7 +621,7 @@ block_waits_selftest_kernel(float *mail, unsigned int *readers, int *status, uns
         if (tid < SLAB)
             for (int q = 0; q < N; ++q)
                 if (q != MISSING) mail_put(mail + q * SLAB + tid, 1.f);
-        (void)mail_sum<SLAB, TK_THREADS>(mail, SLAB, N, 1.f, sum, status, limit_ns);
+        (void)mail_sum_wide<SLAB, TK_THREADS>(mail, SLAB, N, sum, status, limit_ns);
         if (tid < SLAB) mail_put(mail + MISSING * SLAB + tid, 1e30f);
         return;
     }
