@@ -7,7 +7,7 @@ import pytest
 
 import dip_inputs as di
 import oracle
-from gpu_util import check_step, upload_layer
+from gpu_util import bits_to_mask, check_step, upload_layer
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -128,4 +128,25 @@ def test_rows_of_one_segment_leave_room_for_both_updates():
     for t in range(2):
         kinds = launch_kinds(ctx, lambda: check_step(dip, ctx, lw, w, di.heavy_tail_vector(t, d_model), 100, 5000, 0.3, *refs, *mine))
         assert kinds == ["gemv_gate_up", "gemv_down"]           # (no launch for the updates)
+    ctx.close()
+
+
+@pytest.mark.parametrize("n_tied", [1, 2, 7, 8, 9, 128, 129, 256, 257])
+def test_stand_alone_selects_with_threshold_bins_of_every_size(n_tied):
+    """Eight columns are the last that one thread each ranks, 128 the last that the block ranks in one go; half of them have
+    equal keys, the others keys of the same 16 bits."""
+    import paper_2412_01380_b200 as dip
+    ctx = dip.Context(0)
+    d, above = 1000, 100
+    rng = np.random.default_rng(n_tied)
+    tied = np.full(n_tied, 1.5, np.float32)
+    tied[::2] = (tied[::2].view(np.uint32) + rng.integers(0, 1000, tied[::2].size).astype(np.uint32)).view(np.float32)
+    x = np.concatenate([rng.uniform(4.0, 9.0, above), tied, rng.uniform(0.01, 1.0, d - above - n_tied)]).astype(np.float32)
+    x = (rng.permutation(x) * rng.choice([-1, 1], d)).astype(np.float32)
+    bits = torch.zeros((d + 31) // 32, dtype=torch.int32, device="cuda")
+    for kept in sorted({1, (n_tied + 1) // 2, n_tied}):
+        idx = torch.zeros(above + kept, dtype=torch.int32, device="cuda")
+        dip.dip_mask_topk(ctx, torch.from_numpy(x).cuda(), above + kept, bits, idx)
+        m, i = oracle.dip_ca_mask(x, above + kept, 1.0, None)
+        assert np.array_equal(bits_to_mask(bits, d), m) and np.array_equal(idx.cpu().numpy(), i), kept
     ctx.close()
