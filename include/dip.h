@@ -82,8 +82,10 @@ typedef struct dip_ctx dip_ctx;   /* opaque; owns scratch workspace on one devic
  *                      down product (INT4 weights, several tokens, select_in_product < 0) ranks
  *                      h from the 16-bit keys that the gate/up product leaves behind: 0 = default
  *                      (4096), negative = every size.  Either way the masks are the same bits.
- *   wait_limit_us      bound of every in-kernel wait (on an asynchronous copy, on another thread
- *                      block's flag), in microseconds (0 = one second); see dip_device_status.
+ *   wait_limit_us      bound of every in-kernel wait on an asynchronous copy, in microseconds (0 =
+ *                      one second); see dip_device_status.  Waits on another thread block of the
+ *                      same launch, which products with row parts make in the normal course, have
+ *                      this bound or one second, whichever is longer.
  *   select_in_product  0 = default: in a single-token step with F32 / BF16 weights each product
  *                      kernel builds the mask of its own input (every thread block finds the
  *                      columns that are certainly kept and streams them at once, one extra block

@@ -135,6 +135,8 @@ dip_status dip_create_ex(dip_ctx **out, int device, const dip_options *opt)
     ctx->coarse_min_d = o.coarse_min_d == 0 ? 4096 : (o.coarse_min_d < 0 ? 0 : o.coarse_min_d);
     ctx->fuse_select = o.select_in_product < 0 ? 0 : 1;
     ctx->wait_limit_ns = o.wait_limit_us ? 1000ull * (unsigned long long)o.wait_limit_us : 1000000000ull;
+    // (blocks wait for one another whenever a product has row parts: a short limit is not for them)
+    ctx->block_wait_ns = ctx->wait_limit_ns > 1000000000ull ? ctx->wait_limit_ns : 1000000000ull;
     // split-row partial sums: up to one part per SM of a whole output row per token
     ctx->partials_floats = PARTIALS_FLOATS;
     ctx->n_tickets = N_TICKETS;

@@ -23,7 +23,8 @@ struct dip_ctx {
     int max_batch;       // most tokens per call the workspace was sized for
     int gemv_seg;        // 0 = choose per launch; else force the GEMV segment width (dip_options)
     int gemv_direct;     // one token, F32/BF16: plain-load kernel instead of the copy ring
-    unsigned long long wait_limit_ns;   // bound of every in-kernel wait
+    unsigned long long wait_limit_ns;   // bound of every in-kernel wait on an asynchronous copy
+    unsigned long long block_wait_ns;   // and on other blocks of the launch
     // split-row partial sums of the two GEMVs (binary32)
     float *partials;
     size_t partials_floats;

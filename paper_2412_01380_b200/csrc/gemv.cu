@@ -606,6 +606,7 @@ dip_status launch_direct_cfg(dip_ctx *ctx, GemvParams &p, int n_kept_max, cudaSt
     const int n_slabs = (int)((p.row_bytes + GD_SEG - 1) / GD_SEG);   // (parts only with one CTA per SM: the mail boxes suffice)
     const int nparts = row_parts(ctx->sm_count / n_slabs, n_kept_max, NW);
     static_assert(SLAB <= DIP_MAIL_FLOATS, "");
+    p.wait_limit_ns = ctx->block_wait_ns;
     p.defer = 0;
     p.part_base = 0;
     DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_direct_kernel<WT, WHICH, NW, U>, dim3(n_slabs, nparts), dim3(NW * 32), 0,

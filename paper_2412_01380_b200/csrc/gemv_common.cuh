@@ -24,7 +24,7 @@ struct GemvParams {
     float *mail;               // row parts on their way between CTAs of a launch; DIP_MAIL_EMPTY outside one
     unsigned int *tickets;
     int *status;               // device status word (0 = fine)
-    unsigned long long wait_limit_ns;   // a wait on a copy's arrival gives up after this long
+    unsigned long long wait_limit_ns;   // a wait on a copy's arrival, or on another block, gives up after this long
     unsigned long long *tr;    // timeline slot or nullptr
     const int32_t *loc;        // two-tier: packed row of column i is W + loc[i] * row_bytes (nullptr: row i)
     int defer;                 // 1: leave the row parts in `partials` for combine_parts_kernel

@@ -216,6 +216,7 @@ dip_status launch_cfg(dip_ctx *ctx, GemvParams &p, int n_kept_max, cudaStream_t 
     const int n_slabs = (int)((p.row_bytes + GB_SEG - 1) / GB_SEG);
     const int nparts = row_parts(ctx->sm_count / n_slabs, n_kept_max, NW);
     static_assert(BT * SLAB <= DIP_MAIL_FLOATS, "");        // (parts only with one CTA per SM: the mail boxes suffice)
+    p.wait_limit_ns = ctx->block_wait_ns;
     p.defer = 0;
     p.part_base = 0;
     const size_t smem = sizeof(GemvBtSmem) + sizeof(float) * (NW + 1) * BT * SLAB;

@@ -684,7 +684,6 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
         g.batch = 1;
         g.mail = ctx->mail;
         g.status = ctx->status;
-        g.wait_limit_ns = ctx->wait_limit_ns;
         g.tr = dip_trace_slot(ctx, which == 0 ? 4 : 5);
         g.key_gamma = 1.0f;
         if (keys) keys->written = 0;
@@ -702,7 +701,7 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
     p.out = out;
     p.mail = ctx->mail;
     p.status = ctx->status;
-    p.wait_limit_ns = ctx->wait_limit_ns;
+    p.wait_limit_ns = ctx->block_wait_ns;
     p.tr = dip_trace_slot(ctx, which == 0 ? 4 : 5);
     p.key_coarse = nullptr;
     p.key_stamp = nullptr;

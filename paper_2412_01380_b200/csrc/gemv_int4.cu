@@ -767,6 +767,7 @@ dip_status dip_launch_gemv_int4(dip_ctx *ctx, GemvParams &p, int which, int n_ke
     const int seg_elems = seg_chunks * 128;
     const int total_parts = mode ? 2 * nparts : nparts;
     if (mode && (size_t)total_parts * n_slabs * seg_elems > ctx->partials_floats) return DIP_ERR_WORKSPACE;
+    p.wait_limit_ns = ctx->block_wait_ns;
     p.defer = mode != 0;
     p.part_base = mode == 2 ? nparts : 0;
     dip_status st;

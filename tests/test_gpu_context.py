@@ -110,7 +110,8 @@ def test_options_size_the_workspace_and_pick_the_kernels(dip):
     assert used_small < used_full
     # forced kernels: copy ring with each segment width, and the 16-bit keys at every size
     for kw in ({"gemv_copy_ring": True}, {"gemv_copy_ring": True, "gemv_segment_bytes": 512},
-               {"gemv_copy_ring": True, "gemv_segment_bytes": 1024}, {"coarse_min_d": -1}):
+               {"gemv_copy_ring": True, "gemv_segment_bytes": 1024}, {"coarse_min_d": -1},
+               {"wait_limit_us": 1}):            # (for copies: the default kernels make none)
         c = dip.Context(0, **kw)
         try:
             w = upload_layer(dip, c, lw)
