@@ -162,7 +162,6 @@ dip_status dip_create_ex(dip_ctx **out, int device, const dip_options *opt)
     if ((st = dev_alloc(ctx, &ctx->coarse, vec)) != DIP_OK) return fail(st);
     if ((st = dev_alloc(ctx, &ctx->xt, (size_t)ctx->max_d * 32)) != DIP_OK) return fail(st);
     if ((st = dev_alloc(ctx, &ctx->status, (size_t)1)) != DIP_OK) return fail(st);
-    if (cudaMemset(ctx->status, 0, sizeof(int)) != cudaSuccess) return fail(DIP_ERR_CUDA);
     if ((st = dev_alloc(ctx, &ctx->trace, (size_t)DIP_TRACE_SLOTS * DIP_TRACE_WORDS)) != DIP_OK) return fail(st);
     for (int i = 0; i < 2; ++i) {
         if (cudaStreamCreateWithFlags(&ctx->tier_fetch[i], cudaStreamNonBlocking) != cudaSuccess) return fail(DIP_ERR_CUDA);
@@ -176,10 +175,15 @@ dip_status dip_create_ex(dip_ctx **out, int device, const dip_options *opt)
         if (cudaEventCreateWithFlags(&ctx->ev_fork[i], cudaEventDisableTiming) != cudaSuccess) return fail(DIP_ERR_CUDA);
         if (cudaEventCreateWithFlags(&ctx->ev_join[i], cudaEventDisableTiming) != cudaSuccess) return fail(DIP_ERR_CUDA);
     }
-    if (cudaMemset(ctx->mail, 0xff, (size_t)ctx->sm_count * DIP_MAIL_FLOATS * sizeof(float)) != cudaSuccess) return fail(DIP_ERR_CUDA);
-    if (cudaMemset(ctx->readers, 0, sizeof(unsigned int)) != cudaSuccess) return fail(DIP_ERR_CUDA);
-    if (cudaMemset(ctx->tickets, 0, N_TICKETS * sizeof(unsigned int)) != cudaSuccess) return fail(DIP_ERR_CUDA);
-    if (cudaMemset(ctx->counts, 0, 8 * sizeof(int32_t)) != cudaSuccess) return fail(DIP_ERR_CUDA);
+    // through by the time the context is handed out, whatever stream its first call is on (a memset on the legacy stream is
+    // ordered with blocking streams only, and a product must not find its boxes unset)
+    cudaStream_t set = ctx->side[0];
+    if (cudaMemsetAsync(ctx->status, 0, sizeof(int), set) != cudaSuccess) return fail(DIP_ERR_CUDA);
+    if (cudaMemsetAsync(ctx->mail, 0xff, (size_t)ctx->sm_count * DIP_MAIL_FLOATS * sizeof(float), set) != cudaSuccess) return fail(DIP_ERR_CUDA);
+    if (cudaMemsetAsync(ctx->readers, 0, sizeof(unsigned int), set) != cudaSuccess) return fail(DIP_ERR_CUDA);
+    if (cudaMemsetAsync(ctx->tickets, 0, N_TICKETS * sizeof(unsigned int), set) != cudaSuccess) return fail(DIP_ERR_CUDA);
+    if (cudaMemsetAsync(ctx->counts, 0, 8 * sizeof(int32_t), set) != cudaSuccess) return fail(DIP_ERR_CUDA);
+    if (cudaStreamSynchronize(set) != cudaSuccess) return fail(DIP_ERR_CUDA);
     if ((st = dip_init_mask_kernels(ctx)) != DIP_OK) return fail(st);
     if (cudaSetDevice(prev_device) != cudaSuccess) return fail(DIP_ERR_CUDA);
     *out = ctx;

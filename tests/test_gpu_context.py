@@ -171,6 +171,29 @@ def test_misaligned_pointers_are_rejected_before_any_launch(dip):
         c.close()
 
 
+def test_a_new_context_serves_any_stream_at_once(dip):
+    """The first call on a context, on a stream that the default one does not order, finds the workspace set up."""
+    lw = di.layer_weights(di.WORKLOADS["phi3_mini"].scaled(seed=6, d_model=256, d_ff=1536, n_layers=1), 0)
+    first = dip.Context(0)
+    w = upload_layer(dip, first, lw)
+    x = torch.from_numpy(di.heavy_tail_vector(3, 256)).cuda()
+    want = torch.empty(256, device="cuda")
+    dip.dip_mlp_step(first, w, x, 128, 1056, 1.0, None, None, want)
+    torch.cuda.synchronize()
+    first.close()
+    for _ in range(5):
+        y = torch.empty(256, device="cuda")
+        torch.cuda.synchronize()
+        c = dip.Context(0)
+        s = torch.cuda.Stream()                                # (torch's streams do not wait for the default stream)
+        with torch.cuda.stream(s):
+            dip.dip_mlp_step(c, w, x, 128, 1056, 1.0, None, None, y)
+            assert c.device_status() == dip.DEVICE_OK
+        assert torch.equal(y, want)
+        torch.cuda.synchronize()
+        c.close()
+
+
 @pytest.mark.parametrize("wtype", [di.W_BF16, di.W_INT4_G128])
 def test_a_stack_with_a_bad_block_launches_nothing(dip, wtype):
     """A cache state that only the last block refuses: an error code, no launch, states untouched; the next good call is right."""
