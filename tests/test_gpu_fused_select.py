@@ -1,13 +1,14 @@
 """Single-token steps whose products select for themselves, at the sizes where the kernel's branches meet: one and several
-chunks of columns per thread (8192 / 8224 columns), the variants of the cache update that rides along (8192, 20480), rows
-of one segment up to one per SM (where the update gets a launch of its own), row parts of one row, keep counts 1 and d,
-and threshold bins of 256 and 257 columns (the last that is ranked in place, the first that is not)."""
+chunks of columns per thread (8192 / 8224 columns), the variants of the cache update that rides along (8192, 20480), down
+products that leave SMs for updates, fill the SMs to the last one (the updates get launches of their own) or take a second
+wave, row parts of one row, keep counts 1 and d, and threshold bins of 256 and 257 columns (the last that is ranked in
+place, the first that is not).  What a call launches is read from the library's own timeline."""
 import numpy as np
 import pytest
 
 import dip_inputs as di
 import oracle
-from gpu_util import bits_to_mask, check_step, upload_layer
+from gpu_util import REL_TOL, bits_to_mask, check_step, rel_err, upload_layer
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -26,6 +27,16 @@ SHAPES = [
 
 def _layer(d_model, d_ff, wtype, seed):
     return di.layer_weights(di.WORKLOADS["phi3_mini"].scaled(seed=seed, d_model=d_model, d_ff=d_ff, wtype=wtype, n_layers=1), 0)
+
+
+def launch_kinds(ctx, call):
+    """The kinds of the library's launches in a call, as its own timeline records them."""
+    ctx.trace_begin()
+    call()
+    torch.cuda.synchronize()
+    kinds = [r["kind"] for r in ctx.trace_read()]
+    ctx.trace_end()
+    return kinds
 
 
 @pytest.mark.parametrize("policy", [None, "lru", "lfu"])
@@ -106,14 +117,91 @@ def test_stacks_leave_their_cache_updates_to_later_launches(n_layers, caches, wt
     ctx.close()
 
 
-def launch_kinds(ctx, call):
-    """The kinds of the library's launches in a call, as its own timeline records them."""
-    ctx.trace_begin()
-    call()
+# launches for cache updates alone in a stack of 1, 3, 4, 9 blocks: at most seven updates wait, for the last down product
+# (F32 / BF16 with a cache) or a launch beside it; a 4-bit call ends with one for the last down input
+UPDATE_LAUNCHES = {("both", False): {1: 0, 3: 0, 4: 0, 9: 2}, ("x", False): {1: 1, 3: 1, 4: 1, 9: 2}, ("h", False): {1: 0, 3: 0, 4: 0, 9: 1},
+                   ("both", True): {1: 2, 3: 2, 4: 2, 9: 4}, ("x", True): {1: 1, 3: 1, 4: 1, 9: 2}, ("h", True): {1: 1, 3: 2, 4: 2, 9: 3}}
+
+
+@pytest.mark.parametrize("caches", ["both", "x", "h"])
+@pytest.mark.parametrize("n_layers", [1, 3, 4, 9])
+@pytest.mark.parametrize("wtype,d_model,policy", [(di.W_BF16, 256, "lru"), (di.W_BF16, 5120, "lfu"), (di.W_INT4_G128, 256, "lru")])
+def test_updates_of_a_stack_by_launch(n_layers, caches, wtype, d_model, policy):
+    """A stack's cache states equal those of its blocks stepped one by one on a context whose selects and updates are launches
+    of their own (blocks whose updates ride with the last down product, fill a launch beside the products, or have no
+    product with a cache to ride with)."""
+    import paper_2412_01380_b200 as dip
+    ctx, plain = dip.Context(0), dip.Context(0, select_in_product=-1)
+    d_ff = 640
+    k_x, k_h = d_model // 4, 200
+    ws = [upload_layer(dip, ctx, _layer(d_model, d_ff, wtype, 100 + l)) for l in range(n_layers)]
+
+    def states():
+        return [[dip.CacheState(d, d // 2, "cuda", policy) for _ in ws] if caches in (c, "both") else None
+                for d, c in ((d_model, "x"), (d_ff, "h"))]
+    gu, d = states()
+    gu1, d1 = states()
+    stack = dip.Stack(ws, gu, d)
+    out = torch.empty(d_model, device="cuda")
+    y = torch.empty(d_model, device="cuda")
+    probe = dip.StackProbe(n_layers, 1, d_model, d_ff, "cuda")
+    for t in range(5):
+        x = torch.from_numpy(di.heavy_tail_vector(300 + t, d_model)).cuda()
+        kinds = launch_kinds(ctx, lambda: dip.dip_stack_step_probed(ctx, stack, x, k_x, k_h, 0.2, out, probe))
+        assert kinds.count("cache_update") == UPDATE_LAUNCHES[caches, wtype == di.W_INT4_G128][n_layers], kinds
+        for l, w in enumerate(ws):
+            # (each block on the stack's own input, each mask on its own h: sums in another order swap no columns)
+            for v, k, c, want in ((probe.x[l, 0], k_x, gu1, probe.mask_x[l, 0]), (probe.h[l, 0], k_h, d1, probe.mask_h[l, 0])):
+                mask = torch.zeros(v.numel() // 32, dtype=torch.int32, device="cuda")
+                if c:
+                    dip.dip_ca_mask(plain, v.clone(), k, 0.2, c[l], mask, None)
+                else:
+                    dip.dip_mask_topk(plain, v.clone(), k, mask, None)
+                assert torch.equal(mask, want), (t, l)
+        torch.cuda.synchronize()
+        for a, b in ((gu, gu1), (d, d1)):
+            for p, q in zip(a or [], b or []):
+                assert torch.equal(p.stamp, q.stamp) and torch.equal(p.meta, q.meta), t
+                assert policy == "lru" or torch.equal(p.count, q.count), t
+    # and the call without the intermediates does the same
+    again = states()
+    twin = dip.Stack(ws, *again)
+    for t in range(5):
+        dip.dip_stack_step(ctx, twin, torch.from_numpy(di.heavy_tail_vector(300 + t, d_model)).cuda(), k_x, k_h, 0.2, y)
     torch.cuda.synchronize()
-    kinds = [r["kind"] for r in ctx.trace_read()]
-    ctx.trace_end()
-    return kinds
+    assert torch.equal(y, out)
+    for a, b in zip((gu, d), again):
+        for p, q in zip(a or [], b or []):
+            assert torch.equal(p.stamp, q.stamp) and torch.equal(p.meta, q.meta)
+    assert ctx.device_status() == 0
+    ctx.close()
+    plain.close()
+
+
+@pytest.mark.parametrize("policy", ["lru", "lfu"])
+@pytest.mark.parametrize("wtype,d_model,d_ff,rho,launches", [
+    # updates that ride: columns of the three variants, and a launch of two waves (149 segments: its last block waits for
+    # blocks that start when others end)
+    (di.W_BF16, 544, 8192, 0.25, 0), (di.W_BF16, 544, 8224, 0.25, 0), (di.W_BF16, 1056, 20480, 0.2, 0), (di.W_BF16, 544, 20512, 0.2, 0),
+    (di.W_F32, 19072, 128, 0.5, 0),
+    # products on all 148 SMs: 4, 2 and 1 row parts
+    (di.W_BF16, 9472, 640, 0.5, 2), (di.W_BF16, 18944, 256, 0.5, 2), (di.W_F32, 18944, 128, 0.5, 2),
+])
+def test_updates_ride_where_a_down_product_leaves_sms(wtype, d_model, d_ff, rho, launches, policy):
+    import paper_2412_01380_b200 as dip
+    ctx = dip.Context(0)
+    if ctx.sm_count != 148:
+        pytest.skip("shapes chosen for 148 SMs")
+    lw = _layer(d_model, d_ff, wtype, d_model + d_ff)
+    w = upload_layer(dip, ctx, lw)
+    refs = [oracle.Cache(d, int(0.4 * d), policy) for d in (d_model, d_ff)]
+    mine = [dip.CacheState(d, int(0.4 * d), "cuda", policy) for d in (d_model, d_ff)]
+    for t in range(3):
+        kinds = launch_kinds(ctx, lambda: check_step(dip, ctx, lw, w, di.heavy_tail_vector(t, d_model), int(rho * d_model), int(rho * d_ff),
+                                                     0.2, *refs, *mine))
+        assert sorted(kinds) == ["cache_update"] * launches + ["gemv_down", "gemv_gate_up"]
+    assert ctx.device_status() == 0
+    ctx.close()
 
 
 def test_rows_of_one_segment_leave_room_for_both_updates():
@@ -150,3 +238,39 @@ def test_stand_alone_selects_with_threshold_bins_of_every_size(n_tied):
         m, i = oracle.dip_ca_mask(x, above + kept, 1.0, None)
         assert np.array_equal(bits_to_mask(bits, d), m) and np.array_equal(idx.cpu().numpy(), i), kept
     ctx.close()
+
+
+@pytest.mark.parametrize("wtype", [di.W_BF16, di.W_F32])
+@pytest.mark.parametrize("where", ["weights", "x"])
+def test_values_that_are_not_finite(wtype, where):
+    """NaN of any bit pattern (all ones is the mark of an empty box) and infinities give what the kernel gives that adds its
+    row parts up in memory, and no wait runs out."""
+    import paper_2412_01380_b200 as dip
+    d_model, d_ff = 256, 1536
+    lw = _layer(d_model, d_ff, wtype, 77)
+    x = di.heavy_tail_vector(8, d_model)
+    if where == "weights":
+        for m in (lw.gate, lw.up, lw.down):
+            m = m.reshape(-1).view(np.uint32 if wtype == di.W_F32 else np.uint16)
+            bits = (0xffffffff, 0x7fc00000, 0x7f800000, 0xff800000) if wtype == di.W_F32 else (0xffff, 0x7fc0, 0x7f80, 0xff80)
+            for i, v in enumerate(bits):
+                m[m.size // 5 * (i + 1)] = v
+    else:
+        x.view(np.uint32)[[3, 50, 99]] = (0xffffffff, 0x7f800000, 0x7fc00001)
+    got = []
+    for kw in ({}, {"gemv_copy_ring": True}):
+        ctx = dip.Context(0, **kw)
+        w = upload_layer(dip, ctx, lw)
+        y, h = torch.empty(d_model, device="cuda"), torch.empty(d_ff, device="cuda")
+        bits = torch.zeros(d_ff // 32, dtype=torch.int32, device="cuda")
+        dip.dip_mlp_step(ctx, w, torch.from_numpy(x).cuda(), 128, 1056, 1.0, None, None, y, h=h, mask_h=bits)
+        torch.cuda.synchronize()
+        assert ctx.device_status() == 0
+        got.append((h.cpu().numpy(), bits_to_mask(bits, d_ff), y.cpu().numpy()))
+        ctx.close()
+    (h0, m0, y0), (h1, m1, y1) = got
+    assert not np.isfinite(h0).all() and not np.isfinite(y0).all()
+    assert np.array_equal(m0, m1)
+    for a, b in ((h0, h1), (y0, y1)):
+        ok = np.isfinite(a)
+        assert np.array_equal(a[~ok], b[~ok], equal_nan=True) and (not ok.any() or rel_err(a[ok], b[ok]) <= REL_TOL)
