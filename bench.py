@@ -172,7 +172,20 @@ def GATE_UP_KERNEL(w, batch, select_in_product=True):
         return "gemv_int4_kernel"
     if batch == 1:
         return "gemv_fused_kernel" if select_in_product else "gemv_direct_kernel"
-    return "gemv_kernel" if batch == 2 else "gemv_tc_kernel"
+    if batch == 2:
+        return "gemv_direct_bt_kernel"
+    return "gemv_tc_kernel" if w.wtype == di.W_BF16 else "gemv_kernel"
+
+
+def traced(ctx, torch, call):
+    """The library's launches in a call, from its device-side timeline.  (The residual + rmsnorm that closes a stack, the value
+    gathers and part sums of several tokens, and index lists have no slot there.)"""
+    ctx.trace_begin()
+    call()
+    torch.cuda.synchronize()
+    recs = ctx.trace_read()
+    ctx.trace_end()
+    return recs
 
 
 def max_over_ranks(ms, dist, torch, device):
@@ -349,8 +362,20 @@ def run_config(dip, ctx, torch, w, layers, xs_host, keep_ratio, budget, steps, w
                       "h2d_bytes_per_step": 4 * d_model * batch, "d2h_bytes_per_step": 4 * d_model * batch,
                       "wall_ms": (time.perf_counter() - t0) * 1e3}
 
+    # ---- the launches of one token (counted, + the residual + rmsnorm) ----
+    st3 = fresh_stack()
+    for t in range(3):
+        recs = traced(ctx, torch, lambda: dip.dip_stack_step(ctx, st3, xs_dev[t % n_tok], k_x, k_h, gamma, x_out))
+    res["launches"] = len(recs) + 1
+    n_select = sum(r["kind"] in ("select", "select_ca") for r in recs)
+    res["select_in_product"] = batch == 1 and n_select < L
+
     # ---- per-kernel durations (separate instrumented pass, one event pair per launch) ----
-    if kernel_pass and batch == 1:
+    if kernel_pass and batch == 1 and w.wtype == di.W_INT4_G128:
+        # (the products that select for themselves are no calls of their own here: inputs ready -> last block's end)
+        res["kernels"] = {k + "_timeline_us": float(np.mean([r["end"] - r["ready"] for r in recs if r["kind"] == "gemv_" + k]))
+                          for k in ("gate_up", "down")}
+    elif kernel_pass and batch == 1:
         st2 = fresh_stack()
         mask_x = torch.zeros((d_model + 31) // 32, dtype=torch.int32, device="cuda")
         idx_x = torch.zeros(k_x, dtype=torch.int32, device="cuda")
@@ -359,15 +384,8 @@ def run_config(dip, ctx, torch, w, layers, xs_host, keep_ratio, budget, steps, w
         h = torch.empty(d_ff, device="cuda")
         y = torch.empty(d_model, device="cuda")
         n_pass_tok = 6
-        # A step of this configuration runs each mask together with its product (one launch each) when the
-        # library supports that for the weights and shape; otherwise a select kernel precedes each product.
-        try:
-            dip.dip_select_gemv_gate_up(ctx, layers[0], xs_dev[0].clone(), k_x, gamma,
-                                        st2.cache_gu[0] if ca else None, st2.cache_d[0] if ca else None, mask_x, h)
-            fused = True
-        except dip.DipError:
-            fused = False
-        res["select_in_product"] = fused
+        # (a step of this configuration runs each mask together with its product, one launch each, or a select kernel first)
+        fused = res["select_in_product"]
         cg = (lambda l: st2.cache_gu[l]) if ca else (lambda l: None)
         cd = (lambda l: st2.cache_d[l]) if ca else (lambda l: None)
         if fused:
@@ -704,7 +722,7 @@ def main_neuron_pruned(args, dip, ctx, torch, w, keep_ratio, rank, world, local)
         "clocks": clocks,
         "e2e": {"value": L * n_e2e / (ms_e * 1e-3), "unit": UNIT, "h2d_bytes_per_step": 4 * d_model,
                 "d2h_bytes_per_step": 4 * d_model},
-        # per layer: 2 row products, select, mask->list, memset, down GEMV, rmsnorm
+        # per layer: 2 row products, select, mask->list, down GEMV, rmsnorm
         "gpu_launches": 6 * L * args.steps,
         "roofline": {"bound": "hbm", "kernel": "rowdot_kernel (dense ranking product)", "achieved": achieved,
                      "peak": peak, "peak_kind": "of " + peak_kind, "unit": "GB/s", "frac": achieved / peak,
@@ -748,8 +766,9 @@ def main_two_tier(args, dip, ctx, torch, w, keep_ratio, budget, rank, world, loc
                    "parallelism": "replicas only"},
         "mlp_step_us": r["ms_per_step"] * 1e3 / L, "hit_rate": r["hit_rate"], "clocks": r["clocks"],
         "e2e": r["e2e"],
-        # per layer: 2 selects, 2 cache updates, 2 slot assignments, 2 fetches, 4 GEMVs, 2 combines, 1 rmsnorm
-        "gpu_launches": 15 * L * args.steps,
+        # per layer: 2 selects, 2 splits, 2 miss lists, 2 cache updates, 2 slot assignments, 2 fetches, 2 installs, 4 GEMVs,
+        # 2 combines, 1 rmsnorm
+        "gpu_launches": 21 * L * args.steps,
         # the fetch kernel: bytes it brought in / its own device time (timeline of 8 replays); the
         # same bytes over the whole step's time are in fetch_gbs_over_step
         "roofline": {"bound": "host_link", "kernel": "tier_fetch_kernel", "achieved": r["fetch_kernel_gbs"],
@@ -764,26 +783,6 @@ def main_two_tier(args, dip, ctx, torch, w, keep_ratio, budget, rank, world, loc
         line["cpu_baseline"] = {k: v for k, v in oracle_rate(w, keep_ratio, budget, 1, 60).items()
                                 if k in ("value", "unit", "cores", "kind", "sample")}
     print(json.dumps(line))
-
-
-def launches_per_token(n_layers, batch, caches, int4):
-    """Kernels of one dip_stack_step.  One token: two products per layer that build their own masks; the cache updates
-    ride with the last down product, seven at a time in a launch of their own before that (4-bit weights: the last layer's
-    down half is select, update and product, and a launch for the updates that are due).  Several tokens: two selects
-    and two products (their value gathers and part sums not counted).  One residual + rmsnorm closes the stack."""
-    if batch > 1:
-        return 4 * n_layers + 1
-    n, due = 2 * n_layers + 1, 0
-    for layer in range(n_layers if caches else 0):
-        last = layer == n_layers - 1 or layer % 128 == 127        # (the mask slots are used again)
-        due += 1
-        if (last and int4) or (not last and due + 2 > 7):
-            n, due = n + 1, 0
-        if last:
-            n, due = n + (2 if int4 else 0), 0
-        else:
-            due += 1
-    return n
 
 
 def print_timeline(dip, ctx, torch, w, layers, xs_host, keep_ratio, budget):
@@ -991,14 +990,13 @@ def main():
     peak, peak_kind = measured_peak()
     gu_bytes = head["bytes"]["gate_up"]
     if "kernels" in head:
-        gu_us = head["kernels"]["gate_up_train_us"]
+        gu_us = head["kernels"].get("gate_up_train_us") or head["kernels"]["gate_up_timeline_us"]
         achieved = gu_bytes / (gu_us * 1e-6) / 1e9
     else:
         # batched decode: no per-kernel pass; the whole step on the bytes of the union of the masks
         gu_us = None
         achieved = head.get("union_gbs", head["step_gbs"])
     fused = bool(head.get("select_in_product"))
-    launches_per_step = launches_per_token(L, args.batch, budget is not None, w.wtype == di.W_INT4_G128)
     kernel_name = GATE_UP_KERNEL(w, args.batch, fused) + (" (select of x + gate/up bundle)" if fused else " (gate/up bundle)")
     line = {
         "metric": METRIC, "value": whole_job_rate(L * args.steps, world, head["ms_total"]), "unit": UNIT, "n_gpus": world,
@@ -1021,7 +1019,7 @@ def main():
         "paper_simulator_view": head.get("paper_simulator_view"),
         "clocks": head["clocks"],
         "e2e": {k: head["e2e"][k] for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")},
-        "gpu_launches": launches_per_step * args.steps,
+        "gpu_launches": head["launches"] * args.steps,
         "roofline": {"bound": "hbm", "kernel": kernel_name, "achieved": achieved, "peak": peak,
                      "peak_kind": "of " + peak_kind, "unit": "GB/s", "frac": achieved / peak,
                      "frac_of_nominal_8tbs": achieved / NOMINAL_HBM_GBS, "bytes_per_launch": gu_bytes,
