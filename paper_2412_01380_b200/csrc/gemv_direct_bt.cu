@@ -24,7 +24,8 @@ struct __align__(16) GemvBtSmem {
 };
 // after GemvBtSmem (dynamic): float red[NW][BT][SLAB], float sum[BT][SLAB]
 
-template <int WT, int WHICH, int BT, int NW, int U>
+// WIDE: more parts than one trip collects (a variant of its own: the others do without that code).
+template <int WT, int WHICH, int BT, int NW, int U, bool WIDE>
 __global__ void __launch_bounds__(NW * 32, 1)
 gemv_direct_bt_kernel(const GemvParams p)
 {
@@ -165,30 +166,35 @@ gemv_direct_bt_kernel(const GemvParams p)
         for (int e = 0; e < E; ++e) s_red[(warp * BT + b) * SLAB + lane * E + e] = acc[b][e];
     __syncthreads();
     // ---- 5. the parts, in part order, in the last part's CTA: a sum is its own message (see gemv_fused.cu) ----
-    float t = 0.f;
     static_assert(BT * SLAB <= THREADS, "one sum per thread");
-    if (tid < BT * SLAB) {
-        const int b = tid / SLAB, el = tid % SLAB;
+    const size_t stride = (size_t)gridDim.x * (BT * SLAB);
+    float *boxes = p.mail + (size_t)slab * (BT * SLAB);
+    for (int i = tid; i < BT * SLAB; i += THREADS) {
+        const int b = i / SLAB, el = i % SLAB;
+        float t = 0.f;
 #pragma unroll
         for (int w = 0; w < NW; ++w) t += s_red[(w * BT + b) * SLAB + el];
-    }
-    if (nparts > 1) {
-        const size_t stride = (size_t)gridDim.x * (BT * SLAB);
-        float *boxes = p.mail + (size_t)slab * (BT * SLAB);
         if (part != nparts - 1) {
-            if (tid < BT * SLAB) mail_put(boxes + (size_t)part * stride + tid, t);
-            DIP_TRACE_MAX(p.tr, 2);
-            return;
+            mail_put(boxes + (size_t)part * stride + i, t);
+            continue;
         }
-        if (nparts - 1 > MAIL_N) {
-            __syncthreads();           // everyone has read s_red
-            t = mail_sum_wide<BT * SLAB, THREADS>(boxes, stride, nparts - 1, s_red, p.status, p.wait_limit_ns) + t;
-        } else if (tid < BT * SLAB) {
-            t = mail_sum(boxes + tid, stride, nparts - 1, p.status, p.wait_limit_ns) + t;
-        }
+        // (a loop although there is no more than one trip: without it the compiler schedules the rows' stream differently,
+        // 63.1 instead of 61.8 us per step of 5120 / 17920)
+        float others = 0.f;
+        for (int q0 = 0; !WIDE && q0 < nparts - 1; q0 += MAIL_N)
+            others += mail_sum(boxes + i + (size_t)q0 * stride, stride, nparts - 1 - q0, p.status, p.wait_limit_ns);
+        s_sum[i] = nparts > 1 ? others + t : t;
     }
-    if (tid < BT * SLAB) s_sum[tid] = t;
+    if (part != nparts - 1) {
+        DIP_TRACE_MAX(p.tr, 2);
+        return;
+    }
     __syncthreads();
+    if constexpr (WIDE) {
+        const float others = mail_sum_wide<BT * SLAB, THREADS>(boxes, stride, nparts - 1, s_red, p.status, p.wait_limit_ns);
+        if (tid < BT * SLAB) s_sum[tid] = others + s_sum[tid];
+        __syncthreads();
+    }
     // ---- 6. epilogue ----
     for (int i = tid; i < BT * OUT_PER_SLAB; i += THREADS) {
         const int b = i / OUT_PER_SLAB, o = i % OUT_PER_SLAB, j = slab * OUT_PER_SLAB + o;
@@ -209,20 +215,18 @@ gemv_direct_bt_kernel(const GemvParams p)
     DIP_TRACE_MAX(p.tr, 2);
 }
 
-template <int WT, int WHICH, int BT, int NW, int U>
-dip_status launch_cfg(dip_ctx *ctx, GemvParams &p, int n_kept_max, cudaStream_t stream)
+template <int WT, int WHICH, int BT, int NW, int U, bool WIDE>
+dip_status launch_cfg(dip_ctx *ctx, GemvParams &p, int n_slabs, int nparts, cudaStream_t stream)
 {
     constexpr int SLAB = 32 * WTraits<WT>::E;
-    const int n_slabs = (int)((p.row_bytes + GB_SEG - 1) / GB_SEG);
-    const int nparts = row_parts(ctx->sm_count / n_slabs, n_kept_max, NW);
     static_assert(BT * SLAB <= DIP_MAIL_FLOATS, "");        // (parts only with one CTA per SM: the mail boxes suffice)
     p.wait_limit_ns = ctx->block_wait_ns;
     p.defer = 0;
     p.part_base = 0;
     const size_t smem = sizeof(GemvBtSmem) + sizeof(float) * (NW + 1) * BT * SLAB;
     static dip_per_device_once once;
-    DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once, ctx->device, gemv_direct_bt_kernel<WT, WHICH, BT, NW, U>, smem));
-    DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_direct_bt_kernel<WT, WHICH, BT, NW, U>, dim3(n_slabs, nparts), dim3(NW * 32), smem,
+    DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once, ctx->device, gemv_direct_bt_kernel<WT, WHICH, BT, NW, U, WIDE>, smem));
+    DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_direct_bt_kernel<WT, WHICH, BT, NW, U, WIDE>, dim3(n_slabs, nparts), dim3(NW * 32), smem,
                                      stream, p));
     return DIP_OK;
 }
@@ -230,7 +234,11 @@ dip_status launch_cfg(dip_ctx *ctx, GemvParams &p, int n_kept_max, cudaStream_t 
 template <int WT, int WHICH>
 dip_status launch_wt(dip_ctx *ctx, GemvParams &p, int n_kept_max, cudaStream_t stream)
 {
-    return launch_cfg<WT, WHICH, 2, 32, 4>(ctx, p, n_kept_max, stream);
+    constexpr int NW = 32;
+    const int n_slabs = (int)((p.row_bytes + GB_SEG - 1) / GB_SEG);
+    const int nparts = row_parts(ctx->sm_count / n_slabs, n_kept_max, NW);
+    return nparts - 1 > MAIL_N ? launch_cfg<WT, WHICH, 2, NW, 4, true>(ctx, p, n_slabs, nparts, stream)
+                               : launch_cfg<WT, WHICH, 2, NW, 4, false>(ctx, p, n_slabs, nparts, stream);
 }
 
 }  // namespace
