@@ -33,6 +33,13 @@ __device__ __forceinline__ void cache_update_clear(TkShared &s, unsigned int *sm
     small[2 * tid] = small[2 * tid + 1] = 0;
 }
 
+// The counters as they were before the uses of this mask (out of line: only after a wait that ran out).
+__device__ __noinline__ void take_uses_back(const uint32_t *mask_bits, int d, int32_t *count)
+{
+    for (int c = threadIdx.x; c < d; c += TK_THREADS)
+        if ((mask_bits[c >> 5] >> (c & 31)) & 1u) --count[c];
+}
+
 template <int NB, bool LFU, typename Poll, typename MayWrite>
 __device__ __forceinline__ void block_cache_update(const uint32_t *mask_bits, int d, const int32_t *stamp_now, int32_t *stamp,
                                                    int32_t *count, int32_t *meta, int capacity, TkShared &s, unsigned int *small,
@@ -221,9 +228,7 @@ __device__ __forceinline__ void block_cache_update(const uint32_t *mask_bits, in
 
     // ---- the new stamps ----
     if (!may_write()) {
-        if (LFU)                                        // the uses are taken back (from the mask: nothing is kept for this)
-            for (int c = tid; c < d; c += TK_THREADS)
-                if ((mask_bits[c >> 5] >> (c & 31)) & 1u) --count[c];
+        if (LFU) take_uses_back(mask_bits, d, count);
         return;
     }
 #pragma unroll
