@@ -78,20 +78,24 @@ typedef struct dip_ctx dip_ctx;   /* opaque; owns scratch workspace on one devic
  *                      row that one thread block of the copy-ring product kernel handles.
  *   gemv_copy_ring     non-zero: single-token F32 / BF16 products also go through the
  *                      copy-ring kernel (by default they use the plain-load kernel).
- *   coarse_min_d       smallest d_ff for which a step that runs a select kernel in front of the
- *                      down product (INT4 weights, several tokens, select_in_product < 0) ranks
- *                      h from the 16-bit keys that the gate/up product leaves behind: 0 = default
- *                      (4096), negative = every size.  Either way the masks are the same bits.
+ *   coarse_min_d       smallest d_ff for which a step that runs select kernels in front of its products
+ *                      (several tokens, select_in_product < 0, gemv_copy_ring, inputs too wide for
+ *                      a thread block's shared memory) ranks h from the 16-bit keys that the gate/up
+ *                      product leaves behind: 0 = default (4096), negative = every size.  Products
+ *                      that select for themselves rank h from those keys at every size.  Either
+ *                      way the masks are the same bits.
  *   wait_limit_us      bound of every in-kernel wait on an asynchronous copy, in microseconds (0 =
  *                      one second); see dip_device_status.  Waits on another thread block of the
  *                      same launch, which products with row parts make in the normal course, have
  *                      this bound or one second, whichever is longer.
- *   select_in_product  0 = default: in a single-token step with F32 / BF16 weights each product
- *                      kernel builds the mask of its own input (every thread block finds the
- *                      columns that are certainly kept and streams them at once, one extra block
- *                      completes the mask meanwhile); negative: a select kernel runs in front of
- *                      each product instead.  The masks are the same bits either way; the
- *                      products add the same rows in a different order. */
+ *   select_in_product  0 = default: in a single-token step each product kernel builds the mask of its
+ *                      own input (every thread block selects for itself and goes straight on to its
+ *                      rows; the last block also writes the mask; in a down launch that carries
+ *                      cache updates that is a block without rows).  With INT4 weights the down
+ *                      half of a call's last block keeps its select kernel if it has a cache.
+ *                      Negative: a select kernel runs in front of each product instead.  The masks
+ *                      are the same bits either way; the products add the same rows in a different
+ *                      order. */
 typedef struct {
     int32_t max_d;
     int32_t max_batch;

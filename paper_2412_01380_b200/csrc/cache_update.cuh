@@ -11,7 +11,8 @@ namespace {
 // other SMs, and a chain of exchanges between CTAs would cost more than the few thousand columns an SM
 // has to look at.
 // A warp owns NB consecutive blocks of 128 columns, a lane four consecutive columns of each (one
-// 16-byte load and one 16-byte store), and everything in between stays in registers.  The eviction
+// 16-byte load and one 16-byte store), and what lies in between never goes through shared memory (64 registers
+// do not hold all of it in the wider variants: 416 bytes of spill stores in cache_update_kernel, which stay in L1).  The eviction
 // key of a column that may be evicted (resident and outside the mask) is the age of its last use
 // (LFU: t + 1 - uses), of any other column 0.
 // Bound by the SM's issue rate and its trips through shared memory.  Alone, LRU, after 38 updates:

@@ -17,7 +17,8 @@
 // One token with F32 / BF16 weights takes gemv_direct_kernel further down instead: plain loads, a
 // 512-byte segment per CTA, and for gate/up no row parts at all.  INT4 weights (gemv_int4.cu) and
 // BF16 batches of three or more tokens (gemv_tc.cu) run on the tensor cores; this kernel serves
-// batches of F32 weights, two BF16 tokens, and the two-tier step.
+// batches of three and more tokens with F32 weights, and the two-tier step; two tokens run on
+// gemv_direct_bt.cu.
 //
 // which = 0 (gate/up bundle): the epilogue applies silu(gate) * up (Eq. 2).  which = 1: down.
 // Every wait on an mbarrier is bounded; on expiry the kernel records a status word and leaves.
@@ -418,7 +419,7 @@ gemv_kernel(const GemvParams p)
 // the rows round robin, each lane keeps the E sums of its piece, U loads per lane are in flight
 // (NW x U x 512 bytes per SM), the warps' sums meet in shared memory and the epilogue writes
 // the outputs.  Only when the rows have few segments (down: 20) are the rows split into parts,
-// combined as above by the last CTA of a segment.  At any moment all CTAs read neighbouring
+// whose sums meet in the last part's CTA.  At any moment all CTAs read neighbouring
 // segments of the same few rows, so DRAM sees whole rows.
 // ---------------------------------------------------------------------------------------------
 constexpr int GD_SEG = 512;

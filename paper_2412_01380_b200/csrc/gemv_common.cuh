@@ -123,8 +123,8 @@ __device__ __forceinline__ void mail_take(float *box, size_t stride, int n, floa
 // over the T / SLAB groups of the last part's CTA (all T threads call it): the sum of the n boxes boxes[0], boxes[stride], ...
 // of element tid % SLAB, the groups' sums in order of the groups.  (Narrow rows have up to one part per SM, and a trip to L2
 // for every eight added up: the down product of 704 rows of 256 BF16 outputs took 12.3 us, with both this and row_parts
-// 5.8.)  Out of line: in line it cost the launches that carry cache updates, which never come here at these widths, 0.4 us
-// (one step with caches, 3072 / 8192: 19.1 us, 18.8 like this).
+// 5.8.)  Out of line: in line it cost the launches that carry cache updates, which are bound by fetching instructions
+// already, 0.4 us (one step with caches: 3072 / 8192 19.1 us and 18.8 like this, 5120 / 17920 34.4 and 34.1).
 // scratch: T floats of shared memory that nobody reads or writes any more.
 constexpr int MAIL_N = 8;
 template <int SLAB, int T>

@@ -525,8 +525,8 @@ gemv_int4_kernel(const GemvParams p, int n_chunks, const std::conditional_t<SEL,
         }
         __syncthreads();
 
-        // ---- 5. stream: warp (chunk, kgroup) takes the K-blocks kgroup, kgroup + kgroups, ... of
-        //         its chunk; accumulators of the current quad in d[], flushed when the quad changes ----
+        // ---- 5. stream: warp (chunk, kgroup) takes the kgroup-th run of its chunk's K-blocks; accumulators
+        //         of the current quad in d[], flushed when the quad changes ----
         float d[9][4];
 #pragma unroll
         for (int m = 0; m < 9; ++m) d[m][0] = d[m][1] = d[m][2] = d[m][3] = 0.f;
