@@ -337,9 +337,7 @@ dip_status dip_mask_topk(dip_ctx *ctx, const float *x, int batch, int d, int k,
     if (!fits(ctx, d, 0, batch)) return DIP_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     uint32_t *m = mask_bits ? mask_bits : ctx->mask;
-    dip_status st = dip_launch_select(ctx, x, nullptr, nullptr, batch, d, k, 1.0f, nullptr, m, s);
-    if (st == DIP_OK && kept_idx) st = dip_launch_mask_to_idx(ctx, m, batch, 1, d, kept_idx, k, nullptr, s);
-    return st;
+    return dip_launch_select(ctx, x, nullptr, nullptr, batch, d, k, 1.0f, nullptr, m, s, nullptr, kept_idx);
 }
 
 dip_status dip_ca_mask(dip_ctx *ctx, const float *x, int d, int k, float gamma,
@@ -353,13 +351,8 @@ dip_status dip_ca_mask(dip_ctx *ctx, const float *x, int d, int k, float gamma,
     if (!fits(ctx, d, 0, 1)) return DIP_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     uint32_t *m = mask_bits ? mask_bits : ctx->mask;
-    dip_status rc = dip_launch_select(ctx, x, nullptr, nullptr, 1, d, k, gamma, st->stamp, m, s);
-    dip_cache_updates u;
-    u.n = 1;
-    u.at[0] = dip_update_of(st, m);
-    if (rc == DIP_OK) rc = dip_launch_cache_updates(ctx, u, s);
-    if (rc == DIP_OK && kept_idx) rc = dip_launch_mask_to_idx(ctx, m, 1, 1, d, kept_idx, k, nullptr, s);
-    return rc;
+    const dip_cache_update u = dip_update_of(st, m);
+    return dip_launch_select(ctx, x, nullptr, nullptr, 1, d, k, gamma, st->stamp, m, s, nullptr, kept_idx, &u);
 }
 
 static dip_status gemv_entry(dip_ctx *ctx, const dip_mlp_weights *w, int which, const float *v, int batch,
@@ -374,13 +367,7 @@ static dip_status gemv_entry(dip_ctx *ctx, const dip_mlp_weights *w, int which, 
     if (batch < 1 || batch > DIP_MAX_BATCH || n_kept < 1 || n_kept > d_in) return DIP_ERR_INVALID_ARG;
     if (batch > 1 && !mask_bits) return DIP_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    if (batch == 1 && kept_idx) {
-        // the kernels take the kept columns as a bit set
-        dip_status st = dip_launch_idx_to_mask(ctx, kept_idx, n_kept, d_in, ctx->mask_tmp, s);
-        if (st != DIP_OK) return st;
-        mask_bits = ctx->mask_tmp;
-    }
-    return dip_launch_gemv(ctx, w, which, v, batch, mask_bits, n_kept, out, s);
+    return dip_launch_gemv(ctx, w, which, v, batch, mask_bits, n_kept, out, s, nullptr, nullptr, batch == 1 ? kept_idx : nullptr);
 }
 
 dip_status dip_sparse_gemv_gate_up(dip_ctx *ctx, const dip_mlp_weights *w, const float *x, int batch,
@@ -644,8 +631,7 @@ dip_status dip_mlp_step_neuron_pruned(dip_ctx *ctx, const dip_neuron_weights *w,
                            by_gate ? 1 : 0, nullptr, p, h, s);
     if (st != DIP_OK) return st;
     // m = topK(|p|) over the neurons (Eq. 5), as a bit set and as an ascending list
-    if ((st = dip_launch_select(ctx, p, nullptr, nullptr, 1, w->d_ff, k, 1.0f, nullptr, mask, s)) != DIP_OK) return st;
-    if ((st = dip_launch_mask_to_idx(ctx, mask, 1, 1, w->d_ff, idx, k, nullptr, s)) != DIP_OK) return st;
+    if ((st = dip_launch_select(ctx, p, nullptr, nullptr, 1, w->d_ff, k, 1.0f, nullptr, mask, s, nullptr, idx)) != DIP_OK) return st;
     // the kept rows of the other matrix: h_j = p_j * (W^u x)_j, or p_j * silu((W^g x)_j); 0 elsewhere (from the
     // dense product's launch)
     st = dip_launch_rowdot(ctx, w->wtype, by_gate ? w->up : w->gate, w->d_model, w->d_ff, x, idx, k,

@@ -147,21 +147,25 @@ static inline cudaError_t dip_raise_smem_limit(dip_per_device_once &once, int de
 
 // ---- launchers implemented in the kernel files (host functions) -----------------
 
-// topk.cu: mask of each row: k largest rank keys (|x|, or |x| * (resident ? 1 : gamma) when stamp
-// is given).  xb != nullptr: the row is first formed as (xa + xb) / rms(xa + xb), written to x_out.
-// coarse != nullptr (no xb, d % 32 == 0; several rows only without stamps): the producer of xa has left the top 16 bits of
-// every column's rank key there (dip_gemv_keys), and the launch reads those instead of all of
-// xa and stamp.
-dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, float *x_out, int batch, int d, int k,
-                             float gamma, const int32_t *stamp, uint32_t *mask_bits, cudaStream_t stream,
-                             const uint16_t *coarse = nullptr);
-
-// topk.cu: cache updates from (mask, state), a block per cache.  count != nullptr: LFU (use counters), else LRU.
+// One cache update: from (mask, state).  count != nullptr: LFU (use counters), else LRU.
 struct dip_cache_update {
     const uint32_t *mask;
     int32_t *stamp, *count, *meta;
     int d, capacity;
 };
+
+// topk.cu: mask of each row: k largest rank keys (|x|, or |x| * (resident ? 1 : gamma) when stamp
+// is given).  xb != nullptr: the row is first formed as (xa + xb) / rms(xa + xb), written to x_out.
+// coarse != nullptr (no xb, d % 32 == 0; several rows only without stamps): the producer of xa has left the top 16 bits of
+// every column's rank key there (dip_gemv_keys), and the launch reads those instead of all of
+// xa and stamp.  idx_out != nullptr (no xb, no coarse): the kept columns of each row as an ascending list, k apart.
+// update != nullptr (one row with stamps, no xb, no coarse): the launch also makes this cache's update from the mask.
+dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, float *x_out, int batch, int d, int k,
+                             float gamma, const int32_t *stamp, uint32_t *mask_bits, cudaStream_t stream,
+                             const uint16_t *coarse = nullptr, int32_t *idx_out = nullptr,
+                             const dip_cache_update *update = nullptr);
+
+// topk.cu: several of them, a block per cache.
 constexpr int DIP_CACHE_UPDATES = 7;   // the caches of three blocks and a half; beside 140 products' CTAs on 148 SMs
 struct dip_cache_updates {
     int n;
@@ -208,10 +212,12 @@ struct dip_gemv_keys {
     float gamma;
     int written;             // out
 };
+// list != nullptr (one token, no rows; mask_bits is not read then): the rows are the n_kept_max columns of that list, in
+// any order; a column that comes twice counts once, one outside the input is ignored.
 dip_status dip_launch_gemv(dip_ctx *ctx, const dip_mlp_weights *w, int which,
                            const float *v, int batch, const uint32_t *mask_bits, int n_kept_max,
                            float *out, cudaStream_t stream, const dip_gemv_rows *rows = nullptr,
-                           dip_gemv_keys *keys = nullptr);
+                           dip_gemv_keys *keys = nullptr, const int32_t *list = nullptr);
 
 // gemv_fused.cu: the product `which` of a single-token step together with the select of its input.
 struct dip_fused_select {

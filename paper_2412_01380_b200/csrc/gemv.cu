@@ -428,7 +428,7 @@ template <int NW> struct __align__(16) GemvDirectSmem {
     uint16_t idx[GV_MAX_ROWS];
     uint32_t words[DIP_MAX_D / 32];
     int pre[DIP_MAX_D / 32];
-    int wsum[GV_SCAN_THREADS / 32];
+    int wsum[NW];
     int n_total;
     float red[NW][32 * 8];           // [warp][lane * E + e], E <= 8
     float sum[32 * 8];
@@ -443,7 +443,7 @@ gemv_direct_kernel(const GemvParams p)
     constexpr int OUT_PER_SLAB = WHICH == 0 ? SLAB / 2 : SLAB;
     constexpr int C = WTraits<WT>::C;
     constexpr int THREADS = NW * 32;
-    static_assert(THREADS >= GV_SCAN_THREADS && E <= 8, "");
+    static_assert(THREADS >= DIP_MAX_D / 32 && NW == 32 && E <= 8, "");
     __shared__ GemvDirectSmem<NW> s;
 
     DIP_TRACE_MIN(p.tr, 0);
@@ -451,6 +451,7 @@ gemv_direct_kernel(const GemvParams p)
     const int slab = blockIdx.x, part = blockIdx.y, nparts = gridDim.y;
     const size_t byte_off = (size_t)slab * GD_SEG + lane * 16;
     const bool lane_ok = byte_off < p.row_bytes;
+    if (p.list && tid < p.mask_words) s.words[tid] = 0u;
     dip_grid_dependency_wait();
     DIP_TRACE_MIN(p.tr, 1);
     dip_launch_dependents();
@@ -460,17 +461,20 @@ gemv_direct_kernel(const GemvParams p)
     if (WHICH == 0 && p.key_coarse && p.key_stamp && tid < OUT_PER_SLAB && slab * OUT_PER_SLAB + tid < p.d_out)
         key_stamp = __ldcg(p.key_stamp + slab * OUT_PER_SLAB + tid);
 
-    // ---- 1. the mask words and their popcount prefix (as in gemv_kernel) ----
-    if (tid < GV_SCAN_THREADS) {
-        uint32_t u[4] = {0u, 0u, 0u, 0u};
-        int c = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int w = 4 * tid + j;
-            if (w < p.mask_words) u[j] = p.mask_bits[w];
-            if (w == p.mask_words - 1 && (p.d_in & 31)) u[j] &= (1u << (p.d_in & 31)) - 1u;
-            c += __popc(u[j]);
-        }
+    // ---- 1. the mask words, a thread each, and their popcount prefix ----
+    uint32_t word = 0u;
+    if (p.list) {
+        __syncthreads();
+        list_to_words<THREADS>(p.list, p.n_list, p.d_in, s.words);
+        __syncthreads();
+        if (tid < p.mask_words) word = s.words[tid];
+    } else if (tid < p.mask_words) {
+        word = p.mask_bits[tid];
+        if (tid == p.mask_words - 1 && (p.d_in & 31)) word &= (1u << (p.d_in & 31)) - 1u;
+        s.words[tid] = word;
+    }
+    {
+        const int c = __popc(word);
         int incl = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -478,21 +482,10 @@ gemv_direct_kernel(const GemvParams p)
             if (lane >= o) incl += n;
         }
         if (lane == 31) s.wsum[warp] = incl;
-        asm volatile("bar.sync 1, %0;" ::"n"(GV_SCAN_THREADS) : "memory");
-        int before = 0;
-#pragma unroll
-        for (int w = 0; w < GV_SCAN_THREADS / 32; ++w) before += w < warp ? s.wsum[w] : 0;
-        int pre = before + incl - c;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int w = 4 * tid + j;
-            if (w < p.mask_words) {
-                s.words[w] = u[j];
-                s.pre[w] = pre;
-            }
-            pre += __popc(u[j]);
-        }
-        if (tid == GV_SCAN_THREADS - 1) s.n_total = pre;
+        __syncthreads();
+        const int before = (int)__reduce_add_sync(0xffffffffu, lane < warp ? (unsigned)s.wsum[lane] : 0u);
+        s.pre[tid] = before + incl - c;
+        if (tid == THREADS - 1) s.n_total = before + incl;
     }
     __syncthreads();
     const int n_total = s.n_total;
@@ -507,12 +500,14 @@ gemv_direct_kernel(const GemvParams p)
     for (int round_begin = r_begin; round_begin < r_end; round_begin += GV_MAX_ROWS) {
         const int n_rows = min(r_end - round_begin, GV_MAX_ROWS);
         if (round_begin != r_begin) __syncthreads();
-        // ---- 2. the round's rows in rank order ----
+        // ---- 2. the round's rows in rank order: a thread has a byte of a word ----
         {
             const int lo_rank = round_begin, hi_rank = round_begin + n_rows;
-            for (int w = tid; w < p.mask_words; w += THREADS) {
-                uint32_t u = s.words[w];
-                int rank = s.pre[w];
+            for (int q = tid; q < 4 * p.mask_words; q += THREADS) {
+                const int w = q >> 2, low = 8 * (q & 3);
+                const uint32_t all = s.words[w];
+                uint32_t u = all & (0xffu << low);
+                int rank = s.pre[w] + __popc(all & ((1u << low) - 1u));
                 if (rank >= hi_rank || rank + __popc(u) <= lo_rank) continue;
                 while (u) {
                     const int bit = __ffs(u) - 1;
@@ -835,13 +830,14 @@ dip_status launch_bt(dip_ctx *ctx, GemvParams &p, int n_kept_max, int mode, cuda
 
 dip_status dip_launch_gemv(dip_ctx *ctx, const dip_mlp_weights *w, int which,
                            const float *v, int batch, const uint32_t *mask_bits, int n_kept_max,
-                           float *out, cudaStream_t stream, const dip_gemv_rows *rows, dip_gemv_keys *keys)
+                           float *out, cudaStream_t stream, const dip_gemv_rows *rows, dip_gemv_keys *keys, const int32_t *list)
 {
     const int mode = rows ? rows->mode : 0;
     if (keys) keys->written = 0;
     if (mode && batch != 1) return DIP_ERR_UNSUPPORTED;
     const bool int4 = w->wtype == DIP_W_INT4_G128;
     if (int4 && batch > 1) return DIP_ERR_UNSUPPORTED;      // the 4-bit path is single-token
+    if (list && (batch != 1 || rows)) return DIP_ERR_INVALID_ARG;
     const size_t row_elems = which == 0 ? (size_t)2 * w->d_ff : (size_t)w->d_model;
     GemvParams p;
     p.W = rows ? (const char *)rows->base : (const char *)(which == 0 ? w->gate_up : w->down);
@@ -854,6 +850,17 @@ dip_status dip_launch_gemv(dip_ctx *ctx, const dip_mlp_weights *w, int which,
     p.mask_words = (p.d_in + 31) / 32;
     p.partials = ctx->partials;
     p.mail = ctx->mail;
+    p.list = nullptr;
+    p.n_list = 0;
+    if (list && (int4 || ctx->gemv_direct)) {
+        p.list = list;
+        p.n_list = n_kept_max;
+    } else if (list) {
+        // the copy ring takes the columns as a bit set
+        const dip_status st = dip_launch_idx_to_mask(ctx, list, n_kept_max, p.d_in, ctx->mask_tmp, stream);
+        if (st != DIP_OK) return st;
+        mask_bits = ctx->mask_tmp;
+    }
     p.tickets = ctx->tickets;
     p.status = ctx->status;
     p.wait_limit_ns = ctx->wait_limit_ns;

@@ -17,6 +17,8 @@ struct GemvParams {
     int d_in;
     const uint32_t *mask_bits; // [batch][mask_words]; rows read = OR over the batch
     int mask_words;
+    const int32_t *list;       // one token: the kept columns as a list of n_list (see dip_launch_gemv) instead of mask_bits
+    int n_list;
     float *out;                // [batch][d_out]
     int d_out;
     int batch;                 // tokens in this launch (<= BT)
@@ -234,6 +236,22 @@ __device__ __forceinline__ float silu_f32(float g) { return g / (1.0f + expf(-g)
 __device__ __forceinline__ float half_bits_to_float(uint16_t h)
 {
     return __half2float(__ushort_as_half(h));
+}
+
+// The columns in list[0 .. n) as a bit set: words[] is zero on entry (and that is visible), all T threads call it, no
+// barrier at the end.  (Every CTA of a product for itself: a few KB out of L2, against a launch of its own in front.)
+template <int T>
+__device__ __forceinline__ void list_to_words(const int32_t *list, int n, int d, uint32_t *words)
+{
+    constexpr int U = 4;                       // loads that go out together
+    for (int r0 = threadIdx.x; r0 < n; r0 += U * T) {
+        int i[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) i[u] = r0 + u * T < n ? __ldg(list + r0 + u * T) : -1;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i[u] >= 0 && i[u] < d) atomicOr(&words[i[u] >> 5], 1u << (i[u] & 31));
+    }
 }
 
 namespace {

@@ -320,6 +320,8 @@ gemv_int4_kernel(const GemvParams p, int n_chunks, const std::conditional_t<SEL,
     if constexpr (SEL) {
         fine_zero<I4_THREADS>(f.fine);
         if (tid < 32) f.ts.wa[tid] = f.ts.wb[tid] = f.ts.wc[tid] = f.wsum[tid] = 0;
+    } else if (p.list) {
+        for (int w = tid; w < p.mask_words; w += I4_THREADS) s.words[w] = 0u;
     }
     dip_grid_dependency_wait();
     DIP_TRACE_MIN(p.tr, 1);
@@ -346,11 +348,16 @@ gemv_int4_kernel(const GemvParams p, int n_chunks, const std::conditional_t<SEL,
     } else {
         // ---- 1. the mask words and their popcount prefix ----
         uint32_t u[4] = {0u, 0u, 0u, 0u};
+        if (p.list) {
+            __syncthreads();
+            list_to_words<I4_THREADS>(p.list, p.n_list, p.d_in, s.words);
+            __syncthreads();
+        }
         if (tid < GV_SCAN_THREADS) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int w = 4 * tid + j;
-                if (w < p.mask_words) u[j] = p.mask_bits[w];
+                if (w < p.mask_words) u[j] = p.list ? s.words[w] : p.mask_bits[w];
             }
             int c = 0;
 #pragma unroll

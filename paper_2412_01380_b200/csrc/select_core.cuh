@@ -523,7 +523,7 @@ __device__ __forceinline__ void select_fine_tail(const uint32_t *keys, int d, in
 // all in shared memory except x_out.  Ends with a barrier.
 template <bool CA, bool NORM>
 __device__ __forceinline__ void select_fine(const float *__restrict__ xa, float *__restrict__ x_out, int d,
-                                            int k, float gamma, const int32_t *__restrict__ stamp, float scale,
+                                            int k, float gamma, const int32_t *stamp, float scale,
                                             uint32_t *keys, TkShared &s, TkFine &f, unsigned int *maskw)
 {
     const int tid = threadIdx.x;
@@ -702,6 +702,27 @@ __device__ __forceinline__ void select_fine_coarse(const uint16_t *__restrict__ 
     __syncthreads();
     fine_complete(f, n_c, krem, maskw,
                   [&](int col) { return rank_key<CA>(__ldcg(x + col), CA ? __ldcg(stamp + col) : 0, gamma); });
+}
+
+// The columns of a complete mask in shared memory as an ascending list.  A thread has a byte of the mask (d <= 8 *
+// TK_THREADS) or a word.  All threads call it; one barrier inside, none at the end.
+__device__ __forceinline__ void list_mask(const unsigned int *maskw, int d, TkShared &s, int32_t *idx_out)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int span = d <= 8 * TK_THREADS ? 8 : 32;
+    uint32_t m = 0u;
+    if (tid * span < d) m = span == 8 ? reinterpret_cast<const unsigned char *>(maskw)[tid] : maskw[tid];
+    const int c = __popc(m);
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += n;
+    }
+    if (lane == 31) s.wb[warp] = incl;
+    __syncthreads();
+    int at = (int)__reduce_add_sync(0xffffffffu, lane < warp ? (unsigned)s.wb[lane] : 0u) + incl - c;
+    for (; m; m &= m - 1) idx_out[at++] = tid * span + __ffs(m) - 1;
 }
 
 }  // namespace

@@ -9,6 +9,8 @@
 //                        does not feed the GEMVs and runs beside them on another stream.
 // Everything here is integer work on bit patterns, so results are exact and unique (ties go
 // to the lower column index).
+#include <type_traits>
+
 #include "cache_update.cuh"
 
 namespace {
@@ -29,13 +31,19 @@ namespace {
 // bytes this CTA has to pull in are its floor: two bytes per column instead of the eight of value +
 // stamp.  Needs d % 8 == 0 and d <= 8 * TK_COARSE_ITERS * TK_THREADS.
 // Dynamic shared memory: TkFine, then keys[] (d words rounded up to four).
+// idx_out != nullptr: the kept columns of row r as an ascending list at idx_out + r * k.
+// UPD: the CTA goes on to update the row's cache (one row; Algorithm 1 whole).  What bounds dip_ca_mask is the chain of
+// its launches (select, update and list were three), and the mask is here in shared memory: masks with lists and list
+// products at 2080 / 5472, four calls in a graph, 36.7 us with ten launches and 28.8 with four.
 // ---------------------------------------------------------------------------------------
-template <bool CA, bool NORM>
+template <bool CA, bool NORM, bool UPD>
 __global__ void __launch_bounds__(TK_THREADS, 1)
 select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, float *__restrict__ x_out,
-                   int d, int k, float gamma, const int32_t *__restrict__ stamp,
-                   uint32_t *__restrict__ mask_bits, unsigned long long *tr)
+                   int d, int k, float gamma, const int32_t *stamp,
+                   uint32_t *__restrict__ mask_bits, int32_t *__restrict__ idx_out,
+                   const std::conditional_t<UPD, dip_cache_update, Int<0>> u, unsigned long long *tr)
 {
+    static_assert(!UPD || (CA && !NORM), "");
     DIP_TRACE_MIN(tr, 0);
     extern __shared__ __align__(16) unsigned char dyn[];
     TkFine &f = *reinterpret_cast<TkFine *>(dyn);
@@ -68,6 +76,11 @@ select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, f
         select_fine<CA, NORM>(xa, NORM ? x_out : nullptr, d, k, gamma, stamp, scale, keys, s, f, s_maskw);
     }
     for (int w = tid; w < n_words; w += TK_THREADS) mask_bits[w] = s_maskw[w];
+    if (idx_out) list_mask(s_maskw, d, s, idx_out + (size_t)row * k);
+    if constexpr (UPD) {
+        cache_update_clear(s, f.hist);
+        block_cache_update_any(s_maskw, d, u.stamp, u.stamp, u.count, u.meta, u.capacity, s, f.hist, []() {}, []() { return true; });
+    }
     DIP_TRACE_MAX(tr, 2);
 }
 
@@ -180,8 +193,11 @@ residual_rmsnorm_kernel(const float *x, const float *y, int d, float *x_next)
 // ---------------------------------------------------------------------------------------
 dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, float *x_out, int batch, int d, int k,
                              float gamma, const int32_t *stamp, uint32_t *mask_bits, cudaStream_t stream,
-                             const uint16_t *coarse)
+                             const uint16_t *coarse, int32_t *idx_out, const dip_cache_update *update)
 {
+    if ((idx_out || update) && (coarse || xb)) return DIP_ERR_INVALID_ARG;
+    if (update && (batch != 1 || !stamp)) return DIP_ERR_INVALID_ARG;
+    const Int<0> no;
     const size_t smem = sizeof(TkFine) + (size_t)((d + 3) & ~3) * sizeof(uint32_t);
     const dim3 grid(batch), block(TK_THREADS);
     unsigned long long *tr = dip_trace_slot(ctx, d <= 0 ? 0 : (stamp ? 2 : 1));
@@ -196,17 +212,21 @@ dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, flo
                                (const int32_t *)nullptr, mask_bits, tr);
     } else if (xb) {
         if (stamp)
-            e = dip_launch_pdl(select_fine_kernel<true, true>, grid, block, smem, stream, xa, xb, x_out, d, k, gamma, stamp, mask_bits, tr);
+            e = dip_launch_pdl(select_fine_kernel<true, true, false>, grid, block, smem, stream, xa, xb, x_out, d, k, gamma, stamp,
+                               mask_bits, idx_out, no, tr);
         else
-            e = dip_launch_pdl(select_fine_kernel<false, true>, grid, block, smem, stream, xa, xb, x_out, d, k, 1.0f,
-                               (const int32_t *)nullptr, mask_bits, tr);
+            e = dip_launch_pdl(select_fine_kernel<false, true, false>, grid, block, smem, stream, xa, xb, x_out, d, k, 1.0f,
+                               (const int32_t *)nullptr, mask_bits, idx_out, no, tr);
     } else {
-        if (stamp)
-            e = dip_launch_pdl(select_fine_kernel<true, false>, grid, block, smem, stream, xa, (const float *)nullptr,
-                               (float *)nullptr, d, k, gamma, stamp, mask_bits, tr);
+        if (update)
+            e = dip_launch_pdl(select_fine_kernel<true, false, true>, grid, block, smem, stream, xa, (const float *)nullptr,
+                               (float *)nullptr, d, k, gamma, stamp, mask_bits, idx_out, *update, tr);
+        else if (stamp)
+            e = dip_launch_pdl(select_fine_kernel<true, false, false>, grid, block, smem, stream, xa, (const float *)nullptr,
+                               (float *)nullptr, d, k, gamma, stamp, mask_bits, idx_out, no, tr);
         else
-            e = dip_launch_pdl(select_fine_kernel<false, false>, grid, block, smem, stream, xa, (const float *)nullptr,
-                               (float *)nullptr, d, k, 1.0f, (const int32_t *)nullptr, mask_bits, tr);
+            e = dip_launch_pdl(select_fine_kernel<false, false, false>, grid, block, smem, stream, xa, (const float *)nullptr,
+                               (float *)nullptr, d, k, 1.0f, (const int32_t *)nullptr, mask_bits, idx_out, no, tr);
     }
     DIP_CUDA_TRY(ctx, e);
     return DIP_OK;
@@ -224,10 +244,11 @@ dip_status dip_init_mask_kernels(dip_ctx *ctx)
 {
     const int bytes = DIP_MAX_D * (int)sizeof(uint32_t);
     const int fine_bytes = bytes + (int)sizeof(TkFine);
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
     DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_coarse_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
     DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_coarse_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
     return DIP_OK;
