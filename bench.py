@@ -584,7 +584,7 @@ def run_two_tier(dip, ctx, torch, w, L, rank, xs_host, keep_ratio, budget, steps
     e1.record(stream)
     torch.cuda.synchronize()
     ms_e = e0.elapsed_time(e1)
-    # the fetch kernel by itself: a second capture with the device-side timeline on, a few replays
+    # the reads of the slow tier by themselves: a second capture with the device-side timeline on, a few replays
     ctx.trace_begin()
     graph_t = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph_t):
@@ -766,12 +766,12 @@ def main_two_tier(args, dip, ctx, torch, w, keep_ratio, budget, rank, world, loc
                    "parallelism": "replicas only"},
         "mlp_step_us": r["ms_per_step"] * 1e3 / L, "hit_rate": r["hit_rate"], "clocks": r["clocks"],
         "e2e": r["e2e"],
-        # per layer: 2 selects, 2 splits, 2 miss lists, 2 cache updates, 2 slot assignments, 2 fetches, 2 installs, 4 GEMVs,
-        # 2 combines, 1 rmsnorm
-        "gpu_launches": 21 * L * args.steps,
-        # the fetch kernel: bytes it brought in / its own device time (timeline of 8 replays); the
-        # same bytes over the whole step's time are in fetch_gbs_over_step
-        "roofline": {"bound": "host_link", "kernel": "tier_fetch_kernel", "achieved": r["fetch_kernel_gbs"],
+        # per layer: 2 selects, 2 products, 1 rmsnorm; with 4-bit weights 2 selects, 2 fetches, 4 GEMVs, 2 combines, 1 rmsnorm
+        "gpu_launches": (11 if w.wtype == di.W_INT4_G128 else 5) * L * args.steps,
+        # the reads of the slow tier: bytes brought in / the time from their start to their end within their launches
+        # (timeline of 8 replays); the same bytes over the whole step's time are in fetch_gbs_over_step
+        "roofline": {"bound": "host_link", "kernel": "tier_fetch_kernel" if w.wtype == di.W_INT4_G128 else "tier_product_kernel",
+                     "achieved": r["fetch_kernel_gbs"],
                      "peak": link, "peak_kind": "of a pinned host-to-device copy measured in this run",
                      "unit": "GB/s", "frac": r["fetch_kernel_gbs"] / link,
                      "bytes_per_launch": r["fetch_kernel_bytes"], "us_per_launch": r["fetch_kernel_us"],

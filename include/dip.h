@@ -130,7 +130,8 @@ int dip_sm_count(const dip_ctx *ctx);
  * If a wait runs out, the kernel goes on without what it waited for and a sticky status word on the
  * device becomes non-zero.  From then on the outputs of that call AND OF EVERY LATER CALL on the context
  * are invalid (what came too late is still under way in its workspace) until dip_reset_device_status;
- * a cache state that the failed call was to update may or may not be updated: restore or clear it.
+ * a cache state that the failed call was to update may or may not be updated: restore or clear it; a
+ * dip_tier of that call may name rows that were not moved: start it and its cache cold.
  * No call looks at the word by itself.
  * This call waits for `stream`, then copies the word to *status_out (host). */
 typedef enum {
@@ -160,8 +161,8 @@ dip_status dip_selftest_bounded_wait(dip_ctx *ctx, int limit_us, unsigned long l
  * dip_trace_read returns the records of the launches that ran since.  These
  * calls synchronise the device; the stamps cost one atomic per CTA.
  *   kind: 1 select (DIP), 2 select (cache-aware), 3 cache update, 4 gate/up GEMV,
- *         5 down GEMV, 6 slot assignment, 7 fetch, 8 hit/miss split, 10 install (two-tier
- *         step), 9 neuron-major product (Gate / Up pruning).
+ *         5 down GEMV, 6 cache update and slot assignment, 7 reads of the slow tier (two-tier step; parts
+ *         of a GEMV's launch, or of one that does both), 9 neuron-major product (Gate / Up pruning).
  * ------------------------------------------------------------------------ */
 typedef struct {
     int32_t kind;
@@ -482,7 +483,7 @@ dip_status dip_mlp_step_neuron_pruned(dip_ctx *ctx, const dip_neuron_weights *w,
  *            stamp[i] >= 0; start both cold (all -1)
  *   loc      device int32[d]: scratch; arena row of each column of the current mask
  *   fetch    device int32[4 + 2 * staging]: scratch; [0] = misses of the step,
- *            [1] = rows moved into slots, then the misses' columns, then the moves
+ *            [1] = rows moved into slots, then the misses' columns, then their slots or -1
  *   split    device uint32[2][ceil(d/32)]: scratch; the mask's hits and its misses
  *   counters device uint64[2], accumulated: rows fetched, bytes fetched
  * Which slot a new column gets is the library's choice (the lowest free slots,
@@ -508,12 +509,11 @@ typedef struct {
 /* ------------------------------------------------------------------------
  * dip_mlp_step_tiered — dip_mlp_step for one token with both masked inputs
  * cache-aware and their weights two-tiered.  Per input: mask (Algorithm 1's
- * ranking); the mask's hits are multiplied out of the arena at once while one
- * stream of the context copies its misses from the slow tier into the staging
- * rows and another keeps the books (cache update, slot assignment, the move of
- * the staged rows that the cache keeps into their slots); the misses' product
- * follows the copy and the two partial results are added (hits first).  The
- * book-keeping is joined into `stream` before the call's work ends.  w gives
+ * ranking); the mask's hits are multiplied out of the arena while its misses
+ * come from the slow tier, are multiplied and left in the staging rows (INT4:
+ * are copied there and then multiplied), and the books are kept (cache update,
+ * slot assignment, the move of the staged rows that the cache keeps into their
+ * slots).  All of it is through when the call's work on `stream` ends.  w gives
  * the format and shapes (and the INT4 scales); w->gate_up and w->down are not
  * read and may be NULL.  Results equal dip_mlp_step's on the same cache states
  * up to the order of the binary32 sums.  k_x <= tier_gu->staging and

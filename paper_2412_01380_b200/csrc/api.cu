@@ -143,7 +143,7 @@ dip_status dip_create_ex(dip_ctx **out, int device, const dip_options *opt)
     const size_t vec = (size_t)ctx->max_batch * ctx->max_d;
     if ((st = dev_alloc(ctx, &ctx->partials, ctx->partials_floats)) != DIP_OK) return fail(st);
     if ((st = dev_alloc(ctx, &ctx->mail, (size_t)ctx->sm_count * DIP_MAIL_FLOATS)) != DIP_OK) return fail(st);
-    if ((st = dev_alloc(ctx, &ctx->readers, (size_t)1)) != DIP_OK) return fail(st);
+    if ((st = dev_alloc(ctx, &ctx->readers, (size_t)DIP_SYNC_WORDS)) != DIP_OK) return fail(st);
     if ((st = dev_alloc(ctx, &ctx->tickets, (size_t)N_TICKETS)) != DIP_OK) return fail(st);
     if ((st = dev_alloc(ctx, &ctx->h, vec)) != DIP_OK) return fail(st);
     if ((st = dev_alloc(ctx, &ctx->y, vec)) != DIP_OK) return fail(st);
@@ -163,13 +163,9 @@ dip_status dip_create_ex(dip_ctx **out, int device, const dip_options *opt)
     if ((st = dev_alloc(ctx, &ctx->xt, (size_t)ctx->max_d * 32)) != DIP_OK) return fail(st);
     if ((st = dev_alloc(ctx, &ctx->status, (size_t)1)) != DIP_OK) return fail(st);
     if ((st = dev_alloc(ctx, &ctx->trace, (size_t)DIP_TRACE_SLOTS * DIP_TRACE_WORDS)) != DIP_OK) return fail(st);
-    for (int i = 0; i < 2; ++i) {
-        if (cudaStreamCreateWithFlags(&ctx->tier_fetch[i], cudaStreamNonBlocking) != cudaSuccess) return fail(DIP_ERR_CUDA);
-        if (cudaStreamCreateWithFlags(&ctx->tier_book[i], cudaStreamNonBlocking) != cudaSuccess) return fail(DIP_ERR_CUDA);
-        if (cudaEventCreateWithFlags(&ctx->ev_tier_fork[i], cudaEventDisableTiming) != cudaSuccess) return fail(DIP_ERR_CUDA);
-        if (cudaEventCreateWithFlags(&ctx->ev_tier_fetched[i], cudaEventDisableTiming) != cudaSuccess) return fail(DIP_ERR_CUDA);
-        if (cudaEventCreateWithFlags(&ctx->ev_tier_booked[i], cudaEventDisableTiming) != cudaSuccess) return fail(DIP_ERR_CUDA);
-    }
+    if (cudaStreamCreateWithFlags(&ctx->tier_fetch, cudaStreamNonBlocking) != cudaSuccess) return fail(DIP_ERR_CUDA);
+    if (cudaEventCreateWithFlags(&ctx->ev_tier_fork, cudaEventDisableTiming) != cudaSuccess) return fail(DIP_ERR_CUDA);
+    if (cudaEventCreateWithFlags(&ctx->ev_tier_fetched, cudaEventDisableTiming) != cudaSuccess) return fail(DIP_ERR_CUDA);
     for (int i = 0; i < 2; ++i) {
         if (cudaStreamCreateWithFlags(&ctx->side[i], cudaStreamNonBlocking) != cudaSuccess) return fail(DIP_ERR_CUDA);
         if (cudaEventCreateWithFlags(&ctx->ev_fork[i], cudaEventDisableTiming) != cudaSuccess) return fail(DIP_ERR_CUDA);
@@ -189,7 +185,7 @@ dip_status dip_create_ex(dip_ctx **out, int device, const dip_options *opt)
             return cudaMemcpyAsync(to, from, bytes, cudaMemcpyHostToDevice, ctx->side[0]) == cudaSuccess;
         };
         bool ok = set(ctx->mail, empty, mail_bytes) && set(ctx->status, zeros, sizeof(int)) &&
-                  set(ctx->readers, zeros, sizeof(unsigned int)) && set(ctx->tickets, zeros, sizeof(zeros)) &&
+                  set(ctx->readers, zeros, DIP_SYNC_WORDS * sizeof(unsigned int)) && set(ctx->tickets, zeros, sizeof(zeros)) &&
                   set(ctx->counts, zeros, 8 * sizeof(int32_t));
         ok = cudaStreamSynchronize(ctx->side[0]) == cudaSuccess && ok;
         free(empty);
@@ -230,12 +226,10 @@ dip_status dip_destroy(dip_ctx *ctx)
         if (ctx->side[i]) cudaStreamDestroy(ctx->side[i]);
         if (ctx->ev_fork[i]) cudaEventDestroy(ctx->ev_fork[i]);
         if (ctx->ev_join[i]) cudaEventDestroy(ctx->ev_join[i]);
-        if (ctx->tier_fetch[i]) cudaStreamDestroy(ctx->tier_fetch[i]);
-        if (ctx->tier_book[i]) cudaStreamDestroy(ctx->tier_book[i]);
-        if (ctx->ev_tier_fork[i]) cudaEventDestroy(ctx->ev_tier_fork[i]);
-        if (ctx->ev_tier_fetched[i]) cudaEventDestroy(ctx->ev_tier_fetched[i]);
-        if (ctx->ev_tier_booked[i]) cudaEventDestroy(ctx->ev_tier_booked[i]);
     }
+    if (ctx->tier_fetch) cudaStreamDestroy(ctx->tier_fetch);
+    if (ctx->ev_tier_fork) cudaEventDestroy(ctx->ev_tier_fork);
+    if (ctx->ev_tier_fetched) cudaEventDestroy(ctx->ev_tier_fetched);
     delete ctx;
     return DIP_OK;
 }
@@ -279,7 +273,7 @@ dip_status dip_reset_device_status(dip_ctx *ctx, void *stream)
     if (!ctx_ok(ctx)) return DIP_ERR_INVALID_ARG;
     DIP_CUDA_TRY(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(int), (cudaStream_t)stream));
     // (a launch that gave up a wait leaves behind what comes too late: counts, and sums nobody takes)
-    DIP_CUDA_TRY(ctx, cudaMemsetAsync(ctx->readers, 0, sizeof(unsigned int), (cudaStream_t)stream));
+    DIP_CUDA_TRY(ctx, cudaMemsetAsync(ctx->readers, 0, DIP_SYNC_WORDS * sizeof(unsigned int), (cudaStream_t)stream));
     DIP_CUDA_TRY(ctx, cudaMemsetAsync(ctx->mail, 0xff, (size_t)ctx->sm_count * DIP_MAIL_FLOATS * sizeof(float), (cudaStream_t)stream));
     return DIP_OK;
 }
@@ -525,37 +519,25 @@ dip_status dip_mlp_step(dip_ctx *ctx, const dip_mlp_weights *w,
                      ctx->mask, ctx->mask_h, false, &due, true, stream);
 }
 
-// One masked input of the two-tier step.  On the step's path: the hit / miss split, the list of
-// the misses, the hits' product; beside it one stream fetches the misses into the staging rows
-// (the misses' product waits for that) and another keeps the books: cache update, slot
-// assignment, and the move of the staged rows of the inserted columns into their slots.  The
-// book-keeping is joined at the end of the call.
+// One masked input of the two-tier step: the mask from the cache-aware ranking (Algorithm 1) with its hits and misses, then
+// one launch for the rest.  Products that do not read the slow tier themselves (4-bit weights; the copy ring) take the hits,
+// while a launch on another stream fetches the misses into the staging rows and keeps the books, and then the misses.
 static dip_status tiered_half(dip_ctx *ctx, const dip_mlp_weights *w, int which, const dip_tier *t,
-                              const dip_cache_state *c, const float *v, const uint32_t *mask_bits, int k,
+                              const dip_cache_state *c, const float *v, uint32_t *mask_bits, int k, float gamma,
                               float *out, cudaStream_t s)
 {
     const int words = (t->d + 31) / 32;
-    dip_status st = dip_launch_tier_split(ctx, t, mask_bits, s);
+    dip_status st = dip_launch_select(ctx, v, nullptr, nullptr, 1, t->d, k, gamma, c->stamp, mask_bits, s, nullptr, nullptr, nullptr, t);
     if (st != DIP_OK) return st;
-    // the misses as an ascending list: fetch[0] = how many, fetch[4 ..] = their columns
-    if ((st = dip_launch_mask_to_idx(ctx, t->split + words, 1, 1, t->d, t->fetch + 4, 0, t->fetch, s)) != DIP_OK) return st;
-    cudaStream_t sf = ctx->tier_fetch[which], sb = ctx->tier_book[which];
-    DIP_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_tier_fork[which], s));
-    DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(sf, ctx->ev_tier_fork[which], 0));
-    DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(sb, ctx->ev_tier_fork[which], 0));
-    if ((st = dip_launch_tier_fetch(ctx, t, sf)) != DIP_OK) return st;
-    DIP_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_tier_fetched[which], sf));
-    dip_cache_updates u;
-    u.n = 1;
-    u.at[0] = dip_update_of(c, mask_bits);
-    if ((st = dip_launch_cache_updates(ctx, u, sb)) != DIP_OK) return st;
-    if ((st = dip_launch_tier_assign(ctx, t, mask_bits, c->stamp, sb)) != DIP_OK) return st;
-    DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(sb, ctx->ev_tier_fetched[which], 0));
-    if ((st = dip_launch_tier_install(ctx, t, sb)) != DIP_OK) return st;
-    DIP_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_tier_booked[which], sb));
+    const dip_cache_update u = dip_update_of(c, mask_bits);
+    if (ctx->gemv_direct && w->wtype != DIP_W_INT4_G128) return dip_launch_tier_product(ctx, w, which, t, u, v, k, out, s);
+    DIP_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_tier_fork, s));
+    DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->tier_fetch, ctx->ev_tier_fork, 0));
+    if ((st = dip_launch_tier_fetch(ctx, t, u, ctx->tier_fetch)) != DIP_OK) return st;
+    DIP_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_tier_fetched, ctx->tier_fetch));
     dip_gemv_rows rows = {t->arena, t->loc, 1};
     if ((st = dip_launch_gemv(ctx, w, which, v, 1, t->split, k, out, s, &rows)) != DIP_OK) return st;
-    DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(s, ctx->ev_tier_fetched[which], 0));
+    DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(s, ctx->ev_tier_fetched, 0));
     rows.mode = 2;
     return dip_launch_gemv(ctx, w, which, v, 1, t->split + words, k, out, s, &rows);
 }
@@ -586,21 +568,13 @@ dip_status dip_mlp_step_tiered(dip_ctx *ctx, const dip_mlp_weights *w,
     float *h = out && out->h ? out->h : ctx->h;
     uint32_t *mask_h = out && out->mask_h ? out->mask_h : ctx->mask_h;
     dip_status st;
-    // m_x from the cache-aware ranking (Algorithm 1), then the gate/up half out of the two tiers
-    st = dip_launch_select(ctx, x, nullptr, nullptr, 1, w->d_model, k_x, gamma, cache_gu->stamp, mask_x, s);
-    if (st != DIP_OK) return st;
-    if ((st = tiered_half(ctx, w, 0, tier_gu, cache_gu, x, mask_x, k_x, h, s)) != DIP_OK) return st;
-    // m_h likewise (Eq. 8), then the down half
-    st = dip_launch_select(ctx, h, nullptr, nullptr, 1, w->d_ff, k_h, gamma, cache_d->stamp, mask_h, s);
-    if (st != DIP_OK) return st;
-    if ((st = tiered_half(ctx, w, 1, tier_d, cache_d, h, mask_h, k_h, y, s)) != DIP_OK) return st;
+    // m_x and the gate/up half out of the two tiers, then m_h (Eq. 8) and the down half likewise
+    if ((st = tiered_half(ctx, w, 0, tier_gu, cache_gu, x, mask_x, k_x, gamma, h, s)) != DIP_OK) return st;
+    if ((st = tiered_half(ctx, w, 1, tier_d, cache_d, h, mask_h, k_h, gamma, y, s)) != DIP_OK) return st;
     if (out && out->idx_x && (st = dip_launch_mask_to_idx(ctx, mask_x, 1, 1, w->d_model, out->idx_x, k_x, nullptr, s)) != DIP_OK)
         return st;
     if (out && out->idx_h && (st = dip_launch_mask_to_idx(ctx, mask_h, 1, 1, w->d_ff, out->idx_h, k_h, nullptr, s)) != DIP_OK)
         return st;
-    // the book-keeping of both inputs has to be through before the call's work ends
-    DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(s, ctx->ev_tier_booked[0], 0));
-    DIP_CUDA_TRY(ctx, cudaStreamWaitEvent(s, ctx->ev_tier_booked[1], 0));
     return DIP_OK;
 }
 

@@ -12,6 +12,7 @@
 constexpr int DIP_RING_LAYERS = 128;
 constexpr int DIP_TRACE_SLOTS = 1024;
 constexpr uint32_t DIP_MAIL_EMPTY = 0xffffffffu;
+constexpr int DIP_SYNC_WORDS = 3;
 constexpr int DIP_MAIL_FLOATS = 2048;  // boxes per SM: one CTA's segment of sums (INT4: up to 2048, F32 / BF16: 256)
 constexpr int DIP_TRACE_WORDS = 4;   // first start, dependency ready, last end, auxiliary
 
@@ -29,7 +30,8 @@ struct dip_ctx {
     float *partials;
     size_t partials_floats;
     float *mail;         // [sm_count][DIP_MAIL_FLOATS] row parts of one- and two-token products on their way to the CTA that adds them up
-    unsigned int *readers; // [1] CTAs of a fused product that have read the stamps; zero between launches
+    unsigned int *readers; // [DIP_SYNC_WORDS] zero between launches: CTAs of a fused product that have read the stamps; in a
+                           // two-tier launch: the moves are known, CTAs that are through
     // one arrival counter per output slab; zero between launches
     unsigned int *tickets;
     int n_tickets;
@@ -57,9 +59,9 @@ struct dip_ctx {
     cudaStream_t side[2];
     cudaEvent_t ev_fork[2], ev_join[2];
     bool side_busy[2];
-    // two-tier step, per masked input: a stream that fetches the misses and one that keeps the books
-    cudaStream_t tier_fetch[2], tier_book[2];
-    cudaEvent_t ev_tier_fork[2], ev_tier_fetched[2], ev_tier_booked[2];
+    // two-tier step out of the copy ring or with 4-bit weights: the misses are fetched on a stream of their own
+    cudaStream_t tier_fetch;
+    cudaEvent_t ev_tier_fork, ev_tier_fetched;
     // device-side timeline (diagnostics): one slot of DIP_TRACE_WORDS words per launch
     unsigned long long *trace;
     int trace_on;
@@ -160,10 +162,11 @@ struct dip_cache_update {
 // every column's rank key there (dip_gemv_keys), and the launch reads those instead of all of
 // xa and stamp.  idx_out != nullptr (no xb, no coarse): the kept columns of each row as an ascending list, k apart.
 // update != nullptr (one row with stamps, no xb, no coarse): the launch also makes this cache's update from the mask.
+// split != nullptr (likewise): the launch also parts the mask into this tier's hits and misses (split, loc, fetch).
 dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, float *x_out, int batch, int d, int k,
                              float gamma, const int32_t *stamp, uint32_t *mask_bits, cudaStream_t stream,
                              const uint16_t *coarse = nullptr, int32_t *idx_out = nullptr,
-                             const dip_cache_update *update = nullptr);
+                             const dip_cache_update *update = nullptr, const dip_tier *split = nullptr);
 
 // topk.cu: several of them, a block per cache.
 constexpr int DIP_CACHE_UPDATES = 7;   // the caches of three blocks and a half; beside 140 products' CTAs on 148 SMs
@@ -251,18 +254,14 @@ dip_status dip_launch_block_waits_selftest(dip_ctx *ctx, unsigned long long limi
 // gemv.cu: bit set from an ascending index list.
 dip_status dip_launch_idx_to_mask(dip_ctx *ctx, const int32_t *idx, int n, int d, uint32_t *mask, cudaStream_t stream);
 
-// tier.cu: before the cache update of a mask: its hits (resident columns, with their arena rows)
-// and its misses.
-dip_status dip_launch_tier_split(dip_ctx *ctx, const dip_tier *t, const uint32_t *mask_bits, cudaStream_t stream);
-// tier.cu: after the cache update: evicted columns free their slots, inserted columns get slots,
-// and the install list says which staging rows move where.
-dip_status dip_launch_tier_assign(dip_ctx *ctx, const dip_tier *t, const uint32_t *mask_bits, const int32_t *stamp,
-                                  cudaStream_t stream);
-// tier.cu: copy the rows of the miss list (fetch[0] columns at fetch + 4) from the slow tier into
-// the staging rows of the arena, in list order, and point loc at them.
-dip_status dip_launch_tier_fetch(dip_ctx *ctx, const dip_tier *t, cudaStream_t stream);
-// tier.cu: move the staged rows of the inserted columns into their cache slots (install list).
-dip_status dip_launch_tier_install(dip_ctx *ctx, const dip_tier *t, cudaStream_t stream);
+// tier.cu: everything after the select of a two-tier half (F32 / BF16): the product over hits and misses, which are read from
+// the slow tier and staged on the way, the cache update, the slots, and the moves of the staged rows that the cache keeps.
+dip_status dip_launch_tier_product(dip_ctx *ctx, const dip_mlp_weights *w, int which, const dip_tier *t, const dip_cache_update &c,
+                                   const float *v, int k, float *out, cudaStream_t stream);
+// tier.cu: the same without a product, for those that take hits and misses in launches of their own: fetch, books and moves
+// on DIP_TIER_CTAS SMs.
+constexpr int DIP_TIER_CTAS = 17;
+dip_status dip_launch_tier_fetch(dip_ctx *ctx, const dip_tier *t, const dip_cache_update &c, cudaStream_t stream);
 
 // rowdot.cu: out_j = [silu](W[j, :] . x) [* mul_j] for the listed rows (rows == nullptr: rows
 // 0 .. n_rows-1) of a row-major [d_ff][d_model] matrix; F32 or BF16.  zero != nullptr: also zero_j = 0 for these rows.

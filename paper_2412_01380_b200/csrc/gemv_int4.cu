@@ -751,13 +751,14 @@ dip_status dip_launch_gemv_int4(dip_ctx *ctx, GemvParams &p, int which, int n_ke
                                 cudaStream_t stream)
 {
     const int n_chunks = (int)(p.row_bytes / 64);
+    const int sms = ctx->sm_count - (mode ? DIP_TIER_CTAS : 0);   // (two-tier: the misses are fetched beside it)
     int seg_chunks = 16, n_slabs = 0, nparts = 1;
     // wide rows: the widest segment with which the segments alone occupy most of the SMs, so that
     // one CTA sees all kept rows of its segment and nothing is combined across CTAs
     bool whole = false;
     for (int sc = 16; sc >= 1 && !whole; sc >>= 1) {
         const int ns = (n_chunks + sc - 1) / sc;
-        if (ns <= ctx->sm_count && 5 * ns >= 3 * ctx->sm_count) {
+        if (ns <= sms && 5 * ns >= 3 * sms) {
             seg_chunks = sc;
             n_slabs = ns;
             whole = true;
@@ -765,7 +766,7 @@ dip_status dip_launch_gemv_int4(dip_ctx *ctx, GemvParams &p, int which, int n_ke
     }
     for (; !whole; seg_chunks >>= 1) {
         n_slabs = (n_chunks + seg_chunks - 1) / seg_chunks;
-        nparts = ctx->sm_count / n_slabs;
+        nparts = sms / n_slabs;
         if (nparts > n_kept_max / 16) nparts = n_kept_max / 16;     // at least one K-block of rows per part
         if (nparts < 1) nparts = 1;
         const long long tail = (long long)nparts * seg_chunks * 128 * 4;

@@ -704,9 +704,10 @@ __device__ __forceinline__ void select_fine_coarse(const uint16_t *__restrict__ 
                   [&](int col) { return rank_key<CA>(__ldcg(x + col), CA ? __ldcg(stamp + col) : 0, gamma); });
 }
 
-// The columns of a complete mask in shared memory as an ascending list.  A thread has a byte of the mask (d <= 8 *
-// TK_THREADS) or a word.  All threads call it; one barrier inside, none at the end.
-__device__ __forceinline__ void list_mask(const unsigned int *maskw, int d, TkShared &s, int32_t *idx_out)
+// put(rank, column) for the columns of a complete mask in shared memory, by ascending column; returns how many there are.
+// A thread has a byte of the mask (d <= 8 * TK_THREADS) or a word.  All threads call it; one barrier inside, none at the end.
+template <typename Put>
+__device__ __forceinline__ int list_mask(const unsigned int *maskw, int d, TkShared &s, const Put &put)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int span = d <= 8 * TK_THREADS ? 8 : 32;
@@ -722,7 +723,8 @@ __device__ __forceinline__ void list_mask(const unsigned int *maskw, int d, TkSh
     if (lane == 31) s.wb[warp] = incl;
     __syncthreads();
     int at = (int)__reduce_add_sync(0xffffffffu, lane < warp ? (unsigned)s.wb[lane] : 0u) + incl - c;
-    for (; m; m &= m - 1) idx_out[at++] = tid * span + __ffs(m) - 1;
+    for (; m; m &= m - 1, ++at) put(at, tid * span + __ffs(m) - 1);
+    return (int)__reduce_add_sync(0xffffffffu, (unsigned)s.wb[lane]);
 }
 
 }  // namespace

@@ -32,18 +32,23 @@ namespace {
 // stamp.  Needs d % 8 == 0 and d <= 8 * TK_COARSE_ITERS * TK_THREADS.
 // Dynamic shared memory: TkFine, then keys[] (d words rounded up to four).
 // idx_out != nullptr: the kept columns of row r as an ascending list at idx_out + r * k.
-// UPD: the CTA goes on to update the row's cache (one row; Algorithm 1 whole).  What bounds dip_ca_mask is the chain of
+// THEN (one row): THEN_UPDATE: the CTA goes on to update the row's cache (Algorithm 1 whole).  What bounds dip_ca_mask is the chain of
 // its launches (select, update and list were three), and the mask is here in shared memory: masks with lists and list
 // products at 2080 / 5472, four calls in a graph, 36.7 us with ten launches and 28.8 with four.
+// THEN_SPLIT: it goes on to part the mask into the tier's hits (columns in a slot, whose arena rows go to loc) and its misses (a
+// list; their arena rows are the staging rows, in order).
 // ---------------------------------------------------------------------------------------
-template <bool CA, bool NORM, bool UPD>
+constexpr int THEN_NOTHING = 0, THEN_UPDATE = 1, THEN_SPLIT = 2;
+template <int THEN> using ThenArg = std::conditional_t<THEN == THEN_UPDATE, dip_cache_update, std::conditional_t<THEN == THEN_SPLIT, dip_tier, Int<0>>>;
+
+template <bool CA, bool NORM, int THEN>
 __global__ void __launch_bounds__(TK_THREADS, 1)
 select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, float *__restrict__ x_out,
                    int d, int k, float gamma, const int32_t *stamp,
                    uint32_t *__restrict__ mask_bits, int32_t *__restrict__ idx_out,
-                   const std::conditional_t<UPD, dip_cache_update, Int<0>> u, unsigned long long *tr)
+                   const ThenArg<THEN> then, unsigned long long *tr)
 {
-    static_assert(!UPD || (CA && !NORM), "");
+    static_assert(THEN == THEN_NOTHING || (CA && !NORM), "");
     DIP_TRACE_MIN(tr, 0);
     extern __shared__ __align__(16) unsigned char dyn[];
     TkFine &f = *reinterpret_cast<TkFine *>(dyn);
@@ -76,10 +81,44 @@ select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, f
         select_fine<CA, NORM>(xa, NORM ? x_out : nullptr, d, k, gamma, stamp, scale, keys, s, f, s_maskw);
     }
     for (int w = tid; w < n_words; w += TK_THREADS) mask_bits[w] = s_maskw[w];
-    if (idx_out) list_mask(s_maskw, d, s, idx_out + (size_t)row * k);
-    if constexpr (UPD) {
+    if (idx_out) {
+        int32_t *o = idx_out + (size_t)row * k;
+        list_mask(s_maskw, d, s, [&](int r, int col) { o[r] = col; });
+    }
+    if constexpr (THEN == THEN_UPDATE) {
         cache_update_clear(s, f.hist);
-        block_cache_update_any(s_maskw, d, u.stamp, u.stamp, u.count, u.meta, u.capacity, s, f.hist, []() {}, []() { return true; });
+        block_cache_update_any(s_maskw, d, then.stamp, then.stamp, then.count, then.meta, then.capacity, s, f.hist, []() {},
+                               []() { return true; });
+    }
+    if constexpr (THEN == THEN_SPLIT) {
+        // a mask word per warp, a column per lane (d is a multiple of 32 here)
+        const int lane = tid & 31, warp = tid >> 5;
+        unsigned int *missw = f.hist;
+        constexpr int U = 8;                       // words whose loads go out together
+        for (int w0 = warp; w0 < n_words; w0 += U * TK_WARPS) {
+            int sl[U];
+#pragma unroll
+            for (int v = 0; v < U; ++v) sl[v] = w0 + v * TK_WARPS < n_words ? then.slot[(w0 + v * TK_WARPS) * 32 + lane] : -1;
+#pragma unroll
+            for (int v = 0; v < U; ++v) {
+                const int w = w0 + v * TK_WARPS;
+                if (w >= n_words) break;
+                const uint32_t m = s_maskw[w];
+                const bool hit = ((m >> lane) & 1u) && sl[v] >= 0 && sl[v] < then.capacity;   // (a slot outside the arena is none)
+                const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+                if (hit) then.loc[w * 32 + lane] = sl[v];
+                if (lane == 0) {
+                    then.split[w] = hits;
+                    then.split[n_words + w] = missw[w] = m & ~hits;
+                }
+            }
+        }
+        __syncthreads();
+        const int n = list_mask(missw, d, s, [&](int r, int col) {
+            then.fetch[4 + r] = col;
+            then.loc[col] = then.capacity + r;
+        });
+        if (tid == 0) then.fetch[0] = n;
     }
     DIP_TRACE_MAX(tr, 2);
 }
@@ -193,10 +232,10 @@ residual_rmsnorm_kernel(const float *x, const float *y, int d, float *x_next)
 // ---------------------------------------------------------------------------------------
 dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, float *x_out, int batch, int d, int k,
                              float gamma, const int32_t *stamp, uint32_t *mask_bits, cudaStream_t stream,
-                             const uint16_t *coarse, int32_t *idx_out, const dip_cache_update *update)
+                             const uint16_t *coarse, int32_t *idx_out, const dip_cache_update *update, const dip_tier *split)
 {
-    if ((idx_out || update) && (coarse || xb)) return DIP_ERR_INVALID_ARG;
-    if (update && (batch != 1 || !stamp)) return DIP_ERR_INVALID_ARG;
+    if ((idx_out || update || split) && (coarse || xb)) return DIP_ERR_INVALID_ARG;
+    if ((update || split) && (batch != 1 || !stamp)) return DIP_ERR_INVALID_ARG;
     const Int<0> no;
     const size_t smem = sizeof(TkFine) + (size_t)((d + 3) & ~3) * sizeof(uint32_t);
     const dim3 grid(batch), block(TK_THREADS);
@@ -212,20 +251,23 @@ dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, flo
                                (const int32_t *)nullptr, mask_bits, tr);
     } else if (xb) {
         if (stamp)
-            e = dip_launch_pdl(select_fine_kernel<true, true, false>, grid, block, smem, stream, xa, xb, x_out, d, k, gamma, stamp,
+            e = dip_launch_pdl(select_fine_kernel<true, true, THEN_NOTHING>, grid, block, smem, stream, xa, xb, x_out, d, k, gamma, stamp,
                                mask_bits, idx_out, no, tr);
         else
-            e = dip_launch_pdl(select_fine_kernel<false, true, false>, grid, block, smem, stream, xa, xb, x_out, d, k, 1.0f,
+            e = dip_launch_pdl(select_fine_kernel<false, true, THEN_NOTHING>, grid, block, smem, stream, xa, xb, x_out, d, k, 1.0f,
                                (const int32_t *)nullptr, mask_bits, idx_out, no, tr);
     } else {
         if (update)
-            e = dip_launch_pdl(select_fine_kernel<true, false, true>, grid, block, smem, stream, xa, (const float *)nullptr,
+            e = dip_launch_pdl(select_fine_kernel<true, false, THEN_UPDATE>, grid, block, smem, stream, xa, (const float *)nullptr,
                                (float *)nullptr, d, k, gamma, stamp, mask_bits, idx_out, *update, tr);
+        else if (split)
+            e = dip_launch_pdl(select_fine_kernel<true, false, THEN_SPLIT>, grid, block, smem, stream, xa, (const float *)nullptr,
+                               (float *)nullptr, d, k, gamma, stamp, mask_bits, idx_out, *split, tr);
         else if (stamp)
-            e = dip_launch_pdl(select_fine_kernel<true, false, false>, grid, block, smem, stream, xa, (const float *)nullptr,
+            e = dip_launch_pdl(select_fine_kernel<true, false, THEN_NOTHING>, grid, block, smem, stream, xa, (const float *)nullptr,
                                (float *)nullptr, d, k, gamma, stamp, mask_bits, idx_out, no, tr);
         else
-            e = dip_launch_pdl(select_fine_kernel<false, false, false>, grid, block, smem, stream, xa, (const float *)nullptr,
+            e = dip_launch_pdl(select_fine_kernel<false, false, THEN_NOTHING>, grid, block, smem, stream, xa, (const float *)nullptr,
                                (float *)nullptr, d, k, 1.0f, (const int32_t *)nullptr, mask_bits, idx_out, no, tr);
     }
     DIP_CUDA_TRY(ctx, e);
@@ -244,11 +286,12 @@ dip_status dip_init_mask_kernels(dip_ctx *ctx)
 {
     const int bytes = DIP_MAX_D * (int)sizeof(uint32_t);
     const int fine_bytes = bytes + (int)sizeof(TkFine);
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false, THEN_UPDATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false, THEN_SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false, THEN_NOTHING>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<false, false, THEN_NOTHING>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, true, THEN_NOTHING>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<false, true, THEN_NOTHING>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
     DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_coarse_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
     DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_coarse_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
     return DIP_OK;

@@ -1,0 +1,60 @@
+"""The two-tier product at the edges of its plan: parts of more rows than one list, as many parts as SMs, rows of one segment and of a
+ragged one, budgets of nothing and of everything, and a tier whose slots lie outside its arena."""
+import numpy as np
+import pytest
+import torch
+
+import dip_inputs as di
+import oracle
+from gpu_util import check_step, upload_layer
+from test_gpu_tiered import _check_tier, _layer, _tiers
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("wtype,d_model,d_ff,k_x,k_h,beta,steps", [
+    (di.W_BF16, 4160, 9504, 4160, 9504, 0.5, 2),      # 75 segments, one part: 4160 misses, then hits and misses, in lists of 2048
+    (di.W_BF16, 256, 8224, 200, 5000, 0.5, 4),        # down rows of one segment: a part per SM
+    (di.W_F32, 96, 1056, 1, 33, 0.4, 4),              # ragged segments, one row
+    (di.W_BF16, 288, 1056, 96, 400, 0.0, 3),          # nothing cached: every column a miss
+    (di.W_BF16, 288, 1056, 96, 400, 1.0, 4),          # everything fits: hits only, after a while
+    (di.W_INT4_G128, 384, 1152, 100, 500, 0.5, 4),    # (fetched by a launch of its own)
+])
+def test_tiers_of_every_plan(wtype, d_model, d_ff, k_x, k_h, beta, steps):
+    import paper_2412_01380_b200 as dip
+    ctx = dip.Context(0)
+    lw = _layer(d_ff, d_model, d_ff, wtype)
+    w = upload_layer(dip, ctx, lw)
+    gate_up, down = w.gate_up.clone(), w.down.clone()
+    g_gu, g_d, t_gu, t_d = _tiers(dip, w, k_x, k_h, beta, "lru", True)
+    ref_gu, ref_d = oracle.Cache(d_model, g_gu.capacity, "lru"), oracle.Cache(d_ff, g_d.capacity, "lru")
+    w.struct.gate_up = w.struct.down = None
+    for x in di.token_inputs(di.WORKLOADS["phi3_mini"].scaled(seed=d_ff + 1), n_tokens=steps, batch=1, d=d_model)[:, 0]:
+        check_step(dip, ctx, lw, w, x, k_x, k_h, 0.2, ref_gu, ref_d, g_gu, g_d, tiers=(t_gu, t_d))
+        for t, packed, ref in ((t_gu, gate_up, ref_gu), (t_d, down, ref_d)):
+            _check_tier(t, packed, ref, int(ref.counters[1]))
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
+def test_slots_outside_the_arena_are_reported_and_not_read():
+    import paper_2412_01380_b200 as dip
+    d_model, d_ff, k_x, k_h = 512, 1024, 128, 256
+    ctx = dip.Context(0)
+    lw = _layer(9, d_model, d_ff, di.W_BF16)
+    w = upload_layer(dip, ctx, lw)
+    g_gu, g_d, t_gu, t_d = _tiers(dip, w, k_x, k_h, 0.5, "lru", False)
+    stamp = np.full(d_model, -1, dtype=np.int32)
+    stamp[: g_gu.capacity] = 0
+    g_gu.load(stamp, g_gu.capacity, 1)
+    t_gu.slot[: g_gu.capacity] = 1 << 20
+    x = torch.from_numpy(di.token_inputs(di.WORKLOADS["phi3_mini"].scaled(seed=3), 1, 1, d_model)[0, 0]).cuda()
+    h = torch.empty(d_ff, device="cuda")
+    dip.dip_mlp_step_tiered(ctx, w, t_gu, t_d, x, k_x, k_h, 0.2, torch.empty(d_model, device="cuda"), h=h)
+    assert ctx.device_status() == 2 and int(t_gu.fetch[1]) == 0
+    want = torch.empty(d_ff, device="cuda")
+    c2 = dip.CacheState(d_model, g_gu.capacity, "cuda")
+    c2.load(stamp, g_gu.capacity, 1)
+    dip.dip_mlp_step(ctx, w, x, k_x, k_h, 0.2, c2, None, torch.empty(d_model, device="cuda"), h=want)
+    assert torch.allclose(h, want, rtol=1e-4, atol=1e-5 * float(want.abs().max()))    # its columns came from the slow tier
+    ctx.close()
