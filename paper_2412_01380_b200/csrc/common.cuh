@@ -13,7 +13,7 @@ constexpr int DIP_RING_LAYERS = 128;
 constexpr int DIP_TRACE_SLOTS = 1024;
 constexpr uint32_t DIP_MAIL_EMPTY = 0xffffffffu;
 constexpr int DIP_SYNC_WORDS = 3;
-constexpr int DIP_MAIL_FLOATS = 2048;  // boxes per SM: one CTA's segment of sums (INT4: up to 2048, F32 / BF16: 256)
+constexpr int DIP_MAIL_FLOATS = 4096;  // boxes per SM: one CTA's segment of sums (INT4: up to 2048, F32 / BF16: 256 per token)
 constexpr int DIP_TRACE_WORDS = 4;   // first start, dependency ready, last end, auxiliary
 
 // Scratch workspace of a context.  All device memory the library itself owns.
@@ -29,9 +29,9 @@ struct dip_ctx {
     // split-row partial sums of the two GEMVs (binary32)
     float *partials;
     size_t partials_floats;
-    float *mail;         // [sm_count][DIP_MAIL_FLOATS] row parts of one- and two-token products on their way to the CTA that adds them up
+    float *mail;         // [sm_count][DIP_MAIL_FLOATS] row parts on their way to the CTA that adds them up
     unsigned int *readers; // [DIP_SYNC_WORDS] zero between launches: CTAs of a fused product that have read the stamps; in a
-                           // two-tier launch: the moves are known, CTAs that are through
+                           // two-tier or tensor-core launch: what other CTAs wait for is there, CTAs that have seen it
     // one arrival counter per output slab; zero between launches
     unsigned int *tickets;
     int n_tickets;
@@ -51,7 +51,7 @@ struct dip_ctx {
     uint32_t *mask_ring; // [2][DIP_RING_LAYERS][max_d/32] per-layer mask slots of the stack runner
     uint32_t *mask_tmp;  // [max_d/32] list-based GEMV entry points
     uint16_t *coarse;    // [max_batch][max_d] top 16 bits of the rank keys of h, left by the gate/up product
-    uint16_t *xt;        // [max_d][32] batched decode: per row of the union, the tokens' values as bfloat16 (16 high, 16 low halves)
+    uint16_t *xt;        // [max_d][32] batched decode: per column, the tokens' values as bfloat16 (16 high, 16 low halves)
     int coarse_min_d;    // smallest d_ff for which the step ranks h from those
     int *status;         // sticky device status word (0 = fine)
     int fuse_select;     // single-token F32 / BF16 steps: the products build their own masks

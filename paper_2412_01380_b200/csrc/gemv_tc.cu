@@ -8,18 +8,19 @@
 //     into shared memory in the layout that a 128-byte-swizzled
 //     MN-major operand descriptor names: the outputs of a row are contiguous, so the weights are the
 //     B operand (N = 256) as they arrive, untransposed, and each byte is read by one MMA only;
-//   * the tokens' values of the union's rows, zeroed where a token drops the row and split into two
-//     bfloat16, are gathered ONCE per product by xt_build_kernel (16 scattered loads per row), 64
-//     bytes per column of the union; the loaders copy them as the MN-major A operand: row n = the
-//     high halves of token n, row 16 + n the low halves, the other rows of the M = 128 tile zero;
+//   * the tokens' values of all columns, zeroed where a token drops the column and split into two bfloat16, are gathered
+//     ONCE per product into a table of 64 bytes per column: each block makes its share while its first rows are on their way (a
+//     launch of its own in front took 2.5 us).  The loaders copy a row's 64 bytes as the MN-major A operand: row n = the high
+//     halves of token n, row 16 + n the low halves, the other rows of the M = 128 tile zero.  (Every CTA gathering its rows'
+//     values for itself, four bytes at a time, is what the load path cannot take: 16 tokens' gate/up product 86 us
+//     with registers and warps of their own, 105 us with asynchronous copies of four bytes, 60 us like this);
 //   * one thread of a seventeenth warp issues one tcgen05.mma (M = 128, N = 256, K = 16) per 16 rows
 //     once the loader warps have arrived on the buffer's "full" barrier; the accumulator lives in
 //     tensor memory (256 columns) for the whole kernel, and a tcgen05.commit per round tells the
 //     loaders through a second mbarrier when a buffer may be overwritten;
-//   * the epilogue (one warp: the 32 useful accumulator rows are its 32 lanes) reads 16 columns at a
-//     time with tcgen05.ld, adds the low-half row to the high-half row, and either applies
-//     silu(gate) * up (a 16-column chunk is 8 gate outputs and their 8 up outputs; gate/up rows have
-//     enough segments for one CTA to see all rows) or leaves the row part for combine_parts_kernel.
+//   * four warps read the 32 useful accumulator rows with tcgen05.ld, add the low-half row to the high-half row and leave the
+//     sums in shared memory; then all threads apply silu(gate) * up (a 16-column chunk is 8 gate outputs and
+//     their 8 up outputs), or send the row part to the last part's CTA, which adds the parts up first.
 // All products are exact in binary32 (bf16 x bf16); sums are binary32 in the tensor core's order.
 // Every wait on an mbarrier is bounded; on expiry the kernel records a status word, frees its
 // tensor memory and leaves.
@@ -30,8 +31,9 @@
 
 namespace {
 
-constexpr int TC_LOAD_WARPS = 16;                // warps that stream rows; one more warp issues the MMAs
-constexpr int TC_THREADS = (TC_LOAD_WARPS + 1) * 32;
+constexpr int TC_LOAD_WARPS = 16;                // warps that stream rows, and one that issues the MMAs
+constexpr int TC_WARPS = TC_LOAD_WARPS + 1;
+constexpr int TC_THREADS = TC_WARPS * 32;
 constexpr int TC_U = 4;                          // rows per lane and round
 constexpr int TC_ROUND_ROWS = TC_LOAD_WARPS * TC_U;   // 64 rows = 4 K-blocks of 16 per round
 constexpr int TC_KB = TC_ROUND_ROWS / 16;
@@ -46,6 +48,11 @@ constexpr int TC_TMEM_COLS = 256;                // one accumulator: 128 lanes x
 // (16 tokens at keep ratio 0.25 keep ~5100 of 5120 gate/up rows, ~2500 down rows per part).
 constexpr int TC_LIST_ROWS = 8192;
 
+constexpr int TC_BUILD_WORDS = 4;              // words whose loads go out together
+constexpr int TC_BUILD_ROW = 17;               // 4-byte words
+constexpr size_t TC_BUILD_SMEM = (size_t)TC_BUILD_WORDS * 32 * TC_BUILD_ROW * 4;
+constexpr unsigned long long TC_TABLE_WAIT_NS = 100000ull;   // for the other blocks' shares
+
 struct __align__(1024) TcSmem {
     unsigned char a[TC_BUFS][TC_KB * TC_A_KB_BYTES];   // weights, 4 x 32 KB
     unsigned char b[TC_BUFS][TC_KB * TC_B_KB_BYTES];   // token values, 4 x 16 KB
@@ -54,7 +61,9 @@ struct __align__(1024) TcSmem {
     uint32_t tmem_base;
     int n_total;
     int fail;
-    int wsum[GV_SCAN_THREADS / 32];
+    int table;                                   // all blocks have written their shares of the table
+    uint32_t build[TC_BUILD_SMEM / 4];
+    int wsum[TC_WARPS];
     uint32_t words[DIP_MAX_D / 32];
     int pre[DIP_MAX_D / 32];
     uint16_t idx[TC_LIST_ROWS];
@@ -102,47 +111,63 @@ __device__ __forceinline__ void tc_ld64(uint32_t taddr, float (&v)[64])
     for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-}  // namespace
+struct TcParams {
+    int n_slabs, nparts;
+    uint16_t *xt;              // [d_in][32] the table: 16 high, 16 low halves
+    unsigned int *ready;       // blocks whose share of it is written; zero between launches
+    unsigned int *through;     // blocks that need it no more; zero between launches
+    unsigned long long block_wait_ns;
+};
 
-namespace {
-
-// The tokens' values of every column of the union, ready for the tensor core: xt[i][n] = bfloat16 high
-// half of token n's value at column i (zero where the token's own mask drops the column or
-// n >= batch), xt[i][16 + n] = the low half; columns outside the union are not written (and never
-// read).  Built once per product instead of once per CTA (the values are 16 scattered 4-byte loads
-// per column).  A block takes two mask words per pass; 16 consecutive threads are the 16 tokens of
-// one column.
-__global__ void __launch_bounds__(1024, 1)
-xt_build_kernel(const uint32_t *__restrict__ mask_bits, const float *__restrict__ v, int batch, int d_in, int mask_words,
-                uint16_t *__restrict__ xt)
+// The table's columns of the mask words first, first + step, ...: warp n < 16 takes token n's, a column per lane, and a tile in
+// shared memory (rows of 64 bytes, 68 apart: no bank conflicts) turns them round.  The TC_LOAD_WARPS warps call it.
+__device__ __forceinline__ void xt_build(const GemvParams &p, uint16_t *xt, int first, int step, uint32_t *buf)
 {
-    const int tid = threadIdx.x;
-    const int n = tid & 15, bit = (tid >> 4) & 31, half = tid >> 9;
-    dip_grid_dependency_wait();
-    dip_launch_dependents();
-    for (int w = 2 * blockIdx.x + half; w < mask_words; w += 2 * gridDim.x) {
-        const int idx = w * 32 + bit;
-        const bool mine = n < batch && idx < d_in && ((mask_bits[(size_t)n * mask_words + w] >> bit) & 1u);
-        // in the union if any of the 16 tokens (a half-warp) keeps the column
-        const unsigned any = __ballot_sync(0xffffffffu, mine) & (0xffffu << (tid & 16));
-        if (!any) continue;
-        const float x = mine ? __ldg(v + (size_t)n * d_in + idx) : 0.f;
-        const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(x - __bfloat162float(hi));
-        xt[(size_t)idx * 32 + n] = __bfloat16_as_ushort(hi);
-        xt[(size_t)idx * 32 + 16 + n] = __bfloat16_as_ushort(lo);
+    constexpr int T = TC_LOAD_WARPS * 32;
+    static_assert(TC_LOAD_WARPS == TC_N, "a warp per token");
+    const int tid = threadIdx.x, lane = tid & 31, n = tid >> 5;
+    for (int w0 = first; w0 < p.mask_words; w0 += TC_BUILD_WORDS * step) {
+        float x[TC_BUILD_WORDS];
+        uint32_t m[TC_BUILD_WORDS];
+#pragma unroll
+        for (int u = 0; u < TC_BUILD_WORDS; ++u) {
+            const int w = w0 + u * step;
+            x[u] = 0.f;
+            m[u] = 0u;
+            if (n < p.batch && w < p.mask_words) {
+                m[u] = __ldg(p.mask_bits + (size_t)n * p.mask_words + w);
+                if (w * 32 + lane < p.d_in) x[u] = __ldg(p.v + (size_t)n * p.d_in + w * 32 + lane);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < TC_BUILD_WORDS; ++u) {
+            const float v = (m[u] >> lane) & 1u ? x[u] : 0.f;
+            const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+            const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
+            __nv_bfloat16 *row = reinterpret_cast<__nv_bfloat16 *>(buf + (u * 32 + lane) * TC_BUILD_ROW);
+            row[n] = hi;
+            row[16 + n] = lo;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory");
+        for (int i = tid; i < TC_BUILD_WORDS * 128; i += T) {
+            const int w = w0 + (i >> 7) * step, col = w * 32 + ((i & 127) >> 2);
+            const uint32_t *at = buf + (i >> 2) * TC_BUILD_ROW + 4 * (i & 3);
+            if (w < p.mask_words && col < p.d_in) reinterpret_cast<uint4 *>(xt)[(size_t)col * 4 + (i & 3)] = make_uint4(at[0], at[1], at[2], at[3]);
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory");
     }
 }
 
 template <int WHICH>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-gemv_tc_kernel(const GemvParams p, const uint16_t *__restrict__ xt)
+gemv_tc_kernel(const GemvParams p, const TcParams q)
 {
     extern __shared__ unsigned char tc_smem_raw[];
     TcSmem &s = *reinterpret_cast<TcSmem *>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
     DIP_TRACE_MIN(p.tr, 0);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int slab = blockIdx.x, part = blockIdx.y, nparts = gridDim.y;
+    const int block = blockIdx.x;
+    const int slab = block % q.n_slabs, part = block / q.n_slabs, nparts = q.nparts;
     const size_t byte_off = (size_t)slab * TC_SEG + lane * 16;
     const bool lane_ok = byte_off < p.row_bytes;
 
@@ -164,22 +189,26 @@ gemv_tc_kernel(const GemvParams p, const uint16_t *__restrict__ xt)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = s.tmem_base;
+    // the rows of the M = 128 tile that no token uses stay zero
+    for (int i = tid; i < (int)(sizeof(s.b) / 16); i += TC_THREADS) reinterpret_cast<uint4 *>(&s.b[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // (the block barriers below order them before any MMA)
     dip_grid_dependency_wait();        // the masks and the vectors come from the previous kernels
     DIP_TRACE_MIN(p.tr, 1);
     dip_launch_dependents();
 
-    // ---- 1. the union of the tokens' mask words and its popcount prefix ----
-    if (tid < GV_SCAN_THREADS) {
-        uint32_t u[4] = {0u, 0u, 0u, 0u};
-        int c = 0;
+    // ---- 1. the union of the tokens' mask words (two neighbours per thread) and its popcount prefix ----
+    {
+        static_assert(2 * TC_THREADS >= DIP_MAX_D / 32, "");
+        uint32_t u[2] = {0u, 0u};
+#pragma unroll 4
+        for (int b = 0; b < p.batch; ++b)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int w = 4 * tid + j;
-            if (w < p.mask_words)
-                for (int b = 0; b < p.batch; ++b) u[j] |= p.mask_bits[(size_t)b * p.mask_words + w];
-            if (w == p.mask_words - 1 && (p.d_in & 31)) u[j] &= (1u << (p.d_in & 31)) - 1u;
-            c += __popc(u[j]);
-        }
+            for (int j = 0; j < 2; ++j)
+                if (2 * tid + j < p.mask_words) u[j] |= __ldg(p.mask_bits + (size_t)b * p.mask_words + 2 * tid + j);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (2 * tid + j == p.mask_words - 1 && (p.d_in & 31)) u[j] &= (1u << (p.d_in & 31)) - 1u;
+        const int c = __popc(u[0]) + __popc(u[1]);
         int incl = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -187,21 +216,18 @@ gemv_tc_kernel(const GemvParams p, const uint16_t *__restrict__ xt)
             if (lane >= o) incl += n;
         }
         if (lane == 31) s.wsum[warp] = incl;
-        asm volatile("bar.sync 1, %0;" ::"n"(GV_SCAN_THREADS) : "memory");
-        int before = 0;
+        __syncthreads();
+        int pre = (int)__reduce_add_sync(0xffffffffu, lane < warp ? (unsigned)s.wsum[lane] : 0u) + incl - c;
 #pragma unroll
-        for (int w = 0; w < GV_SCAN_THREADS / 32; ++w) before += w < warp ? s.wsum[w] : 0;
-        int pre = before + incl - c;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int w = 4 * tid + j;
+        for (int j = 0; j < 2; ++j) {
+            const int w = 2 * tid + j;
             if (w < p.mask_words) {
                 s.words[w] = u[j];
                 s.pre[w] = pre;
             }
             pre += __popc(u[j]);
         }
-        if (tid == GV_SCAN_THREADS - 1) s.n_total = pre;
+        if (tid == TC_THREADS - 1) s.n_total = pre;
     }
     __syncthreads();
     const int n_total = s.n_total;
@@ -209,18 +235,36 @@ gemv_tc_kernel(const GemvParams p, const uint16_t *__restrict__ xt)
     const int r_end = (int)(((long long)(part + 1) * n_total) / nparts);
     const char *base = p.W + byte_off;
 
-    // this thread's places in a round: as a loader (warps 0-15), row slot k = warp of K-block u,
-    // 16-byte chunk `lane` of the segment; as a builder of B, row tid / 4 and tokens 4 (tid % 4) .. + 3
+    // this lane's place in a round of weights: row slot k = warp of K-block u, 16-byte chunk `lane` of the segment
     const uint32_t a_off = (uint32_t)(((warp & 15) >> 3) * 4096 + (lane >> 3) * 1024 + (warp & 7) * 128 + (((lane & 7) ^ (warp & 7)) << 4));
-    // as a mover of the values: row tid / 4 of the round, 16-byte chunk tid % 4 of its 64 bytes in xt
+    // and, of threads 0 .. 4 TC_ROUND_ROWS - 1, of values: row tid / 4 of the round, 16-byte chunk tid % 4 of its 64 bytes in xt
     // (the high halves of tokens 0-7, 8-15, the low halves of tokens 0-7, 8-15) = A rows 8 (tid % 4) .. + 7
     // at that k: core matrices of 8 k x 16 bytes, the 16 row groups 128 B apart, the two k groups 2 KB apart
-    const int bb_row = (tid >> 2) & (TC_ROUND_ROWS - 1), bb_mg = tid & 3;   // (threads 0 .. 4 TC_ROUND_ROWS - 1)
+    const int bb_row = (tid >> 2) & (TC_ROUND_ROWS - 1), bb_mg = tid & 3;
     const uint32_t b_off = (uint32_t)((bb_row >> 4) * TC_B_KB_BYTES + ((bb_row & 15) >> 3) * 2048 + bb_mg * 128 + (bb_row & 7) * 16);
-    // the rows of the M = 128 tile that no token uses stay zero
-    for (int i = tid; i < (int)(sizeof(s.b) / 16); i += TC_THREADS) reinterpret_cast<uint4 *>(&s.b[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // (the block barriers below order them before any MMA)
 
+    // This block's share of the table, and a wait for the others' (warps 0 - 15).  Blocks wait for one another here without any
+    // order among them, and nothing promises that they all run at the same time: one that has waited long enough makes the
+    // whole table by itself (the same bytes as whoever else writes them).
+    auto make_table = [&]() {
+        const unsigned int n_blocks = q.n_slabs * nparts;
+        xt_build(p, q.xt, block, n_blocks, s.build);
+        if (tid == 0) {
+            __threadfence();
+            count_one(q.ready);
+            unsigned int n = 0u;
+            const unsigned long long t0 = dip_gtime();
+            do asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(q.ready) : "memory");
+            while (n < n_blocks && dip_gtime() - t0 < TC_TABLE_WAIT_NS);
+            s.table = n >= n_blocks;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(TC_LOAD_WARPS * 32) : "memory");
+        if (!s.table) {
+            xt_build(p, q.xt, 0, 1, s.build);
+            __threadfence();
+            asm volatile("bar.sync 1, %0;" ::"n"(TC_LOAD_WARPS * 32) : "memory");
+        }
+    };
     int g = 0;                         // rounds so far (buffer g & 1)
     bool failed = false;
 
@@ -231,65 +275,67 @@ gemv_tc_kernel(const GemvParams p, const uint16_t *__restrict__ xt)
         if (list_begin != r_begin) __syncthreads();               // everyone is done with the previous list
         {
             const int lo_rank = list_begin, hi_rank = list_begin + n_rows;
-            for (int w = tid; w < p.mask_words; w += TC_THREADS) {
-                uint32_t u = s.words[w];
-                int rank = s.pre[w];
+            for (int b = tid; b < 4 * p.mask_words; b += TC_THREADS) {        // a byte of a word
+                const int w = b >> 2, low = 8 * (b & 3);
+                const uint32_t all = s.words[w];
+                uint32_t u = all & (0xffu << low);
+                int rank = s.pre[w] + __popc(all & ((1u << low) - 1u));
                 if (rank >= hi_rank || rank + __popc(u) <= lo_rank) continue;
-                while (u) {
-                    const int bit = __ffs(u) - 1;
-                    u &= u - 1;
-                    if (rank >= lo_rank && rank < hi_rank) s.idx[rank - lo_rank] = (uint16_t)(w * 32 + bit);
-                    ++rank;
-                }
+                for (; u; u &= u - 1, ++rank)
+                    if (rank >= lo_rank && rank < hi_rank) s.idx[rank - lo_rank] = (uint16_t)(w * 32 + __ffs(u) - 1);
             }
         }
         __syncthreads();
         const int n_rounds = (n_rows + TC_ROUND_ROWS - 1) / TC_ROUND_ROWS;
 
         if (warp < TC_LOAD_WARPS) {
-            // copies of one round, global -> shared memory, 16 bytes each (zero-filled past the end of the
-            // list): this lane's piece of rows warp, warp + 16, ... and (threads 0-255) this thread's 16
-            // bytes of the tokens' values of row tid / 4; one copy group per round
-            auto copy_round = [&](int mr) {
+            // copies of one round, global -> shared memory, 16 bytes each (zero-filled past the end of the list): this lane's
+            // piece of rows warp, warp + 16, ... and (threads 0-255) this thread's 16 bytes of the tokens' values of row tid / 4
+            auto copy_weights = [&](int mr) {
                 const int gr = g + mr;                                      // round number over the whole kernel
-                if (mr < n_rounds) {
-                    // the MMAs that read this ring slot four rounds ago must be through
-                    if (gr >= TC_BUFS && !failed) {
-                        if (s.fail || !mbar_wait(&s.done[gr % TC_BUFS], ((gr / TC_BUFS) - 1) & 1, p.wait_limit_ns)) failed = true;
-                    }
-                    const uint32_t ab = smem_u32(s.a[gr % TC_BUFS]) + a_off, bb = smem_u32(s.b[gr % TC_BUFS]) + b_off;
+                if (mr >= n_rounds) return;
+                // the MMAs that read this ring slot four rounds ago must be through
+                if (gr >= TC_BUFS && !failed) {
+                    if (s.fail || !mbar_wait(&s.done[gr % TC_BUFS], ((gr / TC_BUFS) - 1) & 1, p.wait_limit_ns)) failed = true;
+                }
+                const uint32_t ab = smem_u32(s.a[gr % TC_BUFS]) + a_off;
 #pragma unroll
-                    for (int u = 0; u < TC_U; ++u) {
-                        const int r = mr * TC_ROUND_ROWS + warp + u * TC_LOAD_WARPS;
-                        const bool ok = r < n_rows && lane_ok;
-                        const char *src = ok ? base + (size_t)s.idx[r] * p.row_bytes : p.W;
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ab + u * TC_A_KB_BYTES), "l"(src),
-                                     "r"(ok ? 16 : 0) : "memory");
-                    }
-                    if (tid < TC_ROUND_ROWS * 4) {
-                        const int r = mr * TC_ROUND_ROWS + bb_row;
-                        const bool ok = r < n_rows;
-                        const uint16_t *src = ok ? xt + (size_t)s.idx[r] * 32 + bb_mg * 8 : xt;
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(bb), "l"(src), "r"(ok ? 16 : 0) : "memory");
-                    }
+                for (int u = 0; u < TC_U; ++u) {
+                    const int r = mr * TC_ROUND_ROWS + warp + u * TC_LOAD_WARPS;
+                    const bool ok = r < n_rows && lane_ok;
+                    const char *src = ok ? base + (size_t)s.idx[r] * p.row_bytes : p.W;
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ab + u * TC_A_KB_BYTES), "l"(src),
+                                 "r"(ok ? 16 : 0) : "memory");
+                }
+            };
+            auto copy_values = [&](int mr) {
+                if (mr < n_rounds && tid < TC_ROUND_ROWS * 4) {
+                    const int r = mr * TC_ROUND_ROWS + bb_row;
+                    const bool ok = r < n_rows;
+                    const uint16_t *src = ok ? q.xt + (size_t)s.idx[r] * 32 + bb_mg * 8 : q.xt;
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(s.b[(g + mr) % TC_BUFS]) + b_off), "l"(src),
+                                 "r"(ok ? 16 : 0) : "memory");
                 }
                 asm volatile("cp.async.commit_group;" ::: "memory");           // (an empty group past the last round)
             };
 #pragma unroll
-            for (int mr = 0; mr < TC_BUFS - 1; ++mr) copy_round(mr);
+            for (int mr = 0; mr < TC_BUFS - 1; ++mr) copy_weights(mr);
+            if (list_begin == r_begin) make_table();
+#pragma unroll
+            for (int mr = 0; mr < TC_BUFS - 1; ++mr) copy_values(mr);
             for (int mr = 0; mr < n_rounds; ++mr) {
-                const int gg = g + mr;
                 // this thread's copies of round mr have landed (the two younger groups may be in flight)
                 asm volatile("cp.async.wait_group %0;" ::"n"(TC_BUFS - 2) : "memory");
                 // -> visible to the tensor core's (async proxy) reads
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&s.full[gg % TC_BUFS]);
-                copy_round(mr + TC_BUFS - 1);
+                if (lane == 0) mbar_arrive(&s.full[(g + mr) % TC_BUFS]);
+                copy_weights(mr + TC_BUFS - 1);
+                copy_values(mr + TC_BUFS - 1);
             }
             asm volatile("cp.async.wait_group 0;" ::: "memory");              // (only empty groups are left)
         } else if (lane == 0) {
-            // the MMA thread: per round, wait for the 16 loader warps, then two tiles x (hi, lo) per K-block
+            // the MMA thread: per round, wait for the 16 loader warps, then one MMA per K-block
             for (int mr = 0; mr < n_rounds; ++mr) {
                 const int gg = g + mr, buf = gg % TC_BUFS;
                 if (failed) break;
@@ -317,6 +363,16 @@ gemv_tc_kernel(const GemvParams p, const uint16_t *__restrict__ xt)
     if (failed) s.fail = 1;
     __syncthreads();
     failed = s.fail != 0;
+    // (a block without rows has not been there)
+    if (r_begin == r_end && warp < TC_LOAD_WARPS) make_table();
+    // the last block that needs the table no more makes the words ready for the next launch
+    if (tid == 0) {
+        __threadfence();
+        if (atomicAdd(q.through, 1u) == (unsigned)(q.n_slabs * nparts) - 1u) {
+            *q.ready = 0u;
+            *q.through = 0u;
+        }
+    }
 
     // ---- the last round's commit covers every MMA of the kernel ----
     if (g > 0 && !failed) {
@@ -325,11 +381,13 @@ gemv_tc_kernel(const GemvParams p, const uint16_t *__restrict__ xt)
     if (failed && lane == 0) atomicExch(p.status, 1);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-    // ---- epilogue: the useful accumulator rows 0-31 are tensor-memory lanes 0-31, which the warps 0, 4, 8
-    //      and 12 reach (a warp reads the lane quarter warp % 4): token n's high-half sums in lane n, the
-    //      low-half sums in lane 16 + n; 16 columns = 16 packed outputs at a time, four such chunks per warp ----
+    // ---- the useful accumulator rows 0-31 are tensor-memory lanes 0-31, which the warps 0, 4, 8 and 12 reach (a warp reads
+    //      the lane quarter warp % 4): token n's high-half sums in lane n, the low-half sums in lane 16 + n.  64 packed outputs per
+    //      warp, over the ring's first buffer ----
+    constexpr int ROW = 256 + 4;
+    float *sums = reinterpret_cast<float *>(&s.a[0][0]);           // [token][ROW]
     if ((warp & 3) == 0 && warp < 16) {
-        const int n = lane & 15, c0 = warp;                        // this warp's columns: 16 c0 .. 16 c0 + 63 (c0 = 0, 4, 8, 12)
+        const int c0 = warp;                                       // this warp's columns: 16 c0 .. 16 c0 + 63 (c0 = 0, 4, 8, 12)
         float v[64];
         if (g > 0 && !failed) {
             tc_ld64(tmem + 16 * c0, v);
@@ -339,61 +397,57 @@ gemv_tc_kernel(const GemvParams p, const uint16_t *__restrict__ xt)
         }
 #pragma unroll
         for (int i = 0; i < 64; ++i) v[i] += __shfl_down_sync(0xffffffffu, v[i], 16);       // + the low halves' sums
-        if (lane < TC_N) {
-            if (nparts > 1 || p.defer) {
-                // row parts: [part][segment][token][256 packed elements], added up by combine_parts_kernel
-                float *dst = p.partials + ((size_t)(p.part_base + part) * gridDim.x + slab) * (TC_N * 256) + n * 256 + 16 * c0;
+        if (lane < p.batch) {
 #pragma unroll
-                for (int i = 0; i < 64; i += 4)
-                    *reinterpret_cast<float4 *>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-            } else if (n < p.batch) {
-                if (WHICH == 0) {
-                    // every 16 columns: 8 gate outputs followed by their 8 up outputs
-                    const int j = slab * 128 + c0 * 8;
-                    float *dst = p.out + (size_t)n * p.d_out + j;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        float h[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) h[i] = silu_f32(v[16 * c + i]) * v[16 * c + 8 + i];
-                        if (j + 8 * c + 8 <= p.d_out) {
-                            *reinterpret_cast<float4 *>(dst + 8 * c) = make_float4(h[0], h[1], h[2], h[3]);
-                            *reinterpret_cast<float4 *>(dst + 8 * c + 4) = make_float4(h[4], h[5], h[6], h[7]);
-                            if (p.key_coarse) {
-                                // top 16 bits of the rank keys |h_j| for the select that follows (no cache with several tokens)
-                                uint32_t kk[4];
-#pragma unroll
-                                for (int i = 0; i < 4; ++i)
-                                    kk[i] = ((__float_as_uint(h[2 * i]) & 0x7fffffffu) >> 16) |
-                                            ((__float_as_uint(h[2 * i + 1]) & 0x7fffffffu) & 0xffff0000u);
-                                *reinterpret_cast<uint4 *>(p.key_coarse + (size_t)n * p.d_out + j + 8 * c) = make_uint4(kk[0], kk[1], kk[2], kk[3]);
-                            }
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 8; ++i)
-                                if (j + 8 * c + i < p.d_out) dst[8 * c + i] = h[i];
-                        }
-                    }
-                } else {
-                    const int j = slab * 256 + 16 * c0;
-                    float *dst = p.out + (size_t)n * p.d_out + j;
-#pragma unroll
-                    for (int i = 0; i < 64; i += 4) {
-                        if (j + i + 4 <= p.d_out) {
-                            *reinterpret_cast<float4 *>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                if (j + i + e < p.d_out) dst[i + e] = v[i + e];
-                        }
-                    }
-                }
-            }
+            for (int i = 0; i < 64; i += 4)
+                *reinterpret_cast<float4 *>(sums + lane * ROW + 16 * c0 + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
         }
     }
-    // ---- free the tensor memory ----
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    // ---- row parts: to the last part's CTA, which adds them up in part order (see gemv_fused.cu) ----
+    const size_t stride = (size_t)q.n_slabs * p.batch * 256;
+    float *box = p.mail + (size_t)slab * p.batch * 256;
+    if (part != nparts - 1) {
+        for (int e = tid; e < p.batch * 64; e += TC_THREADS)
+            mail_put4(box + (size_t)part * stride + 4 * e, *reinterpret_cast<const float4 *>(sums + (e >> 6) * ROW + 4 * (e & 63)));
+    } else {
+        if (nparts > 1) {
+            for (int e = tid; e < p.batch * 64; e += TC_THREADS) {
+                float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int b0 = 0; b0 < nparts - 1; b0 += MAIL_N) {
+                    float4 a[MAIL_N];
+                    mail_take4<MAIL_N>(box + (size_t)b0 * stride + 4 * e, stride, nparts - 1 - b0, a, p.status, q.block_wait_ns);
+#pragma unroll
+                    for (int b = 0; b < MAIL_N; ++b) { t.x += a[b].x; t.y += a[b].y; t.z += a[b].z; t.w += a[b].w; }
+                }
+                float4 &mine = *reinterpret_cast<float4 *>(sums + (e >> 6) * ROW + 4 * (e & 63));
+                mine = make_float4(t.x + mine.x, t.y + mine.y, t.z + mine.z, t.w + mine.w);
+            }
+            __syncthreads();
+        }
+        // ---- epilogue: four outputs per thread ----
+        constexpr int QUADS = WHICH == 0 ? 32 : 64;
+        for (int e = tid; e < p.batch * QUADS; e += TC_THREADS) {
+            const int n = e / QUADS, o = 4 * (e % QUADS), j = slab * 4 * QUADS + o;
+            if (j >= p.d_out) continue;                            // (d_out is a multiple of 32)
+            // gate/up: every 16 columns are 8 gate outputs followed by their 8 up outputs
+            const float *at = sums + n * ROW + (WHICH == 0 ? (o >> 3) * 16 + (o & 7) : o);
+            float4 r = *reinterpret_cast<const float4 *>(at);
+            if (WHICH == 0) {
+                const float4 up = *reinterpret_cast<const float4 *>(at + 8);
+                r = make_float4(silu_f32(r.x) * up.x, silu_f32(r.y) * up.y, silu_f32(r.z) * up.z, silu_f32(r.w) * up.w);
+                // top 16 bits of the rank keys |h_j| for the select that follows (no cache with several tokens)
+                if (p.key_coarse)
+                    *reinterpret_cast<uint2 *>(p.key_coarse + (size_t)n * p.d_out + j) =
+                        make_uint2(((__float_as_uint(r.x) & 0x7fffffffu) >> 16) | ((__float_as_uint(r.y) & 0x7fffffffu) & 0xffff0000u),
+                                   ((__float_as_uint(r.z) & 0x7fffffffu) >> 16) | ((__float_as_uint(r.w) & 0x7fffffffu) & 0xffff0000u));
+            }
+            *reinterpret_cast<float4 *>(p.out + (size_t)n * p.d_out + j) = r;
+        }
+    }
+    // ---- free the tensor memory (its last use lies before the barrier above) ----
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TC_TMEM_COLS) : "memory");
     DIP_TRACE_MAX(p.tr, 2);
@@ -402,34 +456,31 @@ gemv_tc_kernel(const GemvParams p, const uint16_t *__restrict__ xt)
 }  // namespace
 
 // One CTA per 512-byte segment and row part; all resident at once.  Rows with at least as many
-// segments as SMs' worth of work need no parts (gate/up); otherwise the parts are summed by
-// combine_parts_kernel right after.
+// segments as SMs' worth of work need no parts (gate/up); otherwise the parts meet in the last part's CTA (5120 / 17920, down: 4.6 us
+// after its last row for 16 tokens, 1.8 for 5; a launch of its own for the sums, 8.6 until the next select could start).
 dip_status dip_launch_gemv_tc(dip_ctx *ctx, GemvParams &p, int which, int n_kept_max, cudaStream_t stream)
 {
     const int n_slabs = (int)((p.row_bytes + TC_SEG - 1) / TC_SEG);
-    int nparts = ctx->sm_count / n_slabs;
-    if (nparts > n_kept_max / TC_ROUND_ROWS) nparts = n_kept_max / TC_ROUND_ROWS;   // at least a round of rows per part
-    if (nparts < 1) nparts = 1;
-    if (nparts > 1 && (size_t)nparts * n_slabs * TC_N * 256 > ctx->partials_floats) return DIP_ERR_WORKSPACE;
+    const int nparts = row_parts(ctx->sm_count / n_slabs, n_kept_max, TC_ROUND_ROWS);   // at least a round of rows per part
+    static_assert(TC_N * 256 <= DIP_MAIL_FLOATS, "");        // (parts only with one CTA per SM: the mail boxes suffice)
     p.defer = 0;
     p.part_base = 0;
-    if (nparts > 1 || which != 0 || (p.d_out & 7)) p.key_coarse = nullptr;      // only the epilogue that sees whole sums forms the keys
+    TcParams q;
+    q.n_slabs = n_slabs;
+    q.nparts = nparts;
+    q.xt = ctx->xt;
+    q.ready = ctx->readers + 1;
+    q.through = ctx->readers + 2;
+    q.block_wait_ns = ctx->block_wait_ns;
     const size_t smem = sizeof(TcSmem) + 1024;
     static_assert(sizeof(TcSmem) + 1024 <= 227 * 1024, "fits a CTA's shared memory");
     static dip_per_device_once once[2];
-    // the tokens' values of the union's rows, once for all CTAs
-    const int xt_ctas = min((p.mask_words + 1) / 2, 2 * ctx->sm_count);
-    DIP_CUDA_TRY(ctx, dip_launch_pdl(xt_build_kernel, dim3(xt_ctas), dim3(1024), 0, stream, p.mask_bits, p.v, p.batch, p.d_in,
-                                     p.mask_words, ctx->xt));
-    const uint16_t *xt = ctx->xt;
     if (which == 0) {
         DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once[0], ctx->device, gemv_tc_kernel<0>, smem));
-        DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_tc_kernel<0>, dim3(n_slabs, nparts), dim3(TC_THREADS), smem, stream, p, xt));
+        DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_tc_kernel<0>, dim3(n_slabs * nparts), dim3(TC_THREADS), smem, stream, p, q));
     } else {
         DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once[1], ctx->device, gemv_tc_kernel<1>, smem));
-        DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_tc_kernel<1>, dim3(n_slabs, nparts), dim3(TC_THREADS), smem, stream, p, xt));
+        DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_tc_kernel<1>, dim3(n_slabs * nparts), dim3(TC_THREADS), smem, stream, p, q));
     }
-    if (nparts > 1)
-        return dip_launch_combine_parts(ctx, which, nparts, n_slabs, TC_N, 256, 8, p.batch, p.d_out, p.out, stream);
     return DIP_OK;
 }
