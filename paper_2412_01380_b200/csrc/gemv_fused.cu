@@ -21,6 +21,9 @@
 // (UPD).  The down input's own cache is among them: its block makes the mask together with the others and
 // writes the cache's state once all of them have read it.  Other launches do without that code, which would
 // cost each of them 1.3 us (block_f32 shapes, 14.3 against 16.9 us per step of two launches).
+#include <math.h>
+#include <string.h>
+
 #include <type_traits>
 
 #include "cache_update.cuh"
@@ -31,7 +34,9 @@ namespace {
 constexpr int GF_SEG = 512;
 constexpr int GF_NW = TK_THREADS / 32;     // 32 warps
 constexpr int GF_U = 4;                    // loads in flight per lane
-constexpr double GF_AHEAD_BYTES = 15e6;   // rows asked for ahead of the stream, see own_ahead
+constexpr double GF_AHEAD_BYTES = 10e6;        // rows asked for once the threshold's bin is known: gate/up,
+constexpr double GF_AHEAD_DOWN_BYTES = 16e6;   // down,
+constexpr double GF_EARLY_BYTES = 25e6;        // and before that (see `early`)
 constexpr size_t GF_SMEM_LIMIT = (size_t)224 * 1024;   // dynamic shared memory a launch may ask for
 
 struct FusedParams {
@@ -40,7 +45,11 @@ struct FusedParams {
     size_t row_bytes;
     int d_in, d_out;
     int n_slabs, nparts;
-    int own_ahead;               // gate/up: quads of columns whose rows are asked for as soon as the threshold's bin is known
+    int ahead;                   // the columns of how many threads (of each part's 1024 / nparts) have their rows asked for
+                                 // as soon as the threshold's bin is known
+    int early;                   // gate/up, chained: of how many threads before that, if their keys are larger than
+    uint32_t sure;               // this: rms is 1, so fewer than k columns can be larger than sqrt(d / k)
+    uint32_t by_prod;            // ceil(2^32 / blocks with rows)
     int x_near;                  // gate/up: room in shared memory for the values of x
     float *out;
     float *mail;                 // [nparts][n_slabs][segment elements]; DIP_MAIL_EMPTY outside a launch
@@ -236,6 +245,9 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
     int key_stamp = 0;
     if (WHICH == 0 && p.key_coarse && p.key_stamp && out_ok) key_stamp = __ldcg(p.key_stamp + j_out);
 
+    // (rows asked for ahead are shared out over the blocks: this one's are those of groups q of columns with q % n_prod its index)
+    const auto mine = [&](int q) { return q - (int)__umulhi((unsigned)q, p.by_prod) * n_prod == (int)blockIdx.x; };
+
     // ---- the rank keys of the input and their histogram, in every CTA ----
     const int n_q = p.d_in / W;
     uint32_t kk[NQ][4];                    // gate/up: full keys of four columns; down: 16-bit keys of eight
@@ -285,6 +297,11 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
                 kk[j][1] = rank_key<CA>(r[j].y, st[j].y, p.gamma);
                 kk[j][2] = rank_key<CA>(r[j].z, st[j].z, p.gamma);
                 kk[j][3] = rank_key<CA>(r[j].w, st[j].w, p.gamma);
+                if (NORM && tid < p.early && mine(q)) {
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+                        if (kk[j][t] > p.sure) l2_prefetch(p.W + (size_t)(4 * q + t) * p.row_bytes, (unsigned)p.row_bytes);
+                }
                 if (!every) {
 #pragma unroll
                     for (int t = 0; t < 4; ++t) fine_count_hi(s.fine, kk[j][t]);
@@ -326,17 +343,23 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
         const uint32_t b = (uint32_t)s.ts.bcast[0];
         krem = s.ts.bcast[1];
         n_c = s.ts.bcast[2];
-        if constexpr (WHICH == 0) {
-            // The first rows on their way to L2 while the list is made: whole rows, shared out over the CTAs.  As many as
-            // come in that time: with 15 MB three Phi-3-Medium blocks took 112.7 us, with none 115.4, with 30 MB 116.1,
-            // with 60 MB 120.9 (what is still under way delays the first rows that are waited for)
+        // The first rows of each part on their way to L2 while the list is made (which has the threads' columns in thread
+        // order): whole rows, and of chained gate/up inputs the surely kept ones before that.  As many as come in that time.  Three
+        // Phi-3-Medium blocks, graph, us: none at all 110; gate/up only, 15 MB here 108.0, 10 MB here and up to 25 MB early 105.5; with 16 MB
+        // for down, too, 103.1 (12 MB 103.3, 7 or 13 MB for gate/up 103.4 and 104.1).  What is still under way when the
+        // first rows are waited for delays them
+        if (((tid * nparts) & (TK_THREADS - 1)) < p.ahead) {
 #pragma unroll
             for (int j = 0; j < NQ; ++j) {
                 const int q = tid + j * TK_THREADS;
-                if (q < p.own_ahead && q % n_prod == (int)blockIdx.x) {
+                if (q < n_q && mine(q)) {
 #pragma unroll
-                    for (int t = 0; t < 4; ++t)
-                        if (kk[j][t] > ((b << 16) | 0xffffu)) l2_prefetch(p.W + (size_t)(4 * q + t) * p.row_bytes, (unsigned)p.row_bytes);
+                    for (int t = 0; t < W; ++t) {
+                        bool ask;
+                        if constexpr (WHICH == 0) ask = kk[j][t] > ((b << 16) | 0xffffu) && !(NORM && tid < p.early && kk[j][t] > p.sure);
+                        else ask = ((kk[j][t >> 1] >> (16 * (t & 1))) & 0xffffu) > b;
+                        if (ask) l2_prefetch(p.W + (size_t)(W * q + t) * p.row_bytes, (unsigned)p.row_bytes);
+                    }
                 }
             }
         }
@@ -713,9 +736,16 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
         p.key_gamma = keys->gamma;
         keys->written = 1;
     }
-    const double quads = GF_AHEAD_BYTES / (double)p.row_bytes / sel->k * p.d_in / 4;
-    // (a product of fewer bytes than that gains nothing, and 0.4 us go into asking: two blocks of 1088 / 2816)
-    p.own_ahead = which == 0 && quads < p.d_in / 4 ? (int)quads : 0;
+    // (a product of little more bytes than that gains nothing, and 0.4 us go into asking: three blocks of 3072 / 8192 61.9 us with 12 of
+    // the 12.6 MB of a down product asked for, 61.1 without)
+    const double bytes = (double)p.row_bytes * sel->k, ahead = which == 0 ? GF_AHEAD_BYTES : GF_AHEAD_DOWN_BYTES;
+    p.ahead = 2 * ahead < bytes ? (int)(TK_THREADS * ahead / bytes) : 0;
+    // (of Laplace or Student-t inputs a quarter of the kept columns are that large, hence the quarter)
+    p.early = 0;
+    if (norm && p.ahead) p.early = GF_EARLY_BYTES < bytes / 4 ? (int)(TK_THREADS * GF_EARLY_BYTES / (bytes / 4)) : TK_THREADS;
+    const float sure = sqrtf((float)p.d_in / (float)sel->k) * 1.001f;
+    memcpy(&p.sure, &sure, sizeof(sure));
+    p.by_prod = (uint32_t)((0x100000000ull + (unsigned)(p.n_slabs * p.nparts) - 1) / (unsigned)(p.n_slabs * p.nparts));
     p.xa = sel->xa;
     p.xb = sel->xb;
     p.x_out = sel->x_out;
