@@ -166,8 +166,18 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
 
-def _stream() -> int:
+def _current_stream() -> int:
     return torch.cuda.current_stream().cuda_stream
+
+
+def _raw_stream() -> int:
+    # the current device's current stream without a Stream object around it: 0.2 us instead of 3.2 of the 13 us that the host
+    # spends on one step of two launches
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+# (both names are torch's own; builds of torch without CUDA lack them)
+_stream = _raw_stream if hasattr(torch._C, "_cuda_getCurrentRawStream") and hasattr(torch._C, "_cuda_getDevice") else _current_stream
 
 
 class Context:
