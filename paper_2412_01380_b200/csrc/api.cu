@@ -599,17 +599,18 @@ dip_status dip_mlp_step_neuron_pruned(dip_ctx *ctx, const dip_neuron_weights *w,
     uint32_t *mask = mask_out ? mask_out : ctx->mask_h;
     int32_t *idx = idx_out ? idx_out : ctx->idx_h;
     const bool by_gate = prune_by == DIP_PRUNE_BY_GATE;
+    const void *other = by_gate ? w->up : w->gate;
+    uint16_t *coarse = w->d_ff >= ctx->coarse_min_d ? ctx->coarse : nullptr;
     dip_status st;
     // the dense, ranking activation: p = silu(W^g x) (Gate pruning) or W^u x (Up pruning)
     st = dip_launch_rowdot(ctx, w->wtype, by_gate ? w->gate : w->up, w->d_model, w->d_ff, x, nullptr, w->d_ff,
-                           by_gate ? 1 : 0, nullptr, p, h, s);
+                           by_gate ? 1 : 0, nullptr, p, h, coarse, s);
     if (st != DIP_OK) return st;
     // m = topK(|p|) over the neurons (Eq. 5), as a bit set and as an ascending list
-    if ((st = dip_launch_select(ctx, p, nullptr, nullptr, 1, w->d_ff, k, 1.0f, nullptr, mask, s, nullptr, idx)) != DIP_OK) return st;
+    if ((st = dip_launch_select(ctx, p, nullptr, nullptr, 1, w->d_ff, k, 1.0f, nullptr, mask, s, coarse, idx)) != DIP_OK) return st;
     // the kept rows of the other matrix: h_j = p_j * (W^u x)_j, or p_j * silu((W^g x)_j); 0 elsewhere (from the
     // dense product's launch)
-    st = dip_launch_rowdot(ctx, w->wtype, by_gate ? w->up : w->gate, w->d_model, w->d_ff, x, idx, k,
-                           by_gate ? 0 : 1, p, h, nullptr, s);
+    st = dip_launch_rowdot(ctx, w->wtype, other, w->d_model, w->d_ff, x, idx, k, by_gate ? 0 : 1, p, h, nullptr, nullptr, s);
     if (st != DIP_OK) return st;
     // y = sum over the kept neurons of W^d[:, j] h_j
     dip_mlp_weights wd = {};

@@ -160,7 +160,7 @@ struct dip_cache_update {
 // is given).  xb != nullptr: the row is first formed as (xa + xb) / rms(xa + xb), written to x_out.
 // coarse != nullptr (no xb, d % 32 == 0; several rows only without stamps): the producer of xa has left the top 16 bits of
 // every column's rank key there (dip_gemv_keys), and the launch reads those instead of all of
-// xa and stamp.  idx_out != nullptr (no xb, no coarse): the kept columns of each row as an ascending list, k apart.
+// xa and stamp.   idx_out != nullptr (no xb): the kept columns of each row as an ascending list, k apart.
 // update != nullptr (one row with stamps, no xb, no coarse): the launch also makes this cache's update from the mask.
 // split != nullptr (likewise): the launch also parts the mask into this tier's hits and misses (split, loc, fetch).
 dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, float *x_out, int batch, int d, int k,
@@ -265,9 +265,10 @@ dip_status dip_launch_tier_fetch(dip_ctx *ctx, const dip_tier *t, const dip_cach
 
 // rowdot.cu: out_j = [silu](W[j, :] . x) [* mul_j] for the listed rows (rows == nullptr: rows
 // 0 .. n_rows-1) of a row-major [d_ff][d_model] matrix; F32 or BF16.  zero != nullptr: also zero_j = 0 for these rows.
+// coarse != nullptr: also the top 16 bits of |out_j| to coarse_j.
 dip_status dip_launch_rowdot(dip_ctx *ctx, int wtype, const void *W, int d_model, int d_ff, const float *x,
                              const int32_t *rows, int n_rows, int silu, const float *mul, float *out, float *zero,
-                             cudaStream_t stream);
+                             uint16_t *coarse, cudaStream_t stream);
 
 // pack.cu
 dip_status dip_launch_pack(dip_ctx *ctx, int wtype, int d_model, int d_ff,

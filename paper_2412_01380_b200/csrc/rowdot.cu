@@ -22,6 +22,7 @@ struct RowdotParams {
     const float *mul;          // [d_ff] or nullptr: out_j *= mul_j
     float *out;                // [d_ff]
     float *zero;               // [d_ff] or nullptr: zero_j = 0 for each row done
+    uint16_t *coarse;          // [d_ff] or nullptr: top 16 bits of |out_j|, the rank keys for the select behind
     unsigned long long *tr;
 };
 
@@ -98,16 +99,26 @@ rowdot_kernel(const RowdotParams p)
             if (p.mul) v *= p.mul[j];
             p.out[j] = v;
             if (p.zero) p.zero[j] = 0.f;
+            if (p.coarse) p.coarse[j] = (uint16_t)((__float_as_uint(v) & 0x7fffffffu) >> 16);
         }
     }
     DIP_TRACE_MAX(p.tr, 2);
+}
+
+template <int WT>
+dip_status launch_rowdot(dip_ctx *ctx, const RowdotParams &p, int blocks, size_t smem, cudaStream_t stream)
+{
+    static dip_per_device_once once;
+    DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once, ctx->device, rowdot_kernel<WT>, sizeof(float) * DIP_MAX_D));
+    DIP_CUDA_TRY(ctx, dip_launch_pdl(rowdot_kernel<WT>, dim3(blocks), dim3(RD_THREADS), smem, stream, p));
+    return DIP_OK;
 }
 
 }  // namespace
 
 dip_status dip_launch_rowdot(dip_ctx *ctx, int wtype, const void *W, int d_model, int d_ff, const float *x,
                              const int32_t *rows, int n_rows, int silu, const float *mul, float *out, float *zero,
-                             cudaStream_t stream)
+                             uint16_t *coarse, cudaStream_t stream)
 {
     if (wtype != DIP_W_F32 && wtype != DIP_W_BF16) return DIP_ERR_UNSUPPORTED;
     RowdotParams p;
@@ -121,20 +132,12 @@ dip_status dip_launch_rowdot(dip_ctx *ctx, int wtype, const void *W, int d_model
     p.mul = mul;
     p.out = out;
     p.zero = zero;
+    p.coarse = coarse;
     p.tr = dip_trace_slot(ctx, 9);
     const size_t smem = sizeof(float) * (size_t)d_model;
     const int warps_needed = n_rows;
     int blocks = (warps_needed + RD_THREADS / 32 - 1) / (RD_THREADS / 32);
     if (blocks > ctx->sm_count) blocks = ctx->sm_count;
     if (blocks < 1) blocks = 1;
-    if (wtype == DIP_W_F32) {
-        static dip_per_device_once once;
-        DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once, ctx->device, rowdot_kernel<DIP_W_F32>, sizeof(float) * DIP_MAX_D));
-        DIP_CUDA_TRY(ctx, dip_launch_pdl(rowdot_kernel<DIP_W_F32>, dim3(blocks), dim3(RD_THREADS), smem, stream, p));
-    } else {
-        static dip_per_device_once once;
-        DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once, ctx->device, rowdot_kernel<DIP_W_BF16>, sizeof(float) * DIP_MAX_D));
-        DIP_CUDA_TRY(ctx, dip_launch_pdl(rowdot_kernel<DIP_W_BF16>, dim3(blocks), dim3(RD_THREADS), smem, stream, p));
-    }
-    return DIP_OK;
+    return wtype == DIP_W_F32 ? launch_rowdot<DIP_W_F32>(ctx, p, blocks, smem, stream) : launch_rowdot<DIP_W_BF16>(ctx, p, blocks, smem, stream);
 }

@@ -126,7 +126,8 @@ select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, f
 template <bool CA>
 __global__ void __launch_bounds__(TK_THREADS, 1)
 select_fine_coarse_kernel(const float *__restrict__ x, const uint16_t *__restrict__ coarse, int d, int k, float gamma,
-                          const int32_t *__restrict__ stamp, uint32_t *__restrict__ mask_bits, unsigned long long *tr)
+                          const int32_t *__restrict__ stamp, uint32_t *__restrict__ mask_bits, int32_t *__restrict__ idx_out,
+                          unsigned long long *tr)
 {
     DIP_TRACE_MIN(tr, 0);
     extern __shared__ __align__(16) unsigned char dyn[];
@@ -147,6 +148,10 @@ select_fine_coarse_kernel(const float *__restrict__ x, const uint16_t *__restric
     __syncthreads();                                                  // histogram zeroed
     select_fine_coarse<CA>(coarse, x, stamp, gamma, d, k, keys, s, f, s_maskw);
     for (int w = tid; w < (d >> 5); w += TK_THREADS) mask_bits[w] = s_maskw[w];
+    if (idx_out) {
+        int32_t *o = idx_out + (size_t)row * k;
+        list_mask(s_maskw, d, s, [&](int r, int col) { o[r] = col; });
+    }
     DIP_TRACE_MAX(tr, 2);
 }
 
@@ -234,7 +239,8 @@ dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, flo
                              float gamma, const int32_t *stamp, uint32_t *mask_bits, cudaStream_t stream,
                              const uint16_t *coarse, int32_t *idx_out, const dip_cache_update *update, const dip_tier *split)
 {
-    if ((idx_out || update || split) && (coarse || xb)) return DIP_ERR_INVALID_ARG;
+    if ((update || split) && (coarse || xb)) return DIP_ERR_INVALID_ARG;
+    if (idx_out && xb) return DIP_ERR_INVALID_ARG;
     if ((update || split) && (batch != 1 || !stamp)) return DIP_ERR_INVALID_ARG;
     const Int<0> no;
     const size_t smem = sizeof(TkFine) + (size_t)((d + 3) & ~3) * sizeof(uint32_t);
@@ -245,10 +251,10 @@ dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, flo
         if (xb || (batch != 1 && stamp) || (d & 31)) return DIP_ERR_INVALID_ARG;
         if (stamp)
             e = dip_launch_pdl(select_fine_coarse_kernel<true>, grid, block, smem, stream, xa, coarse, d, k, gamma, stamp,
-                               mask_bits, tr);
+                               mask_bits, idx_out, tr);
         else
             e = dip_launch_pdl(select_fine_coarse_kernel<false>, grid, block, smem, stream, xa, coarse, d, k, 1.0f,
-                               (const int32_t *)nullptr, mask_bits, tr);
+                               (const int32_t *)nullptr, mask_bits, idx_out, tr);
     } else if (xb) {
         if (stamp)
             e = dip_launch_pdl(select_fine_kernel<true, true, THEN_NOTHING>, grid, block, smem, stream, xa, xb, x_out, d, k, gamma, stamp,
