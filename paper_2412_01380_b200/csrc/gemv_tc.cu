@@ -8,12 +8,14 @@
 //     into shared memory in the layout that a 128-byte-swizzled
 //     MN-major operand descriptor names: the outputs of a row are contiguous, so the weights are the
 //     B operand (N = 256) as they arrive, untransposed, and each byte is read by one MMA only;
-//   * the tokens' values of all columns, zeroed where a token drops the column and split into two bfloat16, are gathered
-//     ONCE per product into a table of 64 bytes per column: each block makes its share while its first rows are on their way (a
-//     launch of its own in front took 2.5 us).  The loaders copy a row's 64 bytes as the MN-major A operand: row n = the high
-//     halves of token n, row 16 + n the low halves, the other rows of the M = 128 tile zero.  (Every CTA gathering its rows'
-//     values for itself, four bytes at a time, is what the load path cannot take: 16 tokens' gate/up product 86 us
-//     with registers and warps of their own, 105 us with asynchronous copies of four bytes, 60 us like this);
+//   * the tokens' values of the union's rows, zeroed where a token drops the row and split into two bfloat16, are gathered
+//     ONCE per product by xt_build_kernel (16 scattered loads per row) into a table of 64 bytes per column.  The loaders copy a
+//     row's 64 bytes as the MN-major A operand: row n = the high halves of token n, row 16 + n the low halves, the other rows of
+//     the M = 128 tile zero.  (Every CTA gathering its rows' values for itself, four bytes at a time, is what the load path
+//     cannot take: 16 tokens' gate/up product 86 us with registers and warps of their own, 105 us with asynchronous copies of four
+//     bytes, 60 us like this.  The product's blocks sharing the gathering and waiting for one another saves a launch and is slower
+//     all the same (16 tokens at 5120 / 17920, keep ratio 0.25: 122.4 us per step against 116.5; a union of 64 of 8192 columns, one segment:
+//     47.6 against 7.9), and where there are more segments than SMs the first blocks wait for some that start after them);
 //   * one thread of a seventeenth warp issues one tcgen05.mma (M = 128, N = 256, K = 16) per 16 rows
 //     once the loader warps have arrived on the buffer's "full" barrier; the accumulator lives in
 //     tensor memory (256 columns) for the whole kernel, and a tcgen05.commit per round tells the
@@ -48,11 +50,6 @@ constexpr int TC_TMEM_COLS = 256;                // one accumulator: 128 lanes x
 // (16 tokens at keep ratio 0.25 keep ~5100 of 5120 gate/up rows, ~2500 down rows per part).
 constexpr int TC_LIST_ROWS = 8192;
 
-constexpr int TC_BUILD_WORDS = 4;              // words whose loads go out together
-constexpr int TC_BUILD_ROW = 17;               // 4-byte words
-constexpr size_t TC_BUILD_SMEM = (size_t)TC_BUILD_WORDS * 32 * TC_BUILD_ROW * 4;
-constexpr unsigned long long TC_TABLE_WAIT_NS = 100000ull;   // for the other blocks' shares
-
 struct __align__(1024) TcSmem {
     unsigned char a[TC_BUFS][TC_KB * TC_A_KB_BYTES];   // weights, 4 x 32 KB
     unsigned char b[TC_BUFS][TC_KB * TC_B_KB_BYTES];   // token values, 4 x 16 KB
@@ -61,8 +58,6 @@ struct __align__(1024) TcSmem {
     uint32_t tmem_base;
     int n_total;
     int fail;
-    int table;                                   // all blocks have written their shares of the table
-    uint32_t build[TC_BUILD_SMEM / 4];
     int wsum[TC_WARPS];
     uint32_t words[DIP_MAX_D / 32];
     int pre[DIP_MAX_D / 32];
@@ -113,48 +108,35 @@ __device__ __forceinline__ void tc_ld64(uint32_t taddr, float (&v)[64])
 
 struct TcParams {
     int n_slabs, nparts;
-    uint16_t *xt;              // [d_in][32] the table: 16 high, 16 low halves
-    unsigned int *ready;       // blocks whose share of it is written; zero between launches
-    unsigned int *through;     // blocks that need it no more; zero between launches
+    const uint16_t *xt;        // [d_in][32] the table: 16 high, 16 low halves
     unsigned long long block_wait_ns;
 };
 
-// The table's columns of the mask words first, first + step, ...: warp n < 16 takes token n's, a column per lane, and a tile in
-// shared memory (rows of 64 bytes, 68 apart: no bank conflicts) turns them round.  The TC_LOAD_WARPS warps call it.
-__device__ __forceinline__ void xt_build(const GemvParams &p, uint16_t *xt, int first, int step, uint32_t *buf)
+// The tokens' values of every column of the union, ready for the tensor core: xt[i][n] = bfloat16 high
+// half of token n's value at column i (zero where the token's own mask drops the column or
+// n >= batch), xt[i][16 + n] = the low half; columns outside the union are not written (and never
+// read).  Built once per product instead of once per CTA (the values are 16 scattered 4-byte loads
+// per column).  A block takes two mask words per pass; 16 consecutive threads are the 16 tokens of
+// one column.
+__global__ void __launch_bounds__(1024, 1)
+xt_build_kernel(const uint32_t *__restrict__ mask_bits, const float *__restrict__ v, int batch, int d_in, int mask_words,
+                uint16_t *__restrict__ xt)
 {
-    constexpr int T = TC_LOAD_WARPS * 32;
-    static_assert(TC_LOAD_WARPS == TC_N, "a warp per token");
-    const int tid = threadIdx.x, lane = tid & 31, n = tid >> 5;
-    for (int w0 = first; w0 < p.mask_words; w0 += TC_BUILD_WORDS * step) {
-        float x[TC_BUILD_WORDS];
-        uint32_t m[TC_BUILD_WORDS];
-#pragma unroll
-        for (int u = 0; u < TC_BUILD_WORDS; ++u) {
-            const int w = w0 + u * step;
-            x[u] = 0.f;
-            m[u] = 0u;
-            if (n < p.batch && w < p.mask_words) {
-                m[u] = __ldg(p.mask_bits + (size_t)n * p.mask_words + w);
-                if (w * 32 + lane < p.d_in) x[u] = __ldg(p.v + (size_t)n * p.d_in + w * 32 + lane);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < TC_BUILD_WORDS; ++u) {
-            const float v = (m[u] >> lane) & 1u ? x[u] : 0.f;
-            const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-            const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-            __nv_bfloat16 *row = reinterpret_cast<__nv_bfloat16 *>(buf + (u * 32 + lane) * TC_BUILD_ROW);
-            row[n] = hi;
-            row[16 + n] = lo;
-        }
-        asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory");
-        for (int i = tid; i < TC_BUILD_WORDS * 128; i += T) {
-            const int w = w0 + (i >> 7) * step, col = w * 32 + ((i & 127) >> 2);
-            const uint32_t *at = buf + (i >> 2) * TC_BUILD_ROW + 4 * (i & 3);
-            if (w < p.mask_words && col < p.d_in) reinterpret_cast<uint4 *>(xt)[(size_t)col * 4 + (i & 3)] = make_uint4(at[0], at[1], at[2], at[3]);
-        }
-        asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory");
+    const int tid = threadIdx.x;
+    const int n = tid & 15, bit = (tid >> 4) & 31, half = tid >> 9;
+    dip_grid_dependency_wait();
+    dip_launch_dependents();
+    for (int w = 2 * blockIdx.x + half; w < mask_words; w += 2 * gridDim.x) {
+        const int idx = w * 32 + bit;
+        const bool mine = n < batch && idx < d_in && ((mask_bits[(size_t)n * mask_words + w] >> bit) & 1u);
+        // in the union if any of the 16 tokens (a half-warp) keeps the column
+        const unsigned any = __ballot_sync(0xffffffffu, mine) & (0xffffu << (tid & 16));
+        if (!any) continue;
+        const float x = mine ? __ldg(v + (size_t)n * d_in + idx) : 0.f;
+        const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+        const __nv_bfloat16 lo = __float2bfloat16_rn(x - __bfloat162float(hi));
+        xt[(size_t)idx * 32 + n] = __bfloat16_as_ushort(hi);
+        xt[(size_t)idx * 32 + 16 + n] = __bfloat16_as_ushort(lo);
     }
 }
 
@@ -166,8 +148,7 @@ gemv_tc_kernel(const GemvParams p, const TcParams q)
     TcSmem &s = *reinterpret_cast<TcSmem *>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
     DIP_TRACE_MIN(p.tr, 0);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int block = blockIdx.x;
-    const int slab = block % q.n_slabs, part = block / q.n_slabs, nparts = q.nparts;
+    const int slab = (int)blockIdx.x % q.n_slabs, part = (int)blockIdx.x / q.n_slabs, nparts = q.nparts;
     const size_t byte_off = (size_t)slab * TC_SEG + lane * 16;
     const bool lane_ok = byte_off < p.row_bytes;
 
@@ -243,28 +224,6 @@ gemv_tc_kernel(const GemvParams p, const TcParams q)
     const int bb_row = (tid >> 2) & (TC_ROUND_ROWS - 1), bb_mg = tid & 3;
     const uint32_t b_off = (uint32_t)((bb_row >> 4) * TC_B_KB_BYTES + ((bb_row & 15) >> 3) * 2048 + bb_mg * 128 + (bb_row & 7) * 16);
 
-    // This block's share of the table, and a wait for the others' (warps 0 - 15).  Blocks wait for one another here without any
-    // order among them, and nothing promises that they all run at the same time: one that has waited long enough makes the
-    // whole table by itself (the same bytes as whoever else writes them).
-    auto make_table = [&]() {
-        const unsigned int n_blocks = q.n_slabs * nparts;
-        xt_build(p, q.xt, block, n_blocks, s.build);
-        if (tid == 0) {
-            __threadfence();
-            count_one(q.ready);
-            unsigned int n = 0u;
-            const unsigned long long t0 = dip_gtime();
-            do asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(q.ready) : "memory");
-            while (n < n_blocks && dip_gtime() - t0 < TC_TABLE_WAIT_NS);
-            s.table = n >= n_blocks;
-        }
-        asm volatile("bar.sync 1, %0;" ::"n"(TC_LOAD_WARPS * 32) : "memory");
-        if (!s.table) {
-            xt_build(p, q.xt, 0, 1, s.build);
-            __threadfence();
-            asm volatile("bar.sync 1, %0;" ::"n"(TC_LOAD_WARPS * 32) : "memory");
-        }
-    };
     int g = 0;                         // rounds so far (buffer g & 1)
     bool failed = false;
 
@@ -291,38 +250,34 @@ gemv_tc_kernel(const GemvParams p, const TcParams q)
         if (warp < TC_LOAD_WARPS) {
             // copies of one round, global -> shared memory, 16 bytes each (zero-filled past the end of the list): this lane's
             // piece of rows warp, warp + 16, ... and (threads 0-255) this thread's 16 bytes of the tokens' values of row tid / 4
-            auto copy_weights = [&](int mr) {
+            auto copy_round = [&](int mr) {
                 const int gr = g + mr;                                      // round number over the whole kernel
-                if (mr >= n_rounds) return;
-                // the MMAs that read this ring slot four rounds ago must be through
-                if (gr >= TC_BUFS && !failed) {
-                    if (s.fail || !mbar_wait(&s.done[gr % TC_BUFS], ((gr / TC_BUFS) - 1) & 1, p.wait_limit_ns)) failed = true;
-                }
-                const uint32_t ab = smem_u32(s.a[gr % TC_BUFS]) + a_off;
+                if (mr < n_rounds) {
+                    // the MMAs that read this ring slot four rounds ago must be through
+                    if (gr >= TC_BUFS && !failed) {
+                        if (s.fail || !mbar_wait(&s.done[gr % TC_BUFS], ((gr / TC_BUFS) - 1) & 1, p.wait_limit_ns)) failed = true;
+                    }
+                    const uint32_t ab = smem_u32(s.a[gr % TC_BUFS]) + a_off;
 #pragma unroll
-                for (int u = 0; u < TC_U; ++u) {
-                    const int r = mr * TC_ROUND_ROWS + warp + u * TC_LOAD_WARPS;
-                    const bool ok = r < n_rows && lane_ok;
-                    const char *src = ok ? base + (size_t)s.idx[r] * p.row_bytes : p.W;
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ab + u * TC_A_KB_BYTES), "l"(src),
-                                 "r"(ok ? 16 : 0) : "memory");
-                }
-            };
-            auto copy_values = [&](int mr) {
-                if (mr < n_rounds && tid < TC_ROUND_ROWS * 4) {
-                    const int r = mr * TC_ROUND_ROWS + bb_row;
-                    const bool ok = r < n_rows;
-                    const uint16_t *src = ok ? q.xt + (size_t)s.idx[r] * 32 + bb_mg * 8 : q.xt;
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(s.b[(g + mr) % TC_BUFS]) + b_off), "l"(src),
-                                 "r"(ok ? 16 : 0) : "memory");
+                    for (int u = 0; u < TC_U; ++u) {
+                        const int r = mr * TC_ROUND_ROWS + warp + u * TC_LOAD_WARPS;
+                        const bool ok = r < n_rows && lane_ok;
+                        const char *src = ok ? base + (size_t)s.idx[r] * p.row_bytes : p.W;
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ab + u * TC_A_KB_BYTES), "l"(src),
+                                     "r"(ok ? 16 : 0) : "memory");
+                    }
+                    if (tid < TC_ROUND_ROWS * 4) {
+                        const int r = mr * TC_ROUND_ROWS + bb_row;
+                        const bool ok = r < n_rows;
+                        const uint16_t *src = ok ? q.xt + (size_t)s.idx[r] * 32 + bb_mg * 8 : q.xt;
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(s.b[gr % TC_BUFS]) + b_off), "l"(src),
+                                     "r"(ok ? 16 : 0) : "memory");
+                    }
                 }
                 asm volatile("cp.async.commit_group;" ::: "memory");           // (an empty group past the last round)
             };
 #pragma unroll
-            for (int mr = 0; mr < TC_BUFS - 1; ++mr) copy_weights(mr);
-            if (list_begin == r_begin) make_table();
-#pragma unroll
-            for (int mr = 0; mr < TC_BUFS - 1; ++mr) copy_values(mr);
+            for (int mr = 0; mr < TC_BUFS - 1; ++mr) copy_round(mr);
             for (int mr = 0; mr < n_rounds; ++mr) {
                 // this thread's copies of round mr have landed (the two younger groups may be in flight)
                 asm volatile("cp.async.wait_group %0;" ::"n"(TC_BUFS - 2) : "memory");
@@ -330,8 +285,7 @@ gemv_tc_kernel(const GemvParams p, const TcParams q)
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&s.full[(g + mr) % TC_BUFS]);
-                copy_weights(mr + TC_BUFS - 1);
-                copy_values(mr + TC_BUFS - 1);
+                copy_round(mr + TC_BUFS - 1);
             }
             asm volatile("cp.async.wait_group 0;" ::: "memory");              // (only empty groups are left)
         } else if (lane == 0) {
@@ -363,17 +317,6 @@ gemv_tc_kernel(const GemvParams p, const TcParams q)
     if (failed) s.fail = 1;
     __syncthreads();
     failed = s.fail != 0;
-    // (a block without rows has not been there)
-    if (r_begin == r_end && warp < TC_LOAD_WARPS) make_table();
-    // the last block that needs the table no more makes the words ready for the next launch
-    if (tid == 0) {
-        __threadfence();
-        if (atomicAdd(q.through, 1u) == (unsigned)(q.n_slabs * nparts) - 1u) {
-            *q.ready = 0u;
-            *q.through = 0u;
-        }
-    }
-
     // ---- the last round's commit covers every MMA of the kernel ----
     if (g > 0 && !failed) {
         if (!mbar_wait(&s.done[(g - 1) % TC_BUFS], ((g - 1) / TC_BUFS) & 1, p.wait_limit_ns)) failed = true;
@@ -455,8 +398,8 @@ gemv_tc_kernel(const GemvParams p, const TcParams q)
 
 }  // namespace
 
-// One CTA per 512-byte segment and row part; all resident at once.  Rows with at least as many
-// segments as SMs' worth of work need no parts (gate/up); otherwise the parts meet in the last part's CTA (5120 / 17920, down: 4.6 us
+// One CTA per 512-byte segment and row part.  Rows of half as many segments as SMs or more need no parts (gate/up, whose segments
+// may be more than SMs); otherwise the parts, all resident at once, meet in the last part's CTA (5120 / 17920, down: 4.6 us
 // after its last row for 16 tokens, 1.8 for 5; a launch of its own for the sums, 8.6 until the next select could start).
 dip_status dip_launch_gemv_tc(dip_ctx *ctx, GemvParams &p, int which, int n_kept_max, cudaStream_t stream)
 {
@@ -469,12 +412,13 @@ dip_status dip_launch_gemv_tc(dip_ctx *ctx, GemvParams &p, int which, int n_kept
     q.n_slabs = n_slabs;
     q.nparts = nparts;
     q.xt = ctx->xt;
-    q.ready = ctx->readers + 1;
-    q.through = ctx->readers + 2;
     q.block_wait_ns = ctx->block_wait_ns;
     const size_t smem = sizeof(TcSmem) + 1024;
     static_assert(sizeof(TcSmem) + 1024 <= 227 * 1024, "fits a CTA's shared memory");
     static dip_per_device_once once[2];
+    const int xt_ctas = min((p.mask_words + 1) / 2, 2 * ctx->sm_count);
+    DIP_CUDA_TRY(ctx, dip_launch_pdl(xt_build_kernel, dim3(xt_ctas), dim3(1024), 0, stream, p.mask_bits, p.v, p.batch, p.d_in,
+                                     p.mask_words, ctx->xt));
     if (which == 0) {
         DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once[0], ctx->device, gemv_tc_kernel<0>, smem));
         DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_tc_kernel<0>, dim3(n_slabs * nparts), dim3(TC_THREADS), smem, stream, p, q));

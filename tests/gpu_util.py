@@ -112,3 +112,22 @@ def check_step(dip, ctx, lw, w, x, k_x, k_h, gamma, ref_gu, ref_d, g_gu, g_d, ti
     if ref_gu is not None:
         assert cache_equal(g_gu, ref_gu) and cache_equal(g_d, ref_d)
     return y.cpu().numpy()
+
+
+def graph_us(call, n=8, replays=15) -> float:
+    """Device time of one call in microseconds: the shortest replay of a CUDA graph of n of them (for comparisons inside one test)."""
+    call()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(n):
+            call()
+    best = float("inf")
+    for _ in range(replays):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        graph.replay()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3 / n)
+    return best

@@ -1,12 +1,12 @@
-"""Batched products on the tensor cores, whose blocks share the making of a table of the tokens' values and send their row parts to
-one of them: unions of a round, of less, of none in some parts, of all columns; as many parts as SMs and rows without parts; columns
-that no multiple of 128 is; and every number of tokens."""
+"""Batched products on the tensor cores, which read a table of the tokens' values and send their row parts to one of their blocks:
+unions of a round, of less, of none in some parts, of all columns; as many parts as SMs and rows without parts; columns
+that no multiple of 128 is; every number of tokens; and what a wide row, a wide input and a short limit of the waits cost."""
 import numpy as np
 import pytest
 
 import dip_inputs as di
 import oracle
-from gpu_util import REL_TOL, oracle_mats, rel_err, upload_layer
+from gpu_util import REL_TOL, graph_us, oracle_mats, rel_err, upload_layer
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -35,4 +35,58 @@ def test_batched_products_from_masks(d_model, d_ff, batches):
                         if which == 0 else oracle.masked_matvec(Wd, v[b], masks[b])
                     assert rel_err(out[b].cpu().numpy(), want) <= REL_TOL, (batch, which, k, b)
     assert ctx.device_status() == 0
+    ctx.close()
+
+
+def _product(dip, d_model, d_ff, which, batch, k, **options):
+    """A call of one product, all tokens keeping the same k columns; its context and output."""
+    ctx = dip.Context(0, **options)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d_ff + k)
+    mats = [torch.randn(s, generator=gen, device="cuda").mul_(0.02).bfloat16() for s in ((d_ff, d_model), (d_ff, d_model), (d_model, d_ff))]
+    w = dip.dip_pack_weights(ctx, dip.W_BF16, d_model, d_ff, *mats)
+    d = d_model if which == 0 else d_ff
+    v = torch.randn((batch, d), generator=gen, device="cuda")
+    bits = torch.zeros((batch, (d + 31) // 32), dtype=torch.int32, device="cuda")
+    dip.dip_mask_topk(ctx, v[0].contiguous(), k, bits[0], None)
+    bits[1:] = bits[0]
+    out = torch.empty((batch, d_ff if which == 0 else d_model), device="cuda")
+    product = dip.dip_sparse_gemv_gate_up if which == 0 else dip.dip_sparse_gemv_down
+    return ctx, out, lambda: product(ctx, w, v, None, k, bits, out), (mats, v, bits)
+
+
+@pytest.mark.parametrize("batch", [4, 16])
+def test_a_segment_more_than_sms_does_not_stall(batch):
+    """One segment more than fits at a time takes a second wave, a few microseconds; no block waits for that wave to start."""
+    import paper_2412_01380_b200 as dip
+    us = {}
+    for extra in (0, 64):
+        ctx, _, call, _ = _product(dip, 288, 128 * dip.Context(0).sm_count + extra, 0, batch, 64)
+        us[extra] = graph_us(call)
+        assert ctx.device_status() == 0
+        ctx.close()
+    assert us[64] < us[0] + 30, us
+
+
+@pytest.mark.parametrize("d_model,d_ff,which", [(256, 8192, 1), (8192, 256, 0)])
+def test_few_rows_of_a_wide_input_take_no_longer_than_many(d_model, d_ff, which):
+    import paper_2412_01380_b200 as dip
+    us = {}
+    for k in (64, 4096):
+        ctx, _, call, _ = _product(dip, d_model, d_ff, which, 3, k)
+        us[k] = graph_us(call)
+        ctx.close()
+    assert us[64] < us[4096] + 2, us
+
+
+def test_a_short_limit_for_copies_bounds_copies_only():
+    import paper_2412_01380_b200 as dip
+    d_ff = 128 * dip.Context(0).sm_count + 64
+    ctx, out, call, (mats, v, bits) = _product(dip, 288, d_ff, 0, 4, 64, wait_limit_us=60)
+    call()
+    assert ctx.device_status() == 0
+    keep = torch.from_numpy(np.unpackbits(bits.cpu().numpy().view(np.uint8), axis=1, bitorder="little")[:, :288].astype(np.float64)).cuda()
+    x = v.double() * keep
+    want = torch.nn.functional.silu(x @ mats[0].double().t()) * (x @ mats[1].double().t())
+    assert rel_err(out.cpu().numpy(), want.cpu().numpy()) <= REL_TOL
     ctx.close()
