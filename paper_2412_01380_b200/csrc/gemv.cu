@@ -670,7 +670,7 @@ idx_to_mask_kernel(const int32_t *__restrict__ idx, int n, int d, uint32_t *__re
     for (int w = tid; w < n_words; w += 1024) mask[w] = words[w];
 }
 
-// Sum of the row parts and the epilogue as a kernel of its own (large batches; the two launches
+// Sum of the row parts and the epilogue as a kernel of its own (many parts of large batches; the two launches
 // of the two-tier step).  CP_LANES (1 or 8) neighbouring lanes share four outputs: lane l adds the
 // parts l, l + CP_LANES, ... (its loads in flight together), then the lanes' sums meet in a fixed
 // shuffle tree, so the result is reproducible.  Eight lanes pay when there are many parts.  partials: [nparts][n_slabs][bt][slab]; gate/up rows are
@@ -912,7 +912,7 @@ dip_status dip_launch_gemv(dip_ctx *ctx, const dip_mlp_weights *w, int which,
         else if (p.batch >= 3 && !mode) {
             if (keys && which == 0 && keys->coarse && batch <= 16) p.key_coarse = keys->coarse;
             st = dip_launch_gemv_tc(ctx, p, which, n_kept_max, stream);       // a dense contraction: tensor cores
-            if (st == DIP_OK && p.key_coarse) keys->written = 1;      // (the launcher drops the request when it splits the rows)
+            if (st == DIP_OK && p.key_coarse) keys->written = 1;      // (the launcher drops the request when a launch behind adds up the row parts)
         }
         else
             st = which == 0 ? launch_bt<DIP_W_BF16, 0>(ctx, p, n_kept_max, mode, stream)

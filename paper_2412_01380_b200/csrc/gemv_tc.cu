@@ -348,10 +348,14 @@ gemv_tc_kernel(const GemvParams p, const TcParams q)
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    // ---- row parts: to the last part's CTA, which adds them up in part order (see gemv_fused.cu) ----
+    // ---- row parts: for a launch behind this one, or to the last part's CTA, which adds them up in part order (see gemv_fused.cu) ----
     const size_t stride = (size_t)q.n_slabs * p.batch * 256;
     float *box = p.mail + (size_t)slab * p.batch * 256;
-    if (part != nparts - 1) {
+    if (p.defer) {
+        float *to = p.partials + (size_t)part * stride + (size_t)slab * p.batch * 256;
+        for (int e = tid; e < p.batch * 64; e += TC_THREADS)
+            *reinterpret_cast<float4 *>(to + 4 * e) = *reinterpret_cast<const float4 *>(sums + (e >> 6) * ROW + 4 * (e & 63));
+    } else if (part != nparts - 1) {
         for (int e = tid; e < p.batch * 64; e += TC_THREADS)
             mail_put4(box + (size_t)part * stride + 4 * e, *reinterpret_cast<const float4 *>(sums + (e >> 6) * ROW + 4 * (e & 63)));
     } else {
@@ -398,16 +402,25 @@ gemv_tc_kernel(const GemvParams p, const TcParams q)
 
 }  // namespace
 
-// One CTA per 512-byte segment and row part.  Rows of half as many segments as SMs or more need no parts (gate/up, whose segments
-// may be more than SMs); otherwise the parts, all resident at once, meet in the last part's CTA (5120 / 17920, down: 4.6 us
-// after its last row for 16 tokens, 1.8 for 5; a launch of its own for the sums, 8.6 until the next select could start).
+// One CTA per 512-byte segment and row part.  Rows of more segments than half the SMs need no parts (gate/up, whose segments may be
+// more than SMs); otherwise the parts, all resident at once, meet in the last part's CTA (5120 / 17920, down: 4.6 us
+// after its last row for 16 tokens, 1.8 for 5; a launch of its own for the sums, 8.6 until the next select could start).  That
+// CTA takes parts x tokens KB, and its SM's share of L2's rate makes that the longer way where both are many: 16 tokens,
+// union of 1024 / 4096, one segment (16 / 64 parts) 15.0 / 32.4 us and 10.6 / 12.0 with a launch behind; 8 tokens, 16 parts 11.4 and 9.9;
+// 3 tokens, 32 parts 11.6 and 10.4.  The other way: 5 tokens, 16 parts 10.3 and 9.7, 18 parts of 8 segments 11.1 and 12.0; 16 tokens, 12 parts
+// 14.9 and 16.0.
+constexpr int TC_APART_PARTS = 16, TC_APART_KB = 96;
 dip_status dip_launch_gemv_tc(dip_ctx *ctx, GemvParams &p, int which, int n_kept_max, cudaStream_t stream)
 {
     const int n_slabs = (int)((p.row_bytes + TC_SEG - 1) / TC_SEG);
     const int nparts = row_parts(ctx->sm_count / n_slabs, n_kept_max, TC_ROUND_ROWS);   // at least a round of rows per part
     static_assert(TC_N * 256 <= DIP_MAIL_FLOATS, "");        // (parts only with one CTA per SM: the mail boxes suffice)
-    p.defer = 0;
+    p.defer = nparts >= TC_APART_PARTS && nparts * p.batch >= TC_APART_KB;
     p.part_base = 0;
+    if (p.defer) {
+        if ((size_t)nparts * n_slabs * p.batch * 256 > ctx->partials_floats) return DIP_ERR_WORKSPACE;
+        p.key_coarse = nullptr;                              // (nobody in this launch sees h)
+    }
     TcParams q;
     q.n_slabs = n_slabs;
     q.nparts = nparts;
@@ -426,5 +439,6 @@ dip_status dip_launch_gemv_tc(dip_ctx *ctx, GemvParams &p, int which, int n_kept
         DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once[1], ctx->device, gemv_tc_kernel<1>, smem));
         DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_tc_kernel<1>, dim3(n_slabs * nparts), dim3(TC_THREADS), smem, stream, p, q));
     }
+    if (p.defer) return dip_launch_combine_parts(ctx, which, nparts, n_slabs, p.batch, 256, 8, p.batch, p.d_out, p.out, stream);
     return DIP_OK;
 }

@@ -12,7 +12,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("d_model,d_ff,batches", [(256, 8224, (3, 5, 16)), (1056, 2080, tuple(range(3, 17))), (288, 19008, (4, 9))])
+@pytest.mark.parametrize("d_model,d_ff,batches", [(256, 8224, (3, 5, 16)), (1056, 2080, tuple(range(3, 17))), (288, 19008, (4, 9)), (288, 6176, (5, 6, 8))])
 def test_batched_products_from_masks(d_model, d_ff, batches):
     import paper_2412_01380_b200 as dip
     ctx = dip.Context(0)
@@ -90,3 +90,16 @@ def test_a_short_limit_for_copies_bounds_copies_only():
     want = torch.nn.functional.silu(x @ mats[0].double().t()) * (x @ mats[1].double().t())
     assert rel_err(out.cpu().numpy(), want.cpu().numpy()) <= REL_TOL
     ctx.close()
+
+
+@pytest.mark.parametrize("d_model,batch,k", [(256, 16, 4096), (256, 16, 1024), (256, 8, 1024), (1024, 16, 4096)])
+def test_many_parts_of_many_tokens_are_not_one_blocks_work(d_model, batch, k):
+    """The parts of 3 tokens and of many: what lies between the two times is the collecting of the parts (15 us and more by one block)."""
+    import paper_2412_01380_b200 as dip
+    us = {}
+    for b in (3, batch):
+        ctx, _, call, _ = _product(dip, d_model, 8192, 1, b, k)
+        us[b] = graph_us(call)
+        assert ctx.device_status() == 0
+        ctx.close()
+    assert us[batch] < us[3] + (2 if batch == 16 else 0.7), us
