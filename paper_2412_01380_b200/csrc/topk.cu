@@ -82,8 +82,8 @@ select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, f
     }
     for (int w = tid; w < n_words; w += TK_THREADS) mask_bits[w] = s_maskw[w];
     if (idx_out) {
-        int32_t *o = idx_out + (size_t)row * k;
-        list_mask(s_maskw, d, s, [&](int r, int col) { o[r] = col; });
+        static_assert(sizeof(f.hist) >= sizeof(uint16_t) * DIP_MAX_D, "the list fits where the histogram was");
+        write_list(s_maskw, d, k, s, reinterpret_cast<uint16_t *>(f.hist), idx_out + (size_t)row * k);
     }
     if constexpr (THEN == THEN_UPDATE) {
         cache_update_clear(s, f.hist);
@@ -148,10 +148,7 @@ select_fine_coarse_kernel(const float *__restrict__ x, const uint16_t *__restric
     __syncthreads();                                                  // histogram zeroed
     select_fine_coarse<CA>(coarse, x, stamp, gamma, d, k, keys, s, f, s_maskw);
     for (int w = tid; w < (d >> 5); w += TK_THREADS) mask_bits[w] = s_maskw[w];
-    if (idx_out) {
-        int32_t *o = idx_out + (size_t)row * k;
-        list_mask(s_maskw, d, s, [&](int r, int col) { o[r] = col; });
-    }
+    if (idx_out) write_list(s_maskw, d, k, s, reinterpret_cast<uint16_t *>(f.hist), idx_out + (size_t)row * k);
     DIP_TRACE_MAX(tr, 2);
 }
 
