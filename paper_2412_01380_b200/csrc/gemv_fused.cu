@@ -48,7 +48,7 @@ struct FusedParams {
     int ahead;                   // the columns of how many threads (of each part's 1024 / nparts) have their rows asked for
                                  // as soon as the threshold's bin is known
     int early;                   // gate/up, chained: of how many threads before that, if their keys are larger than
-    uint32_t sure;               // this: rms is 1, so fewer than k columns can be larger than sqrt(d / k)
+    uint32_t sure;               // this: rms is 1, so fewer than k columns can be larger than sqrt(d / k) (times gamma, where that is above 1)
     uint32_t by_prod;            // ceil(2^32 / blocks with rows)
     int x_near;                  // gate/up: room in shared memory for the values of x
     float *out;
@@ -743,7 +743,9 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
     // (of Laplace or Student-t inputs a quarter of the kept columns are that large, hence the quarter)
     p.early = 0;
     if (norm && p.ahead) p.early = GF_EARLY_BYTES < bytes / 4 ? (int)(TK_THREADS * GF_EARLY_BYTES / (bytes / 4)) : TK_THREADS;
-    const float sure = sqrtf((float)p.d_in / (float)sel->k) * 1.001f;
+    // (a gamma of 64 and nothing resident, two blocks of 4096 / 11008 at keep ratio 0.25: 63.8 us where every row with a key above
+    // sqrt(d / k) was asked for, 52.9 with gamma 1)
+    const float sure = sqrtf((float)p.d_in / (float)sel->k) * 1.001f * (sel->stamp ? fmaxf(1.0f, sel->gamma) : 1.0f);
     memcpy(&p.sure, &sure, sizeof(sure));
     p.by_prod = (uint32_t)((0x100000000ull + (unsigned)(p.n_slabs * p.nparts) - 1) / (unsigned)(p.n_slabs * p.nparts));
     p.xa = sel->xa;

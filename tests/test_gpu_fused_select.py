@@ -8,7 +8,7 @@ import pytest
 
 import dip_inputs as di
 import oracle
-from gpu_util import REL_TOL, bits_to_mask, check_step, rel_err, upload_layer
+from gpu_util import REL_TOL, bits_to_mask, check_step, graph_us, rel_err, upload_layer
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -274,3 +274,28 @@ def test_values_that_are_not_finite(wtype, where):
     for a, b in ((h0, h1), (y0, y1)):
         ok = np.isfinite(a)
         assert np.array_equal(a[~ok], b[~ok], equal_nan=True) and (not ok.any() or rel_err(a[ok], b[ok]) <= REL_TOL)
+
+
+def test_rows_asked_for_before_the_select_are_kept_rows_for_every_gamma():
+    """With nothing resident a gamma of 64 is a factor of all keys: the masks are those of gamma 1, and so are the rows that are read
+    (asked for by the key alone, 4096 rows of 44 KB instead of 1024 were: 135 MB, 20 us and more)."""
+    import paper_2412_01380_b200 as dip
+    ctx = dip.Context(0)
+    d_model, d_ff = 4096, 11008
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    layers = []
+    for _ in range(2):
+        mats = [torch.randn(s, generator=gen, device="cuda").mul_(0.02).bfloat16() for s in ((d_ff, d_model), (d_ff, d_model), (d_model, d_ff))]
+        layers.append(dip.dip_pack_weights(ctx, dip.W_BF16, d_model, d_ff, *mats))
+    x = torch.randn(d_model, generator=gen, device="cuda")
+    us, out = {}, {}
+    for gamma in (1.0, 64.0):
+        caches = [[dip.CacheState(d, 0, "cuda") for _ in layers] for d in (d_model, d_ff)]
+        stack = dip.Stack(layers, *caches)
+        out[gamma] = torch.empty_like(x)
+        us[gamma] = graph_us(lambda: dip.dip_stack_step(ctx, stack, x, d_model // 4, d_ff // 4, gamma, out[gamma]))
+    assert torch.equal(out[1.0], out[64.0])
+    assert us[64.0] < us[1.0] + 8, us
+    assert ctx.device_status() == 0
+    ctx.close()
