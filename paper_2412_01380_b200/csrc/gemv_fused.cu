@@ -172,12 +172,12 @@ __device__ __forceinline__ void stream_rows(const uint16_t *idx, int first, int 
 
 // Block part * n_slabs + slab owns segment `slab`, row part `part`.  UPD: then come the blocks without rows, one
 // for each cache of u.beside, and last the one that completes the mask and updates this input's cache.  NQ =
-// chunks of columns per thread (gate/up: 4 columns each, down: 8).  Dynamic shared memory: FusedSmem, then d_in
+// chunks of columns per thread (gate/up: 4 columns each, down: 8).  AHEAD: rows are asked for ahead.  Dynamic shared memory: FusedSmem, then d_in
 // words (rounded up to four: the CTA's row list; the updating block's copy of the stamps; under heavy ties the rank
 // keys before that), then for gate/up (x_near) the d_in values of x.  Shared memory is kept small: what it does not
 // take is L1, which the rows in flight pass through (with the 72 KB of h beside the rest, 224 KB in all, the down
 // product of 17920 dense rows took 11 us longer).
-template <int WT, int WHICH, bool CA, bool NORM, int NQ, bool UPD>
+template <int WT, int WHICH, bool CA, bool NORM, int NQ, bool UPD, bool AHEAD>
 __global__ void __launch_bounds__(TK_THREADS, 1)
 gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdates, Int<0>> u)
 {
@@ -297,7 +297,7 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
                 kk[j][1] = rank_key<CA>(r[j].y, st[j].y, p.gamma);
                 kk[j][2] = rank_key<CA>(r[j].z, st[j].z, p.gamma);
                 kk[j][3] = rank_key<CA>(r[j].w, st[j].w, p.gamma);
-                if (NORM && tid < p.early && mine(q)) {
+                if (AHEAD && NORM && tid < p.early && mine(q)) {
 #pragma unroll
                     for (int t = 0; t < 4; ++t)
                         if (kk[j][t] > p.sure) l2_prefetch(p.W + (size_t)(4 * q + t) * p.row_bytes, (unsigned)p.row_bytes);
@@ -348,7 +348,7 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
         // Phi-3-Medium blocks, graph, us: none at all 110; gate/up only, 15 MB here 108.0, 10 MB here and up to 25 MB early 105.5; with 16 MB
         // for down, too, 103.1 (12 MB 103.3, 7 or 13 MB for gate/up 103.4 and 104.1).  What is still under way when the
         // first rows are waited for delays them
-        if (((tid * nparts) & (TK_THREADS - 1)) < p.ahead) {
+        if (AHEAD && ((tid * nparts) & (TK_THREADS - 1)) < p.ahead) {
 #pragma unroll
             for (int j = 0; j < NQ; ++j) {
                 const int q = tid + j * TK_THREADS;
@@ -567,15 +567,24 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
     DIP_TRACE_MAX(p.tr, 2);
 }
 
+template <int WT, int WHICH, bool CA, bool NORM, int NQ, bool UPD, bool AHEAD>
+dip_status launch_fused_as(dip_ctx *ctx, const FusedParams &p, const std::conditional_t<UPD, FusedUpdates, Int<0>> &u, int extra,
+                           size_t smem, cudaStream_t stream)
+{
+    static dip_per_device_once once;
+    const auto kernel = gemv_fused_kernel<WT, WHICH, CA, NORM, NQ, UPD, AHEAD>;
+    DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once, ctx->device, kernel, GF_SMEM_LIMIT));
+    DIP_CUDA_TRY(ctx, dip_launch_pdl(kernel, dim3(p.n_slabs * p.nparts + extra), dim3(TK_THREADS), smem, stream, p, u));
+    return DIP_OK;
+}
+
+// (launches that ask for no rows ahead do without that code: 2048 / 8192, BF16, keep ratio 0.1, steps with other weights each, 13.6 us with it and 13.1 without)
 template <int WT, int WHICH, bool CA, bool NORM, int NQ, bool UPD>
 dip_status launch_fused(dip_ctx *ctx, const FusedParams &p, const std::conditional_t<UPD, FusedUpdates, Int<0>> &u, int extra,
                         size_t smem, cudaStream_t stream)
 {
-    static dip_per_device_once once;
-    DIP_CUDA_TRY(ctx, dip_raise_smem_limit(once, ctx->device, gemv_fused_kernel<WT, WHICH, CA, NORM, NQ, UPD>, GF_SMEM_LIMIT));
-    DIP_CUDA_TRY(ctx, dip_launch_pdl(gemv_fused_kernel<WT, WHICH, CA, NORM, NQ, UPD>, dim3(p.n_slabs * p.nparts + extra),
-                                     dim3(TK_THREADS), smem, stream, p, u));
-    return DIP_OK;
+    return p.ahead ? launch_fused_as<WT, WHICH, CA, NORM, NQ, UPD, true>(ctx, p, u, extra, smem, stream)
+                   : launch_fused_as<WT, WHICH, CA, NORM, NQ, UPD, false>(ctx, p, u, extra, smem, stream);
 }
 
 // Columns per thread: a row's keys stay in registers, so the variant for wide inputs (which spills) only takes
@@ -739,7 +748,8 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
     // (a product of little more bytes than that gains nothing, and 0.4 us go into asking: three blocks of 3072 / 8192 61.9 us with 12 of
     // the 12.6 MB of a down product asked for, 61.1 without)
     const double bytes = (double)p.row_bytes * sel->k, ahead = which == 0 ? GF_AHEAD_BYTES : GF_AHEAD_DOWN_BYTES;
-    p.ahead = 2 * ahead < bytes ? (int)(TK_THREADS * ahead / bytes) : 0;
+    // (and where every column is kept nothing is searched for: three dense blocks of 4096 / 11008 181.8 us with rows asked for early, 179.4 without)
+    p.ahead = 2 * ahead < bytes && sel->k < p.d_in ? (int)(TK_THREADS * ahead / bytes) : 0;
     // (of Laplace or Student-t inputs a quarter of the kept columns are that large, hence the quarter)
     p.early = 0;
     if (norm && p.ahead) p.early = GF_EARLY_BYTES < bytes / 4 ? (int)(TK_THREADS * GF_EARLY_BYTES / (bytes / 4)) : TK_THREADS;
