@@ -34,7 +34,8 @@ namespace {
 constexpr int GF_SEG = 512;
 constexpr int GF_NW = TK_THREADS / 32;     // 32 warps
 constexpr int GF_U = 4;                    // loads in flight per lane
-constexpr double GF_AHEAD_BYTES = 10e6;        // rows asked for once the threshold's bin is known: gate/up,
+constexpr double GF_AHEAD_BYTES = 15e6;        // rows asked for once the threshold's bin is known: gate/up,
+constexpr double GF_AHEAD_MORE_BYTES = 12e6;   // gate/up that has asked for some before,
 constexpr double GF_AHEAD_DOWN_BYTES = 16e6;   // down,
 constexpr double GF_EARLY_BYTES = 25e6;        // and before that (see `early`)
 constexpr size_t GF_SMEM_LIMIT = (size_t)224 * 1024;   // dynamic shared memory a launch may ask for
@@ -45,11 +46,11 @@ struct FusedParams {
     size_t row_bytes;
     int d_in, d_out;
     int n_slabs, nparts;
-    int ahead;                   // the columns of how many threads (of each part's 1024 / nparts) have their rows asked for
-                                 // as soon as the threshold's bin is known
-    int early;                   // gate/up, chained: of how many threads before that, if their keys are larger than
+    int ahead, ahead_of;         // the rows of how many groups of columns out of how many (the parts together) are asked for as soon
+                                 // as the threshold's bin is known; see there
+    int early;                   // gate/up, chained: of how many groups before that, if their keys are larger than
     uint32_t sure;               // this: rms is 1, so fewer than k columns can be larger than sqrt(d / k) (times gamma, where that is above 1)
-    uint32_t by_prod;            // ceil(2^32 / blocks with rows)
+    uint32_t by_prod, by_ahead;  // ceil(2^32 / n), n = blocks with rows; ahead_of
     int x_near;                  // gate/up: room in shared memory for the values of x
     float *out;
     float *mail;                 // [nparts][n_slabs][segment elements]; DIP_MAIL_EMPTY outside a launch
@@ -250,6 +251,8 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
 
     // ---- the rank keys of the input and their histogram, in every CTA ----
     const int n_q = p.d_in / W;
+    // groups of the threads before this one: the list has the threads' columns in thread order
+    const int before = tid * (n_q / TK_THREADS) + min(tid, n_q % TK_THREADS);
     uint32_t kk[NQ][4];                    // gate/up: full keys of four columns; down: 16-bit keys of eight
     if constexpr (WHICH == 0) {
         // one trip to memory for x (or the two vectors that make it) and the stamps
@@ -297,7 +300,7 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
                 kk[j][1] = rank_key<CA>(r[j].y, st[j].y, p.gamma);
                 kk[j][2] = rank_key<CA>(r[j].z, st[j].z, p.gamma);
                 kk[j][3] = rank_key<CA>(r[j].w, st[j].w, p.gamma);
-                if (AHEAD && NORM && tid < p.early && mine(q)) {
+                if (AHEAD && NORM && before < p.early && mine(q)) {
 #pragma unroll
                     for (int t = 0; t < 4; ++t)
                         if (kk[j][t] > p.sure) l2_prefetch(p.W + (size_t)(4 * q + t) * p.row_bytes, (unsigned)p.row_bytes);
@@ -343,12 +346,13 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
         const uint32_t b = (uint32_t)s.ts.bcast[0];
         krem = s.ts.bcast[1];
         n_c = s.ts.bcast[2];
-        // The first rows of each part on their way to L2 while the list is made (which has the threads' columns in thread
-        // order): whole rows, and of chained gate/up inputs the surely kept ones before that.  As many as come in that time.  Three
-        // Phi-3-Medium blocks, graph, us: none at all 110; gate/up only, 15 MB here 108.0, 10 MB here and up to 25 MB early 105.5; with 16 MB
-        // for down, too, 103.1 (12 MB 103.3, 7 or 13 MB for gate/up 103.4 and 104.1).  What is still under way when the
-        // first rows are waited for delays them
-        if (AHEAD && ((tid * nparts) & (TK_THREADS - 1)) < p.ahead) {
+        // Rows of each part on their way to L2 while the list is made: whole rows, and of chained gate/up inputs the surely kept ones
+        // before that.  As many as come in that time; what is still under way when the first rows are waited for delays them.  Three
+        // Phi-3-Medium blocks, graph, us: none at all 111; gate/up only, 15 MB 108; with up to 25 MB before that 105; and 16 MB for
+        // down 104.  Gate/up: the first rows of each part.  Down: of the threads as if they had equally many groups each, which
+        // is some way into the list for most parts (at their very starts: one step of 5120 / 17920 33.0 us, 32.7 like this)
+        const unsigned at = (unsigned)((WHICH == 0 ? before : tid) * nparts);
+        if (AHEAD && at - __umulhi(at, p.by_ahead) * p.ahead_of < (unsigned)p.ahead) {
 #pragma unroll
             for (int j = 0; j < NQ; ++j) {
                 const int q = tid + j * TK_THREADS;
@@ -356,7 +360,7 @@ gemv_fused_kernel(const FusedParams p, const std::conditional_t<UPD, FusedUpdate
 #pragma unroll
                     for (int t = 0; t < W; ++t) {
                         bool ask;
-                        if constexpr (WHICH == 0) ask = kk[j][t] > ((b << 16) | 0xffffu) && !(NORM && tid < p.early && kk[j][t] > p.sure);
+                        if constexpr (WHICH == 0) ask = kk[j][t] > ((b << 16) | 0xffffu) && !(NORM && before < p.early && kk[j][t] > p.sure);
                         else ask = ((kk[j][t >> 1] >> (16 * (t & 1))) & 0xffffu) > b;
                         if (ask) l2_prefetch(p.W + (size_t)(W * q + t) * p.row_bytes, (unsigned)p.row_bytes);
                     }
@@ -745,14 +749,24 @@ dip_status dip_launch_gemv_fused(dip_ctx *ctx, const dip_mlp_weights *w, int whi
         p.key_gamma = keys->gamma;
         keys->written = 1;
     }
-    // (a product of little more bytes than that gains nothing, and 0.4 us go into asking: three blocks of 3072 / 8192 61.9 us with 12 of
-    // the 12.6 MB of a down product asked for, 61.1 without)
-    const double bytes = (double)p.row_bytes * sel->k, ahead = which == 0 ? GF_AHEAD_BYTES : GF_AHEAD_DOWN_BYTES;
-    // (and where every column is kept nothing is searched for: three dense blocks of 4096 / 11008 181.8 us with rows asked for early, 179.4 without)
-    p.ahead = 2 * ahead < bytes && sel->k < p.d_in ? (int)(TK_THREADS * ahead / bytes) : 0;
+    // Whether rows are asked for ahead, and how many.  Gate/up: from 8 MB on, all rows if there are no more (less gains nothing: keep
+    // ratio 0.1 of 2048 / 8192, 6.7 MB).  One step, BF16, each with other weights: 3072 / 8192 with 10 MB 14.37 us without and 13.9
+    // with, 4096 / 11008 with 18 MB 16.3 and 16.1; F32 2048 / 5632, 23 MB, 15.9 with 15 MB and 16.6 with 20.  The surely kept rows before
+    // that from 20 MB on (3072 / 8192, 25 MB, twelve chained blocks 19.0 us a block without and 18.6 with; 17 MB 16.5 either way) and from
+    // a fifth of the columns kept: of a tenth, few are that large.  Down: from 32 MB on (22 MB, 4096 / 11008, step 23.6 us without
+    // and 24.0 with; 46 MB, 5120 / 17920, 32.9 and 32.3).  Where every column is kept nothing is searched for (three dense blocks of
+    // 4096 / 11008 181.8 us with rows asked for early, 179.4 without)
+    const int n_q = p.d_in / (which == 0 ? 4 : 8);
+    const double bytes = (double)p.row_bytes * sel->k;
+    const bool early = norm && bytes > 20e6 && 5 * (long long)sel->k >= p.d_in;
+    const double ahead = which == 1 ? GF_AHEAD_DOWN_BYTES : early ? GF_AHEAD_MORE_BYTES : GF_AHEAD_BYTES;
+    const double from = which == 1 ? 2 * GF_AHEAD_DOWN_BYTES : 8e6;
+    p.ahead_of = which == 1 && n_q > TK_THREADS ? TK_THREADS : n_q;
+    p.by_ahead = (uint32_t)((0x100000000ull + (unsigned)p.ahead_of - 1) / (unsigned)p.ahead_of);
+    p.ahead = bytes > from && sel->k < p.d_in ? (int)(p.ahead_of * (ahead < bytes ? ahead / bytes : 1.0)) : 0;
     // (of Laplace or Student-t inputs a quarter of the kept columns are that large, hence the quarter)
     p.early = 0;
-    if (norm && p.ahead) p.early = GF_EARLY_BYTES < bytes / 4 ? (int)(TK_THREADS * GF_EARLY_BYTES / (bytes / 4)) : TK_THREADS;
+    if (early && p.ahead) p.early = GF_EARLY_BYTES < bytes / 4 ? (int)(n_q * GF_EARLY_BYTES / (bytes / 4)) : n_q;
     // (a gamma of 64 and nothing resident, two blocks of 4096 / 11008 at keep ratio 0.25: 63.8 us where every row with a key above
     // sqrt(d / k) was asked for, 52.9 with gamma 1)
     const float sure = sqrtf((float)p.d_in / (float)sel->k) * 1.001f * (sel->stamp ? fmaxf(1.0f, sel->gamma) : 1.0f);

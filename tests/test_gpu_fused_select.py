@@ -299,3 +299,23 @@ def test_rows_asked_for_before_the_select_are_kept_rows_for_every_gamma():
     assert us[64.0] < us[1.0] + 8, us
     assert ctx.device_status() == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("policy", [None, "lru"])
+@pytest.mark.parametrize("wtype,d_model,d_ff,rho", [
+    (di.W_BF16, 8224, 1056, 0.23),       # gate/up rows of 8 MB and just above it: all of them are asked for; the wide variant
+    (di.W_BF16, 8224, 1056, 0.24), (di.W_BF16, 4096, 6144, 0.19), (di.W_F32, 2048, 4096, 0.31),   # few kept; 20 MB
+    (di.W_BF16, 1024, 16416, 0.96),      # down rows of 32 MB, with updates beside them
+])
+def test_rows_asked_for_ahead(wtype, d_model, d_ff, rho, policy):
+    import paper_2412_01380_b200 as dip
+    ctx = dip.Context(0)
+    lw = _layer(d_model, d_ff, wtype, 12)
+    w = upload_layer(dip, ctx, lw)
+    k_x, k_h = int(rho * d_model), int(rho * d_ff)
+    refs = [oracle.Cache(d, d // 2, policy) if policy else None for d in (d_model, d_ff)]
+    mine = [dip.CacheState(d, d // 2, "cuda", policy) if policy else None for d in (d_model, d_ff)]
+    for t in range(2):
+        check_step(dip, ctx, lw, w, di.heavy_tail_vector(300 + t, d_model), k_x, k_h, 0.2 if policy else 1.0, *refs, *mine)
+    assert ctx.device_status() == 0
+    ctx.close()
