@@ -58,3 +58,36 @@ def test_slots_outside_the_arena_are_reported_and_not_read():
     dip.dip_mlp_step(ctx, w, x, k_x, k_h, 0.2, c2, None, torch.empty(d_model, device="cuda"), h=want)
     assert torch.allclose(h, want, rtol=1e-4, atol=1e-5 * float(want.abs().max()))    # its columns came from the slow tier
     ctx.close()
+
+
+def test_two_tier_products_round_no_more_than_two_products_did():
+    """Root mean square error of h and y against 64 bits, of the columns that the step kept.  A sum of 256 (704) rows meets at most ten
+    roundings: its chain in a warp, five levels over the warps, the parts with their errors carried along; each is 2.5e-8 rms.  h has two
+    such sums and five roundings of its own: sqrt(25) x 2.5e-8, y sqrt(10) x 2.5e-8, and a third more for what is kept unevenly."""
+    import paper_2412_01380_b200 as dip
+    d_model, d_ff, k_x, k_h = 1024, 2816, 256, 704
+    ctx = dip.Context(0)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(17)
+    mats = [torch.randn(s, generator=gen, device="cuda").mul_(0.02).bfloat16() for s in ((d_ff, d_model), (d_ff, d_model), (d_model, d_ff))]
+    w = dip.dip_pack_weights(ctx, dip.W_BF16, d_model, d_ff, *mats)
+    gate, up, down = [m.double() for m in mats]
+    _, _, t_gu, t_d = _tiers(dip, w, k_x, k_h, 0.5, "lru", False)
+    h, y = torch.empty(d_ff, device="cuda"), torch.empty(d_model, device="cuda")
+    m_x, m_h = [torch.zeros(d // 32, dtype=torch.int32, device="cuda") for d in (d_model, d_ff)]
+
+    def kept(v, bits):
+        return v.double() * ((bits.view(-1, 1) >> torch.arange(32, device="cuda").int()) & 1).view(-1)
+
+    errs = []
+    x = torch.randn(d_model, generator=gen, device="cuda")
+    for _ in range(12):
+        x = 0.95 * x + 0.3 * torch.randn(d_model, generator=gen, device="cuda")
+        dip.dip_mlp_step_tiered(ctx, w, t_gu, t_d, x, k_x, k_h, 0.2, y, mask_x=m_x, h=h, mask_h=m_h)
+        want_h = torch.nn.functional.silu(gate @ kept(x, m_x)) * (up @ kept(x, m_x))
+        want_y = down @ kept(h, m_h)
+        errs.append([float((a.double() - b).norm() / b.norm()) for a, b in ((h, want_h), (y, want_y))])
+    err_h, err_y = np.mean(errs, axis=0)
+    assert err_h <= 4 / 3 * 5 * 2.5e-8 and err_y <= 4 / 3 * 10 ** 0.5 * 2.5e-8, (err_h, err_y)
+    assert ctx.device_status() == 0
+    ctx.close()
