@@ -31,7 +31,7 @@ namespace {
 // bytes this CTA has to pull in are its floor: two bytes per column instead of the eight of value +
 // stamp.  Needs d % 8 == 0 and d <= 8 * TK_COARSE_ITERS * TK_THREADS.
 // Dynamic shared memory: TkFine, then keys[] (d words rounded up to four).
-// idx_out != nullptr: the kept columns of row r as an ascending list at idx_out + r * k.
+// LIST: the kept columns of row r as an ascending list at idx_out + r * k (launches without one do without that code).
 // THEN (one row): THEN_UPDATE: the CTA goes on to update the row's cache (Algorithm 1 whole).  What bounds dip_ca_mask is the chain of
 // its launches (select, update and list were three), and the mask is here in shared memory: masks with lists and list
 // products at 2080 / 5472, four calls in a graph, 36.7 us with ten launches and 28.8 with four.
@@ -41,7 +41,7 @@ namespace {
 constexpr int THEN_NOTHING = 0, THEN_UPDATE = 1, THEN_SPLIT = 2;
 template <int THEN> using ThenArg = std::conditional_t<THEN == THEN_UPDATE, dip_cache_update, std::conditional_t<THEN == THEN_SPLIT, dip_tier, Int<0>>>;
 
-template <bool CA, bool NORM, int THEN>
+template <bool CA, bool NORM, int THEN, bool LIST>
 __global__ void __launch_bounds__(TK_THREADS, 1)
 select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, float *__restrict__ x_out,
                    int d, int k, float gamma, const int32_t *stamp,
@@ -81,7 +81,7 @@ select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, f
         select_fine<CA, NORM>(xa, NORM ? x_out : nullptr, d, k, gamma, stamp, scale, keys, s, f, s_maskw);
     }
     for (int w = tid; w < n_words; w += TK_THREADS) mask_bits[w] = s_maskw[w];
-    if (idx_out) {
+    if constexpr (LIST) {
         static_assert(sizeof(f.hist) >= sizeof(uint16_t) * DIP_MAX_D, "the list fits where the histogram was");
         write_list(s_maskw, d, k, s, reinterpret_cast<uint16_t *>(f.hist), idx_out + (size_t)row * k);
     }
@@ -123,7 +123,7 @@ select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, f
     DIP_TRACE_MAX(tr, 2);
 }
 
-template <bool CA>
+template <bool CA, bool LIST>
 __global__ void __launch_bounds__(TK_THREADS, 1)
 select_fine_coarse_kernel(const float *__restrict__ x, const uint16_t *__restrict__ coarse, int d, int k, float gamma,
                           const int32_t *__restrict__ stamp, uint32_t *__restrict__ mask_bits, int32_t *__restrict__ idx_out,
@@ -148,7 +148,7 @@ select_fine_coarse_kernel(const float *__restrict__ x, const uint16_t *__restric
     __syncthreads();                                                  // histogram zeroed
     select_fine_coarse<CA>(coarse, x, stamp, gamma, d, k, keys, s, f, s_maskw);
     for (int w = tid; w < (d >> 5); w += TK_THREADS) mask_bits[w] = s_maskw[w];
-    if (idx_out) write_list(s_maskw, d, k, s, reinterpret_cast<uint16_t *>(f.hist), idx_out + (size_t)row * k);
+    if constexpr (LIST) write_list(s_maskw, d, k, s, reinterpret_cast<uint16_t *>(f.hist), idx_out + (size_t)row * k);
     DIP_TRACE_MAX(tr, 2);
 }
 
@@ -239,39 +239,34 @@ dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, flo
     if ((update || split) && (coarse || xb)) return DIP_ERR_INVALID_ARG;
     if (idx_out && xb) return DIP_ERR_INVALID_ARG;
     if ((update || split) && (batch != 1 || !stamp)) return DIP_ERR_INVALID_ARG;
+    const bool list = idx_out != nullptr;
     const Int<0> no;
     const size_t smem = sizeof(TkFine) + (size_t)((d + 3) & ~3) * sizeof(uint32_t);
     const dim3 grid(batch), block(TK_THREADS);
     unsigned long long *tr = dip_trace_slot(ctx, d <= 0 ? 0 : (stamp ? 2 : 1));
     cudaError_t e;
+    if (!stamp) gamma = 1.0f;
+    const auto fine = [&](auto *kernel, const auto &then) {
+        return dip_launch_pdl(kernel, grid, block, smem, stream, xa, xb, x_out, d, k, gamma, stamp, mask_bits, idx_out, then, tr);
+    };
+    const auto fine_coarse = [&](auto *kernel) {
+        return dip_launch_pdl(kernel, grid, block, smem, stream, xa, coarse, d, k, gamma, stamp, mask_bits, idx_out, tr);
+    };
     if (coarse) {
         if (xb || (batch != 1 && stamp) || (d & 31)) return DIP_ERR_INVALID_ARG;
-        if (stamp)
-            e = dip_launch_pdl(select_fine_coarse_kernel<true>, grid, block, smem, stream, xa, coarse, d, k, gamma, stamp,
-                               mask_bits, idx_out, tr);
-        else
-            e = dip_launch_pdl(select_fine_coarse_kernel<false>, grid, block, smem, stream, xa, coarse, d, k, 1.0f,
-                               (const int32_t *)nullptr, mask_bits, idx_out, tr);
+        if (stamp) e = list ? fine_coarse(select_fine_coarse_kernel<true, true>) : fine_coarse(select_fine_coarse_kernel<true, false>);
+        else e = list ? fine_coarse(select_fine_coarse_kernel<false, true>) : fine_coarse(select_fine_coarse_kernel<false, false>);
     } else if (xb) {
-        if (stamp)
-            e = dip_launch_pdl(select_fine_kernel<true, true, THEN_NOTHING>, grid, block, smem, stream, xa, xb, x_out, d, k, gamma, stamp,
-                               mask_bits, idx_out, no, tr);
-        else
-            e = dip_launch_pdl(select_fine_kernel<false, true, THEN_NOTHING>, grid, block, smem, stream, xa, xb, x_out, d, k, 1.0f,
-                               (const int32_t *)nullptr, mask_bits, idx_out, no, tr);
+        e = stamp ? fine(select_fine_kernel<true, true, THEN_NOTHING, false>, no) : fine(select_fine_kernel<false, true, THEN_NOTHING, false>, no);
+    } else if (update) {
+        e = list ? fine(select_fine_kernel<true, false, THEN_UPDATE, true>, *update) : fine(select_fine_kernel<true, false, THEN_UPDATE, false>, *update);
+    } else if (split) {
+        if (list) return DIP_ERR_INVALID_ARG;
+        e = fine(select_fine_kernel<true, false, THEN_SPLIT, false>, *split);
+    } else if (stamp) {
+        e = list ? fine(select_fine_kernel<true, false, THEN_NOTHING, true>, no) : fine(select_fine_kernel<true, false, THEN_NOTHING, false>, no);
     } else {
-        if (update)
-            e = dip_launch_pdl(select_fine_kernel<true, false, THEN_UPDATE>, grid, block, smem, stream, xa, (const float *)nullptr,
-                               (float *)nullptr, d, k, gamma, stamp, mask_bits, idx_out, *update, tr);
-        else if (split)
-            e = dip_launch_pdl(select_fine_kernel<true, false, THEN_SPLIT>, grid, block, smem, stream, xa, (const float *)nullptr,
-                               (float *)nullptr, d, k, gamma, stamp, mask_bits, idx_out, *split, tr);
-        else if (stamp)
-            e = dip_launch_pdl(select_fine_kernel<true, false, THEN_NOTHING>, grid, block, smem, stream, xa, (const float *)nullptr,
-                               (float *)nullptr, d, k, gamma, stamp, mask_bits, idx_out, no, tr);
-        else
-            e = dip_launch_pdl(select_fine_kernel<false, false, THEN_NOTHING>, grid, block, smem, stream, xa, (const float *)nullptr,
-                               (float *)nullptr, d, k, 1.0f, (const int32_t *)nullptr, mask_bits, idx_out, no, tr);
+        e = list ? fine(select_fine_kernel<false, false, THEN_NOTHING, true>, no) : fine(select_fine_kernel<false, false, THEN_NOTHING, false>, no);
     }
     DIP_CUDA_TRY(ctx, e);
     return DIP_OK;
@@ -289,14 +284,20 @@ dip_status dip_init_mask_kernels(dip_ctx *ctx)
 {
     const int bytes = DIP_MAX_D * (int)sizeof(uint32_t);
     const int fine_bytes = bytes + (int)sizeof(TkFine);
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false, THEN_UPDATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false, THEN_SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, false, THEN_NOTHING>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<false, false, THEN_NOTHING>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<true, true, THEN_NOTHING>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_kernel<false, true, THEN_NOTHING>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_coarse_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
-    DIP_CUDA_TRY(ctx, cudaFuncSetAttribute(select_fine_coarse_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes));
+    const auto raise = [&](auto *kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes); };
+    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, false, THEN_UPDATE, false>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, false, THEN_UPDATE, true>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, false, THEN_SPLIT, false>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, false, THEN_NOTHING, false>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, false, THEN_NOTHING, true>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<false, false, THEN_NOTHING, false>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<false, false, THEN_NOTHING, true>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, true, THEN_NOTHING, false>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<false, true, THEN_NOTHING, false>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_coarse_kernel<true, false>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_coarse_kernel<true, true>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_coarse_kernel<false, false>));
+    DIP_CUDA_TRY(ctx, raise(select_fine_coarse_kernel<false, true>));
     return DIP_OK;
 }
 
