@@ -101,6 +101,7 @@ __device__ __forceinline__ unsigned long long dip_gtime()
 }
 #define DIP_TRACE_MIN(tr, i) do { if ((tr) && threadIdx.x == 0) atomicMin(&(tr)[i], dip_gtime()); } while (0)
 #define DIP_TRACE_MAX(tr, i) do { if ((tr) && threadIdx.x == 0) atomicMax(&(tr)[i], dip_gtime()); } while (0)
+#define DIP_TRACE_MAX_WARP(tr, i) do { if ((tr) && (threadIdx.x & 31) == 0) atomicMax(&(tr)[i], dip_gtime()); } while (0)   // (of any warp)
 
 // Programmatic dependent launch: a kernel may be scheduled before its predecessor in the stream
 // has finished; it must not touch the predecessor's results before this wait returns.

@@ -245,7 +245,7 @@ tier_fetch_kernel(const TierParams t)
         const int e = (int)(u / per_row);
         copy(t.backing + (size_t)cols[e] * t.row_bytes, t.arena + (size_t)(t.capacity + e) * t.row_bytes, (int)(u % per_row));
     }
-    DIP_TRACE_MAX(t.tr_fetch, 2);
+    DIP_TRACE_MAX_WARP(t.tr_fetch, 2);
     if (!moves_known(t, &go, gridDim.x)) return;
     for (long long u = warp; u < (long long)n * per_row; u += n_warps) {
         const int e = (int)(u / per_row), sl = __ldcg(move + e);
@@ -443,7 +443,7 @@ tier_product_kernel(const TierParams t, const TierProduct p)
                 for (int e = 0; e < E; ++e) acc[e] = fmaf(w[e], xv[u], acc[e]);
             }
         }
-        if (on_misses) DIP_TRACE_MAX(t.tr_fetch, 2);
+        if (on_misses) DIP_TRACE_MAX_WARP(t.tr_fetch, 2);
     }
     DIP_TRACE_MAX(p.tr, 3);            // streaming done
 
