@@ -81,7 +81,8 @@ typedef struct dip_ctx dip_ctx;   /* opaque; owns scratch workspace on one devic
  *   coarse_min_d       smallest d_ff for which a step that runs select kernels in front of its products
  *                      (several tokens, select_in_product < 0, gemv_copy_ring, inputs too wide for
  *                      a thread block's shared memory) ranks h from the 16-bit keys that the gate/up
- *                      product leaves behind: 0 = default (4096), negative = every size.  Products
+ *                      product leaves behind, and a neuron-pruned step p from those that its dense
+ *                      product leaves: 0 = default (4096), negative = every size.  Products
  *                      that select for themselves rank h from those keys at every size.  Either
  *                      way the masks are the same bits.
  *   wait_limit_us      bound of every in-kernel wait on an asynchronous copy, in microseconds (0 =
@@ -125,8 +126,9 @@ const char *dip_last_error(const dip_ctx *ctx);
 /* Number of streaming multiprocessors of the context's device. */
 int dip_sm_count(const dip_ctx *ctx);
 /* Every wait inside a kernel is bounded: on the arrival of an asynchronous copy, and on another thread
- * block of the same launch (the blocks of a one- or two-token product hand their row parts to the
- * block that adds them up; the block that updates a cache waits until the others have read its state).
+ * block of the same launch (the blocks of a product hand their row parts to the block that adds them up; the
+ * block that updates a cache waits until the others have read its state; the blocks of a two-tier launch wait
+ * until it is known which rows move into slots).
  * If a wait runs out, the kernel goes on without what it waited for and a sticky status word on the
  * device becomes non-zero.  From then on the outputs of that call AND OF EVERY LATER CALL on the context
  * are invalid (what came too late is still under way in its workspace) until dip_reset_device_status;
@@ -266,8 +268,8 @@ typedef struct {
     int32_t reserved;
 } dip_cache_state;
 
-/* Self-test of the waits between thread blocks (see dip_device_status): enqueues one kernel in which a row part and a reader of the
- * cache state `st` come too late for the limit.  The status word becomes DIP_DEVICE_WAIT_TIMEOUT and the
+/* Self-test of the waits between thread blocks (see dip_device_status): enqueues two kernels in which row parts, a reader of the
+ * cache state `st` and the word on a two-tier launch's moves come too late for the limit.  The status word becomes DIP_DEVICE_WAIT_TIMEOUT and the
  * workspace is as after a real failure (call dip_reset_device_status); the state, whose update with the mask
  * mask_bits [ceil(st->d/32)] is given up, stays as it is.  1 <= limit_us <= 1000000. */
 dip_status dip_selftest_block_waits(dip_ctx *ctx, int limit_us, const dip_cache_state *st, const uint32_t *mask_bits, void *stream);

@@ -288,7 +288,9 @@ dip_status dip_selftest_block_waits(dip_ctx *ctx, int limit_us, const dip_cache_
 {
     if (!ctx_ok(ctx) || limit_us < 1 || limit_us > 1000000 || !mask_bits || !dip_aligned16(mask_bits)) return DIP_ERR_INVALID_ARG;
     if (!st || st->d < 1 || st->d > DIP_MAX_D || !cache_ok(st, st->d)) return DIP_ERR_INVALID_ARG;
-    return dip_launch_block_waits_selftest(ctx, 1000ull * (unsigned long long)limit_us, dip_update_of(st, mask_bits), (cudaStream_t)stream);
+    const unsigned long long limit_ns = 1000ull * (unsigned long long)limit_us;
+    const dip_status rc = dip_launch_block_waits_selftest(ctx, limit_ns, dip_update_of(st, mask_bits), (cudaStream_t)stream);
+    return rc == DIP_OK ? dip_launch_tier_waits_selftest(ctx, limit_ns, (cudaStream_t)stream) : rc;
 }
 
 // Run cache updates beside the main stream (side stream `which`).

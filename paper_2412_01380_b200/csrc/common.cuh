@@ -31,7 +31,7 @@ struct dip_ctx {
     size_t partials_floats;
     float *mail;         // [sm_count][DIP_MAIL_FLOATS] row parts on their way to the CTA that adds them up
     unsigned int *readers; // [DIP_SYNC_WORDS] zero between launches: CTAs of a fused product that have read the stamps; in a
-                           // two-tier or tensor-core launch: what other CTAs wait for is there, CTAs that have seen it
+                           // two-tier launch: what other CTAs wait for is there, CTAs that have seen it
     // one arrival counter per output slab; zero between launches
     unsigned int *tickets;
     int n_tickets;
@@ -251,6 +251,8 @@ dip_status dip_launch_bounded_wait_selftest(dip_ctx *ctx, unsigned long long lim
 
 // gemv_fused.cu: one kernel whose waits between blocks run out (sets the status word to 1, leaves the cache state as it is).
 dip_status dip_launch_block_waits_selftest(dip_ctx *ctx, unsigned long long limit_ns, const dip_cache_update &c, cudaStream_t stream);
+// tier.cu: the same for the moves of a two-tier launch and the row parts of a tensor-core product.
+dip_status dip_launch_tier_waits_selftest(dip_ctx *ctx, unsigned long long limit_ns, cudaStream_t stream);
 
 // gemv.cu: bit set from an ascending index list.
 dip_status dip_launch_idx_to_mask(dip_ctx *ctx, const int32_t *idx, int n, int d, uint32_t *mask, cudaStream_t stream);

@@ -535,7 +535,32 @@ dip_status launch_product(dip_ctx *ctx, const TierParams &t, TierProduct &p, int
     return DIP_OK;
 }
 
+// Self-test of waits between blocks that run out: for block 0's word on the moves, and for four sums of a row part, which come after that.
+__global__ void __launch_bounds__(TK_THREADS, 1)
+tier_waits_selftest_kernel(const TierParams t, float *mail)
+{
+    __shared__ int go;
+    if (moves_known(t, &go, 1)) atomicExch(t.status, 2);       // (nobody has said anything)
+    if (threadIdx.x == 0) {
+        float4 a[1];
+        mail_take4<1>(mail, 0, 1, a, t.status, t.wait_limit_ns);
+        mail_put4(mail, make_float4(1e30f, 1e30f, 1e30f, 1e30f));
+    }
+}
+
 }  // namespace
+
+dip_status dip_launch_tier_waits_selftest(dip_ctx *ctx, unsigned long long limit_ns, cudaStream_t stream)
+{
+    TierParams t = {};
+    t.moves = ctx->readers + 1;
+    t.through = ctx->readers + 2;
+    t.status = ctx->status;
+    t.wait_limit_ns = limit_ns;
+    tier_waits_selftest_kernel<<<1, TK_THREADS, 0, stream>>>(t, ctx->mail);
+    DIP_CUDA_TRY(ctx, cudaGetLastError());
+    return DIP_OK;
+}
 
 dip_status dip_launch_tier_product(dip_ctx *ctx, const dip_mlp_weights *w, int which, const dip_tier *t, const dip_cache_update &c,
                                    const float *v, int k, float *out, cudaStream_t stream)

@@ -6,7 +6,7 @@ import torch
 
 import dip_inputs as di
 import oracle
-from gpu_util import cache_equal, check_step, upload_layer
+from gpu_util import REL_TOL, cache_equal, check_step, rel_err, upload_layer
 
 pytestmark = pytest.mark.gpu
 
@@ -223,6 +223,42 @@ def test_a_stack_with_a_bad_block_launches_nothing(dip, wtype):
         dip.dip_stack_step(c, dip.Stack(ws, *caches), x, 64, 160, 0.2, y)
         torch.cuda.synchronize()
         assert all(int(s.meta[1]) == 1 for half in caches for s in half) and c.device_status() == dip.DEVICE_OK
+    finally:
+        torch.cuda.synchronize()
+        c.close()
+
+
+def test_every_kind_of_block_wait_runs_out(dip):
+    """The self-test's waits come one after another where they are of another kind (row parts and readers; the moves of a two-tier launch;
+    row parts four sums at a time): each takes its limit.  After a reset a two-tier step and a batch, which use the same words and
+    boxes, are right."""
+    c = dip.Context(0)
+    try:
+        d_model, d_ff, k_x, k_h = 512, 2048, 256, 1024
+        lw = di.layer_weights(di.WORKLOADS["phi3_mini"].scaled(seed=6, d_model=d_model, d_ff=d_ff, n_layers=1), 0)
+        w = upload_layer(dip, c, lw)
+        st, bits = dip.CacheState(d_ff, d_ff // 2, "cuda"), torch.zeros(d_ff // 32, dtype=torch.int32, device="cuda")
+        limit_us = 3000
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        c.selftest_block_waits(limit_us, st, bits)
+        b.record()
+        assert c.device_status() == dip.DEVICE_WAIT_TIMEOUT
+        assert 3 * limit_us <= a.elapsed_time(b) * 1e3 <= 4 * limit_us
+        c.reset_device_status()
+
+        refs = [oracle.Cache(n, n // 2) for n in (d_model, d_ff)]
+        mine = [dip.CacheState(n, n // 2, "cuda") for n in (d_model, d_ff)]
+        tiers = [dip.Tier(s, p.cpu().pin_memory(), p.numel() // s.d, k, "cuda") for s, p, k in zip(mine, (w.gate_up, w.down), (k_x, k_h))]
+        for t in range(2):
+            check_step(dip, c, lw, w, di.heavy_tail_vector(60 + t, d_model), k_x, k_h, 0.2, *refs, *mine, tiers=tiers)
+        xs = np.stack([di.heavy_tail_vector(70 + t, d_model) for t in range(4)])
+        ys, y = torch.empty((4, d_model), device="cuda"), torch.empty(d_model, device="cuda")
+        dip.dip_mlp_step(c, w, torch.from_numpy(xs).cuda(), k_x, k_h, 1.0, None, None, ys)
+        for t in range(4):
+            dip.dip_mlp_step(c, w, torch.from_numpy(xs[t]).cuda(), k_x, k_h, 1.0, None, None, y)
+            assert rel_err(ys[t].cpu().numpy(), y.cpu().numpy()) <= REL_TOL
+        assert c.device_status() == dip.DEVICE_OK
     finally:
         torch.cuda.synchronize()
         c.close()
