@@ -12,7 +12,7 @@
 constexpr int DIP_RING_LAYERS = 128;
 constexpr int DIP_TRACE_SLOTS = 1024;
 constexpr uint32_t DIP_MAIL_EMPTY = 0xffffffffu;
-constexpr int DIP_SYNC_WORDS = 3;
+constexpr int DIP_SYNC_WORDS = 2;
 constexpr int DIP_MAIL_FLOATS = 4096;  // boxes per SM: one CTA's segment of sums (INT4: up to 2048, F32 / BF16: 256 per token)
 constexpr int DIP_TRACE_WORDS = 4;   // first start, dependency ready, last end, auxiliary
 
@@ -30,8 +30,8 @@ struct dip_ctx {
     float *partials;
     size_t partials_floats;
     float *mail;         // [sm_count][DIP_MAIL_FLOATS] row parts on their way to the CTA that adds them up
-    unsigned int *readers; // [DIP_SYNC_WORDS] zero between launches: CTAs of a fused product that have read the stamps; in a
-                           // two-tier launch: what other CTAs wait for is there, CTAs that have seen it
+    unsigned int *readers; // [DIP_SYNC_WORDS] CTAs of a fused product that have read the stamps, zero between launches; whether the
+                           // moves of a two-tier launch are known, zero from the select in front of it on
     // one arrival counter per output slab; zero between launches
     unsigned int *tickets;
     int n_tickets;

@@ -32,8 +32,7 @@ struct TierParams {
     char *arena;
     unsigned long long *counters;
     dip_cache_update cache;
-    unsigned int *moves;       // 1 once fetch[1] and the moves are there; zero between launches
-    unsigned int *through;     // blocks that need `moves` no more; zero between launches
+    unsigned int *moves;       // 1 once fetch[1] and the moves are there; the select in front of the launch has made it 0
     int *status;
     unsigned long long wait_limit_ns;
     unsigned long long *tr_book, *tr_fetch;
@@ -161,20 +160,10 @@ __device__ __forceinline__ void assign_slots(const TierParams &t, BookSmem &s)
     }
 }
 
-// This block needs the moves no more; the last of n such blocks makes the words ready for the next launch.  One thread.
-__device__ __forceinline__ void through(const TierParams &t, unsigned int n)
-{
-    __threadfence();
-    if (atomicAdd(t.through, 1u) == n - 1) {
-        *t.moves = 0u;
-        *t.through = 0u;
-    }
-}
-
 // Block 0 of a launch: update, slots, moves.  In line, though its registers do not fit beside the product's (364 to 392 bytes of spills): as a
 // function of its own that spills nothing it is slower to call than the spills are (one step, keep ratio 0.25, budget 0.5: BF16 3072 / 8192
 // 30.9 us in line and 32.6, 5120 / 17920 52.2 and 54.6).
-__device__ __forceinline__ void keep_books(const TierParams &t, BookSmem &s, unsigned int n_blocks)
+__device__ __forceinline__ void keep_books(const TierParams &t, BookSmem &s)
 {
     const dip_cache_update &c = t.cache;
     DIP_TRACE_MIN(t.tr_book, 0);
@@ -188,28 +177,26 @@ __device__ __forceinline__ void keep_books(const TierParams &t, BookSmem &s, uns
     if (threadIdx.x == 0) {
         __threadfence();
         count_one(t.moves);
-        through(t, n_blocks);
     }
     DIP_TRACE_MAX(t.tr_book, 2);
 }
 
 // The blocks that move rows wait here for block 0, which has started before them (blocks start in index order).  False (and
 // status 1) if that takes longer than the limit: then the slot table may name rows that have not moved.
-__device__ __forceinline__ bool moves_known(const TierParams &t, int *go, unsigned int n_blocks)
+__device__ __forceinline__ bool moves_known(const TierParams &t, int *go)
 {
-    if (threadIdx.x == 0) {
-        *go = wait_count(t.moves, 1u, t.status, t.wait_limit_ns);
-        through(t, n_blocks);
-    }
+    if (threadIdx.x == 0) *go = wait_count(t.moves, 1u, t.status, t.wait_limit_ns);
     __syncthreads();
     return *go != 0;
 }
 
 // ---------------------------------------------------------------------------------------------
-// tier_fetch_kernel: block 0 keeps the books, the other warps copy the missing rows from the slow tier into the staging rows,
-// 2 KB a time (16 bytes per lane, four loads in flight; plain loads, since the source may be host memory mapped into the device's
-// address space), and then move their pieces of those that the cache keeps.  A megabyte in flight covers the
-// host link many times over, and the other SMs are the product's.
+// tier_fetch_kernel: block 0 keeps the books, the other warps copy the missing rows from the slow tier into the staging rows and, of
+// those that the cache keeps, into their slots, 2 KB a time (16 bytes per lane, four loads in flight; plain loads, since the source may be host
+// memory mapped into the device's address space).  A megabyte in flight covers the host link many times over, and
+// the other SMs are the product's.  The product of the misses waits for this launch, so nothing may stand behind its last read: a warp
+// waits for block 0 while its first piece is under way (10 us, the reads take 30) and has both places of each piece then.  With a second
+// pass that moved staged rows to their slots a step of 4096 / 14336 with 4-bit weights took 99.2 us, 92.5 like this (nine launches: 96.9).
 // ---------------------------------------------------------------------------------------------
 constexpr int TF_PIECE = 2048;
 
@@ -217,9 +204,8 @@ __global__ void __launch_bounds__(TK_THREADS, 1)
 tier_fetch_kernel(const TierParams t)
 {
     __shared__ BookSmem s;
-    __shared__ int go;
     if (blockIdx.x == 0) {
-        keep_books(t, s, gridDim.x);
+        keep_books(t, s);
         return;
     }
     DIP_TRACE_MIN(t.tr_fetch, 0);
@@ -230,29 +216,37 @@ tier_fetch_kernel(const TierParams t)
     const int32_t *cols = t.fetch + 4, *move = t.fetch + 4 + t.staging;
     const int n = min(t.fetch[0], t.staging);
     const int per_row = (int)((t.row_bytes + TF_PIECE - 1) / TF_PIECE);
-    const auto copy = [&](const char *src, char *dst, int piece) {
-        uint4 q[TF_PIECE / 512];
+    const auto load = [&](const char *src, int piece, uint4 (&q)[TF_PIECE / 512]) {
 #pragma unroll
         for (int j = 0; j < TF_PIECE / 512; ++j) {
             const size_t at = (size_t)piece * TF_PIECE + j * 512 + lane * 16;
             if (at < t.row_bytes) q[j] = __ldcs(reinterpret_cast<const uint4 *>(src + at));
         }
+    };
+    const auto store = [&](int row, int piece, const uint4 (&q)[TF_PIECE / 512]) {
+        char *dst = t.arena + (size_t)row * t.row_bytes;
 #pragma unroll
         for (int j = 0; j < TF_PIECE / 512; ++j) {
             const size_t at = (size_t)piece * TF_PIECE + j * 512 + lane * 16;
             if (at < t.row_bytes) *reinterpret_cast<uint4 *>(dst + at) = q[j];
         }
     };
+    bool asked = false, known = false;
     for (long long u = warp; u < (long long)n * per_row; u += n_warps) {
-        const int e = (int)(u / per_row);
-        copy(t.backing + (size_t)cols[e] * t.row_bytes, t.arena + (size_t)(t.capacity + e) * t.row_bytes, (int)(u % per_row));
+        const int e = (int)(u / per_row), piece = (int)(u % per_row);
+        uint4 q[TF_PIECE / 512];
+        load(t.backing + (size_t)cols[e] * t.row_bytes, piece, q);
+        if (!asked) {                  // (if that takes longer than the limit, the slot table may name rows that are not there)
+            asked = true;
+            int go = 0;
+            if (lane == 0) go = wait_count(t.moves, 1u, t.status, t.wait_limit_ns);
+            known = __shfl_sync(0xffffffffu, go, 0) != 0;
+        }
+        const int sl = known ? __ldcg(move + e) : -1;
+        store(t.capacity + e, piece, q);
+        if (sl >= 0) store(sl, piece, q);
     }
     DIP_TRACE_MAX_WARP(t.tr_fetch, 2);
-    if (!moves_known(t, &go, gridDim.x)) return;
-    for (long long u = warp; u < (long long)n * per_row; u += n_warps) {
-        const int e = (int)(u / per_row), sl = __ldcg(move + e);
-        if (sl >= 0) copy(t.arena + (size_t)(t.capacity + e) * t.row_bytes, t.arena + (size_t)sl * t.row_bytes, (int)(u % per_row));
-    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -339,7 +333,7 @@ tier_product_kernel(const TierParams t, const TierProduct p)
     constexpr int OUT_PER_SLAB = WHICH == 0 ? SLAB / 2 : SLAB;
     extern __shared__ __align__(16) unsigned char dyn[];
     if (blockIdx.x == 0) {
-        keep_books(t, *reinterpret_cast<BookSmem *>(dyn), gridDim.x);
+        keep_books(t, *reinterpret_cast<BookSmem *>(dyn));
         return;
     }
     ProductSmem &s = *reinterpret_cast<ProductSmem *>(dyn);
@@ -482,7 +476,7 @@ tier_product_kernel(const TierParams t, const TierProduct p)
         }
     }
     // ---- 5. this block's pieces of the staged rows that the cache keeps, into their slots ----
-    if (!moves_known(t, &s.go, gridDim.x)) return;            // (the barrier inside: all pieces are staged)
+    if (!moves_known(t, &s.go)) return;            // (the barrier inside: all pieces are staged)
     const int32_t *move = t.fetch + 4 + t.staging;
     for (int r1 = lo[1] + warp; r1 < hi[1]; r1 += TK_WARPS * TP_U) {
         int to[TP_U];
@@ -516,7 +510,6 @@ TierParams tier_params(dip_ctx *ctx, const dip_tier *t, const dip_cache_update &
     p.counters = t->counters;
     p.cache = c;
     p.moves = ctx->readers + 1;
-    p.through = ctx->readers + 2;
     p.status = ctx->status;
     p.wait_limit_ns = ctx->block_wait_ns;
     p.tr_book = dip_trace_slot(ctx, 6);
@@ -542,7 +535,8 @@ __global__ void __launch_bounds__(TK_THREADS, 1)
 tier_waits_selftest_kernel(const TierParams t, float *mail)
 {
     __shared__ int go;
-    if (moves_known(t, &go, 1)) atomicExch(t.status, 2);       // (nobody has said anything)
+    if (threadIdx.x == 0) *t.moves = 0u;
+    if (moves_known(t, &go)) atomicExch(t.status, 2);          // (nobody has said anything)
     if (threadIdx.x == 0) {
         float4 a[1];
         mail_take4<1>(mail, 0, 1, a, t.status, t.wait_limit_ns);
@@ -556,7 +550,6 @@ dip_status dip_launch_tier_waits_selftest(dip_ctx *ctx, unsigned long long limit
 {
     TierParams t = {};
     t.moves = ctx->readers + 1;
-    t.through = ctx->readers + 2;
     t.status = ctx->status;
     t.wait_limit_ns = limit_ns;
     tier_waits_selftest_kernel<<<1, TK_THREADS, 0, stream>>>(t, ctx->mail);

@@ -40,7 +40,11 @@ namespace {
 // list; their arena rows are the staging rows, in order).
 // ---------------------------------------------------------------------------------------
 constexpr int THEN_NOTHING = 0, THEN_UPDATE = 1, THEN_SPLIT = 2;
-template <int THEN> using ThenArg = std::conditional_t<THEN == THEN_UPDATE, dip_cache_update, std::conditional_t<THEN == THEN_SPLIT, dip_tier, Int<0>>>;
+struct ThenSplit {
+    dip_tier t;
+    unsigned int *moves;       // the word in which the launch behind says that its moves are known: 0 from here on
+};
+template <int THEN> using ThenArg = std::conditional_t<THEN == THEN_UPDATE, dip_cache_update, std::conditional_t<THEN == THEN_SPLIT, ThenSplit, Int<0>>>;
 
 template <bool CA, bool NORM, int THEN, bool LIST>
 __global__ void __launch_bounds__(TK_THREADS, 1)
@@ -92,6 +96,7 @@ select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, f
                                []() { return true; });
     }
     if constexpr (THEN == THEN_SPLIT) {
+        const dip_tier &tier = then.t;
         // a mask word per warp, a column per lane (d is a multiple of 32 here)
         const int lane = tid & 31, warp = tid >> 5;
         unsigned int *missw = f.hist;
@@ -99,27 +104,30 @@ select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, f
         for (int w0 = warp; w0 < n_words; w0 += U * TK_WARPS) {
             int sl[U];
 #pragma unroll
-            for (int v = 0; v < U; ++v) sl[v] = w0 + v * TK_WARPS < n_words ? then.slot[(w0 + v * TK_WARPS) * 32 + lane] : -1;
+            for (int v = 0; v < U; ++v) sl[v] = w0 + v * TK_WARPS < n_words ? tier.slot[(w0 + v * TK_WARPS) * 32 + lane] : -1;
 #pragma unroll
             for (int v = 0; v < U; ++v) {
                 const int w = w0 + v * TK_WARPS;
                 if (w >= n_words) break;
                 const uint32_t m = s_maskw[w];
-                const bool hit = ((m >> lane) & 1u) && sl[v] >= 0 && sl[v] < then.capacity;   // (a slot outside the arena is none)
+                const bool hit = ((m >> lane) & 1u) && sl[v] >= 0 && sl[v] < tier.capacity;   // (a slot outside the arena is none)
                 const uint32_t hits = __ballot_sync(0xffffffffu, hit);
-                if (hit) then.loc[w * 32 + lane] = sl[v];
+                if (hit) tier.loc[w * 32 + lane] = sl[v];
                 if (lane == 0) {
-                    then.split[w] = hits;
-                    then.split[n_words + w] = missw[w] = m & ~hits;
+                    tier.split[w] = hits;
+                    tier.split[n_words + w] = missw[w] = m & ~hits;
                 }
             }
         }
         __syncthreads();
         const int n = list_mask(missw, d, s, [&](int r, int col) {
-            then.fetch[4 + r] = col;
-            then.loc[col] = then.capacity + r;
+            tier.fetch[4 + r] = col;
+            tier.loc[col] = tier.capacity + r;
         });
-        if (tid == 0) then.fetch[0] = n;
+        if (tid == 0) {
+            tier.fetch[0] = n;
+            *then.moves = 0u;
+        }
     }
     DIP_TRACE_MAX(tr, 2);
 }
@@ -263,7 +271,7 @@ dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, flo
         e = list ? fine(select_fine_kernel<true, false, THEN_UPDATE, true>, *update) : fine(select_fine_kernel<true, false, THEN_UPDATE, false>, *update);
     } else if (split) {
         if (list) return DIP_ERR_INVALID_ARG;
-        e = fine(select_fine_kernel<true, false, THEN_SPLIT, false>, *split);
+        e = fine(select_fine_kernel<true, false, THEN_SPLIT, false>, ThenSplit{*split, ctx->readers + 1});
     } else if (stamp) {
         e = list ? fine(select_fine_kernel<true, false, THEN_NOTHING, true>, no) : fine(select_fine_kernel<true, false, THEN_NOTHING, false>, no);
     } else {
