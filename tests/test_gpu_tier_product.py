@@ -91,3 +91,27 @@ def test_two_tier_products_round_no_more_than_two_products_did():
     assert err_h <= 4 / 3 * 5 * 2.5e-8 and err_y <= 4 / 3 * 10 ** 0.5 * 2.5e-8, (err_h, err_y)
     assert ctx.device_status() == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("wtype,d_model,d_ff,k_x,k_h,beta,ring", [
+    (di.W_INT4_G128, 256, 5120, 200, 900, 0.5, 0),     # rows of two pieces and a half, of one that is not full
+    (di.W_INT4_G128, 640, 2048, 300, 1500, 0.0, 0),    # nothing cached: no row has a slot
+    (di.W_BF16, 1024, 1056, 700, 1000, 0.6, 1),        # more pieces than warps, behind the copy ring
+    (di.W_F32, 64, 4128, 1, 40, 1.0, 1),               # one miss, then hits only
+])
+def test_fetched_rows_reach_their_slots(wtype, d_model, d_ff, k_x, k_h, beta, ring):
+    """Launches that fetch the misses for products that do not read the slow tier themselves."""
+    import paper_2412_01380_b200 as dip
+    ctx = dip.Context(0, gemv_copy_ring=ring)
+    lw = _layer(d_ff, d_model, d_ff, wtype)
+    w = upload_layer(dip, ctx, lw)
+    gate_up, down = w.gate_up.clone(), w.down.clone()
+    g_gu, g_d, t_gu, t_d = _tiers(dip, w, k_x, k_h, beta, "lru", True)
+    ref_gu, ref_d = oracle.Cache(d_model, g_gu.capacity, "lru"), oracle.Cache(d_ff, g_d.capacity, "lru")
+    w.struct.gate_up = w.struct.down = None
+    for x in di.token_inputs(di.WORKLOADS["phi3_mini"].scaled(seed=d_ff + 2), n_tokens=4, batch=1, d=d_model)[:, 0]:
+        check_step(dip, ctx, lw, w, x, k_x, k_h, 0.2, ref_gu, ref_d, g_gu, g_d, tiers=(t_gu, t_d))
+        for t, packed, ref in ((t_gu, gate_up, ref_gu), (t_d, down, ref_d)):
+            _check_tier(t, packed, ref, int(ref.counters[1]))
+    assert ctx.device_status() == 0
+    ctx.close()
