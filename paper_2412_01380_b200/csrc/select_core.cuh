@@ -728,20 +728,21 @@ __device__ __forceinline__ int list_mask(const unsigned int *maskw, int d, TkSha
 }
 
 // The columns of a complete mask in shared memory as an ascending list out[0 .. k).  All threads call it; whoever uses stage next needs no
-// barrier.  stage: an entry of 16 bits per column in shared memory, in which a list of more than TK_LIST_DIRECT columns is made first: the
+// barrier.  LONG: more than TK_LIST_DIRECT columns; the list is made first in stage, an entry of 16 bits per column in shared memory: the
 // threads' runs of up to 32 entries each take as many store instructions, which touch a sector per lane (32768 of 32768 columns 42.2 us,
 // 20.5 like this; 4480 of 17920 9.2 and 8.2).  A short list pays 0.25 us for the detour (1280 of 5120, 1638 of 32768).
 constexpr int TK_LIST_DIRECT = 2048;
+template <bool LONG>
 __device__ __forceinline__ void write_list(const unsigned int *maskw, int d, int k, TkShared &s, uint16_t *stage, int32_t *out)
 {
-    if (k <= TK_LIST_DIRECT) {
+    if constexpr (!LONG) {
         list_mask(maskw, d, s, [&](int r, int col) { out[r] = col; });
-        return;
+    } else {
+        list_mask(maskw, d, s, [&](int r, int col) { stage[r] = (uint16_t)col; });
+        __syncthreads();
+        for (int r = threadIdx.x; r < k; r += TK_THREADS) out[r] = stage[r];
+        __syncthreads();
     }
-    list_mask(maskw, d, s, [&](int r, int col) { stage[r] = (uint16_t)col; });
-    __syncthreads();
-    for (int r = threadIdx.x; r < k; r += TK_THREADS) out[r] = stage[r];
-    __syncthreads();
 }
 
 }  // namespace

@@ -31,7 +31,8 @@ namespace {
 // bytes this CTA has to pull in are its floor: two bytes per column instead of the eight of value +
 // stamp.  Needs d % 8 == 0 and d <= 8 * TK_COARSE_ITERS * TK_THREADS.
 // Dynamic shared memory: TkFine, then keys[] (d words rounded up to four).
-// LIST: the kept columns of row r as an ascending list at idx_out + r * k (launches without one do without that code).
+// LIST: the kept columns of row r as an ascending list at idx_out + r * k, LIST_SHORT straight from the mask, LIST_LONG through shared memory
+// (variants, since code beside it costs a launch that does not use it 0.1 to 0.25 us).
 // THEN (one row): THEN_UPDATE: the CTA goes on to update the row's cache (Algorithm 1 whole).  What bounds dip_ca_mask is the chain of
 // its launches (select, update and list were three), and the mask is here in shared memory: masks with lists and list
 // products at 2080 / 5472, four calls in a graph, 36.7 us with ten launches and 28.8 with four.  (In line the update spills 308 bytes; as a
@@ -40,13 +41,14 @@ namespace {
 // list; their arena rows are the staging rows, in order).
 // ---------------------------------------------------------------------------------------
 constexpr int THEN_NOTHING = 0, THEN_UPDATE = 1, THEN_SPLIT = 2;
+constexpr int LIST_NONE = 0, LIST_SHORT = 1, LIST_LONG = 2;
 struct ThenSplit {
     dip_tier t;
     unsigned int *moves;       // the word in which the launch behind says that its moves are known: 0 from here on
 };
 template <int THEN> using ThenArg = std::conditional_t<THEN == THEN_UPDATE, dip_cache_update, std::conditional_t<THEN == THEN_SPLIT, ThenSplit, Int<0>>>;
 
-template <bool CA, bool NORM, int THEN, bool LIST>
+template <bool CA, bool NORM, int THEN, int LIST>
 __global__ void __launch_bounds__(TK_THREADS, 1)
 select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, float *__restrict__ x_out,
                    int d, int k, float gamma, const int32_t *stamp,
@@ -86,9 +88,9 @@ select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, f
         select_fine<CA, NORM>(xa, NORM ? x_out : nullptr, d, k, gamma, stamp, scale, keys, s, f, s_maskw);
     }
     for (int w = tid; w < n_words; w += TK_THREADS) mask_bits[w] = s_maskw[w];
-    if constexpr (LIST) {
+    if constexpr (LIST != LIST_NONE) {
         static_assert(sizeof(f.hist) >= sizeof(uint16_t) * DIP_MAX_D, "the list fits where the histogram was");
-        write_list(s_maskw, d, k, s, reinterpret_cast<uint16_t *>(f.hist), idx_out + (size_t)row * k);
+        write_list<LIST == LIST_LONG>(s_maskw, d, k, s, reinterpret_cast<uint16_t *>(f.hist), idx_out + (size_t)row * k);
     }
     if constexpr (THEN == THEN_UPDATE) {
         cache_update_clear(s, f.hist);
@@ -132,7 +134,7 @@ select_fine_kernel(const float *__restrict__ xa, const float *__restrict__ xb, f
     DIP_TRACE_MAX(tr, 2);
 }
 
-template <bool CA, bool LIST>
+template <bool CA, int LIST>
 __global__ void __launch_bounds__(TK_THREADS, 1)
 select_fine_coarse_kernel(const float *__restrict__ x, const uint16_t *__restrict__ coarse, int d, int k, float gamma,
                           const int32_t *__restrict__ stamp, uint32_t *__restrict__ mask_bits, int32_t *__restrict__ idx_out,
@@ -157,7 +159,7 @@ select_fine_coarse_kernel(const float *__restrict__ x, const uint16_t *__restric
     __syncthreads();                                                  // histogram zeroed
     select_fine_coarse<CA>(coarse, x, stamp, gamma, d, k, keys, s, f, s_maskw);
     for (int w = tid; w < (d >> 5); w += TK_THREADS) mask_bits[w] = s_maskw[w];
-    if constexpr (LIST) write_list(s_maskw, d, k, s, reinterpret_cast<uint16_t *>(f.hist), idx_out + (size_t)row * k);
+    if constexpr (LIST != LIST_NONE) write_list<LIST == LIST_LONG>(s_maskw, d, k, s, reinterpret_cast<uint16_t *>(f.hist), idx_out + (size_t)row * k);
     DIP_TRACE_MAX(tr, 2);
 }
 
@@ -248,34 +250,42 @@ dip_status dip_launch_select(dip_ctx *ctx, const float *xa, const float *xb, flo
     if ((update || split) && (coarse || xb)) return DIP_ERR_INVALID_ARG;
     if (idx_out && xb) return DIP_ERR_INVALID_ARG;
     if ((update || split) && (batch != 1 || !stamp)) return DIP_ERR_INVALID_ARG;
-    const bool list = idx_out != nullptr;
+    const int list = !idx_out ? LIST_NONE : k <= TK_LIST_DIRECT ? LIST_SHORT : LIST_LONG;
     const Int<0> no;
     const size_t smem = sizeof(TkFine) + (size_t)((d + 3) & ~3) * sizeof(uint32_t);
     const dim3 grid(batch), block(TK_THREADS);
     unsigned long long *tr = dip_trace_slot(ctx, d <= 0 ? 0 : (stamp ? 2 : 1));
     cudaError_t e;
     if (!stamp) gamma = 1.0f;
-    const auto fine = [&](auto *kernel, const auto &then) {
-        return dip_launch_pdl(kernel, grid, block, smem, stream, xa, xb, x_out, d, k, gamma, stamp, mask_bits, idx_out, then, tr);
+    // (a variant per kind of list)
+    const auto fine = [&](auto *none, auto *direct, auto *staged, const auto &then) {
+        return dip_launch_pdl(list == LIST_NONE ? none : list == LIST_SHORT ? direct : staged, grid, block, smem, stream, xa, xb, x_out, d, k,
+                              gamma, stamp, mask_bits, idx_out, then, tr);
     };
-    const auto fine_coarse = [&](auto *kernel) {
-        return dip_launch_pdl(kernel, grid, block, smem, stream, xa, coarse, d, k, gamma, stamp, mask_bits, idx_out, tr);
+    const auto fine_coarse = [&](auto *none, auto *direct, auto *staged) {
+        return dip_launch_pdl(list == LIST_NONE ? none : list == LIST_SHORT ? direct : staged, grid, block, smem, stream, xa, coarse, d, k,
+                              gamma, stamp, mask_bits, idx_out, tr);
     };
     if (coarse) {
         if (xb || (batch != 1 && stamp) || (d & 31)) return DIP_ERR_INVALID_ARG;
-        if (stamp) e = list ? fine_coarse(select_fine_coarse_kernel<true, true>) : fine_coarse(select_fine_coarse_kernel<true, false>);
-        else e = list ? fine_coarse(select_fine_coarse_kernel<false, true>) : fine_coarse(select_fine_coarse_kernel<false, false>);
+        e = stamp ? fine_coarse(select_fine_coarse_kernel<true, 0>, select_fine_coarse_kernel<true, 1>, select_fine_coarse_kernel<true, 2>)
+                  : fine_coarse(select_fine_coarse_kernel<false, 0>, select_fine_coarse_kernel<false, 1>, select_fine_coarse_kernel<false, 2>);
     } else if (xb) {
-        e = stamp ? fine(select_fine_kernel<true, true, THEN_NOTHING, false>, no) : fine(select_fine_kernel<false, true, THEN_NOTHING, false>, no);
+        const auto one = [&](auto *kernel) { return fine(kernel, kernel, kernel, no); };
+        e = stamp ? one(select_fine_kernel<true, true, THEN_NOTHING, 0>) : one(select_fine_kernel<false, true, THEN_NOTHING, 0>);
     } else if (update) {
-        e = list ? fine(select_fine_kernel<true, false, THEN_UPDATE, true>, *update) : fine(select_fine_kernel<true, false, THEN_UPDATE, false>, *update);
+        e = fine(select_fine_kernel<true, false, THEN_UPDATE, 0>, select_fine_kernel<true, false, THEN_UPDATE, 1>,
+                 select_fine_kernel<true, false, THEN_UPDATE, 2>, *update);
     } else if (split) {
-        if (list) return DIP_ERR_INVALID_ARG;
-        e = fine(select_fine_kernel<true, false, THEN_SPLIT, false>, ThenSplit{*split, ctx->readers + 1});
+        if (idx_out) return DIP_ERR_INVALID_ARG;
+        const auto one = [&](auto *kernel) { return fine(kernel, kernel, kernel, ThenSplit{*split, ctx->readers + 1}); };
+        e = one(select_fine_kernel<true, false, THEN_SPLIT, 0>);
     } else if (stamp) {
-        e = list ? fine(select_fine_kernel<true, false, THEN_NOTHING, true>, no) : fine(select_fine_kernel<true, false, THEN_NOTHING, false>, no);
+        e = fine(select_fine_kernel<true, false, THEN_NOTHING, 0>, select_fine_kernel<true, false, THEN_NOTHING, 1>,
+                 select_fine_kernel<true, false, THEN_NOTHING, 2>, no);
     } else {
-        e = list ? fine(select_fine_kernel<false, false, THEN_NOTHING, true>, no) : fine(select_fine_kernel<false, false, THEN_NOTHING, false>, no);
+        e = fine(select_fine_kernel<false, false, THEN_NOTHING, 0>, select_fine_kernel<false, false, THEN_NOTHING, 1>,
+                 select_fine_kernel<false, false, THEN_NOTHING, 2>, no);
     }
     DIP_CUDA_TRY(ctx, e);
     return DIP_OK;
@@ -293,20 +303,17 @@ dip_status dip_init_mask_kernels(dip_ctx *ctx)
 {
     const int bytes = DIP_MAX_D * (int)sizeof(uint32_t);
     const int fine_bytes = bytes + (int)sizeof(TkFine);
-    const auto raise = [&](auto *kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes); };
-    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, false, THEN_UPDATE, false>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, false, THEN_UPDATE, true>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, false, THEN_SPLIT, false>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, false, THEN_NOTHING, false>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, false, THEN_NOTHING, true>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<false, false, THEN_NOTHING, false>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<false, false, THEN_NOTHING, true>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<true, true, THEN_NOTHING, false>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_kernel<false, true, THEN_NOTHING, false>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_coarse_kernel<true, false>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_coarse_kernel<true, true>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_coarse_kernel<false, false>));
-    DIP_CUDA_TRY(ctx, raise(select_fine_coarse_kernel<false, true>));
+    cudaError_t e = cudaSuccess;
+    const auto raise = [&](auto *...kernels) {
+        ((e = e == cudaSuccess ? cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, fine_bytes) : e), ...);
+    };
+    raise(select_fine_kernel<true, false, THEN_UPDATE, 0>, select_fine_kernel<true, false, THEN_UPDATE, 1>, select_fine_kernel<true, false, THEN_UPDATE, 2>,
+          select_fine_kernel<true, false, THEN_SPLIT, 0>, select_fine_kernel<true, true, THEN_NOTHING, 0>, select_fine_kernel<false, true, THEN_NOTHING, 0>,
+          select_fine_kernel<true, false, THEN_NOTHING, 0>, select_fine_kernel<true, false, THEN_NOTHING, 1>, select_fine_kernel<true, false, THEN_NOTHING, 2>,
+          select_fine_kernel<false, false, THEN_NOTHING, 0>, select_fine_kernel<false, false, THEN_NOTHING, 1>, select_fine_kernel<false, false, THEN_NOTHING, 2>,
+          select_fine_coarse_kernel<true, 0>, select_fine_coarse_kernel<true, 1>, select_fine_coarse_kernel<true, 2>,
+          select_fine_coarse_kernel<false, 0>, select_fine_coarse_kernel<false, 1>, select_fine_coarse_kernel<false, 2>);
+    DIP_CUDA_TRY(ctx, e);
     return DIP_OK;
 }
 
