@@ -9,7 +9,7 @@
 // keeps, each block moves its pieces of them.  What bounds a step is the slow tier's rate and a chain of launches: with launches
 // for split, list, fetch, update, slots, moves, hits, misses and sums on three streams, a step of 3072 / 8192 (BF16, keep ratio
 // 0.25, budget 0.5, tokens correlated by 0.95) took 72 us, of which the host needed all and the device 43; two launches
-// per input take 33 (host 20.5, device 30.5).
+// per input take 31 (host 20.5, device 28.5).
 // Products that cannot read the slow tier themselves (4-bit weights, whose kernel has no room for a block of 1024 threads
 // beside it; the copy ring) run beside tier_fetch_kernel and once more over the misses.
 #include "cache_update.cuh"
