@@ -12,7 +12,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("d_model,d_ff,batches", [(256, 8224, (3, 5, 16)), (1056, 2080, tuple(range(3, 17))), (288, 19008, (4, 9)), (288, 6176, (5, 6, 8))])
+@pytest.mark.parametrize("d_model,d_ff,batches", [(256, 8224, (3, 5, 16)), (1056, 2080, tuple(range(3, 17))), (288, 19008, (4, 9))])
 def test_batched_products_from_masks(d_model, d_ff, batches):
     import paper_2412_01380_b200 as dip
     ctx = dip.Context(0)
@@ -36,6 +36,11 @@ def test_batched_products_from_masks(d_model, d_ff, batches):
                     assert rel_err(out[b].cpu().numpy(), want) <= REL_TOL, (batch, which, k, b)
     assert ctx.device_status() == 0
     ctx.close()
+
+
+def test_batched_products_around_the_parts_that_are_added_up_apart():
+    """Two segments in 1 to 74 parts, collected by one block or, from 16 parts and 96 KB on, by a launch behind."""
+    test_batched_products_from_masks(288, 6176, (5, 6, 8))
 
 
 def _product(dip, d_model, d_ff, which, batch, k, **options):
